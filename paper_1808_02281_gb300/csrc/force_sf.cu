@@ -49,413 +49,11 @@
 #include <atomic>
 #include <mutex>
 
-#include "kernels.h"
-#include "su3.cuh"
+#include "sf_common.cuh"
 
 namespace lqcd {
 
 namespace {
-
-constexpr int kBlock = 128; // four warps: the four directions of 32 sites
-
-__host__ __device__ __forceinline__ int64_t padded_sites(int64_t V) { return (V + 31) & ~(int64_t)31; }
-__host__ __device__ __forceinline__ int64_t virtual_blocks(int64_t V) { return padded_sites(V) / 32; }
-
-enum { SC_BETA6 = 0, SC_CPL, SC_CRT, SC_CCB, SC_ACT, SC_ACTPL, SC_DT };
-
-template <typename R> __device__ __forceinline__ R scalar(const KernelScalars &s, int i)
-{
-    if constexpr (sizeof(R) == 4) return s.f[i];
-    else return s.d[i];
-}
-
-// Storage of the 24 staple planes: compact (rows 0 and 1, 12 reals, the
-// third row rebuilt on load) or full (all 18 reals, nothing rebuilt).  Both
-// are cut into blocks of 32 consecutive sites: inside a block, 16-byte lane
-// q (q < NW = 12/W compact, 18/W full) of the staple of site s is at
-// q*512 + s*16 bytes, and for full FP32 staples the last two reals at
-// NW*512 + s*8 -- 72 bytes per full staple in FP32, 144 in FP64, every
-// access 16- or 8-byte aligned, and the lanes of one staple a constant 512
-// bytes apart, so that a staple costs one address computation (plus one for
-// the FP32 tail) however many lanes it has.  Plane P starts at
-// P * plane_bytes, plane_bytes = the
-// 32-site blocks of the lattice (V rounded up to 32) times the block size.
-// Pass A writes them with evict-first stores: the 3.6 GB (at 32^3x64) would
-// otherwise push the links that pass A re-reads out of L2.
-constexpr int kStaplePlanes = 24;
-
-template <typename R> struct FullBlock {
-    using V4 = typename Vec<R>::type;
-    static constexpr int W = Vec<R>::W;
-    static constexpr int NW = 18 / W;        // whole 16-byte lanes per staple
-    static constexpr int TAIL = 18 - NW * W; // reals in the FP32 tail (2)
-    static constexpr int LANE = 32 * 16;     // bytes of one lane of a block
-    static constexpr int BYTES = NW * LANE + TAIL * (int)sizeof(R) * 32;
-    static_assert(NW * W + TAIL == 18, "a full staple holds 18 reals");
-};
-
-size_t full_plane_bytes(int64_t V, int precision)
-{
-    const size_t blk = precision == LQCD_F64 ? FullBlock<double>::BYTES : FullBlock<float>::BYTES;
-    return (size_t)((V + 31) / 32) * blk;
-}
-
-// Compact planes: the first two rows (12 reals) of every staple, the third
-// rebuilt on load, in the same 32-site blocks (lane q, q < 12/W, of site s at
-// q*512 + s*16).
-template <typename R> struct CompactBlock {
-    using V4 = typename Vec<R>::type;
-    static constexpr int W = Vec<R>::W;
-    static constexpr int NW = 12 / W;
-    static constexpr int LANE = 32 * 16;
-    static constexpr int BYTES = NW * LANE;
-};
-
-template <typename R, bool FULL> struct Planes;
-
-template <typename R> struct Planes<R, false> {
-    using B = CompactBlock<R>;
-    using V4 = typename B::V4;
-    char *base;
-    int64_t plane_bytes;
-    using Ref = char *;
-
-    __device__ __forceinline__ Ref at(int n) const
-    {
-        return base + (int64_t)(n >> 5) * B::BYTES + (n & 31) * 16;
-    }
-
-    __device__ __forceinline__ Mat<R> load(Ref r, int plane) const
-    {
-        const V4 *p = reinterpret_cast<const V4 *>(r + (int64_t)plane * plane_bytes);
-        R x[12];
-#pragma unroll
-        for (int q = 0; q < B::NW; ++q) {
-            const V4 v = __ldg(p + q * (B::LANE / 16));
-            if constexpr (B::W == 4) {
-                x[4 * q + 0] = v.x;
-                x[4 * q + 1] = v.y;
-                x[4 * q + 2] = v.z;
-                x[4 * q + 3] = v.w;
-            } else {
-                x[2 * q + 0] = v.x;
-                x[2 * q + 1] = v.y;
-            }
-        }
-        Mat<R> u;
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                u.re[i][j] = x[6 * i + 2 * j];
-                u.im[i][j] = x[6 * i + 2 * j + 1];
-            }
-        rebuild_row2(u);
-        return u;
-    }
-
-    __device__ __forceinline__ void store(Ref r, int plane, const Mat<R> &u) const
-    {
-        V4 *p = reinterpret_cast<V4 *>(r + (int64_t)plane * plane_bytes);
-        R x[12];
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                x[6 * i + 2 * j] = u.re[i][j];
-                x[6 * i + 2 * j + 1] = u.im[i][j];
-            }
-#pragma unroll
-        for (int q = 0; q < B::NW; ++q) {
-            V4 v;
-            if constexpr (B::W == 4) v = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-            else v = make_double2(x[2 * q], x[2 * q + 1]);
-            __stcs(p + q * (B::LANE / 16), v);
-        }
-    }
-};
-
-template <typename R> struct Planes<R, true> {
-    using B = FullBlock<R>;
-    using V4 = typename B::V4;
-    char *base;          // plane 0
-    int64_t plane_bytes;
-
-    // The lane-0 and tail addresses of site n in plane 0.
-    struct Ref {
-        char *p;
-        char *t;
-    };
-
-    __device__ __forceinline__ Ref at(int n) const
-    {
-        char *b = base + (int64_t)(n >> 5) * B::BYTES;
-        const int s = n & 31;
-        return Ref{b + s * 16, b + B::NW * B::LANE + s * 8};
-    }
-
-    __device__ __forceinline__ Mat<R> load(const Ref &r, int plane) const
-    {
-        const int64_t off = (int64_t)plane * plane_bytes;
-        const V4 *p = reinterpret_cast<const V4 *>(r.p + off);
-        R x[18];
-#pragma unroll
-        for (int q = 0; q < B::NW; ++q) {
-            const V4 v = __ldg(p + q * (B::LANE / 16));
-            if constexpr (B::W == 4) {
-                x[4 * q + 0] = v.x;
-                x[4 * q + 1] = v.y;
-                x[4 * q + 2] = v.z;
-                x[4 * q + 3] = v.w;
-            } else {
-                x[2 * q + 0] = v.x;
-                x[2 * q + 1] = v.y;
-            }
-        }
-        if constexpr (B::TAIL == 2) {
-            const float2 t = __ldg(reinterpret_cast<const float2 *>(r.t + off));
-            x[16] = t.x;
-            x[17] = t.y;
-        }
-        Mat<R> u;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                u.re[i][j] = x[2 * (3 * i + j)];
-                u.im[i][j] = x[2 * (3 * i + j) + 1];
-            }
-        return u;
-    }
-
-    __device__ __forceinline__ void store(const Ref &r, int plane, const Mat<R> &u) const
-    {
-        const int64_t off = (int64_t)plane * plane_bytes;
-        V4 *p = reinterpret_cast<V4 *>(r.p + off);
-        R x[18];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                x[2 * (3 * i + j)] = u.re[i][j];
-                x[2 * (3 * i + j) + 1] = u.im[i][j];
-            }
-#pragma unroll
-        for (int q = 0; q < B::NW; ++q) {
-            V4 v;
-            if constexpr (B::W == 4) v = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-            else v = make_double2(x[2 * q], x[2 * q + 1]);
-            __stcs(p + q * (B::LANE / 16), v);
-        }
-        if constexpr (B::TAIL == 2) __stcs(reinterpret_cast<float2 *>(r.t + off), make_float2(x[16], x[17]));
-    }
-};
-
-template <typename R, bool FULL> __device__ __forceinline__ Planes<R, FULL> planes_of(const SfLattice &L)
-{
-    if constexpr (FULL) {
-        return Planes<R, true>{static_cast<char *>(L.staples), L.plane_bytes};
-    } else {
-        const int64_t V = (int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3];
-        return Planes<R, false>{static_cast<char *>(L.staples),
-                                ((V + 31) / 32) * CompactBlock<R>::BYTES};
-    }
-}
-
-// Lattice geometry in 32-bit arithmetic: the staple-field algorithm runs only
-// for V < 2^31 sites (its workspace, 1728 bytes a site in FP32, could not
-// hold more), so site indices and neighbour offsets fit an int.
-struct G32 {
-    int L0, L1, L2, L3;
-    int s1, s2, s3, V;
-};
-
-__device__ __forceinline__ G32 make_g32(const int dims[4])
-{
-    G32 g;
-    g.L0 = dims[0];
-    g.L1 = dims[1];
-    g.L2 = dims[2];
-    g.L3 = dims[3];
-    g.s1 = dims[0];
-    g.s2 = g.s1 * dims[1];
-    g.s3 = g.s2 * dims[2];
-    g.V = g.s3 * dims[3];
-    return g;
-}
-
-// Slots of SfLattice::div (the magic of each run-time divisor).
-enum { DV_S1, DV_S2, DV_S3, DV_VOL, DV_SLICE, DV_MVOL, DV_MX, DV_MY, DV_NMX, DV_NMY, DV_NBX, DV_NBY };
-
-__device__ __forceinline__ int divi(int n, const DivMagic &d) { return (int)div_by((unsigned)n, d); }
-
-// Coordinates of site n (the divisions by the strides as multiply-highs).
-__device__ __forceinline__ Coord coord32(const G32 &g, const DivMagic *dm, int n)
-{
-    Coord x;
-    x.c3 = divi(n, dm[DV_S3]);
-    int r = n - x.c3 * g.s3;
-    x.c2 = divi(r, dm[DV_S2]);
-    r -= x.c2 * g.s2;
-    x.c1 = divi(r, dm[DV_S1]);
-    x.c0 = r - x.c1 * g.s1;
-    return x;
-}
-
-__device__ __forceinline__ int index32(const G32 &g, const Coord &x)
-{
-    return x.c0 + g.s1 * x.c1 + g.s2 * x.c2 + g.s3 * x.c3;
-}
-
-// Index offset of the step s * hat(mu) (s = +-1) from a site with
-// coordinates x, periodic (the direction picked by a select chain, so that
-// nothing is indexed at run time in per-thread storage).
-__device__ __forceinline__ int step32(const G32 &g, const Coord &x, int mu, int s)
-{
-    const int L = pick(mu, g.L0, g.L1, g.L2, g.L3);
-    const int c = pick(mu, x.c0, x.c1, x.c2, x.c3);
-    const int st = pick(mu, 1, g.s1, g.s2, g.s3);
-    if (s > 0) return c + 1 == L ? (1 - L) * st : st;
-    return c == 0 ? (L - 1) * st : -st;
-}
-
-// Traversal order of pass B: the lattice is cut into spatial blocks of
-// bx x by x bz sites that run over all t; blocks one after the other, inside
-// a block t-slice by t-slice, inside a slice micro-tiles of mx x my x mz
-// sites (x fastest within and between micro-tiles).  The staple planes of
-// three neighbouring t-slices of one block then stay in L2 while the block
-// is swept, and micro-tiles make y and z neighbours L1 hits.
-struct Sweep {
-    int bx, by, bz, mx, my, mz;
-    int nbx, nby, nmx, nmy, mvol;
-    int slice, vol;     // sites per block slice and per block
-    const DivMagic *dm; // magic of vol, slice, mvol, mx, my, nmx, nmy, nbx, nby
-};
-
-__device__ __forceinline__ Sweep make_sweep(const SfLattice &L, const G32 &g)
-{
-    Sweep s;
-    s.bx = L.sweep[0];
-    s.by = L.sweep[1];
-    s.bz = L.sweep[2];
-    s.mx = L.micro[0];
-    s.my = L.micro[1];
-    s.mz = L.micro[2];
-    s.nbx = L.counts[0];
-    s.nby = L.counts[1];
-    s.nmx = L.counts[2];
-    s.nmy = L.counts[3];
-    s.mvol = s.mx * s.my * s.mz;
-    s.slice = s.bx * s.by * s.bz;
-    s.vol = s.slice * g.L3;
-    s.dm = L.div;
-    return s;
-}
-
-__device__ __forceinline__ Coord swept_site(const Sweep &s, int j)
-{
-    const DivMagic *dm = s.dm;
-    const int blk = divi(j, dm[DV_VOL]);
-    const int r = j - blk * s.vol;
-    Coord c;
-    c.c3 = divi(r, dm[DV_SLICE]);
-    const int r2 = r - c.c3 * s.slice;
-    const int mt = divi(r2, dm[DV_MVOL]), w = r2 - mt * s.mvol;
-    const int wq = divi(w, dm[DV_MX]), xin = w - wq * s.mx;
-    const int zin = divi(wq, dm[DV_MY]), yin = wq - zin * s.my;
-    const int mq = divi(mt, dm[DV_NMX]), mxi = mt - mq * s.nmx;
-    const int mzi = divi(mq, dm[DV_NMY]), myi = mq - mzi * s.nmy;
-    const int q = divi(blk, dm[DV_NBX]), bxi = blk - q * s.nbx;
-    const int bzi = divi(q, dm[DV_NBY]), byi = q - bzi * s.nby;
-    c.c0 = bxi * s.bx + mxi * s.mx + xin;
-    c.c1 = byi * s.by + myi * s.my + yin;
-    c.c2 = bzi * s.bz + mzi * s.mz + zin;
-    return c;
-}
-
-// Sum over the block of one double per thread (result in thread 0); the
-// trailing barrier lets the caller run it again in the next virtual block.
-__device__ __forceinline__ double block_sum(double v)
-{
-    __shared__ double part[kBlock / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) part[warp] = v;
-    __syncthreads();
-    double s = 0.0;
-    if (warp == 0) {
-        s = lane < kBlock / 32 ? part[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    }
-    __syncthreads();
-    return s;
-}
-
-// block_sum over the four warps of row group `row` of a CTA of ROWS groups
-// (named barrier 1 + row over its 128 threads; same order of summation).
-template <int ROWS> __device__ __forceinline__ double group_sum(double v, int row)
-{
-    if constexpr (ROWS == 1) {
-        return block_sum(v);
-    } else {
-        __shared__ double part[ROWS * kBlock / 32];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        if (lane == 0) part[warp] = v;
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + row), "r"(kBlock) : "memory");
-        double s = 0.0;
-        if ((warp & 3) == 0) {
-            s = lane < kBlock / 32 ? part[warp + lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        }
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + row), "r"(kBlock) : "memory");
-        return s;
-    }
-}
-
-// Next virtual block for a persistent CTA of a batched launch, taken from a
-// work counter: the blocks in flight stay a contiguous window of the sweep
-// (as with hardware block scheduling), which keeps the L2 reuse of the
-// traversal; a fixed stride per CTA would let the window spread out.
-__device__ __forceinline__ int64_t next_virtual_block(unsigned long long *counter)
-{
-    __shared__ unsigned long long s_vb;
-    if (threadIdx.x == 0) s_vb = atomicAdd(counter, 1ull);
-    __syncthreads();
-    const int64_t vb = (int64_t)s_vb;
-    __syncthreads();
-    return vb;
-}
-
-// The same queue with the next block claimed (by thread 0) when the current
-// one starts and handed to the block when it ends, so that the atomic's
-// latency overlaps the current block's work.
-__device__ __forceinline__ unsigned long long claim_virtual_block(unsigned long long *counter)
-{
-    return threadIdx.x == 0 ? atomicAdd(counter, 1ull) : 0ull;
-}
-
-__device__ __forceinline__ int64_t publish_virtual_block(unsigned long long claimed)
-{
-    __shared__ unsigned long long s_vb;
-    if (threadIdx.x == 0) s_vb = claimed;
-    __syncthreads();
-    const int64_t vb = (int64_t)s_vb;
-    __syncthreads();
-    return vb;
-}
-
-// Lattice of a batch that virtual block vb (global numbering) belongs to.
-__device__ __forceinline__ int batch_entry(const SfBatch &B, int64_t vb)
-{
-    int c = 0;
-    while (c + 1 < B.n && vb >= B.e[c + 1].vb_begin) ++c;
-    return c;
-}
 
 // ---------------------------------------------------------------- pass A
 
@@ -521,145 +119,10 @@ __global__ void __launch_bounds__(kBlock) staple_fields_batched(const __grid_con
 
 // ---------------------------------------------------------------- pass B
 
-// Products of two SU(3) factors are accumulated as y += s * (a * op(b)) with
-// the third row of the product rebuilt from its first two (mul_acc_su3: the
-// third row of a is never rebuilt or loaded), or (DIRECT, full FP64 staples)
-// as plain products accumulated in full, the sum scaled once: for FP64 that
-// measured faster (114 vs 122 ms at 32^3x64: at the 255-register limit the
-// extra temporaries spill); for FP32 the rebuilt form is faster (3.65 vs
-// 3.75 ms).
-template <int FB, bool DIRECT, typename R>
-__device__ __forceinline__ void acc_su3(Mat<R> &y, const Mat<R> &a, const Mat<R> &b, R s)
-{
-    if constexpr (DIRECT) mul_acc<N, FB>(y, a, b); // s applied by the caller
-    else mul_acc_su3<FB>(y, a, b, s);
-}
-
-// Where the staples of a site and of its neighbours are stored: in the
-// lattice-wide staple field, the site index itself.
-struct LatticeSites {
-    const G32 *g;
-    const Coord *c;
-    int k;
-    __device__ __forceinline__ int at0() const { return k; }
-    __device__ __forceinline__ int nb(int mu, int s) const { return k + step32(*g, *c, mu, s); }
-};
-
-// The staples that start with link(k+rho, d), d = +-nu_d (NEG: minus):
-//   t += B_d [ c_cube sum_{b perp rho, d} S_b(k+d) S^{(d)}_b(k) + c_rect S_d(k+d) A_d^dag ]
-// (the orientation of the shared links fixed at compile time, so that each
-// sign has one small loop body).
-template <bool NEG, bool UNROLLQ, bool FULL, bool DIRECT, typename R, typename SI>
-__device__ __forceinline__ void d_terms(Mat<R> &t, const R *__restrict__ links,
-                                        const Planes<R, FULL> &sf, const SI &si, const G32 &g,
-                                        const Coord &c, int rho, int k, int kp, int id, R c_rt,
-                                        R c_cb)
-{
-    constexpr int FD = NEG ? D : N;
-    const int64_t V = g.V;
-    const int base = rho * 6;
-    const int jd = 2 * id + (NEG ? 1 : 0);
-    const int nud = (rho + 1 + id) & 3;
-    const int kd = k + step32(g, c, nud, NEG ? -1 : 1); // k + d
-    // S^{(d)}_b(k): plane nud*6 + j' at k, or (NEG) its dagger at k - nud = kd
-    const auto at_d = sf.at(si.nb(nud, NEG ? -1 : 1));
-    const auto at_2 = NEG ? at_d : sf.at(si.at0());
-    Mat<R> y;
-    set_zero(y);
-    // the four signed b perpendicular to rho and d: two directions, two signs
-#pragma unroll(UNROLLQ ? 2 : 1)
-    for (int q = 0; q < 2; ++q) {
-        const int ib = q == 0 ? (id == 0 ? 1 : 0) : (id == 2 ? 1 : 2);
-        const int nub = (rho + 1 + ib) & 3;
-        const int jp = 2 * ((nub - nud - 1) & 3);
-        acc_su3<FD, DIRECT>(y, sf.load(at_d, base + 2 * ib),
-                            sf.load(at_2, nud * 6 + jp), c_cb);
-        acc_su3<FD, DIRECT>(y, sf.load(at_d, base + 2 * ib + 1),
-                            sf.load(at_2, nud * 6 + jp + 1), c_cb);
-    }
-    Mat<R> r3 = sf.load(at_d, base + jd);
-    if constexpr (DIRECT) {
-        scale(y, c_cb);
-        scale(r3, c_rt);
-    }
-    if constexpr (!NEG) {
-        acc_su3<D, DIRECT>(y, r3, load_link(links, V, nud, k), c_rt); // A_d = U_nud(k)
-        mul_acc<N, N>(t, load_link(links, V, nud, kp), y);         // B_d = U_nud(k+rho)
-    } else {
-        acc_su3<N, DIRECT>(y, r3, load_link(links, V, nud, kd), c_rt);  // A_d = U_nud(k-nud)^dag
-        mul_acc<D, N>(t, load_link(links, V, nud, kp + (kd - k)), y);  // B_d = U_nud(k+rho-nud)^dag
-    }
-}
-
-// Force (and the fused momentum step) on the link (k, rho), k at coordinates
-// c, its staples found through si; returns its share of the action.
-template <typename R, bool ACTION, bool UNROLLQ, bool FULL, bool DIRECT, typename SI>
-__device__ __forceinline__ double force_link(const SfLattice &L, const KernelScalars &sc, const G32 &g,
-                                             const Planes<R, FULL> &sf, const SI &si, const Coord &c,
-                                             int k, int rho)
-{
-    const R *__restrict__ links = static_cast<const R *>(L.links);
-    const int64_t V = g.V;
-    const R c_pl = scalar<R>(sc, SC_CPL), c_rt = scalar<R>(sc, SC_CRT), c_cb = scalar<R>(sc, SC_CCB);
-    const int kp = k + step32(g, c, rho, 1), km = k + step32(g, c, rho, -1);
-    const int base = rho * 6;
-
-    // plaquettes and the two rectangle chains along rho
-    Mat<R> t;
-    R tr_pl = R(0);
-    {
-        Mat<R> pl, p1, p2;
-        set_zero(pl);
-        set_zero(p1);
-        set_zero(p2);
-        const auto at_k = sf.at(si.at0()), at_p = sf.at(si.nb(rho, 1)), at_m = sf.at(si.nb(rho, -1));
-#pragma unroll 1
-        for (int jj = 0; jj < 6; ++jj) {
-            const Mat<R> s = sf.load(at_k, base + jj);
-            add_to(pl, s);
-            acc_su3<N, DIRECT>(p1, sf.load(at_p, base + jj), s, c_rt);
-            mul_acc<N, N>(p2, s, sf.load(at_m, base + jj));
-        }
-        if constexpr (ACTION) tr_pl = re_trace_mul<N, N>(load_link(links, V, rho, k), pl);
-        t = pl;
-        scale(t, c_pl);
-        if constexpr (DIRECT) scale(p1, c_rt);
-        mul_acc<N, N>(t, load_link(links, V, rho, kp), p1);
-        scale(p2, c_rt);
-        mul_acc<N, N>(t, p2, load_link(links, V, rho, km));
-    }
-    // cubes and the rectangles along d: positive, then negative d
-#pragma unroll 1
-    for (int id = 0; id < 3; ++id)
-        d_terms<false, UNROLLQ, FULL, DIRECT>(t, links, sf, si, g, c, rho, k, kp, id, c_rt, c_cb);
-#pragma unroll 1
-    for (int id = 0; id < 3; ++id)
-        d_terms<true, UNROLLQ, FULL, DIRECT>(t, links, sf, si, g, c, rho, k, kp, id, c_rt, c_cb);
-
-    const Mat<R> m = mul<N, N>(load_link(links, V, rho, k), t);
-    R f[8];
-    ta_components(m, scalar<R>(sc, SC_BETA6), f);
-    if (L.force != nullptr) store_algebra(static_cast<R *>(L.force), V, rho, k, f);
-    if (L.mom != nullptr) {
-        R *mom = static_cast<R *>(L.mom);
-        R p[8];
-        load_algebra(mom, V, rho, k, p);
-        const R dt = scalar<R>(sc, SC_DT);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) p[q] = fma(dt, f[q], p[q]);
-        store_algebra(mom, V, rho, k, p);
-    }
-    if constexpr (ACTION) {
-        const R tr_t = m.re[0][0] + m.re[1][1] + m.re[2][2];
-        return (double)(scalar<R>(sc, SC_ACT) - tr_t * R(1.0 / 6.0) - scalar<R>(sc, SC_ACTPL) * tr_pl);
-    }
-    return 0.0;
-}
-
 // Force (and the fused momentum step) on the 128 links of virtual block vb
 // of the sweep; returns the thread's share of the action (0 for a padding
 // site).
-template <typename R, bool ACTION, bool UNROLLQ, bool FULL, bool DIRECT>
+template <typename R, bool ACTION, bool UNROLLQ, bool FULL>
 __device__ __forceinline__ double force_block(const SfLattice &L, const KernelScalars &sc,
                                               const G32 &g, const Sweep &sw, int vb)
 {
@@ -669,27 +132,19 @@ __device__ __forceinline__ double force_block(const SfLattice &L, const KernelSc
     const Coord c = swept_site(sw, j);
     const int k = index32(g, c);
     const LatticeSites si{&g, &c, k};
-    return force_link<R, ACTION, UNROLLQ, FULL, DIRECT>(L, sc, g, planes_of<R, FULL>(L), si, c, k,
-                                                        rho);
+    return force_link<R, ACTION, UNROLLQ, false>(L, sc, g, planes_of<R, FULL>(L), si, c, k, rho);
 }
 
 // Resident CTAs per SM the register allocation aims at: 4 (128 registers)
 // unless the fused action asks for more registers (3) -- or DENSE forces 4.
-template <typename R, bool ACTION, bool DENSE> constexpr int min_blocks()
-{
-    return sizeof(R) == 8 ? 2 : ((ACTION && !DENSE) ? 3 : 4);
-}
-
-// DIRECT products by default for full FP64 planes (see acc_su3).
-template <typename R, bool FULL> constexpr bool direct_default() { return FULL && sizeof(R) == 8; }
+template <bool ACTION, bool DENSE> constexpr int min_blocks() { return (ACTION && !DENSE) ? 3 : 4; }
 
 // ROWS > 1: a CTA of ROWS groups of four warps on consecutive virtual
 // blocks (y-neighbouring x rows of the sweep), so that the staples of a
 // row's +-y neighbours are the own-row staples of another group of the CTA.
-template <typename R, bool ACTION, bool UNROLLQ, bool DENSE = false, bool FULL = false,
-          bool DIRECT = direct_default<R, FULL>(), int ROWS = 1>
-__global__ void __launch_bounds__(ROWS * kBlock, (min_blocks<R, ACTION, DENSE>() / ROWS > 0
-                                                       ? min_blocks<R, ACTION, DENSE>() / ROWS
+template <typename R, bool ACTION, bool UNROLLQ, bool DENSE = false, bool FULL = false, int ROWS = 1>
+__global__ void __launch_bounds__(ROWS * kBlock, (min_blocks<ACTION, DENSE>() / ROWS > 0
+                                                       ? min_blocks<ACTION, DENSE>() / ROWS
                                                        : 1))
     force_from_staples(const __grid_constant__ SfLattice L, const __grid_constant__ KernelScalars sc)
 {
@@ -700,7 +155,7 @@ __global__ void __launch_bounds__(ROWS * kBlock, (min_blocks<R, ACTION, DENSE>()
     for (int vb0 = blockIdx.x * ROWS; vb0 < nvb; vb0 += gridDim.x * ROWS) {
         const int vb = vb0 + row;
         double acc = 0.0;
-        if (vb < nvb) acc = force_block<R, ACTION, UNROLLQ, FULL, DIRECT>(L, sc, g, sw, vb);
+        if (vb < nvb) acc = force_block<R, ACTION, UNROLLQ, FULL>(L, sc, g, sw, vb);
         if constexpr (ACTION) {
             const double s = group_sum<ROWS>(acc, row);
             if ((threadIdx.x & (kBlock - 1)) == 0 && vb < nvb) L.partials[vb] = s;
@@ -708,9 +163,8 @@ __global__ void __launch_bounds__(ROWS * kBlock, (min_blocks<R, ACTION, DENSE>()
     }
 }
 
-template <typename R, bool ACTION, bool UNROLLQ, bool DENSE = false, bool FULL = false,
-          bool DIRECT = direct_default<R, FULL>()>
-__global__ void __launch_bounds__(kBlock, (min_blocks<R, ACTION, DENSE>()))
+template <typename R, bool ACTION, bool UNROLLQ, bool DENSE = false, bool FULL = false>
+__global__ void __launch_bounds__(kBlock, (min_blocks<ACTION, DENSE>()))
     force_from_staples_batched(const __grid_constant__ SfBatch B,
                                const __grid_constant__ KernelScalars sc)
 {
@@ -719,7 +173,7 @@ __global__ void __launch_bounds__(kBlock, (min_blocks<R, ACTION, DENSE>()))
         const int c = batch_entry(B, vb);
         const SfLattice &L = B.e[c];
         const G32 g = make_g32(L.dims);
-        const double acc = force_block<R, ACTION, UNROLLQ, FULL, DIRECT>(
+        const double acc = force_block<R, ACTION, UNROLLQ, FULL>(
             L, sc, g, make_sweep(L, g), (int)(vb - L.vb_begin));
         if constexpr (ACTION) {
             const double s = block_sum(acc);
@@ -752,14 +206,8 @@ __global__ void __launch_bounds__(1024) finish_batched(const __grid_constant__ S
     }
 }
 
-unsigned grid_of(int64_t items)
-{
-    if (items < 1) items = 1;
-    if (items > ((int64_t)1 << 30)) items = (int64_t)1 << 30;
-    return (unsigned)items;
-}
-
-// Pass-B schedules (same arithmetic, different traversal or occupancy):
+// Pass-B schedules (same arithmetic, different traversal or occupancy; FP64
+// has one kernel, force_fx.cu, and takes only the traversal from these):
 //   0  micro-tiles 8x2x2, inner b loop rolled
 //   1  micro-tiles 8x2x2, inner b loop unrolled
 //   2  x rows (no micro-tiles), inner b loop rolled
@@ -780,8 +228,7 @@ constexpr int kSfVariants = 9;
 
 // Built-in choice: full staples with the 4-CTA register cap in FP32 (at
 // 32^3x64 3.42 ms against 3.45-3.46 ms for the two-row CTAs and 3.64-3.66
-// for the others; at 32^4 1.73 against 1.75 ms), uncapped full staples in
-// FP64 (110 against 128 ms with compact ones; two-row CTAs 110.2-110.3).
+// for the others; at 32^4 1.73 against 1.75 ms), the same traversal in FP64.
 // The two-row CTAs won (3.54 against 3.67 ms at 32^3x64) while the sweep
 // still divided by run-time extents; with multiply-high divisions the
 // one-row CTA is ahead.  The dims are kept for shape-dependent choices.
@@ -795,11 +242,12 @@ bool full_staples(int variant) { return variant >= 4; }
 
 // Slot of a kernel instance in the occupancy cache of persistent_grid:
 // kind (0 pass B, 1 pass B capped, 2 pass B full, 3 pass B full capped,
-// 4 pass A compact, 5 pass A full) x precision x action x unrolled.
-int grid_slot(int kind, bool f64, bool action, bool unrolled)
+// 4 pass A compact, 5 pass A full) x action x unrolled.
+int grid_slot(int kind, bool action, bool unrolled)
 {
-    return kind * 8 + (f64 ? 4 : 0) + (action ? 2 : 0) + (unrolled ? 1 : 0);
+    return kind * 4 + (action ? 2 : 0) + (unrolled ? 1 : 0);
 }
+
 std::atomic<int> g_sf_variant[2] = {{-1}, {-1}};
 
 // Largest divisor of L not above cap.
@@ -868,151 +316,85 @@ int resolve_variant(const ForceArgs &a)
     return v < 0 ? default_variant(a.precision, a.dims) : v;
 }
 
-// CTAs of a persistent launch: as many as are resident on the device at
-// once (occupancy of the kernel times the SM count, cached per device).
-template <typename K> unsigned persistent_grid(K kernel, int slot, int64_t work)
-{
-    static std::mutex mu;
-    static int cached[64][48] = {{0}};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return grid_of(work);
-    int resident = 0;
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        if (cached[dev][slot] == 0) {
-            int sms = 0, per_sm = 0;
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, 0);
-            cached[dev][slot] = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
-        }
-        resident = cached[dev][slot];
-    }
-    return grid_of(work < resident ? work : resident);
-}
-
-template <typename R, bool ACTION>
+template <bool ACTION>
 cudaError_t launch_pass_b(const SfLattice &L, const KernelScalars &sc, int variant, cudaStream_t st)
 {
     const int64_t V = (int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3];
     const unsigned grid = grid_of(virtual_blocks(V));
-    if (variant == 1) force_from_staples<R, ACTION, true><<<grid, kBlock, 0, st>>>(L, sc);
-    else if (variant == 3) force_from_staples<R, ACTION, false, true><<<grid, kBlock, 0, st>>>(L, sc);
+    if (variant == 1) force_from_staples<float, ACTION, true><<<grid, kBlock, 0, st>>>(L, sc);
+    else if (variant == 3) force_from_staples<float, ACTION, false, true><<<grid, kBlock, 0, st>>>(L, sc);
     else if (variant == 4 || variant == 6)
-        force_from_staples<R, ACTION, false, false, true><<<grid, kBlock, 0, st>>>(L, sc);
-
+        force_from_staples<float, ACTION, false, false, true><<<grid, kBlock, 0, st>>>(L, sc);
     else if (variant == 5)
-        force_from_staples<R, ACTION, false, true, true><<<grid, kBlock, 0, st>>>(L, sc);
+        force_from_staples<float, ACTION, false, true, true><<<grid, kBlock, 0, st>>>(L, sc);
     else if (variant >= 7)
-        force_from_staples<R, ACTION, false, true, true, direct_default<R, true>(), 2>
+        force_from_staples<float, ACTION, false, true, true, 2>
             <<<grid_of((virtual_blocks(V) + 1) / 2), 2 * kBlock, 0, st>>>(L, sc);
-    else force_from_staples<R, ACTION, false><<<grid, kBlock, 0, st>>>(L, sc);
+    else force_from_staples<float, ACTION, false><<<grid, kBlock, 0, st>>>(L, sc);
     return cudaGetLastError();
 }
 
-template <typename R, bool ACTION>
+template <bool ACTION>
 cudaError_t launch_pass_b_batched(const SfBatch &B, const KernelScalars &sc, int variant,
                                   cudaStream_t st)
 {
-    constexpr bool f64 = sizeof(R) == 8;
     if (variant == 1) {
-        auto k = force_from_staples_batched<R, ACTION, true>;
-        k<<<persistent_grid(k, grid_slot(0, f64, ACTION, true), B.total), kBlock, 0, st>>>(B, sc);
+        auto k = force_from_staples_batched<float, ACTION, true>;
+        k<<<persistent_grid(k, grid_slot(0, ACTION, true), B.total), kBlock, 0, st>>>(B, sc);
     } else if (variant == 3) {
-        auto k = force_from_staples_batched<R, ACTION, false, true>;
-        k<<<persistent_grid(k, grid_slot(1, f64, ACTION, false), B.total), kBlock, 0, st>>>(B, sc);
+        auto k = force_from_staples_batched<float, ACTION, false, true>;
+        k<<<persistent_grid(k, grid_slot(1, ACTION, false), B.total), kBlock, 0, st>>>(B, sc);
     } else if (variant == 4 || variant == 6) {
-        auto k = force_from_staples_batched<R, ACTION, false, false, true>;
-        k<<<persistent_grid(k, grid_slot(2, f64, ACTION, false), B.total), kBlock, 0, st>>>(B, sc);
+        auto k = force_from_staples_batched<float, ACTION, false, false, true>;
+        k<<<persistent_grid(k, grid_slot(2, ACTION, false), B.total), kBlock, 0, st>>>(B, sc);
     } else if (variant == 5 || variant >= 7) {
-        auto k = force_from_staples_batched<R, ACTION, false, true, true>;
-        k<<<persistent_grid(k, grid_slot(3, f64, ACTION, false), B.total), kBlock, 0, st>>>(B, sc);
+        auto k = force_from_staples_batched<float, ACTION, false, true, true>;
+        k<<<persistent_grid(k, grid_slot(3, ACTION, false), B.total), kBlock, 0, st>>>(B, sc);
     } else {
-        auto k = force_from_staples_batched<R, ACTION, false>;
-        k<<<persistent_grid(k, grid_slot(0, f64, ACTION, false), B.total), kBlock, 0, st>>>(B, sc);
+        auto k = force_from_staples_batched<float, ACTION, false>;
+        k<<<persistent_grid(k, grid_slot(0, ACTION, false), B.total), kBlock, 0, st>>>(B, sc);
     }
     return cudaGetLastError();
 }
 
 size_t round_up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-template <typename R> cudaError_t launch_sf_t(const ForceArgs &a, cudaStream_t st)
+cudaError_t launch_passes(const SfLattice &L, const KernelScalars &sc, int variant, bool action, cudaStream_t st)
 {
-    const int variant = resolve_variant(a);
-    SfLattice L{};
-    for (int i = 0; i < 4; ++i) L.dims[i] = a.dims[i];
-    set_traversal(L, variant);
-    L.plane_bytes = (int64_t)full_plane_bytes((int64_t)a.dims[0] * a.dims[1] * a.dims[2] * a.dims[3],
-                                              a.precision);
-    L.links = a.links;
-    L.staples = a.staples;
-    L.force = a.force;
-    L.mom = a.mom;
-    L.partials = a.partials;
-    L.action = a.action;
-    const KernelScalars sc = make_scalars(a);
-    const int64_t nvb = virtual_blocks((int64_t)a.dims[0] * a.dims[1] * a.dims[2] * a.dims[3]);
-    if (full_staples(variant)) staple_fields<R, true><<<grid_of(nvb), kBlock, 0, st>>>(L);
-    else staple_fields<R, false><<<grid_of(nvb), kBlock, 0, st>>>(L);
-    cudaError_t e = cudaGetLastError();
+    const unsigned grid = grid_of(virtual_blocks((int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3]));
+    if (full_staples(variant)) staple_fields<float, true><<<grid, kBlock, 0, st>>>(L);
+    else staple_fields<float, false><<<grid, kBlock, 0, st>>>(L);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (a.action != nullptr) {
-        e = launch_pass_b<R, true>(L, sc, variant, st);
-        if (e != cudaSuccess) return e;
-        return launch_finish_sum(a.partials, (int)nvb, a.beta / 3.0, a.action, st);
-    }
-    return launch_pass_b<R, false>(L, sc, variant, st);
+    return action ? launch_pass_b<true>(L, sc, variant, st) : launch_pass_b<false>(L, sc, variant, st);
 }
 
-template <typename R>
-cudaError_t launch_sf_batched_t(const ForceArgs &a, int n, const SfLattice *items,
-                                unsigned long long *counter, cudaStream_t st)
+cudaError_t launch_passes_batched(const SfBatch &B, const KernelScalars &sc, int variant, bool action,
+                                  cudaStream_t st)
 {
-    const int variant = resolve_variant(a);
-    SfBatch B{};
-    B.n = n;
-    B.counter = counter;
-    bool any_action = false;
-    int64_t vb = 0;
-    for (int c = 0; c < n; ++c) {
-        B.e[c] = items[c];
-        set_traversal(B.e[c], variant);
-        B.e[c].plane_bytes = (int64_t)full_plane_bytes(
-            (int64_t)items[c].dims[0] * items[c].dims[1] * items[c].dims[2] * items[c].dims[3],
-            a.precision);
-        B.e[c].vb_begin = vb;
-        vb += virtual_blocks((int64_t)items[c].dims[0] * items[c].dims[1] * items[c].dims[2] *
-                             items[c].dims[3]);
-        any_action = any_action || items[c].action != nullptr;
-    }
-    B.total = vb;
-    const KernelScalars sc = make_scalars(a);
-    cudaError_t e = cudaMemsetAsync(counter, 0, 2 * sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return e;
     if (full_staples(variant)) {
-        auto ka = staple_fields_batched<R, true>;
-        ka<<<persistent_grid(ka, grid_slot(5, sizeof(R) == 8, false, false), B.total), kBlock, 0, st>>>(B);
+        auto ka = staple_fields_batched<float, true>;
+        ka<<<persistent_grid(ka, grid_slot(5, false, false), B.total), kBlock, 0, st>>>(B);
     } else {
-        auto ka = staple_fields_batched<R, false>;
-        ka<<<persistent_grid(ka, grid_slot(4, sizeof(R) == 8, false, false), B.total), kBlock, 0, st>>>(B);
+        auto ka = staple_fields_batched<float, false>;
+        ka<<<persistent_grid(ka, grid_slot(4, false, false), B.total), kBlock, 0, st>>>(B);
     }
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (!any_action) return launch_pass_b_batched<R, false>(B, sc, variant, st);
-    e = launch_pass_b_batched<R, true>(B, sc, variant, st);
-    if (e != cudaSuccess) return e;
-    finish_batched<<<n, 1024, 0, st>>>(B, a.beta / 3.0);
-    return cudaGetLastError();
+    return action ? launch_pass_b_batched<true>(B, sc, variant, st)
+                  : launch_pass_b_batched<false>(B, sc, variant, st);
 }
 
 } // namespace
 
-// Room for the 24 planes in the larger (full, 18-real, in blocks of 32
+// FP32: room for the 24 planes in the larger (full, 18-real, in blocks of 32
 // sites) of the two storage forms, so that every schedule fits the same
-// workspace.
+// workspace.  FP64: the 24 planes and the 4 planes of the links, in limbs.
 size_t staple_field_bytes(const int dims[4], int precision)
 {
     const int64_t V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
-    return round_up256((size_t)kStaplePlanes * full_plane_bytes(V, precision));
+    const size_t planes = precision == LQCD_F64 ? fx_planes_count() : kStaplePlanes;
+    return round_up256(planes * full_plane_bytes(V, precision));
 }
 
 bool staple_fields_supported(const int dims[4])
@@ -1027,15 +409,55 @@ int staple_force_partials(const int dims[4])
 
 cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
 {
-    return a.precision == LQCD_F64 ? launch_sf_t<double>(a, st) : launch_sf_t<float>(a, st);
+    const int variant = resolve_variant(a);
+    const int64_t V = (int64_t)a.dims[0] * a.dims[1] * a.dims[2] * a.dims[3];
+    SfLattice L{};
+    for (int i = 0; i < 4; ++i) L.dims[i] = a.dims[i];
+    set_traversal(L, variant);
+    L.plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
+    L.links = a.links;
+    L.staples = a.staples;
+    L.force = a.force;
+    L.mom = a.mom;
+    L.partials = a.partials;
+    L.action = a.action;
+    const KernelScalars sc = make_scalars(a);
+    const bool action = a.action != nullptr;
+    const cudaError_t e = a.precision == LQCD_F64 ? launch_fx_passes(L, sc, action, st)
+                                                  : launch_passes(L, sc, variant, action, st);
+    if (e != cudaSuccess || !action) return e;
+    return launch_finish_sum(a.partials, (int)virtual_blocks(V), a.beta / 3.0, a.action, st);
 }
 
 cudaError_t launch_force_staple_fields_batched(const ForceArgs &a, int n, const SfLattice *items,
                                                unsigned long long *counter, cudaStream_t st)
 {
     if (n < 1 || n > kMaxBatch) return cudaErrorInvalidValue;
-    return a.precision == LQCD_F64 ? launch_sf_batched_t<double>(a, n, items, counter, st)
-                                   : launch_sf_batched_t<float>(a, n, items, counter, st);
+    const int variant = resolve_variant(a);
+    SfBatch B{};
+    B.n = n;
+    B.counter = counter;
+    bool any_action = false;
+    int64_t vb = 0;
+    for (int c = 0; c < n; ++c) {
+        const int *d = items[c].dims;
+        const int64_t V = (int64_t)d[0] * d[1] * d[2] * d[3];
+        B.e[c] = items[c];
+        set_traversal(B.e[c], variant);
+        B.e[c].plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
+        B.e[c].vb_begin = vb;
+        vb += virtual_blocks(V);
+        any_action = any_action || items[c].action != nullptr;
+    }
+    B.total = vb;
+    const KernelScalars sc = make_scalars(a);
+    cudaError_t e = cudaMemsetAsync(counter, 0, 3 * sizeof(unsigned long long), st);
+    if (e != cudaSuccess) return e;
+    e = a.precision == LQCD_F64 ? launch_fx_passes_batched(B, sc, any_action, st)
+                                : launch_passes_batched(B, sc, variant, any_action, st);
+    if (e != cudaSuccess || !any_action) return e;
+    finish_batched<<<n, 1024, 0, st>>>(B, a.beta / 3.0);
+    return cudaGetLastError();
 }
 
 int staple_force_variants() { return kSfVariants; }

@@ -95,7 +95,7 @@ struct SfLattice {
     int64_t vb_begin;  // batch: first virtual block of this lattice
     int64_t plane_bytes; // full staple planes: bytes of one plane
     const void *links;
-    void *staples;     // 24 staple planes (workspace)
+    void *staples;     // 24 staple planes (FP64: and 4 link planes; workspace)
     void *force;       // written when set
     void *mom;         // p += dt f when set
     double *partials;  // one action partial per virtual block
@@ -107,7 +107,7 @@ constexpr int kMaxBatch = 64;
 struct SfBatch {
     int n;
     int64_t total;                 // virtual blocks of all lattices
-    unsigned long long *counter;   // work counters (2, zeroed before the passes)
+    unsigned long long *counter;   // work counters (3, zeroed before the passes)
     SfLattice e[kMaxBatch];
 };
 
@@ -128,6 +128,10 @@ cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st);
 // links, staples, force, mom, partials, action), 1 <= n <= kMaxBatch.
 cudaError_t launch_force_staple_fields_batched(const ForceArgs &a, int n, const SfLattice *items,
                                                unsigned long long *counter, cudaStream_t st);
+// The FP64 passes of it (force_fx.cu): planes of the workspace, the launches.
+int fx_planes_count();
+cudaError_t launch_fx_passes(const SfLattice &L, const KernelScalars &sc, bool action, cudaStream_t st);
+cudaError_t launch_fx_passes_batched(const SfBatch &B, const KernelScalars &sc, bool action, cudaStream_t st);
 int staple_force_variants();
 int staple_force_variant(int precision, const int dims[4]); // current choice (default by shape)
 void set_staple_force_variant(int precision, int variant);
