@@ -49,6 +49,27 @@ struct FxPlanes {
         return u;
     }
 
+    // The matrix or (dag) its dagger, chosen at run time: the off-diagonal
+    // entries are read from their mirrored places.
+    __device__ __forceinline__ FMat load_form(const char *r, int plane, bool dag) const
+    {
+        const int4 *p = reinterpret_cast<const int4 *>(r + (int64_t)plane * plane_bytes);
+        constexpr int S = FxBlock::LANE / 16;
+        const int o = dag ? 2 * S : 0, m = dag ? -1 : 0;
+        const int4 *up = p + o, *dn = p - o, *up2 = up + o, *dn2 = dn - o;
+        const int4 v[9] = {__ldg(p),           __ldg(up + S),      __ldg(up2 + 2 * S), __ldg(dn + 3 * S), __ldg(p + 4 * S),
+                           __ldg(up + 5 * S),  __ldg(dn2 + 6 * S), __ldg(dn + 7 * S),  __ldg(p + 8 * S)};
+        FMat u;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            u.rh[e / 3][e % 3] = v[e].x;
+            u.rl[e / 3][e % 3] = v[e].y;
+            u.ih[e / 3][e % 3] = (v[e].z ^ m) - m;
+            u.il[e / 3][e % 3] = (v[e].w ^ m) - m;
+        }
+        return u;
+    }
+
     template <bool STREAM> __device__ __forceinline__ void store(char *r, int plane, const FMat &u) const
     {
         int4 *p = reinterpret_cast<int4 *>(r + (int64_t)plane * plane_bytes);
@@ -146,7 +167,7 @@ template <int FA, int FB> __device__ __forceinline__ FMat fx_mul_top2(const FMat
     FAcc y;
     fx_zero(y);
     fx_mul_acc<FA, FB, 2>(y, a, b);
-    return fx_round<0, 2>(y);
+    return fx_round<0, FA == FB ? 1 : -1, 2>(y);
 }
 
 __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, int vb)
@@ -240,129 +261,126 @@ __device__ __noinline__ double force_link_floating(const SfLattice &L, const Ker
     return force_link<double, ACTION, false, true>(L, sc, g, sf, si, c, k, rho);
 }
 
-// z += B_d [ alpha sum_{b perp rho, d} S_b(k+d) S^{(d)}_b(k) + beta S_d(k+d) A_d^dag ]
-// for d = +-nud (d_terms of sf_common.cuh without the scale z); units 2^-56.
-template <bool NEG>
-__device__ __forceinline__ void fx_d_terms(FInt &z, bool &bad, const FxPlanes &sf, const FxScalars &fx,
-                                           const G32 &g, const Coord &c, int rho, int k, int kp, int id)
-{
-    const int base = rho * 6;
-    const int jd = 2 * id + (NEG ? 1 : 0);
-    const int nud = (rho + 1 + id) & 3;
-    const int dk = step32(g, c, nud, NEG ? -1 : 1);
-    const char *at_d = sf.at(k + dk);
-    const char *at_2 = NEG ? at_d : sf.at(k);
-    FMat y;
-    {
-        FAcc acc;
-        fx_zero(acc);
-#pragma unroll 1
-        for (int q = 0; q < 4; ++q) {
-            const int ib = q < 2 ? (id == 0 ? 1 : 0) : (id == 2 ? 1 : 2);
-            const int nub = (rho + 1 + ib) & 3;
-            const int jp = 2 * ((nub - nud - 1) & 3) + (q & 1);
-            const FMat a = sf.load(at_d, base + 2 * ib + (q & 1)), b = sf.load(at_2, nud * 6 + jp);
-            bad = bad || fx_poisoned(a) || fx_poisoned(b);
-            fx_mul_acc<N, NEG ? D : N>(acc, a, b);
-        }
-        y = fx_round<2>(acc); // up to 4, units 2^-56
-    }
-    FInt w = fx_scaled(fx.alpha, y);
-    {
-        FMat a = sf.load(at_d, base + jd), b = sf.load(NEG ? at_d : sf.at(k), kLinkPlane + nud);
-        bad = bad || fx_poisoned(a) || fx_poisoned(b);
-        if (fx.use_beta) a = fx_round<0>(fx_scaled(fx.beta, a));
-        FAcc acc;
-        fx_zero(acc);
-        fx_mul_acc<N, NEG ? N : D>(acc, a, b);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                w.re[i][j] += (fx_value(acc.rh[i][j], acc.rl[i][j]) + 2) >> 2;
-                w.im[i][j] += (fx_value(acc.ih[i][j], acc.il[i][j]) + 2) >> 2;
-            }
-    }
-    y = fx_round<0>(w);
-    const FMat b = sf.load(sf.at(kp + (NEG ? dk : 0)), kLinkPlane + nud);
-    bad = bad || fx_poisoned(b);
-    FAcc acc;
-    fx_zero(acc);
-    fx_mul_acc<NEG ? D : N, N>(acc, b, y);
-    fx_add(z, acc);
-}
-
 // Force (and the fused momentum step) on the link (k, rho); returns its
 // share of the action (force_link of sf_common.cuh in fixed point).
+//
+// Every sum of products that a link closes is a group of one loop: group 0
+// F sum_b S_b(k+rho) S_b(k), group 1 sum_b S_b(k) S_b(k-rho) E, groups 2..7
+// B_d [ alpha sum_{b perp rho, d} S_b(k+d) S^{(d)}_b(k) + beta S_d(k+d) A_d^dag ]
+// for the six directions d.  One loop, and not a piece of code for each group
+// and sign: a product is 280 instructions, and with eleven copies of it the
+// instruction cache missed (1.5 stalled cycles per instruction).  The sums
+// take 108 registers of the 255 that two CTAs per SM leave, so the total z of
+// the groups stays in shared memory.
 template <bool ACTION>
 __device__ __forceinline__ double fx_force_link(const SfLattice &L, const KernelScalars &sc, const FxScalars &fx,
                                                 const G32 &g, const Coord &c, int k, int rho)
 {
+    __shared__ longlong2 z_s[9][kBlock]; // units 2^-56
+    longlong2 *z = &z_s[0][threadIdx.x];
     const FxPlanes sf = fx_planes(L);
     const int64_t V = g.V;
-    const int kp = k + step32(g, c, rho, 1), km = k + step32(g, c, rho, -1);
+    const int kp = k + step32(g, c, rho, 1);
     const int base = rho * 6;
     bool bad = false;
 
-    FInt pl, z; // plaquette sum, units 2^-58; the rest, units 2^-56
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) pl.re[i][j] = pl.im[i][j] = z.re[i][j] = z.im[i][j] = 0;
-    {
+#pragma unroll 1
+    for (int grp = 0; grp < 8; ++grp) {
+        const bool chain = grp < 2, neg = grp >= 5;
+        const int id = chain ? 0 : (neg ? grp - 5 : grp - 2);
+        const int nud = chain ? rho : (rho + 1 + id) & 3;
+        const int dk = step32(g, c, nud, neg || grp == 1 ? -1 : 1); // k + dk: k+rho, k-rho, k+d
+        const char *at_k = sf.at(k), *at_d = sf.at(k + dk);
+        const char *at_a = grp == 1 ? at_k : at_d;
+        const char *at_b = chain ? (grp == 0 ? at_k : at_d) : (neg ? at_d : at_k);
         FAcc acc;
         fx_zero(acc);
-        const char *at_k = sf.at(k), *at_p = sf.at(kp);
+        const int n = chain ? 6 : 5;
 #pragma unroll 1
-        for (int jj = 0; jj < 6; ++jj) {
-            const FMat s = sf.load(at_k, base + jj), p = sf.load(at_p, base + jj);
-            bad = bad || fx_poisoned(s) || fx_poisoned(p);
+        for (int q = 0; q < n; ++q) {
+            int pa = base + q, pb = base + q;
+            bool dag = neg;
+            if (!chain) {
+                const int ib = q < 2 ? (id == 0 ? 1 : 0) : (id == 2 ? 1 : 2);
+                const int nub = (rho + 1 + ib) & 3;
+                pa = base + 2 * ib + (q & 1);
+                pb = nud * 6 + 2 * ((nub - nud - 1) & 3) + (q & 1);
+                if (q == 4) { // the rectangle along d, onto alpha times the cubes
+                    const FMat y = fx_round<2>(acc); // up to 4, units 2^-56
+                    const FInt w = fx_scaled(fx.alpha, y);
+                    fx_zero(acc);
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
+                    for (int i = 0; i < 3; ++i)
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    pl.re[i][j] += (long long)s.rh[i][j] * (1 << kLimb) + s.rl[i][j];
-                    pl.im[i][j] += (long long)s.ih[i][j] * (1 << kLimb) + s.il[i][j];
+                        for (int j = 0; j < 3; ++j) {
+                            acc.h1[i][j] = 4 * w.re[i][j];
+                            acc.h3[i][j] = 4 * (w.re[i][j] + w.im[i][j]);
+                        }
+                    pa = base + 2 * id + (neg ? 1 : 0);
+                    pb = kLinkPlane + nud;
+                    dag = !neg;
                 }
-            fx_mul_acc<N, N>(acc, p, s);
+            }
+            FMat a = sf.load(at_a, pa);
+            const FMat b = sf.load_form(at_b, pb, dag);
+            bad = bad || fx_poisoned(a) || fx_poisoned(b);
+            if (fx.use_beta && q == 4 && !chain) a = fx_round<0>(fx_scaled(fx.beta, a));
+            fx_mul_acc<N, N>(acc, a, b);
         }
-        FMat p1 = fx_round<2>(acc);
-        if (fx.use_beta) p1 = fx_round<0>(fx_scaled(fx.beta, p1));
-        const FMat F = sf.load(at_p, kLinkPlane + rho);
-        bad = bad || fx_poisoned(F);
-        fx_zero(acc);
-        fx_mul_acc<N, N>(acc, F, p1);
-        fx_add(z, acc);
-    }
-    {
-        FAcc acc;
-        fx_zero(acc);
-        const char *at_k = sf.at(k), *at_m = sf.at(km);
-#pragma unroll 1
-        for (int jj = 0; jj < 6; ++jj) {
-            const FMat s = sf.load(at_k, base + jj), m = sf.load(at_m, base + jj);
-            bad = bad || fx_poisoned(m);
-            fx_mul_acc<N, N>(acc, s, m);
+        FMat y = fx_round<2>(acc);
+        if (fx.use_beta && chain) y = fx_round<0>(fx_scaled(fx.beta, y));
+        FMat x = sf.load_form(grp == 1 ? at_d : sf.at(neg ? kp + dk : kp), kLinkPlane + nud, neg);
+        bad = bad || fx_poisoned(x);
+        if (grp == 1) {
+            const FMat t = x;
+            x = y;
+            y = t;
         }
-        FMat p2 = fx_round<2>(acc);
-        if (fx.use_beta) p2 = fx_round<0>(fx_scaled(fx.beta, p2));
-        const FMat E = sf.load(at_m, kLinkPlane + rho);
-        bad = bad || fx_poisoned(E);
         fx_zero(acc);
-        fx_mul_acc<N, N>(acc, p2, E);
-        fx_add(z, acc);
+        fx_mul_acc<N, N>(acc, x, y);
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            longlong2 s;
+            fx_value_of<1>(acc, e / 3, e % 3, s.x, s.y);
+            if (grp > 0) {
+                const longlong2 o = z[e * kBlock];
+                s.x += o.x;
+                s.y += o.y;
+            }
+            z[e * kBlock] = s;
+        }
     }
-#pragma unroll 1
-    for (int id = 0; id < 3; ++id) fx_d_terms<false>(z, bad, sf, fx, g, c, rho, k, kp, id);
-#pragma unroll 1
-    for (int id = 0; id < 3; ++id) fx_d_terms<true>(z, bad, sf, fx, g, c, rho, k, kp, id);
 
     const FMat u = sf.load(sf.at(k), kLinkPlane + rho);
     bad = bad || fx_poisoned(u);
     if (bad) return force_link_floating<ACTION>(L, sc, k, rho);
 
-    const FMat plm = fx_round<2>(pl);            // units 2^-56
-    FInt t = fx_scaled(fx.z, fx_round<3>(z));    // units 2^-53
+    FMat plm; // plaquette sum, units 2^-56
+    {
+        FInt pl;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) pl.re[e / 3][e % 3] = pl.im[e / 3][e % 3] = 0;
+#pragma unroll 1
+        for (int jj = 0; jj < 6; ++jj) {
+            const FMat s = sf.load(sf.at(k), base + jj);
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    pl.re[i][j] = mad_wide(s.rh[i][j], 1 << kLimb, pl.re[i][j]) + s.rl[i][j];
+                    pl.im[i][j] = mad_wide(s.ih[i][j], 1 << kLimb, pl.im[i][j]) + s.il[i][j];
+                }
+        }
+        plm = fx_round<2>(pl);
+    }
+    FInt t;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        const longlong2 s = z[e * kBlock];
+        t.re[e / 3][e % 3] = s.x;
+        t.im[e / 3][e % 3] = s.y;
+    }
+    t = fx_scaled(fx.z, fx_round<3>(t)); // units 2^-53
     const FInt tp = fx_scaled(fx.pl, plm);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -378,10 +396,7 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            m.re[i][j] = fx_value(acc.rh[i][j], acc.rl[i][j]);
-            m.im[i][j] = fx_value(acc.ih[i][j], acc.il[i][j]);
-        }
+        for (int j = 0; j < 3; ++j) fx_value_of<1>(acc, i, j, m.re[i][j], m.im[i][j]);
     // f = -(beta/6) Im tr(lambda_a U t) (ta_components)
     const double s = -sc.d[SC_BETA6] * fx.m * 0x1p-53;
     double f[8];
