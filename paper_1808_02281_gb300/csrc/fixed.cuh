@@ -1,56 +1,222 @@
 // Fixed-point arithmetic for FP64 fields of SU(3) matrices.
 //
-// GB300 issues 2 FP64 FMAs per clock and SM but 64 integer multiply-adds of
-// 32 x 32 + 64 bits (measured: 1.7 and 63.4).  The entries of an SU(3) matrix
-// are at most 1 in modulus, so instead of a floating point they can have a
-// fixed one: a real x is the 59-bit integer x 2^58 in two signed limbs,
-// x 2^58 = h 2^29 + l with -2^28 <= l < 2^28, and a product is
-//     x y 2^58 = h h' + (h l' + l h') 2^-29 + l l' 2^-58,
-// three multiply-adds into two 64-bit accumulators (the last term, below
-// 2^-60, is left out): 21 real FMAs per clock and SM against 2, and 28 with
-// complex products in three real ones (FAcc).  Rounding is
-// by half a unit of 2^-58, 1.7e-18, where an FP64 result of that size rounds
-// by up to 5.5e-17, so sums of products come out more exact than in FP64.
-// Sums that pass 1 are kept in coarser units (2^-56 up to 8, 2^-53 up to 64),
-// the unit being fixed by the place in the formula.
+// GB300 issues 2 FP64 FMAs per clock and SM, but 32 integer multiply-adds of
+// 32 x 32 + 64 bits and 128 FP32 FMAs.  The entries of an SU(3) matrix are at
+// most 1 in modulus, so instead of a floating point they can have a fixed
+// one.  Two forms share the leading part h, a whole number of 2^-30:
 //
-// Overflow: entries of a product of matrices that are unitary to about 1e-3
-// are bounded by 1 + 1e-2 through every partial sum (Cauchy-Schwarz).  The
-// largest sum is the mixed one of (ar + ai)(br + bi): the high limbs of a row
-// add up to sqrt(6) 2^29, the low limbs are at most 2^29, so the two terms of
-// one product give at most 4.9 2^58 and six products, the most that share
-// accumulators, 29.4 2^58 < 2^63.  Links that are not within 1e-3 of SU(3)
-// or not finite are marked (kPoison) and take the floating-point path.
+//   FLimbs   x = (h 2^28 + l) 2^-58, l a signed 28-bit whole number: all
+//            sums of products are exact, three multiply-adds per product
+//            (h h', h l', l h'; l l' is below 2^-60).  Links, and the few
+//            products that the result sees with a weight near 1.
+//   FMat     x = (h + l) 2^-30, l in FP32: h h' goes into a 64-bit sum
+//            exactly, h l' + l h' into an FP32 sum (the terms are 2^-31 of
+//            the product, so its rounding is near 2^-55 of it).  Staples, and
+//            the many products under the rectangle and cube coefficients.
+//
+// Complex products take three whole-number products (Gauss: exact, so the
+// cancellation costs nothing, and without signs: a negated factor would make
+// a product and a 64-bit subtraction of every multiply-add).  In the second
+// form the integer and the FP32 work run on the two halves of the FMA pipe:
+// about 400 issue slots per 3x3 product and warp against 1730 (108 FMAs of 16
+// clocks) on the FP64 pipe.
+//
+// Sums that pass 1 are kept in coarser units; the unit is fixed by the place
+// in the formula.  High sums wrap modulo 2^64, so only results have to fit:
+// entries of products of matrices that are unitary to about 1e-3 are bounded
+// by 1 + 1e-2.  Links that are not within 1e-3 of SU(3), or not finite, are
+// marked (kPoison) and take the floating-point path.
 #pragma once
 
 #include "su3.cuh"
 
 namespace lqcd {
 
-constexpr int kLimb = 29;        // bits of the low limb
-constexpr int kUnit = 2 * kLimb; // entries in units of 2^-58
+constexpr int kUnit = 30; // entries of links and staples in units of 2^-30
 
 // h of entry (0, 0) of a matrix that has no fixed-point form.
 constexpr int kPoison = (int)0x80000000;
 
 struct FMat {
+    int rh[3][3];
+    float rl[3][3];
+    int ih[3][3];
+    float il[3][3];
+};
+
+struct FLimbs {
     int rh[3][3], rl[3][3], ih[3][3], il[3][3];
 };
 
-// Sums of a matrix of complex products a b in three real ones each (Gauss):
-// 1: sum ar br, 2: sum ai bi, 3: sum (ar + ai)(br + bi), so that
-// Re = 1 - 2, Im = 3 - 1 - 2; high and mixed sums of each.  In whole numbers
-// the cancellation is exact, and no factor is ever negated.
-struct FAcc {
+// High and mixed sums of the three real products of a matrix of complex ones.
+struct FLimbAcc {
     long long h1[3][3], l1[3][3], h2[3][3], l2[3][3], h3[3][3], l3[3][3];
 };
 
-// A matrix of whole numbers (in the units of its place).
-struct FInt {
-    long long re[3][3], im[3][3];
+// Sums of a matrix of complex products a b: whole-number parts of
+// 1: sum ar br, 2: sum ai bi, 3: sum (ar + ai)(br + bi), so that
+// Re = 1 - 2, Im = 3 - 1 - 2; FP32 parts cr, ci of the real and imaginary one.
+struct FAcc {
+    long long h1[3][3], h2[3][3], h3[3][3];
+    float cr[3][3], ci[3][3];
+};
+
+// A sum of products in the units of its place: v + c.
+struct FSum {
+    long long v;
+    float c;
 };
 
 __device__ __forceinline__ void fx_zero(FAcc &y)
+{
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            y.h1[i][j] = y.h2[i][j] = y.h3[i][j] = 0;
+            y.cr[i][j] = y.ci[i][j] = 0.f;
+        }
+}
+
+// x + a b, one instruction.  As a PTX product and sum, which the assembler
+// joins: PTX's own mad.wide comes out as a product and a 64-bit addition
+// (three instructions) in every other place, and from the C expression the
+// compiler may make an unsigned product with corrections.
+__device__ __forceinline__ long long mad_wide(int a, int b, long long x)
+{
+    asm("{\n\t.reg .s64 t;\n\tmul.wide.s32 t, %1, %2;\n\tadd.s64 %0, %0, t;\n\t}" : "+l"(x) : "r"(a), "r"(b));
+    return x;
+}
+
+// y += op_a(a) op_b(b), rows 0..ROWS-1 (the sign of the second whole-number
+// sum is left to fx_total).
+template <int FA, int FB, int ROWS = 3>
+__device__ __forceinline__ void fx_mul_acc(FAcc &y, const FMat &a, const FMat &b)
+{
+    constexpr float SA = FA == N ? 1.f : -1.f, SB = FB == N ? 1.f : -1.f; // signs of the imaginary parts
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        int bs[3];
+        float br[3], bi[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int p = FB == N ? k : j, q = FB == N ? j : k;
+            bs[j] = FB == N ? b.rh[p][q] + b.ih[p][q] : b.rh[p][q] - b.ih[p][q];
+            br[j] = (float)b.rh[p][q];
+            bi[j] = (float)b.ih[p][q];
+        }
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            const int u = FA == N ? i : k, v = FA == N ? k : i;
+            const int arh = a.rh[u][v], aih = a.ih[u][v], as = FA == N ? arh + aih : arh - aih;
+            const float ar = (float)arh, ai = (float)aih, arl = a.rl[u][v], ail = a.il[u][v];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int p = FB == N ? k : j, q = FB == N ? j : k;
+                y.h1[i][j] = mad_wide(arh, b.rh[p][q], y.h1[i][j]);
+                y.h2[i][j] = mad_wide(aih, b.ih[p][q], y.h2[i][j]);
+                y.h3[i][j] = mad_wide(as, bs[j], y.h3[i][j]);
+                float cr = y.cr[i][j], ci = y.ci[i][j];
+                cr = fmaf(ar, b.rl[p][q], cr);
+                ci = fmaf(SB * ar, b.il[p][q], ci);
+                cr = fmaf(arl, br[j], cr);
+                ci = fmaf(SB * arl, bi[j], ci);
+                cr = fmaf(-SA * SB * ai, b.il[p][q], cr);
+                ci = fmaf(SA * ai, b.rl[p][q], ci);
+                cr = fmaf(-SA * SB * ail, bi[j], cr);
+                ci = fmaf(SA * ail, br[j], ci);
+                y.cr[i][j] = cr;
+                y.ci[i][j] = ci;
+            }
+        }
+    }
+}
+
+// Entry (i, j) of the sums; SIGN = -1 where one of the factors is daggered.
+template <int SIGN> __device__ __forceinline__ void fx_total(const FAcc &y, int i, int j, FSum &re, FSum &im)
+{
+    if constexpr (SIGN > 0) {
+        re.v = y.h1[i][j] - y.h2[i][j];
+        im.v = y.h3[i][j] - y.h1[i][j] - y.h2[i][j];
+    } else {
+        re.v = y.h1[i][j] + y.h2[i][j];
+        im.v = y.h3[i][j] - y.h1[i][j] + y.h2[i][j];
+    }
+    re.c = y.cr[i][j];
+    im.c = y.ci[i][j];
+}
+
+// A sum in units 2^SH times coarser, as h + l.
+template <int SH> __device__ __forceinline__ void fx_split(const FSum s, int &h, float &l)
+{
+    static_assert(SH >= 2 && SH <= 33, "shift");
+    if constexpr (SH == 33) {
+        fx_split<32>(FSum{s.v >> 1, 0.5f * s.c}, h, l);
+    } else if constexpr (SH == 32) {
+        const unsigned lo = (unsigned)s.v;
+        h = (int)(s.v >> 32) + (int)(lo >> 31);
+        l = fmaf((float)(int)lo, 0x1p-32f, s.c * 0x1p-32f);
+    } else {
+        constexpr float scale = 1.f / (float)(1ll << SH);
+        h = (int)((s.v + (1ll << (SH - 1))) >> SH);
+        l = fmaf((float)(int)((unsigned)s.v - ((unsigned)h << SH)), scale, s.c * scale);
+    }
+}
+
+// All entries, rows 0..ROWS-1.
+template <int SH, int SIGN = 1, int ROWS = 3> __device__ __forceinline__ FMat fx_round(const FAcc &y)
+{
+    FMat m;
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            FSum re, im;
+            fx_total<SIGN>(y, i, j, re, im);
+            fx_split<SH>(re, m.rh[i][j], m.rl[i][j]);
+            fx_split<SH>(im, m.ih[i][j], m.il[i][j]);
+        }
+    return m;
+}
+
+// A real scalar of modulus at most 1, in units of 2^-30.
+struct FScalar {
+    int h;
+    float l;
+};
+
+inline FScalar fx_scalar(double c)
+{
+    const double x = c * 1073741824.0; // 2^30
+    FScalar s;
+    s.h = (int)(x + (x < 0 ? -0.5 : 0.5));
+    s.l = (float)(x - (double)s.h);
+    return s;
+}
+
+// c x, x = h + l; in units 2^-30 of those of x.
+__device__ __forceinline__ FSum fx_scaled(const FScalar c, int h, float l)
+{
+    return FSum{mad_wide(c.h, h, 0), fmaf((float)c.h, l, c.l * (float)h)};
+}
+
+// c m, in the units of m.
+__device__ __forceinline__ FMat fx_scaled(const FScalar c, const FMat &m)
+{
+    FMat r;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            fx_split<kUnit>(fx_scaled(c, m.rh[i][j], m.rl[i][j]), r.rh[i][j], r.rl[i][j]);
+            fx_split<kUnit>(fx_scaled(c, m.ih[i][j], m.il[i][j]), r.ih[i][j], r.il[i][j]);
+        }
+    return r;
+}
+
+// ------------------------------------------------------------ whole limbs
+
+__device__ __forceinline__ void fx_zero(FLimbAcc &y)
 {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -59,19 +225,7 @@ __device__ __forceinline__ void fx_zero(FAcc &y)
             y.h1[i][j] = y.l1[i][j] = y.h2[i][j] = y.l2[i][j] = y.h3[i][j] = y.l3[i][j] = 0;
 }
 
-// x + a b, one instruction.  As a PTX product and sum, which the assembler
-// joins: PTX's own mad.wide comes out as a product and a 64-bit addition
-// (three instructions) in every other place, and from the C expression the
-// compiler may make an unsigned product with corrections.  Where a factor is
-// a negated register there is a subtraction all the same, which is why the
-// products below have no signs.
-__device__ __forceinline__ long long mad_wide(int a, int b, long long x)
-{
-    asm("{\n\t.reg .s64 t;\n\tmul.wide.s32 t, %1, %2;\n\tadd.s64 %0, %0, t;\n\t}" : "+l"(x) : "r"(a), "r"(b));
-    return x;
-}
-
-// One real product into a pair of sums.
+// One real product into a high and a mixed sum.
 __device__ __forceinline__ void fx_mad(long long &h, long long &l, int ah, int al, int bh, int bl)
 {
     h = mad_wide(ah, bh, h);
@@ -79,54 +233,42 @@ __device__ __forceinline__ void fx_mad(long long &h, long long &l, int ah, int a
     l = mad_wide(al, bh, l);
 }
 
-// y += op_a(a) op_b(b), rows 0..ROWS-1; the signs of daggered factors are
-// left to fx_value_of (SIGN = -1 for one daggered factor).
+// y += op_a(a) op_b(b), rows 0..ROWS-1 (the sign of the second sums is left
+// to fx_total).
 template <int FA, int FB, int ROWS = 3>
-__device__ __forceinline__ void fx_mul_acc(FAcc &y, const FMat &a, const FMat &b)
+__device__ __forceinline__ void fx_mul_acc(FLimbAcc &y, const FLimbs &a, const FLimbs &b)
 {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         int sh[3], sl[3];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const int bi = FB == N ? k : j, bk = FB == N ? j : k;
-            sh[j] = FB == N ? b.rh[bi][bk] + b.ih[bi][bk] : b.rh[bi][bk] - b.ih[bi][bk];
-            sl[j] = FB == N ? b.rl[bi][bk] + b.il[bi][bk] : b.rl[bi][bk] - b.il[bi][bk];
+            const int p = FB == N ? k : j, q = FB == N ? j : k;
+            sh[j] = FB == N ? b.rh[p][q] + b.ih[p][q] : b.rh[p][q] - b.ih[p][q];
+            sl[j] = FB == N ? b.rl[p][q] + b.il[p][q] : b.rl[p][q] - b.il[p][q];
         }
 #pragma unroll
         for (int i = 0; i < ROWS; ++i) {
-            const int ai = FA == N ? i : k, ak = FA == N ? k : i;
-            const int arh = a.rh[ai][ak], arl = a.rl[ai][ak], aih = a.ih[ai][ak], ail = a.il[ai][ak];
+            const int u = FA == N ? i : k, v = FA == N ? k : i;
+            const int arh = a.rh[u][v], arl = a.rl[u][v], aih = a.ih[u][v], ail = a.il[u][v];
             const int ash = FA == N ? arh + aih : arh - aih, asl = FA == N ? arl + ail : arl - ail;
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                const int bi = FB == N ? k : j, bk = FB == N ? j : k;
-                fx_mad(y.h1[i][j], y.l1[i][j], arh, arl, b.rh[bi][bk], b.rl[bi][bk]);
-                fx_mad(y.h2[i][j], y.l2[i][j], aih, ail, b.ih[bi][bk], b.il[bi][bk]);
+                const int p = FB == N ? k : j, q = FB == N ? j : k;
+                fx_mad(y.h1[i][j], y.l1[i][j], arh, arl, b.rh[p][q], b.rl[p][q]);
+                fx_mad(y.h2[i][j], y.l2[i][j], aih, ail, b.ih[p][q], b.il[p][q]);
                 fx_mad(y.h3[i][j], y.l3[i][j], ash, asl, sh[j], sl[j]);
             }
         }
     }
 }
 
-// The value of a pair of sums, in the unit of the high one.
-__device__ __forceinline__ long long fx_value(long long h, long long l)
-{
-    return h + ((l + (1ll << (kLimb - 1))) >> kLimb);
-}
+// A high and a mixed sum in the units of the high one.
+__device__ __forceinline__ long long fx_value(long long h, long long l) { return h + ((l + (1ll << 27)) >> 28); }
 
-// v 2^-SH as two limbs.
-template <int SH> __device__ __forceinline__ void fx_split(long long v, int &h, int &l)
-{
-    if constexpr (SH > 0) v = (v + (1ll << (SH - 1))) >> SH;
-    h = (int)((v + (1ll << (kLimb - 1))) >> kLimb);
-    l = (int)((unsigned)v - ((unsigned)h << kLimb));
-}
-
-// Entry (i, j) of the sums, in the units of the high ones; SIGN = -1 where
-// one of the factors is daggered.
+// Entry (i, j) of the sums; SIGN = -1 where one of the factors is daggered.
 template <int SIGN>
-__device__ __forceinline__ void fx_value_of(const FAcc &y, int i, int j, long long &re, long long &im)
+__device__ __forceinline__ void fx_total(const FLimbAcc &y, int i, int j, long long &re, long long &im)
 {
     if constexpr (SIGN > 0) {
         re = fx_value(y.h1[i][j] - y.h2[i][j], y.l1[i][j] - y.l2[i][j]);
@@ -137,38 +279,33 @@ __device__ __forceinline__ void fx_value_of(const FAcc &y, int i, int j, long lo
     }
 }
 
-// The sums as limbs, in units 2^SH times coarser; rows 0..ROWS-1.
-template <int SH, int SIGN = 1, int ROWS = 3> __device__ __forceinline__ FMat fx_round(const FAcc &y)
+// A whole number v of 2^-(58 + SH) as limbs of 2^-30 and 2^-58.
+template <int SH> __device__ __forceinline__ void fx_limbs(long long v, int &h, int &l)
 {
-    FMat m;
+    if constexpr (SH > 0) v = (v + (1ll << (SH > 0 ? SH - 1 : 0))) >> SH;
+    h = (int)((v + (1ll << 27)) >> 28);
+    l = (int)((unsigned)v - ((unsigned)h << 28));
+}
+
+// The entries of a product (units 2^-60), rows 0..ROWS-1.
+template <int SIGN, int ROWS = 3> __device__ __forceinline__ FLimbs fx_round(const FLimbAcc &y)
+{
+    FLimbs m;
 #pragma unroll
     for (int i = 0; i < ROWS; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             long long re, im;
-            fx_value_of<SIGN>(y, i, j, re, im);
-            fx_split<SH>(re, m.rh[i][j], m.rl[i][j]);
-            fx_split<SH>(im, m.ih[i][j], m.il[i][j]);
-        }
-    return m;
-}
-
-template <int SH> __device__ __forceinline__ FMat fx_round(const FInt &y)
-{
-    FMat m;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            fx_split<SH>(y.re[i][j], m.rh[i][j], m.rl[i][j]);
-            fx_split<SH>(y.im[i][j], m.ih[i][j], m.il[i][j]);
+            fx_total<SIGN>(y, i, j, re, im);
+            fx_limbs<2>(re, m.rh[i][j], m.rl[i][j]);
+            fx_limbs<2>(im, m.ih[i][j], m.il[i][j]);
         }
     return m;
 }
 
 // Row 2 of an SU(3) matrix from rows 0 and 1: row2 = conj(row0 x row1), the
 // terms of either sign in sums of their own.
-__device__ __forceinline__ void fx_row2(FMat &u)
+__device__ __forceinline__ void fx_row2(FLimbs &u)
 {
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -178,50 +315,32 @@ __device__ __forceinline__ void fx_row2(FMat &u)
         fx_mad(mh, ml, u.ih[0][k], u.il[0][k], u.ih[1][l], u.il[1][l]);
         fx_mad(mh, ml, u.rh[0][l], u.rl[0][l], u.rh[1][k], u.rl[1][k]);
         fx_mad(ph, pl, u.ih[0][l], u.il[0][l], u.ih[1][k], u.il[1][k]);
-        fx_split<0>(fx_value(ph - mh, pl - ml), u.rh[2][j], u.rl[2][j]);
+        fx_limbs<2>(fx_value(ph - mh, pl - ml), u.rh[2][j], u.rl[2][j]);
         ph = pl = mh = ml = 0;
         fx_mad(mh, ml, u.rh[0][k], u.rl[0][k], u.ih[1][l], u.il[1][l]);
         fx_mad(mh, ml, u.ih[0][k], u.il[0][k], u.rh[1][l], u.rl[1][l]);
         fx_mad(ph, pl, u.rh[0][l], u.rl[0][l], u.ih[1][k], u.il[1][k]);
         fx_mad(ph, pl, u.ih[0][l], u.il[0][l], u.rh[1][k], u.rl[1][k]);
-        fx_split<0>(fx_value(ph - mh, pl - ml), u.ih[2][j], u.il[2][j]);
+        fx_limbs<2>(fx_value(ph - mh, pl - ml), u.ih[2][j], u.il[2][j]);
     }
 }
 
-// A real scalar of modulus at most 1.
-struct FScalar {
-    int h, l;
-};
-
-inline FScalar fx_scalar(double c)
+// The same matrix with an FP32 remainder.
+__device__ __forceinline__ FMat fx_remainder(const FLimbs &a)
 {
-    const long long v = (long long)(c * 288230376151711744.0 + (c < 0 ? -0.5 : 0.5)); // 2^58
-    FScalar s;
-    s.h = (int)((v + (1ll << (kLimb - 1))) >> kLimb);
-    s.l = (int)(v - (long long)s.h * (1ll << kLimb));
-    return s;
+    FMat m;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        m.rh[e / 3][e % 3] = a.rh[e / 3][e % 3];
+        m.rl[e / 3][e % 3] = 0x1p-28f * (float)a.rl[e / 3][e % 3];
+        m.ih[e / 3][e % 3] = a.ih[e / 3][e % 3];
+        m.il[e / 3][e % 3] = 0x1p-28f * (float)a.il[e / 3][e % 3];
+    }
+    return m;
 }
 
-// c m, in the units of m.
-__device__ __forceinline__ FInt fx_scaled(const FScalar c, const FMat &m)
-{
-    FInt r;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            long long h = 0, l = 0;
-            fx_mad(h, l, c.h, c.l, m.rh[i][j], m.rl[i][j]);
-            r.re[i][j] = fx_value(h, l);
-            h = l = 0;
-            fx_mad(h, l, c.h, c.l, m.ih[i][j], m.il[i][j]);
-            r.im[i][j] = fx_value(h, l);
-        }
-    return r;
-}
-
-// Re tr(a b), in the units of the product.
-__device__ __forceinline__ long long fx_re_trace(const FMat &a, const FMat &b)
+// Re tr(a b): high and mixed sum.
+__device__ __forceinline__ long long fx_re_trace(const FLimbs &a, const FLimbs &b)
 {
     long long h = 0, l = 0, mh = 0, ml = 0;
 #pragma unroll
@@ -234,11 +353,11 @@ __device__ __forceinline__ long long fx_re_trace(const FMat &a, const FMat &b)
     return fx_value(h - mh, l - ml);
 }
 
-// Rows 0 and 1 of a stored FP64 link as limbs, row 2 rebuilt; a link that is
-// not finite or not within 1e-3 of SU(3) is marked.
-__device__ __forceinline__ FMat fx_from_rows(const double r[12])
+// Rows 0 and 1 of a stored FP64 link, row 2 rebuilt; a link that is not
+// finite or not within 1e-3 of SU(3) is marked.
+__device__ __forceinline__ FLimbs fx_from_rows(const double r[12])
 {
-    FMat u;
+    FLimbs u;
     bool ok = true;
 #pragma unroll
     for (int e = 0; e < 6; ++e) {
@@ -247,15 +366,14 @@ __device__ __forceinline__ FMat fx_from_rows(const double r[12])
         // |x| < 1.5 by its bits (false for a NaN)
         ok = ok && (unsigned)(__double2hiint(x) & 0x7fffffff) < 0x3ff80000u &&
              (unsigned)(__double2hiint(y) & 0x7fffffff) < 0x3ff80000u;
-        fx_split<0>(__double2ll_rn(x * 288230376151711744.0), u.rh[i][j], u.rl[i][j]);
-        fx_split<0>(__double2ll_rn(y * 288230376151711744.0), u.ih[i][j], u.il[i][j]);
+        fx_limbs<0>(__double2ll_rn(x * 0x1p58), u.rh[i][j], u.rl[i][j]);
+        fx_limbs<0>(__double2ll_rn(y * 0x1p58), u.ih[i][j], u.il[i][j]);
     }
     float n0 = 0.f, n1 = 0.f, cr = 0.f, ci = 0.f;
-    constexpr float s = 1.0f / (float)(1 << kLimb);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const float ar = s * (float)u.rh[0][j], ai = s * (float)u.ih[0][j];
-        const float br = s * (float)u.rh[1][j], bi = s * (float)u.ih[1][j];
+        const float ar = 0x1p-30f * (float)u.rh[0][j], ai = 0x1p-30f * (float)u.ih[0][j];
+        const float br = 0x1p-30f * (float)u.rh[1][j], bi = 0x1p-30f * (float)u.ih[1][j];
         n0 += ar * ar + ai * ai;
         n1 += br * br + bi * bi;
         cr += ar * br + ai * bi;
@@ -267,6 +385,6 @@ __device__ __forceinline__ FMat fx_from_rows(const double r[12])
     return u;
 }
 
-__device__ __forceinline__ bool fx_poisoned(const FMat &m) { return m.rh[0][0] == kPoison; }
+template <typename M> __device__ __forceinline__ bool fx_poisoned(const M &m) { return m.rh[0][0] == kPoison; }
 
 } // namespace lqcd

@@ -1,16 +1,11 @@
 // Gauge force of the one-loop Symanzik action for FP64 fields: the
 // staple-field algorithm of force_sf.cu (same formulas, traversal and action)
 // in the fixed-point arithmetic of fixed.cuh, three passes:
-//   links_fx     the links as limbs (all three rows), planes 24..27 of the
+//   links_fx     the links in fixed point (all three rows), planes 24..27 of the
 //                workspace: every link is read about 18 times by the next two
 //                passes, so it is converted (and checked) once
 //   staples_fx   the 24 plaquette staples of every site
 //   force_fx     the force (momentum step, action) of every link
-//
-// What bounds it.  In FP64 the force is 7.3 k FMA per link on a pipe that
-// issues 2 a clock and SM (98 ms at 32^3x64 for the pipe alone); here it is
-// three integer multiply-adds each on the pipe that issues 64, and the bytes
-// (144 per staple in either form) start to count.
 //
 // A thread that reads a marked matrix (a link that is not finite or not
 // within 1e-3 of SU(3), or a staple of one) computes its staple or force in
@@ -28,19 +23,26 @@ using FxBlock = FullBlock<double>;        // 9 lanes of 16 bytes: one complex en
 struct FxPlanes {
     char *base;
     int64_t plane_bytes;
+    static constexpr int S = FxBlock::LANE / 16; // lanes of one entry
 
     __device__ __forceinline__ char *at(int n) const
     {
         return base + (int64_t)(n >> 5) * FxBlock::BYTES + (n & 31) * 16;
     }
 
-    __device__ __forceinline__ FMat load(const char *r, int plane) const
+    __device__ __forceinline__ const int4 *ptr(const char *r, int plane) const
     {
-        const int4 *p = reinterpret_cast<const int4 *>(r + (int64_t)plane * plane_bytes);
-        FMat u;
+        return reinterpret_cast<const int4 *>(r + (int64_t)plane * plane_bytes);
+    }
+
+    // A link (planes 24..27).
+    __device__ __forceinline__ FLimbs link(const char *r, int mu) const
+    {
+        const int4 *p = ptr(r, kLinkPlane + mu);
+        FLimbs u;
 #pragma unroll
         for (int e = 0; e < 9; ++e) {
-            const int4 v = __ldg(p + e * (FxBlock::LANE / 16));
+            const int4 v = __ldg(p + e * S);
             u.rh[e / 3][e % 3] = v.x;
             u.rl[e / 3][e % 3] = v.y;
             u.ih[e / 3][e % 3] = v.z;
@@ -49,13 +51,28 @@ struct FxPlanes {
         return u;
     }
 
-    // The matrix or (dag) its dagger, chosen at run time: the off-diagonal
-    // entries are read from their mirrored places.
-    __device__ __forceinline__ FMat load_form(const char *r, int plane, bool dag) const
+    // A staple (planes 0..23).
+    __device__ __forceinline__ FMat staple(const char *r, int plane) const
     {
-        const int4 *p = reinterpret_cast<const int4 *>(r + (int64_t)plane * plane_bytes);
-        constexpr int S = FxBlock::LANE / 16;
-        const int o = dag ? 2 * S : 0, m = dag ? -1 : 0;
+        const int4 *p = ptr(r, plane);
+        FMat u;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const int4 v = __ldg(p + e * S);
+            u.rh[e / 3][e % 3] = v.x;
+            u.rl[e / 3][e % 3] = __int_as_float(v.y);
+            u.ih[e / 3][e % 3] = v.z;
+            u.il[e / 3][e % 3] = __int_as_float(v.w);
+        }
+        return u;
+    }
+
+    // A staple or (is_link) a link, or (dag) its dagger, chosen at run time:
+    // the off-diagonal entries are then read from their mirrored places.
+    __device__ __forceinline__ FMat form(const char *r, int plane, bool is_link, bool dag) const
+    {
+        const int4 *p = ptr(r, plane);
+        const int o = dag ? 2 * S : 0, m = dag ? -1 : 0, f = dag ? (int)0x80000000 : 0;
         const int4 *up = p + o, *dn = p - o, *up2 = up + o, *dn2 = dn - o;
         const int4 v[9] = {__ldg(p),           __ldg(up + S),      __ldg(up2 + 2 * S), __ldg(dn + 3 * S), __ldg(p + 4 * S),
                            __ldg(up + 5 * S),  __ldg(dn2 + 6 * S), __ldg(dn + 7 * S),  __ldg(p + 8 * S)};
@@ -63,22 +80,38 @@ struct FxPlanes {
 #pragma unroll
         for (int e = 0; e < 9; ++e) {
             u.rh[e / 3][e % 3] = v[e].x;
-            u.rl[e / 3][e % 3] = v[e].y;
             u.ih[e / 3][e % 3] = (v[e].z ^ m) - m;
-            u.il[e / 3][e % 3] = (v[e].w ^ m) - m;
+            u.rl[e / 3][e % 3] = __int_as_float(v[e].y);
+            u.il[e / 3][e % 3] = __int_as_float(v[e].w);
         }
+        if (is_link) {
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                u.rl[e / 3][e % 3] = 0x1p-28f * (float)v[e].y;
+                u.il[e / 3][e % 3] = 0x1p-28f * (float)v[e].w;
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 9; ++e)
+            u.il[e / 3][e % 3] = __int_as_float(__float_as_int(u.il[e / 3][e % 3]) ^ f);
         return u;
     }
 
-    template <bool STREAM> __device__ __forceinline__ void store(char *r, int plane, const FMat &u) const
+    __device__ __forceinline__ void store_link(char *r, int mu, const FLimbs &u) const
     {
-        int4 *p = reinterpret_cast<int4 *>(r + (int64_t)plane * plane_bytes);
+        int4 *p = const_cast<int4 *>(ptr(r, kLinkPlane + mu));
 #pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            const int4 v = make_int4(u.rh[e / 3][e % 3], u.rl[e / 3][e % 3], u.ih[e / 3][e % 3], u.il[e / 3][e % 3]);
-            if constexpr (STREAM) __stcs(p + e * (FxBlock::LANE / 16), v);
-            else p[e * (FxBlock::LANE / 16)] = v;
-        }
+        for (int e = 0; e < 9; ++e)
+            p[e * S] = make_int4(u.rh[e / 3][e % 3], u.rl[e / 3][e % 3], u.ih[e / 3][e % 3], u.il[e / 3][e % 3]);
+    }
+
+    __device__ __forceinline__ void store_staple(char *r, int plane, const FMat &u) const
+    {
+        int4 *p = const_cast<int4 *>(ptr(r, plane));
+#pragma unroll
+        for (int e = 0; e < 9; ++e)
+            __stcs(p + e * S, make_int4(u.rh[e / 3][e % 3], __float_as_int(u.rl[e / 3][e % 3]), u.ih[e / 3][e % 3],
+                                        __float_as_int(u.il[e / 3][e % 3])));
     }
 };
 
@@ -88,15 +121,26 @@ __device__ __forceinline__ FxPlanes fx_planes(const SfLattice &L)
 }
 
 // Coefficients for the fixed-point sums.  With t = c_plaq Pl + c_rect Rc +
-// c_cube Cb and z the larger of c_rect, c_cube in modulus, m the larger of
-// c_plaq, z:
-//     t / m = pl Pl + z (beta Rc + alpha Cb),
-// every scalar at most 1 in modulus (use_beta: beta is not 1).
+// c_cube Cb, z the larger of c_rect, c_cube in modulus and m a quarter of the
+// largest that t can be,
+//     t / m = pl Pl + z (beta Rc + alpha Cb)
+// is at most 4 and every scalar at most 1 in modulus (use_beta: beta is not 1).
 struct FxScalars {
-    FScalar pl, z, alpha, beta;
+    int plh, pll, zh, zl; // pl and z in limbs of 2^-30 and 2^-58
+    FScalar alpha, beta;
     int use_beta;
     double m;
+    long long tr0; // Re tr(U t) / m of unit links, units 2^-58
 };
+
+// x in units of 2^-58, as limbs.
+long long limbs_of(double x, int &h, int &l)
+{
+    const long long v = (long long)(x * 0x1p58);
+    h = (int)((v + (1ll << 27)) >> 28);
+    l = (int)(v - (long long)h * (1ll << 28));
+    return v;
+}
 
 FxScalars make_fx_scalars(const KernelScalars &sc)
 {
@@ -113,13 +157,15 @@ FxScalars make_fx_scalars(const KernelScalars &sc)
         alpha = 1.0;
         beta = cr / cc;
     }
-    f.m = mod(cp) > mod(z) ? mod(cp) : mod(z);
+    f.m = 1.5 * mod(cp) + 4.5 * mod(cr) + 6.0 * mod(cc);
     if (f.m == 0.0) f.m = 1.0;
-    f.pl = fx_scalar(cp / f.m);
-    f.z = fx_scalar(z / f.m);
+    const long long pv = limbs_of(cp / f.m, f.plh, f.pll), zv = limbs_of(z / f.m, f.zh, f.zl);
     f.alpha = fx_scalar(alpha);
     f.beta = fx_scalar(beta);
     f.use_beta = beta != 1.0;
+    // with the scalars as rounded, so that unit links have no action at all
+    const long double aq = (long double)f.alpha.h + f.alpha.l, bq = (long double)f.beta.h + f.beta.l;
+    f.tr0 = (long long)(18.0L * pv + 3.0L * zv * (18.0L * bq + 24.0L * aq) / 1073741824.0L);
     return f;
 }
 
@@ -139,7 +185,7 @@ __device__ __forceinline__ void links_block(const SfLattice &L, int V, int vb)
         r[2 * q + 1] = v.y;
     }
     const FxPlanes sf = fx_planes(L);
-    sf.store<false>(sf.at(x), kLinkPlane + mu, fx_from_rows(r));
+    sf.store_link(sf.at(x), mu, fx_from_rows(r));
 }
 
 __global__ void __launch_bounds__(kBlock) links_fx(const __grid_constant__ SfLattice L)
@@ -161,13 +207,13 @@ __global__ void __launch_bounds__(kBlock) links_fx_batched(const __grid_constant
 
 // ---------------------------------------------------------------- staples
 
-// t <- op_a(a) op_b(b), rows 0 and 1 rounded to 2^-58.
-template <int FA, int FB> __device__ __forceinline__ FMat fx_mul_top2(const FMat &a, const FMat &b)
+// op_a(a) op_b(b), rows 0 and 1.
+template <int FA, int FB> __device__ __forceinline__ FLimbs fx_mul_top2(const FLimbs &a, const FLimbs &b)
 {
-    FAcc y;
+    FLimbAcc y;
     fx_zero(y);
     fx_mul_acc<FA, FB, 2>(y, a, b);
-    return fx_round<0, FA == FB ? 1 : -1, 2>(y);
+    return fx_round<FA == FB ? 1 : -1, 2>(y);
 }
 
 __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, int vb)
@@ -183,22 +229,21 @@ __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, 
     for (int iv = 0; iv < 3; ++iv) {
         const int nu = (mu + 1 + iv) & 3;
         const int vp = step32(g, c, nu, 1), vm = step32(g, c, nu, -1);
-        const int pmu = kLinkPlane + mu, pnu = kLinkPlane + nu;
         {
             // b = +nu:  U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-            const FMat a = sf.load(sf.at(xm), pnu), b = sf.load(sf.at(x + vp), pmu), d = sf.load(sf.at(x), pnu);
-            FMat s = fx_mul_top2<N, D>(fx_mul_top2<N, D>(a, b), d);
+            const FLimbs a = sf.link(sf.at(xm), nu), b = sf.link(sf.at(x + vp), mu), d = sf.link(sf.at(x), nu);
+            FLimbs s = fx_mul_top2<N, D>(fx_mul_top2<N, D>(a, b), d);
             fx_row2(s);
             if (fx_poisoned(a) || fx_poisoned(b) || fx_poisoned(d)) s.rh[0][0] = kPoison;
-            sf.store<true>(out, mu * 6 + 2 * iv, s);
+            sf.store_staple(out, mu * 6 + 2 * iv, fx_remainder(s));
         }
         {
             // b = -nu:  U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
-            const FMat a = sf.load(sf.at(xm + vm), pnu), b = sf.load(sf.at(x + vm), pmu), d = sf.load(sf.at(x + vm), pnu);
-            FMat s = fx_mul_top2<N, N>(fx_mul_top2<D, D>(a, b), d);
+            const FLimbs a = sf.link(sf.at(xm + vm), nu), b = sf.link(sf.at(x + vm), mu), d = sf.link(sf.at(x + vm), nu);
+            FLimbs s = fx_mul_top2<N, N>(fx_mul_top2<D, D>(a, b), d);
             fx_row2(s);
             if (fx_poisoned(a) || fx_poisoned(b) || fx_poisoned(d)) s.rh[0][0] = kPoison;
-            sf.store<true>(out, mu * 6 + 2 * iv + 1, s);
+            sf.store_staple(out, mu * 6 + 2 * iv + 1, fx_remainder(s));
         }
     }
 }
@@ -268,16 +313,17 @@ __device__ __noinline__ double force_link_floating(const SfLattice &L, const Ker
 // F sum_b S_b(k+rho) S_b(k), group 1 sum_b S_b(k) S_b(k-rho) E, groups 2..7
 // B_d [ alpha sum_{b perp rho, d} S_b(k+d) S^{(d)}_b(k) + beta S_d(k+d) A_d^dag ]
 // for the six directions d.  One loop, and not a piece of code for each group
-// and sign: a product is 280 instructions, and with eleven copies of it the
-// instruction cache missed (1.5 stalled cycles per instruction).  The sums
-// take 108 registers of the 255 that two CTAs per SM leave, so the total z of
-// the groups stays in shared memory.
+// and sign: a product is about 400 instructions, and with eleven copies of it
+// the instruction cache missed (1.5 stalled cycles per instruction).  The
+// total z of the groups stays in shared memory, out of the registers' way.
 template <bool ACTION>
 __device__ __forceinline__ double fx_force_link(const SfLattice &L, const KernelScalars &sc, const FxScalars &fx,
                                                 const G32 &g, const Coord &c, int k, int rho)
 {
-    __shared__ longlong2 z_s[9][kBlock]; // units 2^-56
-    longlong2 *z = &z_s[0][threadIdx.x];
+    __shared__ longlong2 zv_s[9][kBlock]; // units 2^-56
+    __shared__ float2 zc_s[9][kBlock];
+    longlong2 *zv = &zv_s[0][threadIdx.x];
+    float2 *zc = &zc_s[0][threadIdx.x];
     const FxPlanes sf = fx_planes(L);
     const int64_t V = g.V;
     const int kp = k + step32(g, c, rho, 1);
@@ -306,30 +352,33 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
                 pa = base + 2 * ib + (q & 1);
                 pb = nud * 6 + 2 * ((nub - nud - 1) & 3) + (q & 1);
                 if (q == 4) { // the rectangle along d, onto alpha times the cubes
-                    const FMat y = fx_round<2>(acc); // up to 4, units 2^-56
-                    const FInt w = fx_scaled(fx.alpha, y);
-                    fx_zero(acc);
+                    const FMat y = fx_round<32>(acc); // up to 4, units 2^-28
 #pragma unroll
                     for (int i = 0; i < 3; ++i)
 #pragma unroll
                         for (int j = 0; j < 3; ++j) {
-                            acc.h1[i][j] = 4 * w.re[i][j];
-                            acc.h3[i][j] = 4 * (w.re[i][j] + w.im[i][j]);
+                            const FSum re = fx_scaled(fx.alpha, y.rh[i][j], y.rl[i][j]);
+                            const FSum im = fx_scaled(fx.alpha, y.ih[i][j], y.il[i][j]);
+                            acc.h1[i][j] = 4 * re.v;
+                            acc.h2[i][j] = 0;
+                            acc.h3[i][j] = 4 * (re.v + im.v);
+                            acc.cr[i][j] = 4.f * re.c;
+                            acc.ci[i][j] = 4.f * im.c;
                         }
                     pa = base + 2 * id + (neg ? 1 : 0);
                     pb = kLinkPlane + nud;
                     dag = !neg;
                 }
             }
-            FMat a = sf.load(at_a, pa);
-            const FMat b = sf.load_form(at_b, pb, dag);
+            FMat a = sf.staple(at_a, pa);
+            const FMat b = sf.form(at_b, pb, pb >= kLinkPlane, dag);
             bad = bad || fx_poisoned(a) || fx_poisoned(b);
-            if (fx.use_beta && q == 4 && !chain) a = fx_round<0>(fx_scaled(fx.beta, a));
+            if (fx.use_beta && q == 4 && !chain) a = fx_scaled(fx.beta, a);
             fx_mul_acc<N, N>(acc, a, b);
         }
-        FMat y = fx_round<2>(acc);
-        if (fx.use_beta && chain) y = fx_round<0>(fx_scaled(fx.beta, y));
-        FMat x = sf.load_form(grp == 1 ? at_d : sf.at(neg ? kp + dk : kp), kLinkPlane + nud, neg);
+        FMat y = fx_round<33>(acc); // up to 6, units 2^-27
+        if (fx.use_beta && chain) y = fx_scaled(fx.beta, y);
+        FMat x = sf.form(grp == 1 ? at_d : sf.at(neg ? kp + dk : kp), kLinkPlane + nud, true, neg);
         bad = bad || fx_poisoned(x);
         if (grp == 1) {
             const FMat t = x;
@@ -340,74 +389,83 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
         fx_mul_acc<N, N>(acc, x, y);
 #pragma unroll
         for (int e = 0; e < 9; ++e) {
-            longlong2 s;
-            fx_value_of<1>(acc, e / 3, e % 3, s.x, s.y);
+            FSum re, im;
+            fx_total<1>(acc, e / 3, e % 3, re, im);
+            longlong2 v = make_longlong2(re.v >> 1, im.v >> 1);
+            float2 w = make_float2(0.5f * re.c, 0.5f * im.c);
             if (grp > 0) {
-                const longlong2 o = z[e * kBlock];
-                s.x += o.x;
-                s.y += o.y;
+                const longlong2 ov = zv[e * kBlock];
+                const float2 ow = zc[e * kBlock];
+                v.x += ov.x;
+                v.y += ov.y;
+                w.x += ow.x;
+                w.y += ow.y;
             }
-            z[e * kBlock] = s;
+            zv[e * kBlock] = v;
+            zc[e * kBlock] = w;
         }
     }
 
-    const FMat u = sf.load(sf.at(k), kLinkPlane + rho);
+    const FLimbs u = sf.link(sf.at(k), rho);
     bad = bad || fx_poisoned(u);
     if (bad) return force_link_floating<ACTION>(L, sc, k, rho);
 
-    FMat plm; // plaquette sum, units 2^-56
-    {
-        FInt pl;
+    // The plaquette sum, t / m and U t / m decide the accuracy of the result:
+    // whole limbs.
+    long long pr[9], pi[9]; // plaquette sum, up to 6, units 2^-58
 #pragma unroll
-        for (int e = 0; e < 9; ++e) pl.re[e / 3][e % 3] = pl.im[e / 3][e % 3] = 0;
+    for (int e = 0; e < 9; ++e) pr[e] = pi[e] = 0;
 #pragma unroll 1
-        for (int jj = 0; jj < 6; ++jj) {
-            const FMat s = sf.load(sf.at(k), base + jj);
+    for (int jj = 0; jj < 6; ++jj) {
+        const FMat s = sf.staple(sf.at(k), base + jj);
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    pl.re[i][j] = mad_wide(s.rh[i][j], 1 << kLimb, pl.re[i][j]) + s.rl[i][j];
-                    pl.im[i][j] = mad_wide(s.ih[i][j], 1 << kLimb, pl.im[i][j]) + s.il[i][j];
-                }
+        for (int e = 0; e < 9; ++e) {
+            pr[e] = mad_wide(s.rh[e / 3][e % 3], 1 << 28, pr[e] + __float2int_rn(0x1p28f * s.rl[e / 3][e % 3]));
+            pi[e] = mad_wide(s.ih[e / 3][e % 3], 1 << 28, pi[e] + __float2int_rn(0x1p28f * s.il[e / 3][e % 3]));
         }
-        plm = fx_round<2>(pl);
     }
-    FInt t;
+    FLimbs t; // t / m, up to 4, units 2^-28 and 2^-56
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
-        const longlong2 s = z[e * kBlock];
-        t.re[e / 3][e % 3] = s.x;
-        t.im[e / 3][e % 3] = s.y;
+        const int i = e / 3, j = e % 3;
+        const longlong2 v = zv[e * kBlock];
+        const float2 w = zc[e * kBlock];
+        const auto sum = [&](long long zval, float zrem, long long p, int &th, int &tl) {
+            int zh;
+            float zl;
+            fx_split<31>(FSum{zval, zrem}, zh, zl);    // up to 42, units 2^-25
+            const int p32 = (int)p;
+            const int ph = (int)(p >> 32) + (int)((unsigned)p32 >> 31);
+            // in units 2^-60: pl times p = ph 2^32 + p32, and z times the rest
+            const long long x = 16 * mad_wide(fx.plh, ph, 0) + (mad_wide(fx.plh, p32, 0) >> 28) +
+                                (mad_wide(fx.pll, ph, 0) >> 24) + 32 * mad_wide(fx.zh, zh, 0) +
+                                (mad_wide(fx.zl, zh, 0) >> 23) + 16ll * __float2int_rn(2.f * (float)fx.zh * zl);
+            const long long y = (x + 8) >> 4;
+            th = (int)((y + (1ll << 27)) >> 28);
+            tl = (int)((unsigned)y - ((unsigned)th << 28));
+        };
+        sum(v.x, w.x, pr[e], t.rh[i][j], t.rl[i][j]);
+        sum(v.y, w.y, pi[e], t.ih[i][j], t.il[i][j]);
     }
-    t = fx_scaled(fx.z, fx_round<3>(t)); // units 2^-53
-    const FInt tp = fx_scaled(fx.pl, plm);
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            t.re[i][j] += (tp.re[i][j] + 4) >> 3;
-            t.im[i][j] += (tp.im[i][j] + 4) >> 3;
-        }
-    FAcc acc;
+    FLimbAcc acc;
     fx_zero(acc);
-    fx_mul_acc<N, N>(acc, u, fx_round<0>(t));
-    FInt m;
+    fx_mul_acc<N, N>(acc, u, t);
+    long long re[3][3], im[3][3]; // U t / m, units 2^-58
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) fx_value_of<1>(acc, i, j, m.re[i][j], m.im[i][j]);
+        for (int j = 0; j < 3; ++j) fx_total<1>(acc, i, j, re[i][j], im[i][j]);
     // f = -(beta/6) Im tr(lambda_a U t) (ta_components)
-    const double s = -sc.d[SC_BETA6] * fx.m * 0x1p-53;
+    const double s = -sc.d[SC_BETA6] * fx.m * 0x1p-58;
     double f[8];
-    f[0] = s * (double)(m.im[0][1] + m.im[1][0]);
-    f[1] = s * (double)(m.re[0][1] - m.re[1][0]);
-    f[2] = s * (double)(m.im[0][0] - m.im[1][1]);
-    f[3] = s * (double)(m.im[0][2] + m.im[2][0]);
-    f[4] = s * (double)(m.re[0][2] - m.re[2][0]);
-    f[5] = s * (double)(m.im[1][2] + m.im[2][1]);
-    f[6] = s * (double)(m.re[1][2] - m.re[2][1]);
-    f[7] = s * 0.57735026918962576451 * (double)(m.im[0][0] + m.im[1][1] - 2 * m.im[2][2]);
+    f[0] = s * (double)(im[0][1] + im[1][0]);
+    f[1] = s * (double)(re[0][1] - re[1][0]);
+    f[2] = s * (double)(im[0][0] - im[1][1]);
+    f[3] = s * (double)(im[0][2] + im[2][0]);
+    f[4] = s * (double)(re[0][2] - re[2][0]);
+    f[5] = s * (double)(im[1][2] + im[2][1]);
+    f[6] = s * (double)(re[1][2] - re[2][1]);
+    f[7] = s * 0.57735026918962576451 * (double)(im[0][0] + im[1][1] - 2 * im[2][2]);
     if (L.force != nullptr) store_algebra(static_cast<double *>(L.force), V, rho, k, f);
     if (L.mom != nullptr) {
         double *mom = static_cast<double *>(L.mom);
@@ -419,9 +477,17 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
         store_algebra(mom, V, rho, k, p);
     }
     if constexpr (ACTION) {
-        const double tr_t = (double)(m.re[0][0] + m.re[1][1] + m.re[2][2]);
-        const double tr_pl = (double)fx_re_trace(u, plm) * 0x1p-56;
-        return fma(-sc.d[SC_ACTPL], tr_pl, fma(-fx.m * 0x1p-53 / 6.0, tr_t, sc.d[SC_ACT]));
+        // the differences from unit links, exact; share = 3 (1.5 c_plaq + 3
+        // c_rect + 4 c_cube) - Re tr(U t) / 6 - (c_plaq / 12) Re tr(U Pl)
+        const double d_t = (double)(fx.tr0 - (re[0][0] + re[1][1] + re[2][2]));
+        FLimbs p; // plaquette sum, units 2^-27 and 2^-55
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            fx_limbs<3>(pr[e], p.rh[e / 3][e % 3], p.rl[e / 3][e % 3]);
+            fx_limbs<3>(pi[e], p.ih[e / 3][e % 3], p.il[e / 3][e % 3]);
+        }
+        const double d_pl = (double)((18ll << 57) - fx_re_trace(u, p));
+        return fma(sc.d[SC_ACTPL] * 0x1p-57, d_pl, fx.m * 0x1p-58 / 6.0 * d_t);
     }
     return 0.0;
 }
