@@ -10,18 +10,20 @@
 
 #include <nvtx3/nvToolsExt.h>
 
-#include "kernels.h"
-#include "su3.cuh"
+#include "fx_planes.cuh"
+#include "sites.cuh"
 
 namespace lqcd {
 
 namespace {
 
 constexpr int kBlock = 256;
+constexpr int kActionBlock = 128; // four warps: a quarter of the loops of 32 sites each
 
-__device__ __forceinline__ double block_sum(double v)
+// Sum over a block of B threads (result in thread 0).
+template <int B> __device__ __forceinline__ double block_sum(double v)
 {
-    __shared__ double warp_part[kBlock / 32];
+    __shared__ double warp_part[B / 32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -29,7 +31,7 @@ __device__ __forceinline__ double block_sum(double v)
     __syncthreads();
     double s = 0.0;
     if (warp == 0) {
-        s = lane < kBlock / 32 ? warp_part[lane] : 0.0;
+        s = lane < B / 32 ? warp_part[lane] : 0.0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     }
@@ -49,27 +51,279 @@ __device__ __forceinline__ Mat<R> walk(const R *__restrict__ links, const Geom &
     return dagger(load_link(links, g.V, -d - 1, index_of(g, x)));
 }
 
-template <typename R>
-__global__ void __launch_bounds__(kBlock) action_partials(const ReduceArgs a, const LoopTable tab)
+// The warp of a site's four that a loop of the table belongs to: plaquettes
+// and rectangles to their first (long) direction, cubes to the direction that
+// they leave out.
+__device__ __forceinline__ int loop_owner(const Loop &lp)
+{
+    const auto dir = [](int d) { return (d > 0 ? d : -d) - 1; };
+    return lp.cls < 2 ? dir(lp.d[0]) : 6 - dir(lp.d[0]) - dir(lp.d[1]) - dir(lp.d[2]);
+}
+
+// sum c_P (3 - Re tr P) over the loops of warp w at site n, each walked link
+// by link in floating point: for FP64 links without a fixed-point form.
+__device__ __noinline__ double walked_loops(const ReduceArgs &a, const LoopTable &tab, int64_t n, int w)
 {
     const Geom g = make_geom(a.dims);
-    const R *__restrict__ links = static_cast<const R *>(a.links);
+    const double *links = static_cast<const double *>(a.links);
+    const Coord x0 = coord_of(g, n);
     double acc = 0.0;
-    for (int64_t n = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; n < g.V;
-         n += (int64_t)gridDim.x * blockDim.x) {
-        const Coord x0 = coord_of(g, n);
-        for (int l = 0; l < tab.count; ++l) {
-            const Loop &lp = tab.l[l];
-            Coord x = x0;
-            Mat<R> m = walk(links, g, x, lp.d[0]);
-            for (int j = 1; j < lp.len - 1; ++j) m = mul<N, N>(m, walk(links, g, x, lp.d[j]));
-            const R retr = re_trace_mul<N, N>(m, walk(links, g, x, lp.d[lp.len - 1]));
-            const double c = lp.cls == 0 ? a.c[0] : (lp.cls == 1 ? a.c[1] : a.c[2]);
-            acc += c * (3.0 - (double)retr);
+    for (int l = 0; l < tab.count; ++l) {
+        const Loop &lp = tab.l[l];
+        if (loop_owner(lp) != w) continue;
+        Coord x = x0;
+        // the four cube loops of a site are those of the cube it is the lowest
+        // corner of: one with a step down starts from above
+        if (lp.cls == 2)
+            for (int j = 1; j < 3; ++j)
+                if (lp.d[j] < 0) step(g, x, -lp.d[j] - 1, 1);
+        Mat<double> m = walk(links, g, x, lp.d[0]);
+        for (int j = 1; j < lp.len - 1; ++j) m = mul<N, N>(m, walk(links, g, x, lp.d[j]));
+        const double retr = re_trace_mul<N, N>(m, walk(links, g, x, lp.d[lp.len - 1]));
+        acc += (lp.cls == 0 ? a.c[0] : (lp.cls == 1 ? a.c[1] : a.c[2])) * (3.0 - retr);
+    }
+    return acc;
+}
+
+// The arithmetic of the action kernel.  FP32: matrices in FP32, a class's
+// traces in a sum with its rounding errors kept (FP64 additions, 2 a clock
+// and SM, would take as long as a third of the products).
+struct Plain {
+    using M = Mat<float>;
+    static constexpr int kMinBlocks = 4, kWords = 18;
+    using Word = float;
+    const float *links;
+    int64_t V;
+
+    __device__ __forceinline__ explicit Plain(const ReduceArgs &a, int64_t v)
+        : links(static_cast<const float *>(a.links)), V(v)
+    {
+    }
+    __device__ __forceinline__ M link(int mu, int64_t n) const { return load_link(links, V, mu, n); }
+    template <int FB> __device__ __forceinline__ static M mul(const M &x, const M &y) { return lqcd::mul<N, FB>(x, y); }
+    __device__ __forceinline__ static bool bad(const M &) { return false; }
+    __device__ __forceinline__ static void mark(M &) {}
+    template <int STRIDE> __device__ __forceinline__ static void put(Word *p, const M &x)
+    {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            p[2 * e * STRIDE] = x.re[e / 3][e % 3];
+            p[(2 * e + 1) * STRIDE] = x.im[e / 3][e % 3];
         }
     }
-    const double s = block_sum(acc);
+    template <int STRIDE> __device__ __forceinline__ static M get(const Word *p)
+    {
+        M x;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            x.re[e / 3][e % 3] = p[2 * e * STRIDE];
+            x.im[e / 3][e % 3] = p[(2 * e + 1) * STRIDE];
+        }
+        return x;
+    }
+    struct Traces {
+        float s = 0.f, e = 0.f;
+        // + Re tr(x y^dag)
+        __device__ __forceinline__ void add(const M &x, const M &y)
+        {
+            const float t = re_trace_mul<N, D>(x, y), u = s + t, b = u - s;
+            e += (s - (u - b)) + (t - b);
+            s = u;
+        }
+        // 3 n - the sum
+        __device__ __forceinline__ double below(int n) const { return (3.0 * n - (double)s) - (double)e; }
+    };
+};
+
+// FP64: the fixed point of fixed.cuh (FP32 remainders: their rounding is
+// random from loop to loop, 2^-54 of one); the class sums are exact.  Links
+// from planes made once per call (PLANES), or converted at each of their 23
+// reads: two operations per real on the FP64 pipe, which then bounds the
+// kernel, for callers without a workspace for the planes; the same bits.
+template <bool PLANES> struct Fixed {
+    using M = FMat;
+    static constexpr int kMinBlocks = 2, kWords = 9;
+    using Word = int4;
+    FxPlanes planes;
+    const double *links;
+    int64_t V;
+
+    __device__ __forceinline__ explicit Fixed(const ReduceArgs &a, int64_t v)
+        : planes{static_cast<char *>(a.planes), (v + 31) / 32 * FxPlanes::BYTES},
+          links(static_cast<const double *>(a.links)), V(v)
+    {
+    }
+    __device__ __forceinline__ M link(int mu, int64_t n) const
+    {
+        if constexpr (PLANES) return planes.mat(planes.at(n), mu);
+        else return fx_remainder(fx_load_link(links, V, mu, n));
+    }
+    template <int FB> __device__ __forceinline__ static M mul(const M &x, const M &y)
+    {
+        FAcc acc;
+        fx_zero(acc);
+        fx_mul_acc<N, FB>(acc, x, y);
+        return fx_round<kUnit, FB == N ? 1 : -1>(acc);
+    }
+    __device__ __forceinline__ static bool bad(const M &x) { return fx_poisoned(x); }
+    __device__ __forceinline__ static void mark(M &x) { x.rh[0][0] = kPoison; }
+    template <int STRIDE> __device__ __forceinline__ static void put(Word *p, const M &x)
+    {
+#pragma unroll
+        for (int e = 0; e < 9; ++e)
+            p[e * STRIDE] = make_int4(x.rh[e / 3][e % 3], __float_as_int(x.rl[e / 3][e % 3]), x.ih[e / 3][e % 3],
+                                      __float_as_int(x.il[e / 3][e % 3]));
+    }
+    template <int STRIDE> __device__ __forceinline__ static M get(const Word *p)
+    {
+        M x;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const int4 v = p[e * STRIDE];
+            x.rh[e / 3][e % 3] = v.x;
+            x.rl[e / 3][e % 3] = __int_as_float(v.y);
+            x.ih[e / 3][e % 3] = v.z;
+            x.il[e / 3][e % 3] = __int_as_float(v.w);
+        }
+        return x;
+    }
+    struct Traces {
+        long long v = 0; // units 2^-56
+        float c = 0.f;
+        __device__ __forceinline__ void add(const M &x, const M &y)
+        {
+            const FSum t = fx_re_trace_dag(x, y); // units 2^-60
+            v += (t.v + 8) >> 4;
+            c = fmaf(0.0625f, t.c, c);
+        }
+        __device__ __forceinline__ double below(int n) const
+        {
+            return ((double)(((3ll * n) << 56) - v) - (double)c) * 0x1p-56;
+        }
+    };
+};
+
+// The loops of 32 sites per block, a quarter of them on each of its four
+// warps.  From the corners L_{mu nu}(n) = U_mu(n) U_nu(n+mu), three per warp
+// and shared, every loop is the trace of a product X Y^dag of two halves:
+//   plaquette            X = L_{mu nu},                  Y = L_{nu mu}
+//   rectangle            X = U_mu U_mu(+mu) U_nu(+2mu),  Y = L_{nu mu} U_mu(+mu+nu)
+//   cube from n          X = L_{xy} U_z(+x+y),           Y = L_{zy} U_x(+z+y),
+// (x, y, z) the three rotations of the directions that warp w leaves out w
+// of; and the cube loop that misses n and its opposite corner,
+//   X = U_b(+a) U_a(+b)^dag U_c(+b),  Y = U_c(+a) U_a(+c)^dag U_b(+c).
+// 80 matrix products and 92 link loads per site against 124 and 192 for the
+// loops walked one by one.  Rolled loops: the halves are one piece of code
+// for six of a warp's loops, as the instruction cache holds few of the
+// fixed-point products.
+template <typename P, typename I>
+__global__ void __launch_bounds__(kActionBlock, P::kMinBlocks)
+    action_loops(const __grid_constant__ ReduceArgs a, const __grid_constant__ LoopTable tab)
+{
+    using M = typename P::M;
+    using Word = typename P::Word;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const Sites<I> g = make_sites<I>(a.dims);
+    const P src(a, (int64_t)g.V);
+    const int w = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+    // 12 corners of 32 sites, then one matrix of each thread
+    Word *corners = reinterpret_cast<Word *>(smem) + lane;
+    Word *own = reinterpret_cast<Word *>(smem) + 12 * P::kWords * 32 + threadIdx.x;
+    const auto corner = [&](int mu, int nu) { return corners + (mu * 3 + ((nu - mu) & 3) - 1) * (P::kWords * 32); };
+    double acc = 0.0;
+    const I nvb = (g.V + 31) / 32;
+    for (I vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
+        const I site = vb * 32 + lane;
+        const I n = site < g.V ? site : g.V - 1;
+        Coord c;
+        if constexpr (sizeof(I) == 4) c = coord_fast(g, a.div, n);
+        else c = coord_in(g, n);
+        const auto up = [&](int mu) { return hop_offset(g, c, mu, 1); };
+        const I ow = up(w);
+        bool bad = false;
+        {
+            const M u = src.link(w, n);
+            bad = P::bad(u);
+#pragma unroll 1
+            for (int j = 0; j < 4; ++j) {
+                const M y = src.link((w + j) & 3, n + ow);
+                M p = P::template mul<N>(u, y);
+                if (P::bad(u) || P::bad(y)) {
+                    P::mark(p);
+                    bad = true;
+                }
+                if (j == 0) P::template put<kActionBlock>(own, p);
+                else P::template put<32>(corner(w, (w + j) & 3), p);
+            }
+        }
+        __syncthreads();
+        typename P::Traces pl, rc, cb;
+#pragma unroll 1
+        for (int nu = w + 1; nu < 4; ++nu) {
+            const M x = P::template get<32>(corner(w, nu)), y = P::template get<32>(corner(nu, w));
+            bad = bad || P::bad(x) || P::bad(y);
+            pl.add(x, y);
+        }
+#pragma unroll 1
+        for (int it = 0; it < 6; ++it) {
+            // X = A B, Y = C D
+            const int x = (w + 1 + it % 3) & 3;
+            const int y = it < 3 ? w : (w + 1 + (it + 1) % 3) & 3, z = it < 3 ? w : (w + 1 + (it + 2) % 3) & 3;
+            I nb, nd;
+            if (it < 3) { // rectangle, x = nu
+                Coord c1 = c;
+                step_up(g, c1, w);
+                nb = n + ow + hop_offset(g, c1, w, 1);
+                nd = n + ow + up(x);
+            } else {
+                nb = n + up(x) + up(y);
+                nd = n + up(z) + up(y);
+            }
+            M h;
+            {
+                const M A = it < 3 ? P::template get<kActionBlock>(own) : P::template get<32>(corner(x, y));
+                const M B = src.link(it < 3 ? x : z, nb);
+                bad = bad || P::bad(A) || P::bad(B);
+                h = P::template mul<N>(A, B);
+            }
+            const M C = P::template get<32>(it < 3 ? corner(x, w) : corner(z, y));
+            const M E = src.link(it < 3 ? w : x, nd);
+            bad = bad || P::bad(C) || P::bad(E);
+            const M k = P::template mul<N>(C, E);
+            if (it < 3) rc.add(h, k);
+            else cb.add(h, k);
+        }
+        {
+            const int da = (w + 1) & 3;
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                const int p = (w + (h == 0 ? 2 : 3)) & 3, q = (w + (h == 0 ? 3 : 2)) & 3;
+                const M A = src.link(p, n + up(da)), B = src.link(da, n + up(p)), E = src.link(q, n + up(p));
+                bad = bad || P::bad(A) || P::bad(B) || P::bad(E);
+                const M z = P::template mul<N>(P::template mul<D>(A, B), E);
+                if (h == 0) P::template put<kActionBlock>(own, z);
+                else cb.add(P::template get<kActionBlock>(own), z);
+            }
+        }
+        if (site < g.V) {
+            if (bad) acc += walked_loops(a, tab, (int64_t)n, w);
+            else acc += a.c[0] * pl.below(3 - w) + a.c[1] * rc.below(3) + a.c[2] * cb.below(4);
+        }
+        __syncthreads(); // before the corners of the next sites
+    }
+    const double s = block_sum<kActionBlock>(acc);
     if (threadIdx.x == 0) a.partials[blockIdx.x] = s;
+}
+
+// The links of FP64 fields as planes with FP32 remainders, for action_loops.
+__global__ void __launch_bounds__(kBlock) action_planes(const double *__restrict__ links, FxPlanes planes, int64_t V)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 4 * V;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int mu = (int)(i >= V) + (int)(i >= 2 * V) + (int)(i >= 3 * V);
+        const int64_t n = i - mu * V;
+        planes.store<false>(planes.at(n), mu, fx_remainder(fx_load_link(links, V, mu, n)));
+    }
 }
 
 template <typename R> __global__ void __launch_bounds__(kBlock) kinetic_partials(const ReduceArgs a)
@@ -87,7 +341,7 @@ template <typename R> __global__ void __launch_bounds__(kBlock) kinetic_partials
 #pragma unroll
         for (int c = 0; c < 8; ++c) acc += 0.5 * (double)p[c] * (double)p[c];
     }
-    const double s = block_sum(acc);
+    const double s = block_sum<kBlock>(acc);
     if (threadIdx.x == 0) a.partials[blockIdx.x] = s;
 }
 
@@ -199,13 +453,39 @@ int reduction_blocks(int device)
     return cached[device];
 }
 
-cudaError_t launch_action(const ReduceArgs &a, cudaStream_t st)
+template <typename P, typename I> static cudaError_t launch_action_t(const ReduceArgs &a, cudaStream_t st)
 {
-    if (a.precision == LQCD_F64)
-        action_partials<double><<<a.blocks, kBlock, 0, st>>>(a, loop_table());
-    else
-        action_partials<float><<<a.blocks, kBlock, 0, st>>>(a, loop_table());
-    cudaError_t e = cudaGetLastError();
+    constexpr int bytes = (12 * 32 + kActionBlock) * P::kWords * (int)sizeof(typename P::Word);
+    if constexpr (bytes > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(action_loops<P, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+    }
+    action_loops<P, I><<<a.blocks, kActionBlock, bytes, st>>>(a, loop_table());
+    return cudaGetLastError();
+}
+
+size_t action_plane_bytes(const int dims[4])
+{
+    return 4 * fx_plane_bytes((int64_t)dims[0] * dims[1] * dims[2] * dims[3]);
+}
+
+cudaError_t launch_action(const ReduceArgs &args, cudaStream_t st)
+{
+    ReduceArgs a = args;
+    stride_magic(a.dims, a.div);
+    const int64_t V = (int64_t)a.dims[0] * a.dims[1] * a.dims[2] * a.dims[3];
+    const bool i32 = sites_fit_int(V);
+    cudaError_t e;
+    if (a.precision != LQCD_F64) {
+        e = i32 ? launch_action_t<Plain, int>(a, st) : launch_action_t<Plain, int64_t>(a, st);
+    } else if (a.planes != nullptr && i32) {
+        const FxPlanes p{static_cast<char *>(a.planes), (int64_t)fx_plane_bytes(V)};
+        action_planes<<<(unsigned)((4 * V + kBlock - 1) / kBlock), kBlock, 0, st>>>(static_cast<const double *>(a.links), p, V);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = launch_action_t<Fixed<true>, int>(a, st);
+    } else {
+        e = i32 ? launch_action_t<Fixed<false>, int>(a, st) : launch_action_t<Fixed<false>, int64_t>(a, st);
+    }
     if (e != cudaSuccess) return e;
     finish_sum<<<1, kFinish, 0, st>>>(a.partials, a.blocks, a.scale, a.out);
     return cudaGetLastError();

@@ -444,6 +444,10 @@ int lqcd_gauge_action(const lqcd_desc *desc, const void *links, double *action, 
     a.partials = static_cast<double *>(workspace);
     a.blocks = blocks;
     a.out = action;
+    // FP64 links are converted once per call where the workspace has room
+    const size_t head = round256((size_t)blocks * sizeof(double));
+    if (desc->precision == LQCD_F64 && workspace_bytes >= head && workspace_bytes - head >= lqcd::action_plane_bytes(desc->dims))
+        a.planes = static_cast<char *>(workspace) + head;
     return cuda_status(lqcd::launch_action(a, as_stream(stream)));
 }
 

@@ -214,6 +214,24 @@ __device__ __forceinline__ FMat fx_scaled(const FScalar c, const FMat &m)
     return r;
 }
 
+// Re tr(a b^dag), in the units of the product.
+__device__ __forceinline__ FSum fx_re_trace_dag(const FMat &a, const FMat &b)
+{
+    FSum s{0, 0.f};
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            s.v = mad_wide(a.rh[i][k], b.rh[i][k], s.v);
+            s.v = mad_wide(a.ih[i][k], b.ih[i][k], s.v);
+            s.c = fmaf((float)a.rh[i][k], b.rl[i][k], s.c);
+            s.c = fmaf(a.rl[i][k], (float)b.rh[i][k], s.c);
+            s.c = fmaf((float)a.ih[i][k], b.il[i][k], s.c);
+            s.c = fmaf(a.il[i][k], (float)b.ih[i][k], s.c);
+        }
+    return s;
+}
+
 // ------------------------------------------------------------ whole limbs
 
 __device__ __forceinline__ void fx_zero(FLimbAcc &y)

@@ -10,111 +10,14 @@
 // A thread that reads a marked matrix (a link that is not finite or not
 // within 1e-3 of SU(3), or a staple of one) computes its staple or force in
 // floating point from the stored links instead.
+#include "fx_planes.cuh"
 #include "sf_common.cuh"
-#include "fixed.cuh"
 
 namespace lqcd {
 
 namespace {
 
 constexpr int kLinkPlane = kStaplePlanes; // planes 24..27: the links
-using FxBlock = FullBlock<double>;        // 9 lanes of 16 bytes: one complex entry each
-
-struct FxPlanes {
-    char *base;
-    int64_t plane_bytes;
-    static constexpr int S = FxBlock::LANE / 16; // lanes of one entry
-
-    __device__ __forceinline__ char *at(int n) const
-    {
-        return base + (int64_t)(n >> 5) * FxBlock::BYTES + (n & 31) * 16;
-    }
-
-    __device__ __forceinline__ const int4 *ptr(const char *r, int plane) const
-    {
-        return reinterpret_cast<const int4 *>(r + (int64_t)plane * plane_bytes);
-    }
-
-    // A link (planes 24..27).
-    __device__ __forceinline__ FLimbs link(const char *r, int mu) const
-    {
-        const int4 *p = ptr(r, kLinkPlane + mu);
-        FLimbs u;
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            const int4 v = __ldg(p + e * S);
-            u.rh[e / 3][e % 3] = v.x;
-            u.rl[e / 3][e % 3] = v.y;
-            u.ih[e / 3][e % 3] = v.z;
-            u.il[e / 3][e % 3] = v.w;
-        }
-        return u;
-    }
-
-    // A staple (planes 0..23).
-    __device__ __forceinline__ FMat staple(const char *r, int plane) const
-    {
-        const int4 *p = ptr(r, plane);
-        FMat u;
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            const int4 v = __ldg(p + e * S);
-            u.rh[e / 3][e % 3] = v.x;
-            u.rl[e / 3][e % 3] = __int_as_float(v.y);
-            u.ih[e / 3][e % 3] = v.z;
-            u.il[e / 3][e % 3] = __int_as_float(v.w);
-        }
-        return u;
-    }
-
-    // A staple or (is_link) a link, or (dag) its dagger, chosen at run time:
-    // the off-diagonal entries are then read from their mirrored places.
-    __device__ __forceinline__ FMat form(const char *r, int plane, bool is_link, bool dag) const
-    {
-        const int4 *p = ptr(r, plane);
-        const int o = dag ? 2 * S : 0, m = dag ? -1 : 0, f = dag ? (int)0x80000000 : 0;
-        const int4 *up = p + o, *dn = p - o, *up2 = up + o, *dn2 = dn - o;
-        const int4 v[9] = {__ldg(p),           __ldg(up + S),      __ldg(up2 + 2 * S), __ldg(dn + 3 * S), __ldg(p + 4 * S),
-                           __ldg(up + 5 * S),  __ldg(dn2 + 6 * S), __ldg(dn + 7 * S),  __ldg(p + 8 * S)};
-        FMat u;
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            u.rh[e / 3][e % 3] = v[e].x;
-            u.ih[e / 3][e % 3] = (v[e].z ^ m) - m;
-            u.rl[e / 3][e % 3] = __int_as_float(v[e].y);
-            u.il[e / 3][e % 3] = __int_as_float(v[e].w);
-        }
-        if (is_link) {
-#pragma unroll
-            for (int e = 0; e < 9; ++e) {
-                u.rl[e / 3][e % 3] = 0x1p-28f * (float)v[e].y;
-                u.il[e / 3][e % 3] = 0x1p-28f * (float)v[e].w;
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < 9; ++e)
-            u.il[e / 3][e % 3] = __int_as_float(__float_as_int(u.il[e / 3][e % 3]) ^ f);
-        return u;
-    }
-
-    __device__ __forceinline__ void store_link(char *r, int mu, const FLimbs &u) const
-    {
-        int4 *p = const_cast<int4 *>(ptr(r, kLinkPlane + mu));
-#pragma unroll
-        for (int e = 0; e < 9; ++e)
-            p[e * S] = make_int4(u.rh[e / 3][e % 3], u.rl[e / 3][e % 3], u.ih[e / 3][e % 3], u.il[e / 3][e % 3]);
-    }
-
-    __device__ __forceinline__ void store_staple(char *r, int plane, const FMat &u) const
-    {
-        int4 *p = const_cast<int4 *>(ptr(r, plane));
-#pragma unroll
-        for (int e = 0; e < 9; ++e)
-            __stcs(p + e * S, make_int4(u.rh[e / 3][e % 3], __float_as_int(u.rl[e / 3][e % 3]), u.ih[e / 3][e % 3],
-                                        __float_as_int(u.il[e / 3][e % 3])));
-    }
-};
-
 __device__ __forceinline__ FxPlanes fx_planes(const SfLattice &L)
 {
     return FxPlanes{static_cast<char *>(L.staples), L.plane_bytes};
@@ -176,16 +79,8 @@ __device__ __forceinline__ void links_block(const SfLattice &L, int V, int vb)
     const int mu = (int)(threadIdx.x >> 5);
     const int x = vb * 32 + (int)(threadIdx.x & 31);
     if (x >= V) return;
-    const double2 *p = static_cast<const double2 *>(L.links) + (int64_t)mu * 6 * V + x;
-    double r[12];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        const double2 v = __ldg(p + (int64_t)q * V);
-        r[2 * q] = v.x;
-        r[2 * q + 1] = v.y;
-    }
     const FxPlanes sf = fx_planes(L);
-    sf.store_link(sf.at(x), mu, fx_from_rows(r));
+    sf.store(sf.at(x), kLinkPlane + mu, fx_load_link(static_cast<const double *>(L.links), V, mu, x));
 }
 
 __global__ void __launch_bounds__(kBlock) links_fx(const __grid_constant__ SfLattice L)
@@ -231,19 +126,19 @@ __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, 
         const int vp = step32(g, c, nu, 1), vm = step32(g, c, nu, -1);
         {
             // b = +nu:  U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-            const FLimbs a = sf.link(sf.at(xm), nu), b = sf.link(sf.at(x + vp), mu), d = sf.link(sf.at(x), nu);
+            const FLimbs a = sf.limbs(sf.at(xm), kLinkPlane + nu), b = sf.limbs(sf.at(x + vp), kLinkPlane + mu), d = sf.limbs(sf.at(x), kLinkPlane + nu);
             FLimbs s = fx_mul_top2<N, D>(fx_mul_top2<N, D>(a, b), d);
             fx_row2(s);
             if (fx_poisoned(a) || fx_poisoned(b) || fx_poisoned(d)) s.rh[0][0] = kPoison;
-            sf.store_staple(out, mu * 6 + 2 * iv, fx_remainder(s));
+            sf.store<true>(out, mu * 6 + 2 * iv, fx_remainder(s));
         }
         {
             // b = -nu:  U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
-            const FLimbs a = sf.link(sf.at(xm + vm), nu), b = sf.link(sf.at(x + vm), mu), d = sf.link(sf.at(x + vm), nu);
+            const FLimbs a = sf.limbs(sf.at(xm + vm), kLinkPlane + nu), b = sf.limbs(sf.at(x + vm), kLinkPlane + mu), d = sf.limbs(sf.at(x + vm), kLinkPlane + nu);
             FLimbs s = fx_mul_top2<N, N>(fx_mul_top2<D, D>(a, b), d);
             fx_row2(s);
             if (fx_poisoned(a) || fx_poisoned(b) || fx_poisoned(d)) s.rh[0][0] = kPoison;
-            sf.store_staple(out, mu * 6 + 2 * iv + 1, fx_remainder(s));
+            sf.store<true>(out, mu * 6 + 2 * iv + 1, fx_remainder(s));
         }
     }
 }
@@ -370,7 +265,7 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
                     dag = !neg;
                 }
             }
-            FMat a = sf.staple(at_a, pa);
+            FMat a = sf.mat(at_a, pa);
             const FMat b = sf.form(at_b, pb, pb >= kLinkPlane, dag);
             bad = bad || fx_poisoned(a) || fx_poisoned(b);
             if (fx.use_beta && q == 4 && !chain) a = fx_scaled(fx.beta, a);
@@ -406,7 +301,7 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
         }
     }
 
-    const FLimbs u = sf.link(sf.at(k), rho);
+    const FLimbs u = sf.limbs(sf.at(k), kLinkPlane + rho);
     bad = bad || fx_poisoned(u);
     if (bad) return force_link_floating<ACTION>(L, sc, k, rho);
 
@@ -417,7 +312,7 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
     for (int e = 0; e < 9; ++e) pr[e] = pi[e] = 0;
 #pragma unroll 1
     for (int jj = 0; jj < 6; ++jj) {
-        const FMat s = sf.staple(sf.at(k), base + jj);
+        const FMat s = sf.mat(sf.at(k), base + jj);
 #pragma unroll
         for (int e = 0; e < 9; ++e) {
             pr[e] = mad_wide(s.rh[e / 3][e % 3], 1 << 28, pr[e] + __float2int_rn(0x1p28f * s.rl[e / 3][e % 3]));

@@ -160,7 +160,12 @@ struct ReduceArgs {
     double *partials;  // workspace, one double per block
     int blocks;
     double *out;
+    void *planes;      // action of FP64 links: room for action_plane_bytes, or NULL
+    DivMagic div[3];   // action: the strides' magic (set by the launcher)
 };
+
+// Bytes of the four planes of an FP64 link field in fixed point.
+size_t action_plane_bytes(const int dims[4]);
 
 int reduction_blocks(int device);
 // out = scale * (sum of partials[0..count)), one block, fixed order.

@@ -6,6 +6,7 @@
 
 #include <mutex>
 
+#include "fx_planes.cuh"
 #include "kernels.h"
 #include "su3.cuh"
 
@@ -53,8 +54,7 @@ template <typename R> struct FullBlock {
 
 inline size_t full_plane_bytes(int64_t V, int precision)
 {
-    const size_t blk = precision == LQCD_F64 ? FullBlock<double>::BYTES : FullBlock<float>::BYTES;
-    return (size_t)((V + 31) / 32) * blk;
+    return precision == LQCD_F64 ? fx_plane_bytes(V) : (size_t)((V + 31) / 32) * FullBlock<float>::BYTES;
 }
 
 // Compact planes: the first two rows (12 reals) of every staple, the third

@@ -7,8 +7,7 @@
 // neighbours come from L1/L2 (a time slice of a 32^3 spinor field is 3 MB),
 // and every (1 -+ gamma_mu) is applied as a spin projection to two colour
 // vectors, so that each link multiplies two colour vectors instead of four.
-#include "kernels.h"
-#include "su3.cuh"
+#include "sites.cuh"
 
 namespace lqcd {
 namespace {
@@ -65,71 +64,6 @@ template <typename R> struct Spinor {
 template <typename R> struct Half {
     R re[2][3], im[2][3];
 };
-
-// ------------------------------------------------------- site geometry
-
-// Site coordinates and neighbour indices in type I: int whenever the site
-// loops fit (2 V + a block below 2^31), so that the divisions of the site
-// index and the neighbour offsets take 32-bit arithmetic (a 64-bit division
-// is a long software sequence); the 16-byte lane addresses stay 64-bit.
-// Measured at 32^3x64 FP32: hopping operator 0.176 -> 0.168 ms, force 0.281
-// -> 0.246 ms (32-bit lane addresses as well were slower: 0.171, 0.289).
-template <typename I> struct Sites {
-    int L0, L1, L2, L3;
-    I s1, s2, s3, V;
-};
-
-template <typename I> __device__ __forceinline__ Sites<I> make_sites(const int dims[4])
-{
-    Sites<I> g;
-    g.L0 = dims[0];
-    g.L1 = dims[1];
-    g.L2 = dims[2];
-    g.L3 = dims[3];
-    g.s1 = dims[0];
-    g.s2 = g.s1 * dims[1];
-    g.s3 = g.s2 * dims[2];
-    g.V = g.s3 * dims[3];
-    return g;
-}
-
-// Coordinates of site n < 2^31 with the strides' division magic (three
-// multiply-highs instead of three divisions by run-time values: hopping
-// force 0.242 -> 0.234 ms at 32^3x64 FP32).
-__device__ __forceinline__ Coord coord_fast(const Sites<int> &g, const DivMagic div[3], int n)
-{
-    Coord x;
-    x.c3 = (int)div_by((unsigned)n, div[2]);
-    int r = n - x.c3 * g.s3;
-    x.c2 = (int)div_by((unsigned)r, div[1]);
-    r -= x.c2 * g.s2;
-    x.c1 = (int)div_by((unsigned)r, div[0]);
-    x.c0 = r - x.c1 * g.s1;
-    return x;
-}
-
-template <typename I> __device__ __forceinline__ Coord coord_in(const Sites<I> &g, I n)
-{
-    Coord x;
-    x.c3 = (int)(n / g.s3);
-    I r = n - x.c3 * g.s3;
-    x.c2 = (int)(r / g.s2);
-    r -= x.c2 * g.s2;
-    x.c1 = (int)(r / g.s1);
-    x.c0 = (int)(r - x.c1 * g.s1);
-    return x;
-}
-
-// Index offset of the step s * hat(mu) (s = +-1), periodic.
-template <typename I>
-__device__ __forceinline__ I hop_offset(const Sites<I> &g, const Coord &x, int mu, int s)
-{
-    const int L = pick(mu, g.L0, g.L1, g.L2, g.L3);
-    const int c = pick(mu, x.c0, x.c1, x.c2, x.c3);
-    const I st = mu == 0 ? I(1) : (mu == 1 ? g.s1 : (mu == 2 ? g.s2 : g.s3));
-    if (s > 0) return c + 1 == L ? (I)(1 - L) * st : st;
-    return c == 0 ? (I)(L - 1) * st : -st;
-}
 
 // ------------------------------------------------------------ spinor I/O
 
@@ -462,17 +396,11 @@ unsigned blocks_for(int64_t items, int per_block)
     return (unsigned)b;
 }
 
-// Site loops in int: n + grid stride stays below 2 V + a block.
-bool sites_fit_int(int64_t V) { return 2 * V + 1024 < ((int64_t)1 << 31); }
-
 // The launch copy of the arguments: FP32 scalars and the strides' division
 // magic filled in.
 WilsonArgs launch_args(WilsonArgs a)
 {
-    const int64_t s[3] = {a.dims[0], (int64_t)a.dims[0] * a.dims[1],
-                          (int64_t)a.dims[0] * a.dims[1] * a.dims[2]};
-    for (int i = 0; i < 3; ++i)
-        a.div[i] = div_magic(s[i] < ((int64_t)1 << 31) ? (unsigned)s[i] : 1u);
+    stride_magic(a.dims, a.div);
     a.fca = (float)a.ca;
     a.fcb = (float)a.cb;
     a.fcoef = (float)a.coef;

@@ -102,7 +102,7 @@ def hamiltonian(st: MDState, action_precision: str | None = None) -> float:
         S = lqcd.gauge_action(lat, st.links, workspace=st.workspace)
     else:
         lat2 = lat.with_(precision=prec)
-        S = lqcd.gauge_action(lat2, lqcd.convert_links(lat, st.links, prec))
+        S = lqcd.gauge_action(lat2, lqcd.convert_links(lat, st.links, prec), workspace=st.workspace)
     return float(K.item()) + float(S.item())
 
 
