@@ -6,6 +6,7 @@
 //   links from omega  U = exp(i sum_a omega^a T_a)    (Eq. 18_1_29_3)
 //   pack / unpack  full 3x3 complex <-> first two rows
 #include "kernels.h"
+#include "link_step_fx.cuh"
 #include "su3.cuh"
 
 namespace lqcd {
@@ -19,9 +20,9 @@ int64_t volume(const int dims[4])
     return (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
 }
 
-unsigned grid_for(int64_t items)
+unsigned grid_for(int64_t items, int block = kBlock)
 {
-    int64_t g = (items + kBlock - 1) / kBlock;
+    int64_t g = (items + block - 1) / block;
     if (g < 1) g = 1;
     if (g > ((int64_t)1 << 30)) g = (int64_t)1 << 30;
     return (unsigned)g;
@@ -57,79 +58,17 @@ __global__ void __launch_bounds__(kBlock) update_momenta(typename Vec<R>::type *
     }
 }
 
-// U <- exp(i dt P) U (FROM_UNIT: U = exp(i dt P)), rows 0 and 1 only, then
-// Gram-Schmidt.  The link and algebra planes share the site index.
+// U <- exp(i P) U (FROM_UNIT: U = exp(i P)), rows 0 and 1 only, then
+// Gram-Schmidt, for one link; p the components of P.
 template <typename R, bool FROM_UNIT>
-__global__ void __launch_bounds__(kBlock) update_links(R *__restrict__ links,
-                                                       const R *__restrict__ mom, int64_t V, R dt)
+__device__ __forceinline__ void link_step(R *__restrict__ links, const R p[8], int64_t V, int mu, int64_t n)
 {
-    const int64_t nlinks = 4 * V;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nlinks;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int mu = direction_of(i, V);
-        const int64_t n = i - mu * V;
-        R p[8];
-        load_algebra(mom, V, mu, n, p);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) p[c] *= dt;
-        const Mat<R> e = exp_i_hermitian(algebra_matrix(p));
-        Mat<R> u;
-        if constexpr (FROM_UNIT) {
-            u = e;
-        } else {
-            const Mat<R> v = load_link(links, V, mu, n);
-#pragma unroll
-            for (int r = 0; r < 2; ++r)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    R re = R(0), im = R(0);
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        re = fma(e.re[r][k], v.re[k][j], re);
-                        re = fma(-e.im[r][k], v.im[k][j], re);
-                        im = fma(e.re[r][k], v.im[k][j], im);
-                        im = fma(e.im[r][k], v.re[k][j], im);
-                    }
-                    u.re[r][j] = re;
-                    u.im[r][j] = im;
-                }
-        }
-        reunitarise(u);
-        store_link(links, V, mu, n, u);
-    }
-}
-
-// The link step of update_links for one link of a batch of lattices: the
-// persistent CTAs walk the concatenated link ranges.
-struct LinkBatch {
-    int n;
-    int64_t total;
-    int64_t begin[kMaxBatch + 1]; // first link of each lattice in the concatenation
-    int64_t V[kMaxBatch];
-    void *links[kMaxBatch];
-    const void *mom[kMaxBatch];
-};
-
-template <typename R>
-__global__ void __launch_bounds__(kBlock) update_links_batched(const __grid_constant__ LinkBatch B, R dt)
-{
-    int c = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B.total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        while (c > 0 && i < B.begin[c]) --c;
-        while (c + 1 < B.n && i >= B.begin[c + 1]) ++c;
-        const int64_t V = B.V[c];
-        const int64_t l = i - B.begin[c];
-        const int mu = direction_of(l, V);
-        const int64_t n = l - mu * V;
-        R *links = static_cast<R *>(B.links[c]);
-        R p[8];
-        load_algebra(static_cast<const R *>(B.mom[c]), V, mu, n, p);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) p[q] *= dt;
-        const Mat<R> e = exp_i_hermitian(algebra_matrix(p));
+    const Mat<R> e = exp_i_hermitian(algebra_matrix(p));
+    Mat<R> u;
+    if constexpr (FROM_UNIT) {
+        u = e;
+    } else {
         const Mat<R> v = load_link(links, V, mu, n);
-        Mat<R> u;
 #pragma unroll
         for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -145,8 +84,93 @@ __global__ void __launch_bounds__(kBlock) update_links_batched(const __grid_cons
                 u.re[r][j] = re;
                 u.im[r][j] = im;
             }
-        reunitarise(u);
-        store_link(links, V, mu, n, u);
+    }
+    reunitarise(u);
+    store_link(links, V, mu, n, u);
+}
+
+// The FP64 step in floating point, for links that fx_link_step leaves.
+template <bool FROM_UNIT>
+__device__ __noinline__ void link_step_floating(double *links, const double *mom, double dt, int64_t V, int mu, int64_t n)
+{
+    double p[8];
+    load_algebra(mom, V, mu, n, p);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) p[c] *= dt;
+    link_step<double, FROM_UNIT>(links, p, V, mu, n);
+}
+
+// The step of link (n, mu) with the momenta scaled by dt.
+template <typename R, bool FROM_UNIT>
+__device__ __forceinline__ void update_link(R *__restrict__ links, const R *__restrict__ mom, R dt, int64_t V, int mu,
+                                            int64_t n)
+{
+    R p[8];
+    load_algebra(mom, V, mu, n, p);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) p[c] *= dt;
+    if constexpr (sizeof(R) == 4) {
+        link_step<R, FROM_UNIT>(links, p, V, mu, n);
+    } else {
+        double2 *u = reinterpret_cast<double2 *>(links) + (int64_t)mu * 6 * V + n;
+        double r[12] = {1.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0};
+        if constexpr (!FROM_UNIT) {
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const double2 v = u[q * V];
+                r[2 * q] = v.x;
+                r[2 * q + 1] = v.y;
+            }
+        }
+        if (fx_link_step(p, r)) {
+#pragma unroll
+            for (int q = 0; q < 6; ++q) u[q * V] = make_double2(r[2 * q], r[2 * q + 1]);
+        } else {
+            link_step_floating<FROM_UNIT>(links, mom, dt, V, mu, n);
+        }
+    }
+}
+
+// Threads of a link-step block: the FP64 step takes more registers.
+template <typename R> constexpr int link_block() { return sizeof(R) == 8 ? 128 : kBlock; }
+template <typename R> constexpr int link_min_blocks() { return sizeof(R) == 8 ? 3 : 1; }
+
+// The link and algebra planes share the site index.
+template <typename R, bool FROM_UNIT>
+__global__ void __launch_bounds__(link_block<R>(), link_min_blocks<R>())
+    update_links(R *__restrict__ links, const R *__restrict__ mom, int64_t V, R dt)
+{
+    const int64_t nlinks = 4 * V;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nlinks;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int mu = direction_of(i, V);
+        update_link<R, FROM_UNIT>(links, mom, dt, V, mu, i - mu * V);
+    }
+}
+
+// The link step of update_links for one link of a batch of lattices: the
+// persistent CTAs walk the concatenated link ranges.
+struct LinkBatch {
+    int n;
+    int64_t total;
+    int64_t begin[kMaxBatch + 1]; // first link of each lattice in the concatenation
+    int64_t V[kMaxBatch];
+    void *links[kMaxBatch];
+    const void *mom[kMaxBatch];
+};
+
+template <typename R>
+__global__ void __launch_bounds__(link_block<R>(), link_min_blocks<R>()) update_links_batched(const __grid_constant__ LinkBatch B, R dt)
+{
+    int c = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B.total;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        while (c > 0 && i < B.begin[c]) --c;
+        while (c + 1 < B.n && i >= B.begin[c + 1]) ++c;
+        const int64_t V = B.V[c];
+        const int64_t l = i - B.begin[c];
+        const int mu = direction_of(l, V);
+        update_link<R, false>(static_cast<R *>(B.links[c]), static_cast<const R *>(B.mom[c]), dt, V, mu, l - mu * V);
     }
 }
 
@@ -399,7 +423,7 @@ cudaError_t launch_update_links(const MdArgs &a, cudaStream_t st)
 {
     const int64_t V = volume(a.dims);
     if (a.precision == LQCD_F64)
-        update_links<double, false><<<grid_for(4 * V), kBlock, 0, st>>>(
+        update_links<double, false><<<grid_for(4 * V, link_block<double>()), link_block<double>(), 0, st>>>(
             static_cast<double *>(a.links), static_cast<const double *>(a.mom), V, a.dt);
     else
         update_links<float, false><<<grid_for(4 * V), kBlock, 0, st>>>(
@@ -425,14 +449,15 @@ cudaError_t launch_update_links_batched(int precision, int n, const LinkStepItem
     B.total = pos;
     int dev = 0, sms = 1;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int64_t grid = (pos + kBlock - 1) / kBlock;
+    const int block = precision == LQCD_F64 ? link_block<double>() : link_block<float>();
+    int64_t grid = (pos + block - 1) / block;
     const int64_t cap = (int64_t)(sms > 0 ? sms : 1) * 8;
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
     if (precision == LQCD_F64)
-        update_links_batched<double><<<(unsigned)grid, kBlock, 0, st>>>(B, dt);
+        update_links_batched<double><<<(unsigned)grid, block, 0, st>>>(B, dt);
     else
-        update_links_batched<float><<<(unsigned)grid, kBlock, 0, st>>>(B, (float)dt);
+        update_links_batched<float><<<(unsigned)grid, block, 0, st>>>(B, (float)dt);
     return cudaGetLastError();
 }
 
@@ -440,7 +465,7 @@ cudaError_t launch_links_from_omega(const MdArgs &a, cudaStream_t st)
 {
     const int64_t V = volume(a.dims);
     if (a.precision == LQCD_F64)
-        update_links<double, true><<<grid_for(4 * V), kBlock, 0, st>>>(
+        update_links<double, true><<<grid_for(4 * V, link_block<double>()), link_block<double>(), 0, st>>>(
             static_cast<double *>(a.links), static_cast<const double *>(a.mom), V, 1.0);
     else
         update_links<float, true><<<grid_for(4 * V), kBlock, 0, st>>>(
