@@ -297,12 +297,12 @@ __device__ __forceinline__ void fx_total(const FLimbAcc &y, int i, int j, long l
     }
 }
 
-// A whole number v of 2^-(58 + SH) as limbs of 2^-30 and 2^-58.
+// A whole number v of 2^-(58 + SH) as limbs of 2^-30 and 2^-58 (SH at most 3).
 template <int SH> __device__ __forceinline__ void fx_limbs(long long v, int &h, int &l)
 {
-    if constexpr (SH > 0) v = (v + (1ll << (SH > 0 ? SH - 1 : 0))) >> SH;
-    h = (int)((v + (1ll << 27)) >> 28);
-    l = (int)((unsigned)v - ((unsigned)h << 28));
+    h = (int)((v + (1ll << (27 + SH))) >> (28 + SH));
+    l = (int)((unsigned)v - ((unsigned)h << (28 + SH)));
+    if constexpr (SH > 0) l = (l + (1 << (SH > 0 ? SH - 1 : 0))) >> SH;
 }
 
 // The entries of a product (units 2^-60), rows 0..ROWS-1.
@@ -371,6 +371,40 @@ __device__ __forceinline__ long long fx_re_trace(const FLimbs &a, const FLimbs &
     return fx_value(h - mh, l - ml);
 }
 
+// x 2^-shift in units of 2^-58 for |x| < 2 (shift 0), cut towards zero: 13
+// integer operations, where scaling and converting on the FP64 pipe take two
+// of its slots of 16 clocks.
+// With flip = -1 the negative of it.
+__device__ __forceinline__ long long fx_of_double(double x, int shift, int flip = 0)
+{
+    const int hi = __double2hiint(x);
+    const unsigned lo = (unsigned)__double2loint(x);
+    const int e = (hi >> 20) & 0x7ff;
+    // 53-bit mantissa in units 2^(e - 1075), moved up by 6: the value for e = 1023
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | lo) << 6;
+    const long long v = (long long)(m >> min(1023 - e + shift, 63));
+    const long long s = (long long)((hi >> 31) ^ flip);
+    return (v ^ s) - s;
+}
+
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// Whether rows 0 and 1 are orthonormal to 1e-3.
+__device__ __forceinline__ bool fx_near_su3(const FLimbs &u)
+{
+    float n0 = 0.f, n1 = 0.f, cr = 0.f, ci = 0.f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const float ar = 0x1p-30f * (float)u.rh[0][j], ai = 0x1p-30f * (float)u.ih[0][j];
+        const float br = 0x1p-30f * (float)u.rh[1][j], bi = 0x1p-30f * (float)u.ih[1][j];
+        n0 += ar * ar + ai * ai;
+        n1 += br * br + bi * bi;
+        cr += ar * br + ai * bi;
+        ci += ar * bi - ai * br;
+    }
+    return fabsf(n0 - 1.f) < 1e-3f && fabsf(n1 - 1.f) < 1e-3f && fabsf(cr) < 1e-3f && fabsf(ci) < 1e-3f;
+}
+
 // Rows 0 and 1 of a stored FP64 link, row 2 rebuilt; a link that is not
 // finite or not within 1e-3 of SU(3) is marked.
 __device__ __forceinline__ FLimbs fx_from_rows(const double r[12])
@@ -387,20 +421,24 @@ __device__ __forceinline__ FLimbs fx_from_rows(const double r[12])
         fx_limbs<0>(__double2ll_rn(x * 0x1p58), u.rh[i][j], u.rl[i][j]);
         fx_limbs<0>(__double2ll_rn(y * 0x1p58), u.ih[i][j], u.il[i][j]);
     }
-    float n0 = 0.f, n1 = 0.f, cr = 0.f, ci = 0.f;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const float ar = 0x1p-30f * (float)u.rh[0][j], ai = 0x1p-30f * (float)u.ih[0][j];
-        const float br = 0x1p-30f * (float)u.rh[1][j], bi = 0x1p-30f * (float)u.ih[1][j];
-        n0 += ar * ar + ai * ai;
-        n1 += br * br + bi * bi;
-        cr += ar * br + ai * bi;
-        ci += ar * bi - ai * br;
-    }
-    ok = ok && fabsf(n0 - 1.f) < 1e-3f && fabsf(n1 - 1.f) < 1e-3f && fabsf(cr) < 1e-3f && fabsf(ci) < 1e-3f;
+    ok = ok && fx_near_su3(u);
     fx_row2(u);
     if (!ok) u.rh[0][0] = kPoison;
     return u;
+}
+
+// Rows 0 and 1 of a stored FP64 link by integer operations (row 2 is not
+// set); false where they have no fixed-point form.
+__device__ __forceinline__ bool fx_limbs_of_rows(const double r[12], FLimbs &u)
+{
+    bool ok = true;
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+        ok = ok && exponent_of(r[2 * e]) < 1024 && exponent_of(r[2 * e + 1]) < 1024;
+        fx_limbs<0>(fx_of_double(r[2 * e], 0), u.rh[e / 3][e % 3], u.rl[e / 3][e % 3]);
+        fx_limbs<0>(fx_of_double(r[2 * e + 1], 0), u.ih[e / 3][e % 3], u.il[e / 3][e % 3]);
+    }
+    return ok && fx_near_su3(u);
 }
 
 template <typename M> __device__ __forceinline__ bool fx_poisoned(const M &m) { return m.rh[0][0] == kPoison; }

@@ -45,20 +45,17 @@ __device__ __forceinline__ long long fxs_mul(const FxS a, const FxS b)
     return (fx_value(h, l) + 2) >> 2;
 }
 
-// x 2^-shift in units of 2^-58 for |x| < 2 (shift 0), cut towards zero.
-__device__ __forceinline__ long long fx_of_double(double x, int shift)
+// 2^58 / n!, n = 3 to 12, as limbs.
+constexpr FxS inverse_factorial(int n)
 {
-    const int hi = __double2hiint(x);
-    const unsigned lo = (unsigned)__double2loint(x);
-    const int e = (hi >> 20) & 0x7ff;
-    // 53-bit mantissa in units 2^(e - 1075), moved up by 6: the value for e = 1023
-    unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | lo) << 6;
-    const int sh = 1023 - e + shift;
-    m = sh < 63 ? m >> sh : 0ull;
-    return hi < 0 ? -(long long)m : (long long)m;
+    double f = 288230376151711744.0;
+    for (int i = 2; i <= n; ++i) f /= (double)i;
+    const long long v = (long long)(f + 0.5), h = (v + (1ll << 27)) >> 28;
+    return FxS{(int)h, (int)(v - h * (1ll << 28))};
 }
-
-__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__constant__ const FxS kInverseFactorial[10] = {
+    inverse_factorial(3), inverse_factorial(4), inverse_factorial(5),  inverse_factorial(6),  inverse_factorial(7),
+    inverse_factorial(8), inverse_factorial(9), inverse_factorial(10), inverse_factorial(11), inverse_factorial(12)};
 
 // f0 - 1, f1, f2 for c0, c1 in units of 2^-58 (c1 <= 1/2): the forward
 // recurrence of exp_i_hermitian, the terms from n = 13 (below 2^-32) in FP32.
@@ -69,46 +66,45 @@ __device__ __forceinline__ void fx_exp_coefficients(long long c0, long long c1, 
     f[0] = f[1] = f[2] = f[5] = 0; // f0r - 1, f0i, f1r, f2i
     f[3] = 1ll << 58;              // f1i
     f[4] = -(1ll << 57);           // f2r
-    long long a = 0, b = 0, d = 1ll << 58; // Q^2 = d Q^2
-    double fact = 0.5;
-#pragma unroll
-    for (int n = 3; n <= 12; ++n) {
-        const FxS ds = fxs(d);
-        const long long an = n == 3 ? c0 : fxs_mul(s0, ds), bn = a + (n == 3 ? c1 : fxs_mul(s1, ds)), dn = b;
+    // (a, b, d) with the sign of i^n: it turns from odd to even n
+    long long a = 0, b = 0, d = -(1ll << 58);
+#pragma unroll 1
+    for (int m = 0; m < 5; ++m) {
+        const auto odd = kInverseFactorial[2 * m], even = kInverseFactorial[2 * m + 1];
+        FxS ds = fxs(d);
+        long long an = fxs_mul(s0, ds), bn = a + fxs_mul(s1, ds);
+        d = b;
         a = an;
         b = bn;
-        d = dn;
-        fact /= (double)n;
-        const long long w = (long long)(fact * 288230376151711744.0 + 0.5); // 2^58 / n!
-        const FxS ws{(int)((w + (1ll << 27)) >> 28), (int)(w - (((w + (1ll << 27)) >> 28) << 28))};
-        const long long ta = fxs_mul(ws, fxs(a)), tb = fxs_mul(ws, fxs(b)), td = n == 3 ? 0 : fxs_mul(ws, fxs(d));
-        const int o = n & 1; // odd: imaginary
-        if ((n & 3) < 2) {
-            f[0 + o] += ta;
-            f[2 + o] += tb;
-            f[4 + o] += td;
-        } else {
-            f[0 + o] -= ta;
-            f[2 + o] -= tb;
-            f[4 + o] -= td;
-        }
+        ds = fxs(d);
+        f[1] += fxs_mul(odd, fxs(a));
+        f[3] += fxs_mul(odd, fxs(b));
+        f[5] += fxs_mul(odd, ds);
+        an = -fxs_mul(s0, ds);
+        bn = -a - fxs_mul(s1, ds);
+        d = -b;
+        a = an;
+        b = bn;
+        f[0] += fxs_mul(even, fxs(a));
+        f[2] += fxs_mul(even, fxs(b));
+        f[4] += fxs_mul(even, fxs(d));
     }
     float fa = (float)a, fb = (float)b, fd = (float)d;
     const float g0 = 0x1p-58f * (float)c0, g1 = 0x1p-58f * (float)c1;
     float t[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    float ff = (float)fact;
+    float ff = 1.f / 479001600.f;
 #pragma unroll
     for (int n = 13; n <= 19; ++n) {
-        const float an = g0 * fd, bn = fmaf(g1, fd, fa), dn = fb;
+        const float sign = n & 1 ? 1.f : -1.f;
+        const float an = sign * g0 * fd, bn = sign * fmaf(g1, fd, fa), dn = sign * fb;
         fa = an;
         fb = bn;
         fd = dn;
         ff *= 1.f / (float)n;
         const int o = n & 1;
-        const float w = (n & 3) < 2 ? ff : -ff;
-        t[0 + o] = fmaf(w, fa, t[0 + o]);
-        t[2 + o] = fmaf(w, fb, t[2 + o]);
-        t[4 + o] = fmaf(w, fd, t[4 + o]);
+        t[0 + o] = fmaf(ff, fa, t[0 + o]);
+        t[2 + o] = fmaf(ff, fb, t[2 + o]);
+        t[4 + o] = fmaf(ff, fd, t[4 + o]);
     }
 #pragma unroll
     for (int i = 0; i < 6; ++i) f[i] += (long long)__float2int_rn(t[i]); // below 2^-32: fits 27 bits
@@ -143,25 +139,7 @@ __device__ __forceinline__ bool fx_link_step(const double x[8], double r[12])
     // the link
     FLimbs u;
     {
-        bool ok = true;
-        float n0 = 0.f, n1 = 0.f, cr = 0.f, ci = 0.f;
-#pragma unroll
-        for (int e = 0; e < 6; ++e) {
-            ok = ok && exponent_of(r[2 * e]) < 1024 && exponent_of(r[2 * e + 1]) < 1024;
-            fx_limbs<0>(fx_of_double(r[2 * e], 0), u.rh[e / 3][e % 3], u.rl[e / 3][e % 3]);
-            fx_limbs<0>(fx_of_double(r[2 * e + 1], 0), u.ih[e / 3][e % 3], u.il[e / 3][e % 3]);
-        }
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const float ar = 0x1p-30f * (float)u.rh[0][j], ai = 0x1p-30f * (float)u.ih[0][j];
-            const float br = 0x1p-30f * (float)u.rh[1][j], bi = 0x1p-30f * (float)u.ih[1][j];
-            n0 += ar * ar + ai * ai;
-            n1 += br * br + bi * bi;
-            cr += ar * br + ai * bi;
-            ci += ar * bi - ai * br;
-        }
-        if (!(ok && fabsf(n0 - 1.f) < 1e-3f && fabsf(n1 - 1.f) < 1e-3f && fabsf(cr) < 1e-3f && fabsf(ci) < 1e-3f))
-            return false;
+        if (!fx_limbs_of_rows(r, u)) return false;
         fx_row2(u);
     }
     // Q and its invariants

@@ -131,9 +131,11 @@ __device__ __forceinline__ void update_link(R *__restrict__ links, const R *__re
     }
 }
 
-// Threads of a link-step block: the FP64 step takes more registers.
-template <typename R> constexpr int link_block() { return sizeof(R) == 8 ? 128 : kBlock; }
-template <typename R> constexpr int link_min_blocks() { return sizeof(R) == 8 ? 3 : 1; }
+// Threads of a link-step block and resident blocks: the FP64 step takes more
+// registers (18x14x22x36: 153 us with 2 blocks of 192, 157 with 3 of 128, 170
+// with 2 of 128).
+template <typename R> constexpr int link_block() { return sizeof(R) == 8 ? 192 : kBlock; }
+template <typename R> constexpr int link_min_blocks() { return sizeof(R) == 8 ? 2 : 1; }
 
 // The link and algebra planes share the site index.
 template <typename R, bool FROM_UNIT>

@@ -7,6 +7,7 @@
 // neighbours come from L1/L2 (a time slice of a 32^3 spinor field is 3 MB),
 // and every (1 -+ gamma_mu) is applied as a spin projection to two colour
 // vectors, so that each link multiplies two colour vectors instead of four.
+#include "fixed.cuh"
 #include "sites.cuh"
 
 namespace lqcd {
@@ -352,13 +353,218 @@ __device__ __forceinline__ Mat<R> b_minus_c(const R *__restrict__ links, const R
 
 constexpr int kForceBlock = 128; // 32 sites x 4 directions, one direction per warp
 
-template <typename R, typename I>
+// f = coef h stored and/or applied to the momenta.
+__device__ __forceinline__ void finish_force(const WilsonArgs &a, int64_t V, int rho, int64_t k, const double f[8])
+{
+    if (a.force != nullptr) store_algebra(static_cast<double *>(a.force), V, rho, k, f);
+    if (a.mom != nullptr) {
+        double *mom = static_cast<double *>(a.mom);
+        double p[8];
+        load_algebra(mom, V, rho, k, p);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) p[q] = fma(a.dt, f[q], p[q]);
+        store_algebra(mom, V, rho, k, p);
+    }
+}
+
+// ------------------------------------------ hopping-term force in fixed point
+
+// Two colour vectors in whole limbs of 2^-28 and 2^-56 of their spinor's scale.
+struct FHalf {
+    int rh[2][3], rl[2][3], ih[2][3], il[2][3];
+};
+
+// Rows 0 and 1 of (1 + s gamma_mu) x_n, mu at run time, over 2^(e - 1022) with
+// e the largest exponent field of the spinor's 24 reals; false where that is
+// out of range (the scales of two spinors are multiplied) or not finite.
+__device__ __forceinline__ bool fx_half(const double *__restrict__ x, int64_t V, int64_t n, int mu, bool minus, FHalf &h,
+                                        int &e)
+{
+    // rows 0, 1 go with rows 3, 2 (mu < 2) or 2, 3; where i^gcode is odd the
+    // parts of those are exchanged, by where they are read
+    const double2 *p = reinterpret_cast<const double2 *>(x) + n;
+    const bool turn = mu == 0 || mu == 2;
+    const double *p2 = x + 2 * (n + (mu < 2 ? 9 : 6) * V), *p3 = x + 2 * (n + (mu < 2 ? 6 : 9) * V);
+    const int ore = turn ? 1 : 0, oim = 1 - ore;
+    double2 v[12];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) v[q] = __ldg(p + q * V);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        v[6 + q] = make_double2(__ldg(p2 + 2 * q * V + ore), __ldg(p2 + 2 * q * V + oim));
+        v[9 + q] = make_double2(__ldg(p3 + 2 * q * V + ore), __ldg(p3 + 2 * q * V + oim));
+    }
+    e = 0;
+#pragma unroll
+    for (int q = 0; q < 12; ++q) e = max(e, max(exponent_of(v[q].x), exponent_of(v[q].y)));
+    if (e < 64 || e > 1900) {
+        if (e != 0) return false;
+        bool zero = true; // and no subnormals
+#pragma unroll
+        for (int q = 0; q < 12; ++q) zero = zero && v[q].x == 0.0 && v[q].y == 0.0;
+        if (!zero) return false;
+        e = 64;
+    }
+    const int shift = e - 1022;
+#pragma unroll
+    for (int al = 0; al < 2; ++al) {
+        // times s i^gcode(mu, al)
+        const int code = ((mu == 0 ? 1 : mu == 1 ? (al == 0 ? 2 : 0) : mu == 2 ? (al == 0 ? 1 : 3) : 0) + (minus ? 2 : 0)) & 3;
+        const int sr = code == 1 || code == 2 ? -1 : 0, si = code >= 2 ? -1 : 0; // masks of the signs
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double2 w = v[6 + 3 * al + a], u = v[3 * al + a];
+            const long long re = fx_of_double(u.x, shift) + fx_of_double(w.x, shift, sr);
+            const long long im = fx_of_double(u.y, shift) + fx_of_double(w.y, shift, si);
+            fx_limbs<2>(re, h.rh[al][a], h.rl[al][a]);
+            fx_limbs<2>(im, h.ih[al][a], h.il[al][a]);
+        }
+    }
+    return true;
+}
+
+// u h on both colour vectors.
+__device__ __forceinline__ void fx_colour_mul(const FLimbs &u, FHalf &h)
+{
+#pragma unroll
+    for (int al = 0; al < 2; ++al) {
+        FLimbAcc y; // column 0
+#pragma unroll
+        for (int a = 0; a < 3; ++a) y.h1[a][0] = y.l1[a][0] = y.h2[a][0] = y.l2[a][0] = y.h3[a][0] = y.l3[a][0] = 0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int sh = h.rh[al][b] + h.ih[al][b], sl = h.rl[al][b] + h.il[al][b];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                fx_mad(y.h1[a][0], y.l1[a][0], u.rh[a][b], u.rl[a][b], h.rh[al][b], h.rl[al][b]);
+                fx_mad(y.h2[a][0], y.l2[a][0], u.ih[a][b], u.il[a][b], h.ih[al][b], h.il[al][b]);
+                fx_mad(y.h3[a][0], y.l3[a][0], u.rh[a][b] + u.ih[a][b], u.rl[a][b] + u.il[a][b], sh, sl);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            long long re, im;
+            fx_total<1>(y, a, 0, re, im);
+            fx_limbs<2>(re, h.rh[al][a], h.rl[al][a]);
+            fx_limbs<2>(im, h.ih[al][a], h.il[al][a]);
+        }
+    }
+}
+
+// The force on one FP64 link.  With N_0 = (U (1 - g) X_{k+rho}) (x) ((1 - g) Y_k)^dag
+// and N_1 = (U (1 + g) Y_{k+rho}) (x) ((1 + g) X_k)^dag, spin rows 0 and 1 summed,
+// B = N_0 and C = N_1^dag, so h^i = Im tr(lambda_i N_0) + Im tr(lambda_i N_1): one
+// loop body for both, the direction at run time, so that the four warps of a
+// block run the same code.
+//
+// In floating point this is 720 operations a link on the FP64 pipe (2 a clock
+// and SM) and 108 numbers read.  Here every spinor is a block of whole numbers
+// of its own scale, taken apart by integer operations; the FP64 pipe makes the
+// 16 components.
+__device__ __forceinline__ bool hopping_force_fx(const WilsonArgs &a, int64_t V, int rho, int64_t k, int64_t kp)
+{
+    __shared__ int4 u_s[9][kForceBlock]; // the link, out of the registers' way
+    int4 *us = &u_s[0][threadIdx.x];
+    {
+        FLimbs u;
+        const double2 *p = static_cast<const double2 *>(a.links) + (int64_t)rho * 6 * V + k;
+        double r[12];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const double2 v = __ldg(p + q * V);
+            r[2 * q] = v.x;
+            r[2 * q + 1] = v.y;
+        }
+        if (!fx_limbs_of_rows(r, u)) return false;
+        fx_row2(u);
+#pragma unroll
+        for (int e = 0; e < 9; ++e)
+            us[e * kForceBlock] = make_int4(u.rh[e / 3][e % 3], u.rl[e / 3][e % 3], u.ih[e / 3][e % 3], u.il[e / 3][e % 3]);
+    }
+    double f[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int t = 0; t < 2; ++t) {
+        const double *s0 = static_cast<const double *>(t == 0 ? a.x : a.y), *s1 = static_cast<const double *>(t == 0 ? a.y : a.x);
+        FHalf p, q;
+        int ep, eq;
+        if (!fx_half(s0, V, kp, rho, t == 0, p, ep)) return false;
+        {
+            FLimbs u;
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                const int4 v = us[e * kForceBlock];
+                u.rh[e / 3][e % 3] = v.x;
+                u.rl[e / 3][e % 3] = v.y;
+                u.ih[e / 3][e % 3] = v.z;
+                u.il[e / 3][e % 3] = v.w;
+            }
+            fx_colour_mul(u, p);
+        }
+        if (!fx_half(s1, V, k, rho, t == 0, q, eq)) return false;
+        long long re[3][3], im[3][3]; // N, units 2^-56 of the two scales
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            FLimbAcc y; // row 0
+#pragma unroll
+            for (int j = 0; j < 3; ++j) y.h1[0][j] = y.l1[0][j] = y.h2[0][j] = y.l2[0][j] = y.h3[0][j] = y.l3[0][j] = 0;
+#pragma unroll
+            for (int al = 0; al < 2; ++al) {
+                const int sh = p.rh[al][i] + p.ih[al][i], sl = p.rl[al][i] + p.il[al][i];
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    fx_mad(y.h1[0][j], y.l1[0][j], p.rh[al][i], p.rl[al][i], q.rh[al][j], q.rl[al][j]);
+                    fx_mad(y.h2[0][j], y.l2[0][j], p.ih[al][i], p.il[al][i], q.ih[al][j], q.il[al][j]);
+                    fx_mad(y.h3[0][j], y.l3[0][j], sh, sl, q.rh[al][j] - q.ih[al][j], q.rl[al][j] - q.il[al][j]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 3; ++j) fx_total<-1>(y, 0, j, re[i][j], im[i][j]);
+        }
+        // Im tr(lambda_a N) times coef and the scales 2^(e - 1022)
+        const double s = a.coef * 0x1p-56 * __hiloint2double((ep + 1) << 20, 0), w = __hiloint2double((eq + 1) << 20, 0);
+        f[0] = fma(s * (double)(im[0][1] + im[1][0]), w, f[0]);
+        f[1] = fma(s * (double)(re[0][1] - re[1][0]), w, f[1]);
+        f[2] = fma(s * (double)(im[0][0] - im[1][1]), w, f[2]);
+        f[3] = fma(s * (double)(im[0][2] + im[2][0]), w, f[3]);
+        f[4] = fma(s * (double)(re[0][2] - re[2][0]), w, f[4]);
+        f[5] = fma(s * (double)(im[1][2] + im[2][1]), w, f[5]);
+        f[6] = fma(s * (double)(re[1][2] - re[2][1]), w, f[6]);
+        f[7] = fma(s * 0.57735026918962576451 * (double)(im[0][0] + im[1][1] - 2 * im[2][2]), w, f[7]);
+    }
+    finish_force(a, V, rho, k, f);
+    return true;
+}
+
+// B - C on link (k, rho), the direction at run time.
+template <typename R>
+__device__ __forceinline__ Mat<R> b_minus_c(const R *__restrict__ links, const R *__restrict__ X,
+                                            const R *__restrict__ Y, int64_t V, int rho, int64_t k, int64_t kp)
+{
+    switch (rho) {
+    case 0: return b_minus_c<0>(links, X, Y, V, k, kp);
+    case 1: return b_minus_c<1>(links, X, Y, V, k, kp);
+    case 2: return b_minus_c<2>(links, X, Y, V, k, kp);
+    default: return b_minus_c<3>(links, X, Y, V, k, kp);
+    }
+}
+
+// The FP64 force in floating point, for links that hopping_force_fx leaves.
+__device__ __noinline__ void hopping_force_floating(const WilsonArgs &a, int64_t V, int rho, int64_t k, int64_t kp)
+{
+    const Mat<double> m = b_minus_c(static_cast<const double *>(a.links), static_cast<const double *>(a.x),
+                                    static_cast<const double *>(a.y), V, rho, k, kp);
+    double f[8];
+    ta_components(m, -a.coef, f);
+    finish_force(a, V, rho, k, f);
+}
+
+template <typename I>
 __global__ void __launch_bounds__(kForceBlock) wilson_hopping_force(const __grid_constant__ WilsonArgs a)
 {
     const Sites<I> g = make_sites<I>(a.dims);
-    const R *__restrict__ links = static_cast<const R *>(a.links);
-    const R *__restrict__ X = static_cast<const R *>(a.x);
-    const R *__restrict__ Y = static_cast<const R *>(a.y);
+    const float *__restrict__ links = static_cast<const float *>(a.links);
+    const float *__restrict__ X = static_cast<const float *>(a.x);
+    const float *__restrict__ Y = static_cast<const float *>(a.y);
     const int rho = (int)(threadIdx.x >> 5);
     const I ks = (I)blockIdx.x * 32 + (I)(threadIdx.x & 31);
     if (ks >= g.V) return;
@@ -366,7 +572,7 @@ __global__ void __launch_bounds__(kForceBlock) wilson_hopping_force(const __grid
     if constexpr (sizeof(I) == 4) c = coord_fast(g, a.div, ks);
     else c = coord_in(g, ks);
     const int64_t V = g.V, k = ks, kp = (int64_t)(ks + hop_offset(g, c, rho, 1));
-    Mat<R> m;
+    Mat<float> m;
     switch (rho) {
     case 0: m = b_minus_c<0>(links, X, Y, V, k, kp); break;
     case 1: m = b_minus_c<1>(links, X, Y, V, k, kp); break;
@@ -374,18 +580,36 @@ __global__ void __launch_bounds__(kForceBlock) wilson_hopping_force(const __grid
     default: m = b_minus_c<3>(links, X, Y, V, k, kp); break;
     }
     // f^i = coef * h^i,  h^i = -(tr(i T_i M) + c.c.) = Im tr(lambda_i M)
-    R f[8];
-    ta_components(m, -scalar_of<R>(a.coef, a.fcoef), f);
-    if (a.force != nullptr) store_algebra(static_cast<R *>(a.force), V, rho, k, f);
+    float f[8];
+    ta_components(m, -a.fcoef, f);
+    if (a.force != nullptr) store_algebra(static_cast<float *>(a.force), V, rho, k, f);
     if (a.mom != nullptr) {
-        R *mom = static_cast<R *>(a.mom);
-        R p[8];
+        float *mom = static_cast<float *>(a.mom);
+        float p[8];
         load_algebra(mom, V, rho, k, p);
-        const R dt = scalar_of<R>(a.dt, a.fdt);
+        const float dt = a.fdt;
 #pragma unroll
         for (int q = 0; q < 8; ++q) p[q] = fma(dt, f[q], p[q]);
         store_algebra(mom, V, rho, k, p);
     }
+}
+
+// 4 blocks per SM (128 registers, 172 bytes spilled): 146 us at 20x18x14x30
+// against 149 with 3 and 158 with 5; in floating point 431.  What bounds it
+// now are three pipes alike: instruction issue, the integer half of the FMA
+// pipe and the ALUs would each take about 67 us.
+template <typename I>
+__global__ void __launch_bounds__(kForceBlock, 4) wilson_hopping_force_fx(const __grid_constant__ WilsonArgs a)
+{
+    const Sites<I> g = make_sites<I>(a.dims);
+    const int rho = (int)(threadIdx.x >> 5);
+    const I ks = (I)blockIdx.x * 32 + (I)(threadIdx.x & 31);
+    if (ks >= g.V) return;
+    Coord c;
+    if constexpr (sizeof(I) == 4) c = coord_fast(g, a.div, ks);
+    else c = coord_in(g, ks);
+    const int64_t V = g.V, k = ks, kp = (int64_t)(ks + hop_offset(g, c, rho, 1));
+    if (!hopping_force_fx(a, V, rho, k, kp)) hopping_force_floating(a, V, rho, k, kp);
 }
 
 unsigned blocks_for(int64_t items, int per_block)
@@ -442,11 +666,11 @@ cudaError_t launch_wilson_hopping_force(const WilsonArgs &args, cudaStream_t st)
     const unsigned grid = blocks_for(V, 32);
     const bool i32 = sites_fit_int(V);
     if (a.precision == LQCD_F64) {
-        if (i32) wilson_hopping_force<double, int><<<grid, kForceBlock, 0, st>>>(a);
-        else wilson_hopping_force<double, int64_t><<<grid, kForceBlock, 0, st>>>(a);
+        if (i32) wilson_hopping_force_fx<int><<<grid, kForceBlock, 0, st>>>(a);
+        else wilson_hopping_force_fx<int64_t><<<grid, kForceBlock, 0, st>>>(a);
     } else {
-        if (i32) wilson_hopping_force<float, int><<<grid, kForceBlock, 0, st>>>(a);
-        else wilson_hopping_force<float, int64_t><<<grid, kForceBlock, 0, st>>>(a);
+        if (i32) wilson_hopping_force<int><<<grid, kForceBlock, 0, st>>>(a);
+        else wilson_hopping_force<int64_t><<<grid, kForceBlock, 0, st>>>(a);
     }
     return cudaGetLastError();
 }

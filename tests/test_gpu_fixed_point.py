@@ -136,3 +136,50 @@ def test_any_coefficients(coef):
     assert np.abs(lqcd.algebra_from_device(force) - ref).max() <= 1e-12 * np.abs(ref).max()
     assert abs(float(S.item()) - want) <= 1e-12 * abs(want)
     assert abs(float(lqcd.gauge_action(lat, links).item()) - want) <= 1e-12 * abs(want)
+
+
+@pytest.mark.parametrize("scale_x, scale_y", [(1.0, 1.0), (1e-200, 1e200), (3e140, 2e-90), (0.0, 1.0)])
+@pytest.mark.parametrize("scaled", [(), (5, 6)])
+def test_hopping_force_scales(scale_x, scale_y, scaled):
+    """FP64 hopping-term force of spinors of any size, entries of very
+    different sizes among them, and of links without a fixed-point form."""
+    dims = (3, 4, 2, 5)
+    lat = lqcd.Lattice.symanzik(dims, 6.0, 0.87, "f64")
+    U = O.links_from_omega(synth.omega(dims, 0.4, 3)).reshape(lat.V, 4, 3, 3)
+    for i in scaled:
+        U[i // 4, i % 4, :2] *= 1.01
+    U = _third(U)
+    X, Y = (synth.spinor(dims, s) for s in (11, 12))
+    X[::7] *= 1e-9
+    Y[:, 2] *= 1e-5
+    X, Y = (s[..., 0] + 1j * s[..., 1] for s in (X * scale_x, Y * scale_y))
+    f = lqcd.algebra_from_device(lqcd.wilson_hopping_force(lat, _links(lat, U), lqcd.spinor_to_device(lat, X),
+                                                           lqcd.spinor_to_device(lat, Y), coef=0.5))
+    ref = O.wilson_hopping_force(dims, U, X, Y, 0.5)
+    # each link's force against the size of the spinors it is made of
+    size = np.abs(ref).max(-1, keepdims=True) + 1e-300
+    big = np.abs(f - ref).max(-1, keepdims=True) / size
+    assert (big[np.broadcast_to(size > 1e-290, big.shape)] <= 1e-11).all()
+    if scale_x == 0.0:
+        assert not f.any()
+
+
+@pytest.mark.parametrize("dt", [0.05, 0.6, 3.0, 40.0])
+@pytest.mark.parametrize("scaled", [(), (0, 9)])
+def test_link_step_sizes(dt, scaled):
+    """FP64 link step from small to large exponents (the step is then made 2^s
+    times, or in floating point) and on links that depart from SU(3)."""
+    dims = (3, 4, 2, 5)
+    lat = lqcd.Lattice.symanzik(dims, 6.0, 0.87, "f64")
+    U = O.links_from_omega(synth.omega(dims, 0.4, 3)).reshape(lat.V, 4, 3, 3)
+    for i in scaled:
+        U[i // 4, i % 4, 0] *= 1.0 + 1e-6
+        U[i // 4, i % 4, 1] += 1e-4 * U[i // 4, i % 4, 0]
+    U = _third(U)
+    p = synth.momenta(dims, 4)
+    p[::3] *= 1e-6
+    links = _links(lat, U)
+    lqcd.md_update_links(lat, links, lqcd.algebra_to_device(lat, p), dt)
+    got = lqcd.full_from_device(lqcd.unpack_links(lat, links))
+    # exponents up to about 10 dt: their rounding is that of the angle
+    assert np.abs(got - O.md_update_links(U, p, dt)).max() <= 1e-13 * max(1.0, 10 * dt)
