@@ -111,7 +111,8 @@ template <int FA, int FB> __device__ __forceinline__ FLimbs fx_mul_top2(const FL
     return fx_round<FA == FB ? 1 : -1, 2>(y);
 }
 
-__device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, int vb)
+// Staples j0 to j1 - 1 of each direction.
+__device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, int vb, int j0, int j1)
 {
     const int mu = (int)(threadIdx.x >> 5);
     const int x = vb * 32 + (int)(threadIdx.x & 31);
@@ -121,25 +122,27 @@ __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, 
     const int xm = x + step32(g, c, mu, 1); // x + mu
     char *out = sf.at(x);
 #pragma unroll 1
-    for (int iv = 0; iv < 3; ++iv) {
-        const int nu = (mu + 1 + iv) & 3;
-        const int vp = step32(g, c, nu, 1), vm = step32(g, c, nu, -1);
-        {
+    for (int j = j0; j < j1; ++j) {
+        const int nu = (mu + 1 + (j >> 1)) & 3;
+        FLimbs s;
+        bool bad;
+        if ((j & 1) == 0) {
             // b = +nu:  U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-            const FLimbs a = sf.limbs(sf.at(xm), kLinkPlane + nu), b = sf.limbs(sf.at(x + vp), kLinkPlane + mu), d = sf.limbs(sf.at(x), kLinkPlane + nu);
-            FLimbs s = fx_mul_top2<N, D>(fx_mul_top2<N, D>(a, b), d);
-            fx_row2(s);
-            if (fx_poisoned(a) || fx_poisoned(b) || fx_poisoned(d)) s.rh[0][0] = kPoison;
-            sf.store<true>(out, mu * 6 + 2 * iv, fx_remainder(s));
-        }
-        {
+            const FLimbs a = sf.limbs(sf.at(xm), kLinkPlane + nu),
+                         b = sf.limbs(sf.at(x + step32(g, c, nu, 1)), kLinkPlane + mu), d = sf.limbs(sf.at(x), kLinkPlane + nu);
+            bad = fx_poisoned(a) || fx_poisoned(b) || fx_poisoned(d);
+            s = fx_mul_top2<N, D>(fx_mul_top2<N, D>(a, b), d);
+        } else {
             // b = -nu:  U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
-            const FLimbs a = sf.limbs(sf.at(xm + vm), kLinkPlane + nu), b = sf.limbs(sf.at(x + vm), kLinkPlane + mu), d = sf.limbs(sf.at(x + vm), kLinkPlane + nu);
-            FLimbs s = fx_mul_top2<N, N>(fx_mul_top2<D, D>(a, b), d);
-            fx_row2(s);
-            if (fx_poisoned(a) || fx_poisoned(b) || fx_poisoned(d)) s.rh[0][0] = kPoison;
-            sf.store<true>(out, mu * 6 + 2 * iv + 1, fx_remainder(s));
+            const int vm = step32(g, c, nu, -1);
+            const FLimbs a = sf.limbs(sf.at(xm + vm), kLinkPlane + nu), b = sf.limbs(sf.at(x + vm), kLinkPlane + mu),
+                         d = sf.limbs(sf.at(x + vm), kLinkPlane + nu);
+            bad = fx_poisoned(a) || fx_poisoned(b) || fx_poisoned(d);
+            s = fx_mul_top2<N, N>(fx_mul_top2<D, D>(a, b), d);
         }
+        fx_row2(s);
+        if (bad) s.rh[0][0] = kPoison;
+        sf.store<true>(out, mu * 6 + j, fx_remainder(s));
     }
 }
 
@@ -147,7 +150,12 @@ __global__ void __launch_bounds__(kBlock) staples_fx(const __grid_constant__ SfL
 {
     const G32 g = make_g32(L.dims);
     const int nvb = (int)virtual_blocks(g.V);
-    for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) staples_block(L, g, vb);
+    if (L.split) { // one staple of each direction per block
+        const int vb = blockIdx.x / 6, j = blockIdx.x - 6 * vb;
+        staples_block(L, g, vb, j, j + 1);
+        return;
+    }
+    for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) staples_block(L, g, vb, 0, 6);
 }
 
 __global__ void __launch_bounds__(kBlock) staples_fx_batched(const __grid_constant__ SfBatch B)
@@ -155,7 +163,7 @@ __global__ void __launch_bounds__(kBlock) staples_fx_batched(const __grid_consta
     for (int64_t vb = next_virtual_block(B.counter); vb < B.total;) {
         const unsigned long long next = claim_virtual_block(B.counter);
         const SfLattice &L = B.e[batch_entry(B, vb)];
-        staples_block(L, make_g32(L.dims), (int)(vb - L.vb_begin));
+        staples_block(L, make_g32(L.dims), (int)(vb - L.vb_begin), 0, 6);
         vb = publish_virtual_block(next);
     }
 }
@@ -201,109 +209,91 @@ __device__ __noinline__ double force_link_floating(const SfLattice &L, const Ker
     return force_link<double, ACTION, false, true>(L, sc, g, sf, si, c, k, rho);
 }
 
-// Force (and the fused momentum step) on the link (k, rho); returns its
-// share of the action (force_link of sf_common.cuh in fixed point).
-//
-// Every sum of products that a link closes is a group of one loop: group 0
+// Every sum of products that a link closes is a group: group 0
 // F sum_b S_b(k+rho) S_b(k), group 1 sum_b S_b(k) S_b(k-rho) E, groups 2..7
 // B_d [ alpha sum_{b perp rho, d} S_b(k+d) S^{(d)}_b(k) + beta S_d(k+d) A_d^dag ]
-// for the six directions d.  One loop, and not a piece of code for each group
-// and sign: a product is about 400 instructions, and with eleven copies of it
-// the instruction cache missed (1.5 stalled cycles per instruction).  The
-// total z of the groups stays in shared memory, out of the registers' way.
-template <bool ACTION>
-__device__ __forceinline__ double fx_force_link(const SfLattice &L, const KernelScalars &sc, const FxScalars &fx,
-                                                const G32 &g, const Coord &c, int k, int rho)
+// for the six directions d.  One piece of code for all of them, and not one
+// for each group and sign: a product is about 400 instructions, and with
+// eleven copies of it the instruction cache missed (1.5 stalled cycles per
+// instruction).  z: the nine entries of the sum, units 2^-56.
+__device__ __forceinline__ void fx_group(longlong2 z[9], bool &bad, const FxPlanes &sf, const FxScalars &fx, const G32 &g,
+                                         const Coord &c, int rho, int k, int grp)
 {
-    __shared__ longlong2 zv_s[9][kBlock]; // units 2^-56
-    __shared__ float2 zc_s[9][kBlock];
-    longlong2 *zv = &zv_s[0][threadIdx.x];
-    float2 *zc = &zc_s[0][threadIdx.x];
-    const FxPlanes sf = fx_planes(L);
-    const int64_t V = g.V;
     const int kp = k + step32(g, c, rho, 1);
     const int base = rho * 6;
-    bool bad = false;
-
+    const bool chain = grp < 2, neg = grp >= 5;
+    const int id = chain ? 0 : (neg ? grp - 5 : grp - 2);
+    const int nud = chain ? rho : (rho + 1 + id) & 3;
+    const int dk = step32(g, c, nud, neg || grp == 1 ? -1 : 1); // k + dk: k+rho, k-rho, k+d
+    const char *at_k = sf.at(k), *at_d = sf.at(k + dk);
+    const char *at_a = grp == 1 ? at_k : at_d;
+    const char *at_b = chain ? (grp == 0 ? at_k : at_d) : (neg ? at_d : at_k);
+    FAcc acc;
+    fx_zero(acc);
+    const int n = chain ? 6 : 5;
 #pragma unroll 1
-    for (int grp = 0; grp < 8; ++grp) {
-        const bool chain = grp < 2, neg = grp >= 5;
-        const int id = chain ? 0 : (neg ? grp - 5 : grp - 2);
-        const int nud = chain ? rho : (rho + 1 + id) & 3;
-        const int dk = step32(g, c, nud, neg || grp == 1 ? -1 : 1); // k + dk: k+rho, k-rho, k+d
-        const char *at_k = sf.at(k), *at_d = sf.at(k + dk);
-        const char *at_a = grp == 1 ? at_k : at_d;
-        const char *at_b = chain ? (grp == 0 ? at_k : at_d) : (neg ? at_d : at_k);
-        FAcc acc;
-        fx_zero(acc);
-        const int n = chain ? 6 : 5;
-#pragma unroll 1
-        for (int q = 0; q < n; ++q) {
-            int pa = base + q, pb = base + q;
-            bool dag = neg;
-            if (!chain) {
-                const int ib = q < 2 ? (id == 0 ? 1 : 0) : (id == 2 ? 1 : 2);
-                const int nub = (rho + 1 + ib) & 3;
-                pa = base + 2 * ib + (q & 1);
-                pb = nud * 6 + 2 * ((nub - nud - 1) & 3) + (q & 1);
-                if (q == 4) { // the rectangle along d, onto alpha times the cubes
-                    const FMat y = fx_round<32>(acc); // up to 4, units 2^-28
+    for (int q = 0; q < n; ++q) {
+        int pa = base + q, pb = base + q;
+        bool dag = neg;
+        if (!chain) {
+            const int ib = q < 2 ? (id == 0 ? 1 : 0) : (id == 2 ? 1 : 2);
+            const int nub = (rho + 1 + ib) & 3;
+            pa = base + 2 * ib + (q & 1);
+            pb = nud * 6 + 2 * ((nub - nud - 1) & 3) + (q & 1);
+            if (q == 4) { // the rectangle along d, onto alpha times the cubes
+                const FMat y = fx_round<32>(acc); // up to 4, units 2^-28
 #pragma unroll
-                    for (int i = 0; i < 3; ++i)
+                for (int i = 0; i < 3; ++i)
 #pragma unroll
-                        for (int j = 0; j < 3; ++j) {
-                            const FSum re = fx_scaled(fx.alpha, y.rh[i][j], y.rl[i][j]);
-                            const FSum im = fx_scaled(fx.alpha, y.ih[i][j], y.il[i][j]);
-                            acc.h1[i][j] = 4 * re.v;
-                            acc.h2[i][j] = 0;
-                            acc.h3[i][j] = 4 * (re.v + im.v);
-                            acc.cr[i][j] = 4.f * re.c;
-                            acc.ci[i][j] = 4.f * im.c;
-                        }
-                    pa = base + 2 * id + (neg ? 1 : 0);
-                    pb = kLinkPlane + nud;
-                    dag = !neg;
-                }
+                    for (int j = 0; j < 3; ++j) {
+                        const FSum re = fx_scaled(fx.alpha, y.rh[i][j], y.rl[i][j]);
+                        const FSum im = fx_scaled(fx.alpha, y.ih[i][j], y.il[i][j]);
+                        acc.h1[i][j] = 4 * re.v;
+                        acc.h2[i][j] = 0;
+                        acc.h3[i][j] = 4 * (re.v + im.v);
+                        acc.cr[i][j] = 4.f * re.c;
+                        acc.ci[i][j] = 4.f * im.c;
+                    }
+                pa = base + 2 * id + (neg ? 1 : 0);
+                pb = kLinkPlane + nud;
+                dag = !neg;
             }
-            FMat a = sf.mat(at_a, pa);
-            const FMat b = sf.form(at_b, pb, pb >= kLinkPlane, dag);
-            bad = bad || fx_poisoned(a) || fx_poisoned(b);
-            if (fx.use_beta && q == 4 && !chain) a = fx_scaled(fx.beta, a);
-            fx_mul_acc<N, N>(acc, a, b);
         }
-        FMat y = fx_round<33>(acc); // up to 6, units 2^-27
-        if (fx.use_beta && chain) y = fx_scaled(fx.beta, y);
-        FMat x = sf.form(grp == 1 ? at_d : sf.at(neg ? kp + dk : kp), kLinkPlane + nud, true, neg);
-        bad = bad || fx_poisoned(x);
-        if (grp == 1) {
-            const FMat t = x;
-            x = y;
-            y = t;
-        }
-        fx_zero(acc);
-        fx_mul_acc<N, N>(acc, x, y);
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            FSum re, im;
-            fx_total<1>(acc, e / 3, e % 3, re, im);
-            longlong2 v = make_longlong2(re.v >> 1, im.v >> 1);
-            float2 w = make_float2(0.5f * re.c, 0.5f * im.c);
-            if (grp > 0) {
-                const longlong2 ov = zv[e * kBlock];
-                const float2 ow = zc[e * kBlock];
-                v.x += ov.x;
-                v.y += ov.y;
-                w.x += ow.x;
-                w.y += ow.y;
-            }
-            zv[e * kBlock] = v;
-            zc[e * kBlock] = w;
-        }
+        FMat a = sf.mat(at_a, pa);
+        const FMat b = sf.form(at_b, pb, pb >= kLinkPlane, dag);
+        bad = bad || fx_poisoned(a) || fx_poisoned(b);
+        if (fx.use_beta && q == 4 && !chain) a = fx_scaled(fx.beta, a);
+        fx_mul_acc<N, N>(acc, a, b);
     }
+    FMat y = fx_round<33>(acc); // up to 6, units 2^-27
+    if (fx.use_beta && chain) y = fx_scaled(fx.beta, y);
+    FMat x = sf.form(grp == 1 ? at_d : sf.at(neg ? kp + dk : kp), kLinkPlane + nud, true, neg);
+    bad = bad || fx_poisoned(x);
+    if (grp == 1) {
+        const FMat t = x;
+        x = y;
+        y = t;
+    }
+    fx_zero(acc);
+    fx_mul_acc<N, N>(acc, x, y);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        FSum re, im;
+        fx_total<1>(acc, e / 3, e % 3, re, im);
+        // units 2^-57; the FP32 part in units of 2^-54
+        z[e] = make_longlong2((re.v >> 1) + 4ll * __float2int_rn(0.125f * re.c), (im.v >> 1) + 4ll * __float2int_rn(0.125f * im.c));
+    }
+}
 
+// The force (and the fused momentum step) from the sum z_of(e) of the groups;
+// returns the link's share of the action.
+template <bool ACTION, typename Z>
+__device__ __forceinline__ double fx_finish(const SfLattice &L, const KernelScalars &sc, const FxScalars &fx,
+                                            const FxPlanes &sf, int64_t V, int rho, int k, bool bad, const Z &z_of)
+{
+    const int base = rho * 6;
     const FLimbs u = sf.limbs(sf.at(k), kLinkPlane + rho);
-    bad = bad || fx_poisoned(u);
-    if (bad) return force_link_floating<ACTION>(L, sc, k, rho);
+    if (bad || fx_poisoned(u)) return force_link_floating<ACTION>(L, sc, k, rho);
 
     // The plaquette sum, t / m and U t / m decide the accuracy of the result:
     // whole limbs.
@@ -323,12 +313,11 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
 #pragma unroll
     for (int e = 0; e < 9; ++e) {
         const int i = e / 3, j = e % 3;
-        const longlong2 v = zv[e * kBlock];
-        const float2 w = zc[e * kBlock];
-        const auto sum = [&](long long zval, float zrem, long long p, int &th, int &tl) {
+        const longlong2 v = z_of(e);
+        const auto sum = [&](long long zval, long long p, int &th, int &tl) {
             int zh;
             float zl;
-            fx_split<31>(FSum{zval, zrem}, zh, zl);    // up to 42, units 2^-25
+            fx_split<31>(FSum{zval, 0.f}, zh, zl);     // up to 42, units 2^-25
             const int p32 = (int)p;
             const int ph = (int)(p >> 32) + (int)((unsigned)p32 >> 31);
             // in units 2^-60: pl times p = ph 2^32 + p32, and z times the rest
@@ -339,8 +328,8 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
             th = (int)((y + (1ll << 27)) >> 28);
             tl = (int)((unsigned)y - ((unsigned)th << 28));
         };
-        sum(v.x, w.x, pr[e], t.rh[i][j], t.rl[i][j]);
-        sum(v.y, w.y, pi[e], t.ih[i][j], t.il[i][j]);
+        sum(v.x, pr[e], t.rh[i][j], t.rl[i][j]);
+        sum(v.y, pi[e], t.ih[i][j], t.il[i][j]);
     }
     FLimbAcc acc;
     fx_zero(acc);
@@ -387,15 +376,49 @@ __device__ __forceinline__ double fx_force_link(const SfLattice &L, const Kernel
     return 0.0;
 }
 
+// The four directions of 32 sites, one per warp.  The total of the groups
+// stays in shared memory, out of the registers' way.
 template <bool ACTION>
 __device__ __forceinline__ double fx_force_block(const SfLattice &L, const KernelScalars &sc, const FxScalars &fx,
                                                  const G32 &g, const Sweep &sw, int vb)
 {
+    __shared__ longlong2 z_s[9][kBlock];
+    longlong2 *zs = &z_s[0][threadIdx.x];
     const int rho = (int)(threadIdx.x >> 5);
     const int j = vb * 32 + (int)(threadIdx.x & 31);
     if (j >= g.V) return 0.0;
     const Coord c = swept_site(sw, j);
-    return fx_force_link<ACTION>(L, sc, fx, g, c, index32(g, c), rho);
+    const int k = index32(g, c);
+    const FxPlanes sf = fx_planes(L);
+    bool bad = false;
+#pragma unroll 1
+    for (int grp = 0; grp < 8; ++grp) {
+        longlong2 z[9];
+        fx_group(z, bad, sf, fx, g, c, rho, k, grp);
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            if (grp > 0) {
+                const longlong2 o = zs[e * kBlock];
+                z[e].x += o.x;
+                z[e].y += o.y;
+            }
+            zs[e * kBlock] = z[e];
+        }
+    }
+    return fx_finish<ACTION>(L, sc, fx, sf, g.V, rho, k, bad, [&](int e) { return zs[e * kBlock]; });
+}
+
+// The partial sums of virtual block vb: four for a split lattice, so that the
+// action does not depend on which kernel made them.
+__device__ __forceinline__ void fx_store_partials(const SfLattice &L, int vb, double share)
+{
+    if (L.split) {
+        const double s = warp_sum(share);
+        if ((threadIdx.x & 31) == 0) L.partials[vb * 4 + (threadIdx.x >> 5)] = s;
+    } else {
+        const double s = block_sum(share);
+        if (threadIdx.x == 0) L.partials[vb] = s;
+    }
 }
 
 template <bool ACTION>
@@ -408,10 +431,55 @@ __global__ void __launch_bounds__(kBlock, 2)
     const int nvb = (int)virtual_blocks(g.V);
     for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
         const double acc = fx_force_block<ACTION>(L, sc, fx, g, sw, vb);
-        if constexpr (ACTION) {
-            const double s = block_sum(acc);
-            if (threadIdx.x == 0) L.partials[vb] = s;
+        if constexpr (ACTION) fx_store_partials(L, vb, acc);
+    }
+}
+
+// Split lattices: direction rho of 32 sites, a group on each of eight warps,
+// the first adding them up (whole numbers: the sum of force_fx to the bit).
+constexpr int kSplitBlock = 256;
+
+template <bool ACTION>
+__global__ void __launch_bounds__(kSplitBlock, 1)
+    force_fx_split(const __grid_constant__ SfLattice L, const __grid_constant__ KernelScalars sc,
+                   const __grid_constant__ FxScalars fx)
+{
+    __shared__ longlong2 z_s[7][9][32];
+    __shared__ unsigned bad_s[8];
+    const G32 g = make_g32(L.dims);
+    const Sweep sw = make_sweep(L, g);
+    const int vb = (int)(blockIdx.x >> 2), rho = (int)(blockIdx.x & 3);
+    const int grp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+    const int j = vb * 32 + lane;
+    const Coord c = swept_site(sw, j < g.V ? j : g.V - 1);
+    const int k = index32(g, c);
+    const FxPlanes sf = fx_planes(L);
+    longlong2 z[9];
+    bool bad = false;
+    fx_group(z, bad, sf, fx, g, c, rho, k, grp);
+    const unsigned marks = __ballot_sync(0xffffffffu, bad);
+    if (lane == 0) bad_s[grp] = marks;
+    if (grp > 0) {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) z_s[grp - 1][e][lane] = z[e];
+    }
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int p = 1; p < 8; ++p) bad = bad || (bad_s[p] >> lane & 1);
+#pragma unroll 1
+    for (int p = 0; p < 7; ++p)
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const longlong2 o = z_s[p][e][lane];
+            z[e].x += o.x;
+            z[e].y += o.y;
         }
+    double share = 0.0;
+    if (j < g.V) share = fx_finish<ACTION>(L, sc, fx, sf, g.V, rho, k, bad, [&](int e) { return z[e]; });
+    if constexpr (ACTION) {
+        share = warp_sum(share);
+        if (lane == 0) L.partials[vb * 4 + rho] = share;
     }
 }
 
@@ -424,11 +492,9 @@ __global__ void __launch_bounds__(kBlock, 2)
         const unsigned long long next = claim_virtual_block(B.counter + 1);
         const SfLattice &L = B.e[batch_entry(B, vb)];
         const G32 g = make_g32(L.dims);
-        const double acc = fx_force_block<ACTION>(L, sc, fx, g, make_sweep(L, g), (int)(vb - L.vb_begin));
-        if constexpr (ACTION) {
-            const double s = block_sum(acc);
-            if (threadIdx.x == 0) L.partials[vb - L.vb_begin] = s;
-        }
+        const int v = (int)(vb - L.vb_begin);
+        const double acc = fx_force_block<ACTION>(L, sc, fx, g, make_sweep(L, g), v);
+        if constexpr (ACTION) fx_store_partials(L, v, acc);
         vb = publish_virtual_block(next);
     }
 }
@@ -444,10 +510,13 @@ cudaError_t launch_fx_passes(const SfLattice &L, const KernelScalars &sc, bool a
     links_fx<<<grid, kBlock, 0, st>>>(L);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    staples_fx<<<grid, kBlock, 0, st>>>(L);
+    staples_fx<<<L.split ? 6 * grid : grid, kBlock, 0, st>>>(L);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (action) force_fx<true><<<grid, kBlock, 0, st>>>(L, sc, fx);
+    if (L.split) {
+        if (action) force_fx_split<true><<<4 * grid, kSplitBlock, 0, st>>>(L, sc, fx);
+        else force_fx_split<false><<<4 * grid, kSplitBlock, 0, st>>>(L, sc, fx);
+    } else if (action) force_fx<true><<<grid, kBlock, 0, st>>>(L, sc, fx);
     else force_fx<false><<<grid, kBlock, 0, st>>>(L, sc, fx);
     return cudaGetLastError();
 }

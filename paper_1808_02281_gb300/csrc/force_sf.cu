@@ -86,6 +86,27 @@ __device__ __forceinline__ void site_staples(const R *__restrict__ links, const 
     }
 }
 
+// Staple plane mu*6 + j of site x (site_staples one at a time).
+template <typename R, bool FULL>
+__device__ __forceinline__ void site_staple(const R *__restrict__ links, const G32 &g, const Coord &c, int x, int mu, int j,
+                                            const Planes<R, FULL> &sf)
+{
+    const int64_t V = g.V;
+    const int nu = (mu + 1 + (j >> 1)) & 3;
+    const int xm = x + step32(g, c, mu, 1);
+    Mat<R> s;
+    if ((j & 1) == 0) {
+        const Mat<R> t = mul<N, D>(load_link(links, V, nu, xm), load_link(links, V, mu, x + step32(g, c, nu, 1)));
+        s = mul_top2<N, D>(t, load_link(links, V, nu, x));
+    } else {
+        const int vm = step32(g, c, nu, -1);
+        const Mat<R> t = mul<D, D>(load_link(links, V, nu, xm + vm), load_link(links, V, mu, x + vm));
+        s = mul_top2<N, N>(t, load_link(links, V, nu, x + vm));
+    }
+    if constexpr (FULL) rebuild_row2(s);
+    sf.store(sf.at(x), mu * 6 + j, s);
+}
+
 // The 24 staples of the 32 sites of virtual block vb: thread = (site, mu).
 template <typename R, bool FULL>
 __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, int vb)
@@ -103,6 +124,35 @@ __global__ void __launch_bounds__(kBlock) staple_fields(const __grid_constant__ 
     const G32 g = make_g32(L.dims);
     const int nvb = (int)virtual_blocks(g.V);
     for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x) staples_block<R, FULL>(L, g, vb);
+}
+
+// Staples q, q + 4 of each direction (split lattices: a quarter of the work
+// of staples_block in a CTA of its own).
+template <typename R, bool FULL>
+__device__ __forceinline__ void split_staples_block(const SfLattice &L, const G32 &g, int vb, int q)
+{
+    const int mu = (int)(threadIdx.x >> 5);
+    const int x = vb * 32 + (int)(threadIdx.x & 31);
+    if (x >= g.V) return;
+    const Coord c = coord32(g, L.div, x);
+#pragma unroll 1
+    for (int j = q; j < 6; j += 4)
+        site_staple<R, FULL>(static_cast<const R *>(L.links), g, c, x, mu, j, planes_of<R, FULL>(L));
+}
+
+template <typename R, bool FULL>
+__global__ void __launch_bounds__(kBlock) staple_fields_split(const __grid_constant__ SfLattice L)
+{
+    split_staples_block<R, FULL>(L, make_g32(L.dims), (int)(blockIdx.x >> 2), (int)(blockIdx.x & 3));
+}
+
+// The same for a batch of split lattices only.
+template <typename R, bool FULL>
+__global__ void __launch_bounds__(kBlock) staple_fields_split_batched(const __grid_constant__ SfBatch B)
+{
+    const SfLattice &L = B.e[batch_entry(B, blockIdx.x)];
+    const int v = (int)(blockIdx.x - L.vb_begin);
+    split_staples_block<R, FULL>(L, make_g32(L.dims), v >> 2, v & 3);
 }
 
 template <typename R, bool FULL>
@@ -133,6 +183,76 @@ __device__ __forceinline__ double force_block(const SfLattice &L, const KernelSc
     const int k = index32(g, c);
     const LatticeSites si{&g, &c, k};
     return force_link<R, ACTION, UNROLLQ, false>(L, sc, g, planes_of<R, FULL>(L), si, c, k, rho);
+}
+
+// Split lattices: the links of direction rho of virtual block vb, warp 0 their
+// plaquettes and chains, warps 1 to 3 the terms of one direction d each; warp
+// 0 adds them up.  A quarter of force_block's chain of products (14 against
+// 51 of a thread).  The action's share goes to partial vb*4 + rho.
+template <typename R, bool ACTION>
+__device__ __forceinline__ void split_force_block(const SfLattice &L, const KernelScalars &sc, const G32 &g,
+                                                  const Sweep &sw, int vb, int rho)
+{
+    __shared__ R t_s[3][18][32];
+    const int part = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+    const int j = vb * 32 + lane;
+    const Coord c = swept_site(sw, j < g.V ? j : g.V - 1);
+    const int k = index32(g, c), kp = k + step32(g, c, rho, 1);
+    const LatticeSites si{&g, &c, k};
+    const auto sf = planes_of<R, true>(L);
+    const R *__restrict__ links = static_cast<const R *>(L.links);
+    const R c_rt = scalar<R>(sc, SC_CRT), c_cb = scalar<R>(sc, SC_CCB);
+    Mat<R> t;
+    R tr_pl = R(0);
+    if (part == 0) {
+        chain_terms<R, ACTION, false>(t, tr_pl, links, sf, si, g, c, rho, k, kp, scalar<R>(sc, SC_CPL), c_rt);
+    } else {
+        set_zero(t);
+        d_terms<false, false, false>(t, links, sf, si, g, c, rho, k, kp, part - 1, c_rt, c_cb);
+        d_terms<true, false, false>(t, links, sf, si, g, c, rho, k, kp, part - 1, c_rt, c_cb);
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            t_s[part - 1][2 * e][lane] = t.re[e / 3][e % 3];
+            t_s[part - 1][2 * e + 1][lane] = t.im[e / 3][e % 3];
+        }
+    }
+    __syncthreads();
+    if (part == 0) {
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                t.re[e / 3][e % 3] += t_s[p][2 * e][lane];
+                t.im[e / 3][e % 3] += t_s[p][2 * e + 1][lane];
+            }
+        double share = 0.0;
+        if (j < g.V) share = finish_link<R, ACTION>(L, sc, links, g.V, rho, k, t, tr_pl);
+        if constexpr (ACTION) {
+            share = warp_sum(share);
+            if (lane == 0) L.partials[vb * 4 + rho] = share;
+        }
+    }
+    __syncthreads(); // before t_s is written again
+}
+
+template <typename R, bool ACTION>
+__global__ void __launch_bounds__(kBlock, 4)
+    force_split(const __grid_constant__ SfLattice L, const __grid_constant__ KernelScalars sc)
+{
+    const G32 g = make_g32(L.dims);
+    split_force_block<R, ACTION>(L, sc, g, make_sweep(L, g), (int)(blockIdx.x >> 2), (int)(blockIdx.x & 3));
+}
+
+// The split lattices of a batch, in a launch of their own: with both kinds of
+// block in one kernel the large lattices took 3 to 6 % longer.
+template <typename R, bool ACTION>
+__global__ void __launch_bounds__(kBlock, 4)
+    force_split_batched(const __grid_constant__ SfBatch B, const __grid_constant__ KernelScalars sc)
+{
+    const SfLattice &L = B.e[batch_entry(B, blockIdx.x)];
+    const G32 g = make_g32(L.dims);
+    const int v = (int)(blockIdx.x - L.vb_begin);
+    split_force_block<R, ACTION>(L, sc, g, make_sweep(L, g), v >> 2, v & 3);
 }
 
 // Resident CTAs per SM the register allocation aims at: 4 (128 registers)
@@ -189,7 +309,7 @@ __global__ void __launch_bounds__(1024) finish_batched(const __grid_constant__ S
 {
     const SfLattice &L = B.e[blockIdx.x];
     if (L.action == nullptr) return;
-    const int count = (int)virtual_blocks((int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3]);
+    const int count = (int)virtual_blocks((int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3]) * (L.split ? 4 : 1);
     __shared__ double warp_part[32];
     double v = 0.0;
     for (int i = threadIdx.x; i < count; i += 1024) v += L.partials[i];
@@ -362,6 +482,14 @@ size_t round_up256(size_t b) { return (b + 255) & ~(size_t)255; }
 cudaError_t launch_passes(const SfLattice &L, const KernelScalars &sc, int variant, bool action, cudaStream_t st)
 {
     const unsigned grid = grid_of(virtual_blocks((int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3]));
+    if (L.split) {
+        staple_fields_split<float, true><<<4 * grid, kBlock, 0, st>>>(L);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (action) force_split<float, true><<<4 * grid, kBlock, 0, st>>>(L, sc);
+        else force_split<float, false><<<4 * grid, kBlock, 0, st>>>(L, sc);
+        return cudaGetLastError();
+    }
     if (full_staples(variant)) staple_fields<float, true><<<grid, kBlock, 0, st>>>(L);
     else staple_fields<float, false><<<grid, kBlock, 0, st>>>(L);
     const cudaError_t e = cudaGetLastError();
@@ -369,20 +497,47 @@ cudaError_t launch_passes(const SfLattice &L, const KernelScalars &sc, int varia
     return action ? launch_pass_b<true>(L, sc, variant, st) : launch_pass_b<false>(L, sc, variant, st);
 }
 
-cudaError_t launch_passes_batched(const SfBatch &B, const KernelScalars &sc, int variant, bool action,
-                                  cudaStream_t st)
+// The lattices of B with (or without) split set, numbered anew in blocks of
+// 32 sites or quarters of one.
+SfBatch part_of(const SfBatch &B, bool split)
 {
-    if (full_staples(variant)) {
+    SfBatch p{};
+    p.counter = B.counter;
+    for (int c = 0; c < B.n; ++c) {
+        if ((B.e[c].split != 0) != split) continue;
+        const int *d = B.e[c].dims;
+        SfLattice &L = p.e[p.n++];
+        L = B.e[c];
+        L.vb_begin = p.total;
+        p.total += virtual_blocks((int64_t)d[0] * d[1] * d[2] * d[3]) * (split ? 4 : 1);
+    }
+    return p;
+}
+
+cudaError_t launch_passes_batched(const SfBatch &B, const KernelScalars &sc, int variant, bool action, cudaStream_t st)
+{
+    const SfBatch split = part_of(B, true);
+    if (split.n == B.n) {
+        staple_fields_split_batched<float, true><<<grid_of(split.total), kBlock, 0, st>>>(split);
+    } else if (full_staples(variant)) {
         auto ka = staple_fields_batched<float, true>;
         ka<<<persistent_grid(ka, grid_slot(5, false, false), B.total), kBlock, 0, st>>>(B);
     } else {
         auto ka = staple_fields_batched<float, false>;
         ka<<<persistent_grid(ka, grid_slot(4, false, false), B.total), kBlock, 0, st>>>(B);
     }
-    const cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return action ? launch_pass_b_batched<true>(B, sc, variant, st)
-                  : launch_pass_b_batched<false>(B, sc, variant, st);
+    if (split.n > 0) {
+        if (action) force_split_batched<float, true><<<grid_of(split.total), kBlock, 0, st>>>(split, sc);
+        else force_split_batched<float, false><<<grid_of(split.total), kBlock, 0, st>>>(split, sc);
+        e = cudaGetLastError();
+        if (e != cudaSuccess || split.n == B.n) return e;
+        const SfBatch whole = part_of(B, false);
+        return action ? launch_pass_b_batched<true>(whole, sc, variant, st)
+                      : launch_pass_b_batched<false>(whole, sc, variant, st);
+    }
+    return action ? launch_pass_b_batched<true>(B, sc, variant, st) : launch_pass_b_batched<false>(B, sc, variant, st);
 }
 
 } // namespace
@@ -404,7 +559,8 @@ bool staple_fields_supported(const int dims[4])
 
 int staple_force_partials(const int dims[4])
 {
-    return (int)virtual_blocks((int64_t)dims[0] * dims[1] * dims[2] * dims[3]);
+    const int64_t V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
+    return (int)virtual_blocks(V) * (split_lattice(LQCD_F32, V) || split_lattice(LQCD_F64, V) ? 4 : 1);
 }
 
 cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
@@ -415,6 +571,7 @@ cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
     for (int i = 0; i < 4; ++i) L.dims[i] = a.dims[i];
     set_traversal(L, variant);
     L.plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
+    L.split = split_lattice(a.precision, V) && (a.precision == LQCD_F64 || full_staples(variant));
     L.links = a.links;
     L.staples = a.staples;
     L.force = a.force;
@@ -426,7 +583,7 @@ cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
     const cudaError_t e = a.precision == LQCD_F64 ? launch_fx_passes(L, sc, action, st)
                                                   : launch_passes(L, sc, variant, action, st);
     if (e != cudaSuccess || !action) return e;
-    return launch_finish_sum(a.partials, (int)virtual_blocks(V), a.beta / 3.0, a.action, st);
+    return launch_finish_sum(a.partials, (int)virtual_blocks(V) * (L.split ? 4 : 1), a.beta / 3.0, a.action, st);
 }
 
 cudaError_t launch_force_staple_fields_batched(const ForceArgs &a, int n, const SfLattice *items,
@@ -438,18 +595,17 @@ cudaError_t launch_force_staple_fields_batched(const ForceArgs &a, int n, const 
     B.n = n;
     B.counter = counter;
     bool any_action = false;
-    int64_t vb = 0;
     for (int c = 0; c < n; ++c) {
         const int *d = items[c].dims;
         const int64_t V = (int64_t)d[0] * d[1] * d[2] * d[3];
         B.e[c] = items[c];
         set_traversal(B.e[c], variant);
         B.e[c].plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
-        B.e[c].vb_begin = vb;
-        vb += virtual_blocks(V);
-        any_action = any_action || items[c].action != nullptr;
+        B.e[c].split = split_lattice(a.precision, V) && (a.precision == LQCD_F64 || full_staples(variant));
+        B.e[c].vb_begin = B.total;
+        B.total += virtual_blocks(V);
+        any_action = any_action || B.e[c].action != nullptr;
     }
-    B.total = vb;
     const KernelScalars sc = make_scalars(a);
     cudaError_t e = cudaMemsetAsync(counter, 0, 3 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;

@@ -92,13 +92,14 @@ struct SfLattice {
     // extents, micro-tiles along x and y of a block, blocks along x and y
     DivMagic div[12];
     int counts[4];     // blocks along x and y, micro-tiles along x and y of a block
+    int split;         // a link's sums on several warps (split_lattice), four partials per virtual block
     int64_t vb_begin;  // batch: first virtual block of this lattice
     int64_t plane_bytes; // full staple planes: bytes of one plane
     const void *links;
     void *staples;     // 24 staple planes (FP64: and 4 link planes; workspace)
     void *force;       // written when set
     void *mom;         // p += dt f when set
-    double *partials;  // one action partial per virtual block
+    double *partials;  // one action partial per virtual block, or four
     double *action;    // action written here when set
 };
 

@@ -486,51 +486,43 @@ __device__ __forceinline__ void d_terms(Mat<R> &t, const R *__restrict__ links,
     }
 }
 
-// Force (and the fused momentum step) on the link (k, rho), k at coordinates
-// c, its staples found through si; returns its share of the action.
-template <typename R, bool ACTION, bool UNROLLQ, bool DIRECT, typename SF, typename SI>
-__device__ __forceinline__ double force_link(const SfLattice &L, const KernelScalars &sc, const G32 &g,
-                                             const SF &sf, const SI &si, const Coord &c,
-                                             int k, int rho)
+// The plaquettes and the two rectangle chains along rho: t = c_plaq Pl +
+// c_rect (F sum_b S_b(k+rho) S_b(k) + sum_b S_b(k) S_b(k-rho) E); tr_pl the
+// trace of U Pl for the action.
+template <typename R, bool ACTION, bool DIRECT, typename SF, typename SI>
+__device__ __forceinline__ void chain_terms(Mat<R> &t, R &tr_pl, const R *__restrict__ links, const SF &sf, const SI &si,
+                                            const G32 &g, const Coord &c, int rho, int k, int kp, R c_pl, R c_rt)
 {
-    const R *__restrict__ links = static_cast<const R *>(L.links);
     const int64_t V = g.V;
-    const R c_pl = scalar<R>(sc, SC_CPL), c_rt = scalar<R>(sc, SC_CRT), c_cb = scalar<R>(sc, SC_CCB);
-    const int kp = k + step32(g, c, rho, 1), km = k + step32(g, c, rho, -1);
+    const int km = k + step32(g, c, rho, -1);
     const int base = rho * 6;
-
-    // plaquettes and the two rectangle chains along rho
-    Mat<R> t;
-    R tr_pl = R(0);
-    {
-        Mat<R> pl, p1, p2;
-        set_zero(pl);
-        set_zero(p1);
-        set_zero(p2);
-        const auto at_k = sf.at(si.at0()), at_p = sf.at(si.nb(rho, 1)), at_m = sf.at(si.nb(rho, -1));
+    Mat<R> pl, p1, p2;
+    set_zero(pl);
+    set_zero(p1);
+    set_zero(p2);
+    const auto at_k = sf.at(si.at0()), at_p = sf.at(si.nb(rho, 1)), at_m = sf.at(si.nb(rho, -1));
 #pragma unroll 1
-        for (int jj = 0; jj < 6; ++jj) {
-            const Mat<R> s = sf.load(at_k, base + jj);
-            add_to(pl, s);
-            acc_su3<N, DIRECT>(p1, sf.load(at_p, base + jj), s, c_rt);
-            mul_acc<N, N>(p2, s, sf.load(at_m, base + jj));
-        }
-        if constexpr (ACTION) tr_pl = re_trace_mul<N, N>(load_link(links, V, rho, k), pl);
-        t = pl;
-        scale(t, c_pl);
-        if constexpr (DIRECT) scale(p1, c_rt);
-        mul_acc<N, N>(t, load_link(links, V, rho, kp), p1);
-        scale(p2, c_rt);
-        mul_acc<N, N>(t, p2, load_link(links, V, rho, km));
+    for (int jj = 0; jj < 6; ++jj) {
+        const Mat<R> s = sf.load(at_k, base + jj);
+        add_to(pl, s);
+        acc_su3<N, DIRECT>(p1, sf.load(at_p, base + jj), s, c_rt);
+        mul_acc<N, N>(p2, s, sf.load(at_m, base + jj));
     }
-    // cubes and the rectangles along d: positive, then negative d
-#pragma unroll 1
-    for (int id = 0; id < 3; ++id)
-        d_terms<false, UNROLLQ, DIRECT>(t, links, sf, si, g, c, rho, k, kp, id, c_rt, c_cb);
-#pragma unroll 1
-    for (int id = 0; id < 3; ++id)
-        d_terms<true, UNROLLQ, DIRECT>(t, links, sf, si, g, c, rho, k, kp, id, c_rt, c_cb);
+    if constexpr (ACTION) tr_pl = re_trace_mul<N, N>(load_link(links, V, rho, k), pl);
+    t = pl;
+    scale(t, c_pl);
+    if constexpr (DIRECT) scale(p1, c_rt);
+    mul_acc<N, N>(t, load_link(links, V, rho, kp), p1);
+    scale(p2, c_rt);
+    mul_acc<N, N>(t, p2, load_link(links, V, rho, km));
+}
 
+// The force from the staple sum t (stored, and/or the momentum step); returns
+// the link's share of the action.
+template <typename R, bool ACTION>
+__device__ __forceinline__ double finish_link(const SfLattice &L, const KernelScalars &sc, const R *__restrict__ links,
+                                              int64_t V, int rho, int k, const Mat<R> &t, R tr_pl)
+{
     const Mat<R> m = mul<N, N>(load_link(links, V, rho, k), t);
     R f[8];
     ta_components(m, scalar<R>(sc, SC_BETA6), f);
@@ -551,7 +543,53 @@ __device__ __forceinline__ double force_link(const SfLattice &L, const KernelSca
     return 0.0;
 }
 
+// Force (and the fused momentum step) on the link (k, rho), k at coordinates
+// c, its staples found through si; returns its share of the action.
+template <typename R, bool ACTION, bool UNROLLQ, bool DIRECT, typename SF, typename SI>
+__device__ __forceinline__ double force_link(const SfLattice &L, const KernelScalars &sc, const G32 &g,
+                                             const SF &sf, const SI &si, const Coord &c,
+                                             int k, int rho)
+{
+    const R *__restrict__ links = static_cast<const R *>(L.links);
+    const R c_rt = scalar<R>(sc, SC_CRT), c_cb = scalar<R>(sc, SC_CCB);
+    const int kp = k + step32(g, c, rho, 1);
+    Mat<R> t;
+    R tr_pl = R(0);
+    chain_terms<R, ACTION, DIRECT>(t, tr_pl, links, sf, si, g, c, rho, k, kp, scalar<R>(sc, SC_CPL), c_rt);
+    // cubes and the rectangles along d: positive, then negative d
+#pragma unroll 1
+    for (int id = 0; id < 3; ++id)
+        d_terms<false, UNROLLQ, DIRECT>(t, links, sf, si, g, c, rho, k, kp, id, c_rt, c_cb);
+#pragma unroll 1
+    for (int id = 0; id < 3; ++id)
+        d_terms<true, UNROLLQ, DIRECT>(t, links, sf, si, g, c, rho, k, kp, id, c_rt, c_cb);
+    return finish_link<R, ACTION>(L, sc, links, g.V, rho, k, t, tr_pl);
+}
+
 // ------------------------------------------------------------- launch sizes
+
+// Lattices of up to this many virtual blocks have a link's sums computed by
+// several warps: four in FP32 (force_sf.cu), eight in FP64 (force_fx.cu).
+// While there are fewer blocks than SMs a launch lasts as long as one thread's
+// chain of products.  Measured, whole | split, force and action: FP32 4^4 24.6
+// | 17.4 us, 64 blocks 26.7 | 17.1, 128 28.7 | 20.5, 256 30.5 | 32.7; FP64 8
+// blocks 73.7 | 30.8, 64 75.6 | 45.2, 128 75.9 | 72.4, 256 97 | 123.  FP32
+// stops at 64 because batches that mix both kinds launch the split ones apart
+// (7 us).
+constexpr int kSplitBlocks[2] = {64, 128}; // FP32, FP64
+inline bool split_lattice(int precision, int64_t V)
+{
+    return virtual_blocks(V) <= kSplitBlocks[precision == LQCD_F64 ? 1 : 0];
+}
+
+// Sum over a warp of one double per lane (result in lane 0), the order of
+// block_sum's first stage.
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+}
 
 inline unsigned grid_of(int64_t items)
 {
