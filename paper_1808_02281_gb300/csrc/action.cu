@@ -96,8 +96,8 @@ __device__ __noinline__ double walked_loops(const ReduceArgs &a, const LoopTable
 // and SM, would take as long as a third of the products).
 struct Plain {
     using M = Mat<float>;
-    static constexpr int kMinBlocks = 4, kWords = 18;
-    using Word = float;
+    static constexpr int kMinBlocks = 4, kWords = 5; // the last half full
+    using Word = float4;
     const float *links;
     int64_t V;
 
@@ -112,19 +112,25 @@ struct Plain {
     template <int STRIDE> __device__ __forceinline__ static void put(Word *p, const M &x)
     {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            p[2 * e * STRIDE] = x.re[e / 3][e % 3];
-            p[(2 * e + 1) * STRIDE] = x.im[e / 3][e % 3];
-        }
+        for (int e = 0; e < 8; e += 2)
+            p[(e / 2) * STRIDE] = make_float4(x.re[e / 3][e % 3], x.im[e / 3][e % 3], x.re[(e + 1) / 3][(e + 1) % 3],
+                                              x.im[(e + 1) / 3][(e + 1) % 3]);
+        *reinterpret_cast<float2 *>(p + 4 * STRIDE) = make_float2(x.re[2][2], x.im[2][2]);
     }
     template <int STRIDE> __device__ __forceinline__ static M get(const Word *p)
     {
         M x;
 #pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            x.re[e / 3][e % 3] = p[2 * e * STRIDE];
-            x.im[e / 3][e % 3] = p[(2 * e + 1) * STRIDE];
+        for (int e = 0; e < 8; e += 2) {
+            const float4 v = p[(e / 2) * STRIDE];
+            x.re[e / 3][e % 3] = v.x;
+            x.im[e / 3][e % 3] = v.y;
+            x.re[(e + 1) / 3][(e + 1) % 3] = v.z;
+            x.im[(e + 1) / 3][(e + 1) % 3] = v.w;
         }
+        const float2 v = *reinterpret_cast<const float2 *>(p + 4 * STRIDE);
+        x.re[2][2] = v.x;
+        x.im[2][2] = v.y;
         return x;
     }
     struct Traces {
