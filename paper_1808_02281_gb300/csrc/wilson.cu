@@ -269,17 +269,16 @@ __device__ __forceinline__ void hop_x_shuffled(Spinor<R> &acc, const R *__restri
 
 constexpr int kDslashBlock = 128;
 
-// Register cap: 5 blocks (20 warps, 96 registers, a 64-byte spill) per SM in
-// FP32: at 32^3x64 0.161 against 0.167 ms with 4 blocks (128 registers) and
-// 0.245 ms with the uncapped 138 (12 warps) -- the kernel waits on loads, so
-// warps in flight count more than the spill; FP64 is bound by the FP64 pipe
-// and keeps its registers.
-template <typename R> constexpr int dslash_min_blocks() { return sizeof(R) == 8 ? 1 : 5; }
+// Register cap: 5 blocks (20 warps, 96 registers, a 64-byte spill) per SM: at
+// 32^3x64 0.161 against 0.167 ms with 4 blocks (128 registers) and 0.245 ms
+// with the uncapped 138 (12 warps) -- the kernel waits on loads, so warps in
+// flight count more than the spill.
+constexpr int kDslashMinBlocks = 5;
 
 // out_n = ca x_n + cb (calD x)_n, one thread per site.
 // XSHFL: x hops by shuffles.
 template <typename R, bool XSHFL, typename I>
-__global__ void __launch_bounds__(kDslashBlock, dslash_min_blocks<R>())
+__global__ void __launch_bounds__(kDslashBlock, kDslashMinBlocks)
     wilson_dslash(const __grid_constant__ WilsonArgs a)
 {
     const Sites<I> g = make_sites<I>(a.dims);
@@ -327,6 +326,33 @@ __global__ void __launch_bounds__(kDslashBlock, dslash_min_blocks<R>())
         }
         store_spinor(out, V, (int64_t)n, acc);
     }
+}
+
+// out_n = ca x_n + cb acc (x not read for ca = 0).
+__device__ __forceinline__ void store_dslash(const WilsonArgs &a, const double *__restrict__ x, int64_t V, int64_t n,
+                                             Spinor<double> &acc, double ca, double cb)
+{
+    Spinor<double> xn;
+    if (ca != 0.0) xn = load_spinor(x, V, n);
+#pragma unroll
+    for (int al = 0; al < 4; ++al)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            acc.re[al][b] *= cb;
+            acc.im[al][b] *= cb;
+            if (ca != 0.0) {
+                acc.re[al][b] = fma(ca, xn.re[al][b], acc.re[al][b]);
+                acc.im[al][b] = fma(ca, xn.im[al][b], acc.im[al][b]);
+            }
+        }
+    store_spinor(static_cast<double *>(a.out), V, n, acc);
+}
+
+// gcode at run time.
+__device__ __forceinline__ int gcode_of(int mu, int alpha)
+{
+    return mu == 0 ? (alpha < 2 ? 1 : 3) : mu == 1 ? ((alpha == 0 || alpha == 3) ? 2 : 0)
+           : mu == 2 ? ((alpha == 0 || alpha == 3) ? 1 : 3) : 0;
 }
 
 // --------------------------------------------------- hopping-term force
@@ -423,24 +449,31 @@ __device__ __forceinline__ bool fx_half(const double *__restrict__ x, int64_t V,
     return true;
 }
 
-// u h on both colour vectors.
+// u h (D: u^dagger h) on both colour vectors.
+template <int F> __device__ __forceinline__ void fx_colour_sums(const FLimbs &u, const FHalf &h, int al, FLimbAcc &y)
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a) y.h1[a][0] = y.l1[a][0] = y.h2[a][0] = y.l2[a][0] = y.h3[a][0] = y.l3[a][0] = 0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const int sh = h.rh[al][b] + h.ih[al][b], sl = h.rl[al][b] + h.il[al][b];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int p = F == N ? a : b, q = F == N ? b : a;
+            fx_mad(y.h1[a][0], y.l1[a][0], u.rh[p][q], u.rl[p][q], h.rh[al][b], h.rl[al][b]);
+            fx_mad(y.h2[a][0], y.l2[a][0], u.ih[p][q], u.il[p][q], h.ih[al][b], h.il[al][b]);
+            fx_mad(y.h3[a][0], y.l3[a][0], F == N ? u.rh[p][q] + u.ih[p][q] : u.rh[p][q] - u.ih[p][q],
+                   F == N ? u.rl[p][q] + u.il[p][q] : u.rl[p][q] - u.il[p][q], sh, sl);
+        }
+    }
+}
+
 __device__ __forceinline__ void fx_colour_mul(const FLimbs &u, FHalf &h)
 {
 #pragma unroll
     for (int al = 0; al < 2; ++al) {
         FLimbAcc y; // column 0
-#pragma unroll
-        for (int a = 0; a < 3; ++a) y.h1[a][0] = y.l1[a][0] = y.h2[a][0] = y.l2[a][0] = y.h3[a][0] = y.l3[a][0] = 0;
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const int sh = h.rh[al][b] + h.ih[al][b], sl = h.rl[al][b] + h.il[al][b];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                fx_mad(y.h1[a][0], y.l1[a][0], u.rh[a][b], u.rl[a][b], h.rh[al][b], h.rl[al][b]);
-                fx_mad(y.h2[a][0], y.l2[a][0], u.ih[a][b], u.il[a][b], h.ih[al][b], h.il[al][b]);
-                fx_mad(y.h3[a][0], y.l3[a][0], u.rh[a][b] + u.ih[a][b], u.rl[a][b] + u.il[a][b], sh, sl);
-            }
-        }
+        fx_colour_sums<N>(u, h, al, y);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             long long re, im;
@@ -612,6 +645,125 @@ __global__ void __launch_bounds__(kForceBlock, 4) wilson_hopping_force_fx(const 
     if (!hopping_force_fx(a, V, rho, k, kp)) hopping_force_floating(a, V, rho, k, kp);
 }
 
+// ------------------------------------------------ hopping operator, FP64
+
+// One site of y = ca x + cb calD x in floating point, for sites that
+// dslash_site_fx leaves.
+template <typename I>
+__device__ __noinline__ void dslash_site_floating(const WilsonArgs &a, const Sites<I> &g, const Coord &c, I n)
+{
+    const double *__restrict__ links = static_cast<const double *>(a.links);
+    const double *__restrict__ x = static_cast<const double *>(a.x);
+    Spinor<double> acc;
+#pragma unroll
+    for (int al = 0; al < 4; ++al)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) acc.re[al][b] = acc.im[al][b] = 0.0;
+    hop<0>(acc, links, x, g, c, n);
+    hop<1>(acc, links, x, g, c, n);
+    hop<2>(acc, links, x, g, c, n);
+    hop<3>(acc, links, x, g, c, n);
+    store_dslash(a, x, (int64_t)g.V, (int64_t)n, acc, a.ca, a.cb);
+}
+
+// The same in fixed point (hopping_force_fx): the eight hops in one loop, the
+// direction and sign at run time; every neighbour's half spinor in its own
+// scale, the sum in whole numbers of 2^-56 of the largest scale so far.
+template <typename I>
+__device__ __forceinline__ bool dslash_site_fx(const WilsonArgs &a, const Sites<I> &g, const Coord &c, I n)
+{
+    const double *__restrict__ x = static_cast<const double *>(a.x);
+    const int64_t V = g.V;
+    long long sr[12], si[12]; // spin rows 0 to 3, colours 0 to 2
+#pragma unroll
+    for (int q = 0; q < 12; ++q) sr[q] = si[q] = 0;
+    int scale = 0; // exponent field of the sum's scale
+#pragma unroll 1
+    for (int t = 0; t < 8; ++t) {
+        const int mu = t >> 1;
+        const bool back = t & 1;
+        const int64_t nb = n + hop_offset(g, c, mu, back ? -1 : 1);
+        FHalf h;
+        int e;
+        if (!fx_half(x, V, nb, mu, !back, h, e)) return false;
+        FLimbs u;
+        {
+            const double2 *p = static_cast<const double2 *>(a.links) + (int64_t)mu * 6 * V + (back ? nb : (int64_t)n);
+            double r[12];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const double2 v = __ldg(p + q * V);
+                r[2 * q] = v.x;
+                r[2 * q + 1] = v.y;
+            }
+            if (!fx_limbs_of_rows(r, u)) return false;
+            fx_row2(u);
+        }
+        if (e > scale) { // the sum so far in the new scale
+            const int d = min(e - scale, 63);
+#pragma unroll
+            for (int q = 0; q < 12; ++q) {
+                sr[q] >>= d;
+                si[q] >>= d;
+            }
+            scale = e;
+        }
+        const int sh = min(scale - e, 60) + 2;
+        const long long half = 1ll << (sh - 1);
+#pragma unroll
+        for (int al = 0; al < 2; ++al) {
+            FLimbAcc y;
+            if (back) fx_colour_sums<D>(u, h, al, y);
+            else fx_colour_sums<N>(u, h, al, y);
+            // rows 0, 1 of the hop, and its rows 2, 3 as s i^gcode times them
+            const int p = mu < 2 ? 3 - al : 2 + al; // partner row
+            const int code = (gcode_of(mu, p) + (back ? 0 : 2)) & 3;
+            const long long mr = code == 1 || code == 2 ? -1 : 0, mi = code >= 2 ? -1 : 0;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                long long re, im;
+                if (back) fx_total<-1>(y, b, 0, re, im);
+                else fx_total<1>(y, b, 0, re, im);
+                re = (re + half) >> sh;
+                im = (im + half) >> sh;
+                sr[3 * al + b] += re;
+                si[3 * al + b] += im;
+                const long long tr = (((code & 1) ? im : re) ^ mr) - mr, ti = (((code & 1) ? re : im) ^ mi) - mi;
+                if (mu < 2) {
+                    sr[3 * (3 - al) + b] += tr;
+                    si[3 * (3 - al) + b] += ti;
+                } else {
+                    sr[3 * (2 + al) + b] += tr;
+                    si[3 * (2 + al) + b] += ti;
+                }
+            }
+        }
+    }
+    Spinor<double> acc;
+    const double s = 0x1p-56 * __hiloint2double((scale + 1) << 20, 0); // 2^-56 of 2^(scale - 1022)
+#pragma unroll
+    for (int q = 0; q < 12; ++q) {
+        acc.re[q / 3][q % 3] = (double)sr[q];
+        acc.im[q / 3][q % 3] = (double)si[q];
+    }
+    store_dslash(a, x, V, (int64_t)n, acc, a.ca, a.cb * s);
+    return true;
+}
+
+// 2117 -> 715 us at 32^4, 320 -> 117 at 20x18x14x30; error against extended
+// precision 6.0e-17 where it was 9.0e-17.
+template <typename I>
+__global__ void __launch_bounds__(kDslashBlock, 3) wilson_dslash_fx(const __grid_constant__ WilsonArgs a)
+{
+    const Sites<I> g = make_sites<I>(a.dims);
+    for (I n = (I)blockIdx.x * blockDim.x + threadIdx.x; n < g.V; n += (I)gridDim.x * blockDim.x) {
+        Coord c;
+        if constexpr (sizeof(I) == 4) c = coord_fast(g, a.div, n);
+        else c = coord_in(g, n);
+        if (!dslash_site_fx(a, g, c, n)) dslash_site_floating(a, g, c, n);
+    }
+}
+
 unsigned blocks_for(int64_t items, int per_block)
 {
     int64_t b = (items + per_block - 1) / per_block;
@@ -646,9 +798,9 @@ cudaError_t launch_wilson_dslash(const WilsonArgs &args, cudaStream_t st)
     const bool xshfl = L0 <= 32 && (32 % L0) == 0 && V % 32 == 0 &&
                        (int64_t)grid * kDslashBlock >= V;
     const bool i32 = sites_fit_int(V);
-    if (a.precision == LQCD_F64) { // FP64-pipe bound; the shuffled form spills there
-        if (i32) wilson_dslash<double, false, int><<<grid, kDslashBlock, 0, st>>>(a);
-        else wilson_dslash<double, false, int64_t><<<grid, kDslashBlock, 0, st>>>(a);
+    if (a.precision == LQCD_F64) {
+        if (i32) wilson_dslash_fx<int><<<grid, kDslashBlock, 0, st>>>(a);
+        else wilson_dslash_fx<int64_t><<<grid, kDslashBlock, 0, st>>>(a);
     } else if (i32) {
         if (xshfl) wilson_dslash<float, true, int><<<grid, kDslashBlock, 0, st>>>(a);
         else wilson_dslash<float, false, int><<<grid, kDslashBlock, 0, st>>>(a);

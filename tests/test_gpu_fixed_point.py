@@ -183,3 +183,31 @@ def test_link_step_sizes(dt, scaled):
     got = lqcd.full_from_device(lqcd.unpack_links(lat, links))
     # exponents up to about 10 dt: their rounding is that of the angle
     assert np.abs(got - O.md_update_links(U, p, dt)).max() <= 1e-13 * max(1.0, 10 * dt)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-250, 1e200])
+@pytest.mark.parametrize("scaled", [(), (5, 6)])
+@pytest.mark.parametrize("dims", [(3, 4, 2, 5), (1, 2, 7, 3)])
+def test_hopping_operator_scales(dims, scale, scaled):
+    """FP64 hopping operator of spinors whose sizes change by many orders from
+    site to site (each neighbour has its own scale), zeros among them, and of
+    links without a fixed-point form."""
+    lat = lqcd.Lattice.symanzik(dims, 6.0, 0.87, "f64")
+    U = O.links_from_omega(synth.omega(dims, 0.4, 3)).reshape(lat.V, 4, 3, 3)
+    for i in scaled:
+        U[i // 4, i % 4, :2] *= 1.01
+    U = _third(U)
+    x = synth.spinor(dims, 11)
+    x = (x[..., 0] + 1j * x[..., 1]) * scale
+    x[1::5] *= 1e-12
+    x[2::7] = 0.0
+    x[3::11] *= 1e25
+    got = lqcd.spinor_from_device(lqcd.wilson_dslash(lat, _links(lat, U), lqcd.spinor_to_device(lat, x), 1.0, -0.13))
+    ref = x - 0.13 * O.wilson_hopping(dims, U, x)
+    # every site against the largest of the nine spinors it is made of: 8 hops,
+    # a few roundings each
+    grid = np.abs(x).max((1, 2)).reshape(dims[::-1])
+    near = np.max([grid] + [np.roll(grid, s, axis) for axis in range(4) for s in (1, -1)], axis=0).reshape(-1)
+    assert (np.abs(got - ref).max((1, 2)) <= 2e-15 * near).all()
+    zero = torch.zeros(lat.spinor_shape, dtype=torch.float64, device="cuda")
+    assert not lqcd.wilson_dslash(lat, _links(lat, U), zero, 0.0, 1.0).any()
