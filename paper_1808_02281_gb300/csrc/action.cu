@@ -154,7 +154,7 @@ struct Plain {
 // kernel, for callers without a workspace for the planes; the same bits.
 template <bool PLANES> struct Fixed {
     using M = FMat;
-    static constexpr int kMinBlocks = 2, kWords = 9;
+    static constexpr int kMinBlocks = 3, kWords = 9;
     using Word = int4;
     FxPlanes planes;
     const double *links;
@@ -324,7 +324,10 @@ __global__ void __launch_bounds__(kActionBlock, P::kMinBlocks)
         __syncthreads(); // before the corners of the next sites
     }
     const double s = block_sum<kActionBlock>(acc);
-    if (threadIdx.x == 0) a.partials[blockIdx.x] = s;
+    if (threadIdx.x == 0) {
+        a.partials[blockIdx.x] = s;
+        for (int i = blockIdx.x + gridDim.x; i < a.blocks; i += gridDim.x) a.partials[i] = 0.0;
+    }
 }
 
 // The links of FP64 fields as planes with FP32 remainders, for action_loops.
@@ -506,7 +509,9 @@ template <typename P, typename I> static cudaError_t launch_action_t(const Reduc
         const cudaError_t e = cudaFuncSetAttribute(action_loops<P, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
     }
-    action_loops<P, I><<<a.blocks, kActionBlock, bytes, st>>>(a, loop_table());
+    // the resident blocks (a.blocks is four per SM)
+    const int grid = a.blocks * P::kMinBlocks / 4 > 0 ? a.blocks * P::kMinBlocks / 4 : 1;
+    action_loops<P, I><<<grid, kActionBlock, bytes, st>>>(a, loop_table());
     return cudaGetLastError();
 }
 
