@@ -154,7 +154,7 @@ struct Plain {
 // kernel, for callers without a workspace for the planes; the same bits.
 template <bool PLANES> struct Fixed {
     using M = FMat;
-    static constexpr int kMinBlocks = 3, kWords = 9;
+    static constexpr int kMinBlocks = 2, kWords = 9;
     using Word = int4;
     FxPlanes planes;
     const double *links;
