@@ -51,13 +51,6 @@ template <int K, typename R> __device__ __forceinline__ void times_ipow(R &re, R
     }
 }
 
-// A launch scalar in the kernel's precision (FP32 copies made on the host).
-template <typename R> __device__ __forceinline__ R scalar_of(double d, float f)
-{
-    if constexpr (sizeof(R) == 8) return d;
-    else return f;
-}
-
 template <typename R> struct Spinor {
     R re[4][3], im[4][3];
 };
@@ -254,77 +247,219 @@ template <typename R> __device__ __forceinline__ Half<R> shfl_half(const Half<R>
     return r;
 }
 
-template <typename R>
-__device__ __forceinline__ void hop_x_shuffled(Spinor<R> &acc, const R *__restrict__ links,
-                                               const Spinor<R> &xn, int64_t V, int64_t n, int L0)
-{
-    const int lane = (int)(threadIdx.x & 31), m = L0 - 1;
-    const int up = (lane & ~m) | ((lane + 1) & m), dn = (lane & ~m) | ((lane - 1) & m);
-    const Mat<R> u = load_link(links, V, 0, n);
-    const Half<R> fw = shfl_half(project<0, -1>(xn), up);                  // (1 - g_x) x_{n+x}
-    const Half<R> bw = shfl_half(colour_mul<D>(u, project<0, +1>(xn)), dn); // U_{n-x}^dag (1 + g_x) x_{n-x}
-    accumulate<0, -1>(acc, colour_mul<N>(u, fw));
-    accumulate<0, +1>(acc, bw);
-}
-
 constexpr int kDslashBlock = 128;
 
-// Register cap: 5 blocks (20 warps, 96 registers, a 64-byte spill) per SM: at
-// 32^3x64 0.161 against 0.167 ms with 4 blocks (128 registers) and 0.245 ms
-// with the uncapped 138 (12 warps) -- the kernel waits on loads, so warps in
-// flight count more than the spill.
-constexpr int kDslashMinBlocks = 5;
+// FP32 operator: what bounds it is the latency of HBM and L2 (384 bytes and
+// about 1,400 instructions a site), so what counts is bytes in flight.  Loads
+// into registers keep one hop of a warp in flight, and each site begins with
+// an empty pipe.  Here every thread copies the operands of its hops (a
+// neighbour's spinor and a link: nine 16-byte words) asynchronously into its
+// own words of shared memory, kRing hops ahead and over the end of a site into
+// the next of its sites; no thread reads another's words, so there is no
+// barrier, only the thread's own copy groups.  The copies pass L1 by (through
+// L1, which the ring leaves little of: 178 us).
+// 32^3x64: 159 -> 133 us (5.1 -> 6.1 TB/s of 384 B a site), 32^4: 84 -> 69 us,
+// 24^3x48: 55 -> 51 us; below that the launch is what counts.
+// A ring of two hops and 4 blocks an SM (147 KB of shared memory, up to 128
+// registers): 133 us at 32^3x64; 3 blocks of three hops 131, but more shared
+// memory than a static allocation may have; 5 blocks of two hops at 96
+// registers 145, 4 of three hops 144; 64 or 256 threads a block the same; one
+// site a thread instead of as many blocks as are resident 139.
+constexpr int kRing = 2;
+constexpr int kDslashMinBlocks = 4;
+constexpr int kHopWords = 9;
 
-// out_n = ca x_n + cb (calD x)_n, one thread per site.
-// XSHFL: x hops by shuffles.
-template <typename R, bool XSHFL, typename I>
-__global__ void __launch_bounds__(kDslashBlock, kDslashMinBlocks)
-    wilson_dslash(const __grid_constant__ WilsonArgs a)
+// Asynchronous 16-byte copy to shared memory, past L1.
+__device__ __forceinline__ void copy_async(float4 *dst, const float4 *src)
 {
-    const Sites<I> g = make_sites<I>(a.dims);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT> __device__ __forceinline__ void copies_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+
+// The hops of a site in their order: +-y, +-z, +-t, then +-x.  XSHFL: the x
+// hops both come from the site's own spinor and link, by shuffles.  The last
+// hop brings the site's own spinor in both forms.
+template <bool XSHFL> struct Hops {
+    static constexpr int kCount = XSHFL ? 7 : 9;
+    static constexpr bool own(int s) { return s == kCount - 1; }
+    static constexpr int mu(int s) { return s < 6 ? 1 + s / 2 : 0; }
+    static constexpr int sign(int s) { return (s & 1) ? -1 : 1; }
+};
+
+// Starts the copies of hop S of site n.
+template <bool XSHFL, int S, typename I>
+__device__ __forceinline__ void fetch_hop(float4 *slot, const float *__restrict__ x, const float *__restrict__ links,
+                                          const Sites<I> &g, const Coord &c, I n)
+{
+    using H = Hops<XSHFL>;
+    constexpr int mu = H::mu(S);
+    constexpr bool own = H::own(S);
     const int64_t V = g.V;
-    const R *__restrict__ links = static_cast<const R *>(a.links);
-    const R *__restrict__ x = static_cast<const R *>(a.x);
-    R *__restrict__ out = static_cast<R *>(a.out);
-    const R ca = scalar_of<R>(a.ca, a.fca), cb = scalar_of<R>(a.cb, a.fcb);
-    const bool with_x = a.ca != 0.0;
-    for (I n = (I)blockIdx.x * blockDim.x + threadIdx.x; n < g.V; n += (I)gridDim.x * blockDim.x) {
-        Coord c;
-        if constexpr (sizeof(I) == 4) c = coord_fast(g, a.div, n);
-        else c = coord_in(g, n);
-        Spinor<R> acc;
+    const int64_t m = own ? (int64_t)n : (int64_t)(n + hop_offset(g, c, mu, H::sign(S)));
+    const float4 *px = reinterpret_cast<const float4 *>(x) + m;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) copy_async(slot + q * kDslashBlock, px + q * V);
+    if constexpr (XSHFL || !own) {
+        const float4 *pu = reinterpret_cast<const float4 *>(links) + (int64_t)mu * 3 * V + (H::sign(S) > 0 ? (int64_t)n : m);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) copy_async(slot + (6 + q) * kDslashBlock, pu + q * V);
+    }
+}
+
+__device__ __forceinline__ Spinor<float> slot_spinor(const float4 *slot)
+{
+    Spinor<float> s;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        const float4 v = slot[q * kDslashBlock];
+        s.re[2 * q / 3][2 * q % 3] = v.x;
+        s.im[2 * q / 3][2 * q % 3] = v.y;
+        s.re[(2 * q + 1) / 3][(2 * q + 1) % 3] = v.z;
+        s.im[(2 * q + 1) / 3][(2 * q + 1) % 3] = v.w;
+    }
+    return s;
+}
+__device__ __forceinline__ Mat<float> slot_link(const float4 *slot)
+{
+    Mat<float> u;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float4 v = slot[(6 + q) * kDslashBlock];
+        u.re[2 * q / 3][2 * q % 3] = v.x;
+        u.im[2 * q / 3][2 * q % 3] = v.y;
+        u.re[(2 * q + 1) / 3][(2 * q + 1) % 3] = v.z;
+        u.im[(2 * q + 1) / 3][(2 * q + 1) % 3] = v.w;
+    }
+    rebuild_row2(u);
+    return u;
+}
+
+// One thread's pass over its sites: hop S lies in slot S % kRing, and the slots
+// turn by kCount from site to site.
+template <bool XSHFL, typename I> struct HopRing {
+    using H = Hops<XSHFL>;
+    float4 *slot[kRing];
+    const float *x, *links;
+    Coord c, cn; // of this site and of the thread's next
+    I n, nn;
+    bool more; // there is a next site
+
+    // The copies of hop S, or of hop S - kCount of the next site; always one
+    // group, so that copies_wait counts hops.
+
+    template <int S> __device__ __forceinline__ void fetch(const Sites<I> &g)
+    {
+        if constexpr (S < H::kCount) {
+            fetch_hop<XSHFL, S>(slot[S % kRing], x, links, g, c, n);
+        } else {
+            if (more) fetch_hop<XSHFL, S - H::kCount>(slot[S % kRing], x, links, g, cn, nn);
+        }
+        copies_commit();
+    }
+
+    // acc += hop S (the last: acc = ca x + cb acc), and the copies of hop
+    // S + kRing into the slot that is read out.
+    template <int S> __device__ __forceinline__ void hop(Spinor<float> &acc, const Sites<I> &g, float ca, float cb)
+    {
+        constexpr int mu = H::mu(S);
+        float4 *const p = slot[S % kRing];
+        copies_wait<kRing - 1>();
+        if constexpr (!H::own(S)) {
+            const Half<float> h = project<mu, -H::sign(S)>(slot_spinor(p));
+            const Mat<float> u = slot_link(p);
+            fetch<S + kRing>(g);
+            accumulate<mu, -H::sign(S)>(acc, colour_mul<(H::sign(S) > 0 ? N : D)>(u, h));
+        } else {
+            if constexpr (XSHFL) {
+                const int lane = (int)(threadIdx.x & 31), m = g.L0 - 1;
+                const int up = (lane & ~m) | ((lane + 1) & m), dn = (lane & ~m) | ((lane - 1) & m);
+                const Spinor<float> xn = slot_spinor(p);
+                const Mat<float> u = slot_link(p);
+                const Half<float> fw = shfl_half(project<0, -1>(xn), up);
+                const Half<float> bw = shfl_half(colour_mul<D>(u, project<0, +1>(xn)), dn);
+                accumulate<0, -1>(acc, colour_mul<N>(u, fw));
+                accumulate<0, +1>(acc, bw);
+            }
+            if (ca != 0.0f) {
+                const Spinor<float> xn = slot_spinor(p);
+#pragma unroll
+                for (int al = 0; al < 4; ++al)
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) {
+                        acc.re[al][b] = fma(ca, xn.re[al][b], cb * acc.re[al][b]);
+                        acc.im[al][b] = fma(ca, xn.im[al][b], cb * acc.im[al][b]);
+                    }
+            } else {
+#pragma unroll
+                for (int al = 0; al < 4; ++al)
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) {
+                        acc.re[al][b] *= cb;
+                        acc.im[al][b] *= cb;
+                    }
+            }
+            fetch<S + kRing>(g);
+        }
+    }
+};
+
+// out_n = ca x_n + cb (calD x)_n in FP32.
+template <bool XSHFL, typename I>
+__global__ void __launch_bounds__(kDslashBlock, kDslashMinBlocks) wilson_dslash(const __grid_constant__ WilsonArgs a)
+{
+    using H = Hops<XSHFL>;
+    __shared__ float4 ring_s[kRing * kHopWords * kDslashBlock];
+    const Sites<I> g = make_sites<I>(a.dims);
+    const I step = (I)gridDim.x * blockDim.x;
+    HopRing<XSHFL, I> r;
+    r.x = static_cast<const float *>(a.x);
+    r.links = static_cast<const float *>(a.links);
+    r.n = (I)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r.n >= g.V) return;
+#pragma unroll
+    for (int s = 0; s < kRing; ++s) r.slot[s] = ring_s + s * kHopWords * kDslashBlock + threadIdx.x;
+    if constexpr (sizeof(I) == 4) r.c = coord_fast(g, a.div, r.n);
+    else r.c = coord_in(g, r.n);
+    r.more = false;
+    r.template fetch<0>(g);
+    r.template fetch<1>(g);
+    for (;;) {
+        Spinor<float> acc;
 #pragma unroll
         for (int al = 0; al < 4; ++al)
 #pragma unroll
-            for (int b = 0; b < 3; ++b) acc.re[al][b] = acc.im[al][b] = R(0);
-        if constexpr (XSHFL) {
-            const Spinor<R> xn = load_spinor(x, V, (int64_t)n);
-            hop_x_shuffled(acc, links, xn, V, (int64_t)n, g.L0);
-        } else {
-            hop<0>(acc, links, x, g, c, n);
+            for (int b = 0; b < 3; ++b) acc.re[al][b] = acc.im[al][b] = 0.0f;
+        r.template hop<0>(acc, g, a.fca, a.fcb);
+        r.template hop<1>(acc, g, a.fca, a.fcb);
+        r.template hop<2>(acc, g, a.fca, a.fcb);
+        r.template hop<3>(acc, g, a.fca, a.fcb);
+        r.nn = r.n + step;
+        r.more = r.nn < g.V;
+        if (r.more) {
+            if constexpr (sizeof(I) == 4) r.cn = coord_fast(g, a.div, r.nn);
+            else r.cn = coord_in(g, r.nn);
         }
-        hop<1>(acc, links, x, g, c, n);
-        hop<2>(acc, links, x, g, c, n);
-        hop<3>(acc, links, x, g, c, n);
-        if (with_x) {
-            const Spinor<R> xn = load_spinor(x, V, (int64_t)n);
-#pragma unroll
-            for (int al = 0; al < 4; ++al)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    acc.re[al][b] = fma(ca, xn.re[al][b], cb * acc.re[al][b]);
-                    acc.im[al][b] = fma(ca, xn.im[al][b], cb * acc.im[al][b]);
-                }
-        } else {
-#pragma unroll
-            for (int al = 0; al < 4; ++al)
-#pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    acc.re[al][b] *= cb;
-                    acc.im[al][b] *= cb;
-                }
+        r.template hop<4>(acc, g, a.fca, a.fcb);
+        r.template hop<5>(acc, g, a.fca, a.fcb);
+        r.template hop<6>(acc, g, a.fca, a.fcb);
+        if constexpr (!XSHFL) {
+            r.template hop<7>(acc, g, a.fca, a.fcb);
+            r.template hop<8>(acc, g, a.fca, a.fcb);
         }
-        store_spinor(out, V, (int64_t)n, acc);
+        store_spinor(static_cast<float *>(a.out), (int64_t)g.V, (int64_t)r.n, acc);
+        if (!r.more) break;
+        r.n = r.nn;
+        r.c = r.cn;
+        float4 *old[kRing];
+#pragma unroll
+        for (int s = 0; s < kRing; ++s) old[s] = r.slot[s];
+#pragma unroll
+        for (int s = 0; s < kRing; ++s) r.slot[s] = old[(s + H::kCount) % kRing];
     }
 }
 
@@ -791,22 +926,25 @@ cudaError_t launch_wilson_dslash(const WilsonArgs &args, cudaStream_t st)
     const WilsonArgs a = launch_args(args);
     const int64_t V = (int64_t)a.dims[0] * a.dims[1] * a.dims[2] * a.dims[3];
     const unsigned grid = blocks_for(V, kDslashBlock);
-    // shuffled x hops need whole x rows in every warp: L0 divides 32 (then
-    // V is a multiple of L0 and every warp's first site starts a row), and a
-    // grid-stride loop that never runs a warp past V with only part of it
-    const int L0 = a.dims[0];
-    const bool xshfl = L0 <= 32 && (32 % L0) == 0 && V % 32 == 0 &&
-                       (int64_t)grid * kDslashBlock >= V;
     const bool i32 = sites_fit_int(V);
     if (a.precision == LQCD_F64) {
         if (i32) wilson_dslash_fx<int><<<grid, kDslashBlock, 0, st>>>(a);
         else wilson_dslash_fx<int64_t><<<grid, kDslashBlock, 0, st>>>(a);
-    } else if (i32) {
-        if (xshfl) wilson_dslash<float, true, int><<<grid, kDslashBlock, 0, st>>>(a);
-        else wilson_dslash<float, false, int><<<grid, kDslashBlock, 0, st>>>(a);
     } else {
-        if (xshfl) wilson_dslash<float, true, int64_t><<<grid, kDslashBlock, 0, st>>>(a);
-        else wilson_dslash<float, false, int64_t><<<grid, kDslashBlock, 0, st>>>(a);
+        // shuffled x hops need whole x rows in every warp: L0 divides 32 (every
+        // warp's first site then starts a row) and V is whole warps.  They save
+        // 15 of 78 words a site (0.203 -> 0.184 ms at 32^3x64 when introduced).
+        const int L0 = a.dims[0];
+        const bool xshfl = L0 <= 32 && (32 % L0) == 0 && V % 32 == 0;
+        // as many blocks as are resident, each thread over several sites
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        const unsigned resident = grid < (unsigned)(sms * kDslashMinBlocks) ? grid : (unsigned)(sms * kDslashMinBlocks);
+        const auto k = i32 ? (xshfl ? wilson_dslash<true, int> : wilson_dslash<false, int>)
+                           : (xshfl ? wilson_dslash<true, int64_t> : wilson_dslash<false, int64_t>);
+        k<<<resident, kDslashBlock, 0, st>>>(a);
     }
     return cudaGetLastError();
 }
