@@ -5,6 +5,7 @@
 //   link step      U <- exp(i dt sum_a p^a T_a) U     (left flow of Eq. 18_1_29_3)
 //   links from omega  U = exp(i sum_a omega^a T_a)    (Eq. 18_1_29_3)
 //   pack / unpack  full 3x3 complex <-> first two rows
+#include "async_copy.cuh"
 #include "gaussian.cuh"
 #include "kernels.h"
 #include "link_step_fx.cuh"
@@ -60,16 +61,16 @@ __global__ void __launch_bounds__(kBlock) update_momenta(typename Vec<R>::type *
 }
 
 // U <- exp(i P) U (FROM_UNIT: U = exp(i P)), rows 0 and 1 only, then
-// Gram-Schmidt, for one link; p the components of P.
-template <typename R, bool FROM_UNIT>
-__device__ __forceinline__ void link_step(R *__restrict__ links, const R p[8], int64_t V, int mu, int64_t n)
+// Gram-Schmidt, for one link; p the components of P, load() gives U.
+template <typename R, bool FROM_UNIT, typename Load>
+__device__ __forceinline__ void link_step(R *__restrict__ links, const R p[8], int64_t V, int mu, int64_t n, const Load &load)
 {
     const Mat<R> e = exp_i_hermitian(algebra_matrix(p));
     Mat<R> u;
     if constexpr (FROM_UNIT) {
         u = e;
     } else {
-        const Mat<R> v = load_link(links, V, mu, n);
+        const Mat<R> v = load();
 #pragma unroll
         for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -98,61 +99,55 @@ __device__ __noinline__ void link_step_floating(double *links, const double *mom
     load_algebra(mom, V, mu, n, p);
 #pragma unroll
     for (int c = 0; c < 8; ++c) p[c] *= dt;
-    link_step<double, FROM_UNIT>(links, p, V, mu, n);
+    link_step<double, FROM_UNIT>(links, p, V, mu, n, [&] { return load_link(links, V, mu, n); });
 }
 
-// The step of link (n, mu) with the momenta scaled by dt.
-template <typename R, bool FROM_UNIT>
-__device__ __forceinline__ void update_link(R *__restrict__ links, const R *__restrict__ mom, R dt, int64_t V, int mu,
-                                            int64_t n)
+// The FP64 step of link (n, mu).
+template <bool FROM_UNIT>
+__device__ __forceinline__ void update_link(double *__restrict__ links, const double *__restrict__ mom, double dt, int64_t V,
+                                            int mu, int64_t n)
 {
-    R p[8];
+    double p[8];
     load_algebra(mom, V, mu, n, p);
 #pragma unroll
     for (int c = 0; c < 8; ++c) p[c] *= dt;
-    if constexpr (sizeof(R) == 4) {
-        link_step<R, FROM_UNIT>(links, p, V, mu, n);
+    double2 *u = reinterpret_cast<double2 *>(links) + (int64_t)mu * 6 * V + n;
+    double r[12] = {1.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0};
+    if constexpr (!FROM_UNIT) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const double2 v = u[q * V];
+            r[2 * q] = v.x;
+            r[2 * q + 1] = v.y;
+        }
+    }
+    if (fx_link_step(p, r)) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) u[q * V] = make_double2(r[2 * q], r[2 * q + 1]);
     } else {
-        double2 *u = reinterpret_cast<double2 *>(links) + (int64_t)mu * 6 * V + n;
-        double r[12] = {1.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0};
-        if constexpr (!FROM_UNIT) {
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                const double2 v = u[q * V];
-                r[2 * q] = v.x;
-                r[2 * q + 1] = v.y;
-            }
-        }
-        if (fx_link_step(p, r)) {
-#pragma unroll
-            for (int q = 0; q < 6; ++q) u[q * V] = make_double2(r[2 * q], r[2 * q + 1]);
-        } else {
-            link_step_floating<FROM_UNIT>(links, mom, dt, V, mu, n);
-        }
+        link_step_floating<FROM_UNIT>(links, mom, dt, V, mu, n);
     }
 }
 
-// Threads of a link-step block and resident blocks: the FP64 step takes more
-// registers (18x14x22x36: 153 us with 2 blocks of 192, 157 with 3 of 128, 170
-// with 2 of 128).
-template <typename R> constexpr int link_block() { return sizeof(R) == 8 ? 192 : kBlock; }
-template <typename R> constexpr int link_min_blocks() { return sizeof(R) == 8 ? 2 : 1; }
+// Threads of an FP64 link-step block and resident blocks (18x14x22x36: 153 us
+// with 2 blocks of 192, 157 with 3 of 128, 170 with 2 of 128).
+constexpr int kFxStepBlock = 192, kFxStepBlocks = 2;
 
 // The link and algebra planes share the site index.
-template <typename R, bool FROM_UNIT>
-__global__ void __launch_bounds__(link_block<R>(), link_min_blocks<R>())
-    update_links(R *__restrict__ links, const R *__restrict__ mom, int64_t V, R dt)
+template <bool FROM_UNIT>
+__global__ void __launch_bounds__(kFxStepBlock, kFxStepBlocks)
+    update_links_f64(double *__restrict__ links, const double *__restrict__ mom, int64_t V, double dt)
 {
     const int64_t nlinks = 4 * V;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nlinks;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int mu = direction_of(i, V);
-        update_link<R, FROM_UNIT>(links, mom, dt, V, mu, i - mu * V);
+        update_link<FROM_UNIT>(links, mom, dt, V, mu, i - mu * V);
     }
 }
 
-// The link step of update_links for one link of a batch of lattices: the
-// persistent CTAs walk the concatenated link ranges.
+// The link step for the links of a batch of lattices: the persistent CTAs
+// walk the concatenated link ranges.
 struct LinkBatch {
     int n;
     int64_t total;
@@ -160,21 +155,133 @@ struct LinkBatch {
     int64_t V[kMaxBatch];
     void *links[kMaxBatch];
     const void *mom[kMaxBatch];
+
+    // The lattice of link i of the concatenation, from a near one's number.
+    __device__ __forceinline__ int lattice_of(int64_t i, int c) const
+    {
+        while (c > 0 && i < begin[c]) --c;
+        while (c + 1 < n && i >= begin[c + 1]) ++c;
+        return c;
+    }
 };
 
-template <typename R>
-__global__ void __launch_bounds__(link_block<R>(), link_min_blocks<R>()) update_links_batched(const __grid_constant__ LinkBatch B, R dt)
+__global__ void __launch_bounds__(kFxStepBlock, kFxStepBlocks) update_links_f64_batched(const __grid_constant__ LinkBatch B, double dt)
 {
     int c = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < B.total;
          i += (int64_t)gridDim.x * blockDim.x) {
-        while (c > 0 && i < B.begin[c]) --c;
-        while (c + 1 < B.n && i >= B.begin[c + 1]) ++c;
+        c = B.lattice_of(i, c);
         const int64_t V = B.V[c];
         const int64_t l = i - B.begin[c];
         const int mu = direction_of(l, V);
-        update_link<R, false>(static_cast<R *>(B.links[c]), static_cast<const R *>(B.mom[c]), dt, V, mu, l - mu * V);
+        update_link<false>(static_cast<double *>(B.links[c]), static_cast<const double *>(B.mom[c]), dt, V, mu, l - mu * V);
     }
+}
+
+// FP32 step.  It moves 128 bytes a link and executes about 450 instructions on
+// them; loading and computing took turns (217 us at 32^3x64, the bytes alone
+// 159, the instructions 136).  A thread passes over many links and copies the
+// next one's momentum and link (five words) into shared memory while it
+// computes: 209 -> 174 us at 32^3x64, 70 -> 59 at 24^3x48.  4 blocks of 256
+// as many as the registers allow; 3: 177, 8 of 128: 175.
+constexpr int kStepBlock = 256, kStepBlocks = 4, kStepWords = 5;
+
+// A link: the fields of its lattice, its direction and site.
+struct StepLink {
+    float *links;
+    const float *mom;
+    int64_t V, n;
+    int mu;
+};
+
+// Link i of one lattice, or of the concatenation of a batch.
+struct LatticeLinks {
+    float *links;
+    const float *mom;
+    int64_t V;
+    __device__ __forceinline__ int64_t total() const { return 4 * V; }
+    __device__ __forceinline__ StepLink link(int64_t i, int &) const
+    {
+        const int mu = direction_of(i, V);
+        return {links, mom, V, i - mu * V, mu};
+    }
+};
+struct BatchLinks {
+    const LinkBatch &B;
+    __device__ __forceinline__ int64_t total() const { return B.total; }
+    __device__ __forceinline__ StepLink link(int64_t i, int &c) const
+    {
+        c = B.lattice_of(i, c);
+        const int64_t V = B.V[c], l = i - B.begin[c];
+        const int mu = direction_of(l, V);
+        return {static_cast<float *>(B.links[c]), static_cast<const float *>(B.mom[c]), V, l - mu * V, mu};
+    }
+};
+
+template <bool FROM_UNIT> __device__ __forceinline__ void fetch_step(float4 *slot, const StepLink &s)
+{
+    const float4 *p = reinterpret_cast<const float4 *>(s.mom) + (int64_t)s.mu * 2 * s.V + s.n;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) copy_async(slot + q * kStepBlock, p + q * s.V);
+    if constexpr (!FROM_UNIT) {
+        const float4 *u = reinterpret_cast<const float4 *>(s.links) + (int64_t)s.mu * 3 * s.V + s.n;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) copy_async(slot + (2 + q) * kStepBlock, u + q * s.V);
+    }
+}
+
+template <bool FROM_UNIT, typename Links> __device__ __forceinline__ void step_links(const Links &links, float dt)
+{
+    __shared__ float4 ring[2 * kStepWords * kStepBlock];
+    const int64_t total = links.total(), step = (int64_t)gridDim.x * kStepBlock;
+    int64_t i = blockIdx.x * (int64_t)kStepBlock + threadIdx.x;
+    if (i >= total) return;
+    float4 *slot = ring + threadIdx.x, *next = slot + kStepWords * kStepBlock;
+    int c = 0;
+    StepLink s = links.link(i, c);
+    fetch_step<FROM_UNIT>(slot, s);
+    copies_commit();
+    for (;;) {
+        i += step;
+        StepLink s2 = s;
+        if (i < total) {
+            s2 = links.link(i, c);
+            fetch_step<FROM_UNIT>(next, s2);
+        }
+        copies_commit();
+        copies_wait<1>(); // this link's
+        const float4 a = slot[0], b = slot[kStepBlock];
+        const float p[8] = {a.x * dt, a.y * dt, a.z * dt, a.w * dt, b.x * dt, b.y * dt, b.z * dt, b.w * dt};
+        link_step<float, FROM_UNIT>(s.links, p, s.V, s.mu, s.n, [&] {
+            Mat<float> u;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float4 v = slot[(2 + q) * kStepBlock];
+                u.re[2 * q / 3][2 * q % 3] = v.x;
+                u.im[2 * q / 3][2 * q % 3] = v.y;
+                u.re[(2 * q + 1) / 3][(2 * q + 1) % 3] = v.z;
+                u.im[(2 * q + 1) / 3][(2 * q + 1) % 3] = v.w;
+            }
+            rebuild_row2(u);
+            return u;
+        });
+        if (i >= total) break;
+        s = s2;
+        float4 *const t = slot;
+        slot = next;
+        next = t;
+    }
+}
+
+template <bool FROM_UNIT>
+__global__ void __launch_bounds__(kStepBlock, kStepBlocks) update_links_f32(float *links, const float *mom, int64_t V, float dt)
+{
+    step_links<FROM_UNIT>(LatticeLinks{links, mom, V}, dt);
+}
+
+__global__ void __launch_bounds__(kStepBlock, kStepBlocks) update_links_f32_batched(const __grid_constant__ LinkBatch B, float dt)
+{
+    step_links<false>(BatchLinks{B}, dt);
 }
 
 // Chain rule through U = exp(X) U0, X = i W, W = omega.T (Eq. 18_1_29_3).
@@ -482,17 +589,32 @@ cudaError_t launch_update_momenta(const MdArgs &a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_update_links(const MdArgs &a, cudaStream_t st)
+namespace {
+
+// The blocks of `block` threads for n links, at most `per_sm` on every SM.
+unsigned step_grid(int64_t n, int block, int per_sm)
+{
+    int dev = 0, sms = 1;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t blocks = (n + block - 1) / block, cap = (int64_t)(sms > 0 ? sms : 1) * per_sm;
+    return (unsigned)(blocks < 1 ? 1 : (blocks < cap ? blocks : cap));
+}
+
+template <bool FROM_UNIT> cudaError_t launch_step(const MdArgs &a, double dt, cudaStream_t st)
 {
     const int64_t V = volume(a.dims);
     if (a.precision == LQCD_F64)
-        update_links<double, false><<<grid_for(4 * V, link_block<double>()), link_block<double>(), 0, st>>>(
-            static_cast<double *>(a.links), static_cast<const double *>(a.mom), V, a.dt);
+        update_links_f64<FROM_UNIT><<<grid_for(4 * V, kFxStepBlock), kFxStepBlock, 0, st>>>(
+            static_cast<double *>(a.links), static_cast<const double *>(a.mom), V, dt);
     else
-        update_links<float, false><<<grid_for(4 * V), kBlock, 0, st>>>(
-            static_cast<float *>(a.links), static_cast<const float *>(a.mom), V, (float)a.dt);
+        update_links_f32<FROM_UNIT><<<step_grid(4 * V, kStepBlock, kStepBlocks), kStepBlock, 0, st>>>(
+            static_cast<float *>(a.links), static_cast<const float *>(a.mom), V, (float)dt);
     return cudaGetLastError();
 }
+
+} // namespace
+
+cudaError_t launch_update_links(const MdArgs &a, cudaStream_t st) { return launch_step<false>(a, a.dt, st); }
 
 cudaError_t launch_update_links_batched(int precision, int n, const LinkStepItem *items, double dt,
                                         cudaStream_t st)
@@ -510,31 +632,14 @@ cudaError_t launch_update_links_batched(int precision, int n, const LinkStepItem
     }
     B.begin[n] = pos;
     B.total = pos;
-    int dev = 0, sms = 1;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int block = precision == LQCD_F64 ? link_block<double>() : link_block<float>();
-    int64_t grid = (pos + block - 1) / block;
-    const int64_t cap = (int64_t)(sms > 0 ? sms : 1) * 8;
-    if (grid > cap) grid = cap;
-    if (grid < 1) grid = 1;
     if (precision == LQCD_F64)
-        update_links_batched<double><<<(unsigned)grid, block, 0, st>>>(B, dt);
+        update_links_f64_batched<<<step_grid(pos, kFxStepBlock, 8), kFxStepBlock, 0, st>>>(B, dt);
     else
-        update_links_batched<float><<<(unsigned)grid, block, 0, st>>>(B, (float)dt);
+        update_links_f32_batched<<<step_grid(pos, kStepBlock, kStepBlocks), kStepBlock, 0, st>>>(B, (float)dt);
     return cudaGetLastError();
 }
 
-cudaError_t launch_links_from_omega(const MdArgs &a, cudaStream_t st)
-{
-    const int64_t V = volume(a.dims);
-    if (a.precision == LQCD_F64)
-        update_links<double, true><<<grid_for(4 * V, link_block<double>()), link_block<double>(), 0, st>>>(
-            static_cast<double *>(a.links), static_cast<const double *>(a.mom), V, 1.0);
-    else
-        update_links<float, true><<<grid_for(4 * V), kBlock, 0, st>>>(
-            static_cast<float *>(a.links), static_cast<const float *>(a.mom), V, 1.0f);
-    return cudaGetLastError();
-}
+cudaError_t launch_links_from_omega(const MdArgs &a, cudaStream_t st) { return launch_step<true>(a, 1.0, st); }
 
 cudaError_t launch_omega_gradient(const MdArgs &a, cudaStream_t st)
 {

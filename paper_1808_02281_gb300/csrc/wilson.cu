@@ -7,6 +7,7 @@
 // neighbours come from L1/L2 (a time slice of a 32^3 spinor field is 3 MB),
 // and every (1 -+ gamma_mu) is applied as a spin projection to two colour
 // vectors, so that each link multiplies two colour vectors instead of four.
+#include "async_copy.cuh"
 #include "fixed.cuh"
 #include "sites.cuh"
 
@@ -268,18 +269,6 @@ constexpr int kDslashBlock = 128;
 constexpr int kRing = 2;
 constexpr int kDslashMinBlocks = 4;
 constexpr int kHopWords = 9;
-
-// Asynchronous 16-byte copy to shared memory, past L1.
-__device__ __forceinline__ void copy_async(float4 *dst, const float4 *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int LEFT> __device__ __forceinline__ void copies_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
-}
 
 // The hops of a site in their order: +-y, +-z, +-t, then +-x.  XSHFL: the x
 // hops both come from the site's own spinor and link, by shuffles.  The last
