@@ -11,6 +11,58 @@ namespace lqcd {
 namespace {
 
 
+// The word at p: GLOBAL, of read-only global memory.
+template <bool GLOBAL> __device__ __forceinline__ int4 fx_word(const int4 *p)
+{
+    if constexpr (GLOBAL) return __ldg(p);
+    else return *p;
+}
+
+// The matrix with FP32 remainders whose entries lie S words apart.
+template <int S, bool GLOBAL> __device__ __forceinline__ FMat fx_mat_at(const int4 *p)
+{
+    FMat u;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        const int4 v = fx_word<GLOBAL>(p + e * S);
+        u.rh[e / 3][e % 3] = v.x;
+        u.rl[e / 3][e % 3] = __int_as_float(v.y);
+        u.ih[e / 3][e % 3] = v.z;
+        u.il[e / 3][e % 3] = __int_as_float(v.w);
+    }
+    return u;
+}
+
+// The same, or of whole limbs (whole), or (dag) its dagger: the off-diagonal
+// entries are then read from their mirrored places.
+template <int S, bool GLOBAL> __device__ __forceinline__ FMat fx_form_at(const int4 *p, bool whole, bool dag)
+{
+    const int o = dag ? 2 * S : 0, m = dag ? -1 : 0, f = dag ? (int)0x80000000 : 0;
+    const int4 *up = p + o, *dn = p - o, *up2 = up + o, *dn2 = dn - o;
+    const int4 v[9] = {fx_word<GLOBAL>(p),           fx_word<GLOBAL>(up + S),      fx_word<GLOBAL>(up2 + 2 * S),
+                       fx_word<GLOBAL>(dn + 3 * S),  fx_word<GLOBAL>(p + 4 * S),   fx_word<GLOBAL>(up + 5 * S),
+                       fx_word<GLOBAL>(dn2 + 6 * S), fx_word<GLOBAL>(dn + 7 * S),  fx_word<GLOBAL>(p + 8 * S)};
+    FMat u;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        u.rh[e / 3][e % 3] = v[e].x;
+        u.ih[e / 3][e % 3] = (v[e].z ^ m) - m;
+        u.rl[e / 3][e % 3] = __int_as_float(v[e].y);
+        u.il[e / 3][e % 3] = __int_as_float(v[e].w);
+    }
+    if (whole) {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            u.rl[e / 3][e % 3] = 0x1p-28f * (float)v[e].y;
+            u.il[e / 3][e % 3] = 0x1p-28f * (float)v[e].w;
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 9; ++e)
+        u.il[e / 3][e % 3] = __int_as_float(__float_as_int(u.il[e / 3][e % 3]) ^ f);
+    return u;
+}
+
 struct FxPlanes {
     char *base;
     int64_t plane_bytes;
@@ -45,49 +97,12 @@ struct FxPlanes {
     }
 
     // A matrix with an FP32 remainder.
-    __device__ __forceinline__ FMat mat(const char *r, int plane) const
-    {
-        const int4 *p = ptr(r, plane);
-        FMat u;
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            const int4 v = __ldg(p + e * S);
-            u.rh[e / 3][e % 3] = v.x;
-            u.rl[e / 3][e % 3] = __int_as_float(v.y);
-            u.ih[e / 3][e % 3] = v.z;
-            u.il[e / 3][e % 3] = __int_as_float(v.w);
-        }
-        return u;
-    }
+    __device__ __forceinline__ FMat mat(const char *r, int plane) const { return fx_mat_at<S, true>(ptr(r, plane)); }
 
-    // Either of the two (whole: whole limbs), or (dag) its dagger, chosen at run time:
-    // the off-diagonal entries are then read from their mirrored places.
+    // Either of the two (whole: whole limbs), or (dag) its dagger, chosen at run time.
     __device__ __forceinline__ FMat form(const char *r, int plane, bool whole, bool dag) const
     {
-        const int4 *p = ptr(r, plane);
-        const int o = dag ? 2 * S : 0, m = dag ? -1 : 0, f = dag ? (int)0x80000000 : 0;
-        const int4 *up = p + o, *dn = p - o, *up2 = up + o, *dn2 = dn - o;
-        const int4 v[9] = {__ldg(p),           __ldg(up + S),      __ldg(up2 + 2 * S), __ldg(dn + 3 * S), __ldg(p + 4 * S),
-                           __ldg(up + 5 * S),  __ldg(dn2 + 6 * S), __ldg(dn + 7 * S),  __ldg(p + 8 * S)};
-        FMat u;
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            u.rh[e / 3][e % 3] = v[e].x;
-            u.ih[e / 3][e % 3] = (v[e].z ^ m) - m;
-            u.rl[e / 3][e % 3] = __int_as_float(v[e].y);
-            u.il[e / 3][e % 3] = __int_as_float(v[e].w);
-        }
-        if (whole) {
-#pragma unroll
-            for (int e = 0; e < 9; ++e) {
-                u.rl[e / 3][e % 3] = 0x1p-28f * (float)v[e].y;
-                u.il[e / 3][e % 3] = 0x1p-28f * (float)v[e].w;
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < 9; ++e)
-            u.il[e / 3][e % 3] = __int_as_float(__float_as_int(u.il[e / 3][e % 3]) ^ f);
-        return u;
+        return fx_form_at<S, true>(ptr(r, plane), whole, dag);
     }
 
     __device__ __forceinline__ void store(char *r, int plane, const FLimbs &u) const
