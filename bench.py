@@ -94,7 +94,7 @@ def _source_digest() -> str:
     """Digest of the force kernels' code (comments and whitespace stripped,
     so that only a change of the code itself invalidates a recorded profile)."""
     h = hashlib.sha256()
-    for f in ("force_sf.cu", "su3.cuh"):
+    for f in ("force_sf.cu", "sf_common.cuh", "su3.cuh"):
         with open(os.path.join(ROOT, "paper_1808_02281_gb300", "csrc", f)) as fh:
             text = fh.read()
         text = re.sub(r"/\*.*?\*/", " ", text, flags=re.S)

@@ -61,7 +61,7 @@ namespace {
 // at coordinates c; stored at staple index sx of sf.
 template <typename R, bool FULL>
 __device__ __forceinline__ void site_staples(const R *__restrict__ links, const G32 &g, const Coord &c,
-                                             int x, int mu, const Planes<R, FULL> &sf, int sx)
+                                             int x, int mu, const Planes<FULL> &sf, int sx)
 {
     const int64_t V = g.V;
     const int xm = x + step32(g, c, mu, 1); // x + mu
@@ -89,7 +89,7 @@ __device__ __forceinline__ void site_staples(const R *__restrict__ links, const 
 // Staple plane mu*6 + j of site x (site_staples one at a time).
 template <typename R, bool FULL>
 __device__ __forceinline__ void site_staple(const R *__restrict__ links, const G32 &g, const Coord &c, int x, int mu, int j,
-                                            const Planes<R, FULL> &sf)
+                                            const Planes<FULL> &sf)
 {
     const int64_t V = g.V;
     const int nu = (mu + 1 + (j >> 1)) & 3;
@@ -115,7 +115,7 @@ __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, 
     const int x = vb * 32 + (int)(threadIdx.x & 31);
     if (x >= g.V) return;
     site_staples<R, FULL>(static_cast<const R *>(L.links), g, coord32(g, L.div, x), x, mu,
-                                planes_of<R, FULL>(L), x);
+                                planes_of<FULL>(L), x);
 }
 
 template <typename R, bool FULL>
@@ -137,7 +137,7 @@ __device__ __forceinline__ void split_staples_block(const SfLattice &L, const G3
     const Coord c = coord32(g, L.div, x);
 #pragma unroll 1
     for (int j = q; j < 6; j += 4)
-        site_staple<R, FULL>(static_cast<const R *>(L.links), g, c, x, mu, j, planes_of<R, FULL>(L));
+        site_staple<R, FULL>(static_cast<const R *>(L.links), g, c, x, mu, j, planes_of<FULL>(L));
 }
 
 template <typename R, bool FULL>
@@ -182,7 +182,7 @@ __device__ __forceinline__ double force_block(const SfLattice &L, const KernelSc
     const Coord c = swept_site(sw, j);
     const int k = index32(g, c);
     const LatticeSites si{&g, &c, k};
-    return force_link<R, ACTION, UNROLLQ, false>(L, sc, g, planes_of<R, FULL>(L), si, c, k, rho);
+    return force_link<R, ACTION, UNROLLQ, false>(L, sc, g, planes_of<FULL>(L), si, c, k, rho);
 }
 
 // Split lattices: the links of direction rho of virtual block vb, warp 0 their
@@ -199,7 +199,7 @@ __device__ __forceinline__ void split_force_block(const SfLattice &L, const Kern
     const Coord c = swept_site(sw, j < g.V ? j : g.V - 1);
     const int k = index32(g, c), kp = k + step32(g, c, rho, 1);
     const LatticeSites si{&g, &c, k};
-    const auto sf = planes_of<R, true>(L);
+    const auto sf = planes_of<true>(L);
     const R *__restrict__ links = static_cast<const R *>(L.links);
     const R c_rt = scalar<R>(sc, SC_CRT), c_cb = scalar<R>(sc, SC_CCB);
     Mat<R> t;

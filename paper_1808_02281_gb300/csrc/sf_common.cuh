@@ -27,52 +27,44 @@ template <typename R> __device__ __forceinline__ R scalar(const KernelScalars &s
     else return s.d[i];
 }
 
-// Storage of the 24 staple planes: compact (rows 0 and 1, 12 reals, the
+// Storage of the 24 FP32 staple planes: compact (rows 0 and 1, 12 reals, the
 // third row rebuilt on load) or full (all 18 reals, nothing rebuilt).  Both
 // are cut into blocks of 32 consecutive sites: inside a block, 16-byte lane
-// q (q < NW = 12/W compact, 18/W full) of the staple of site s is at
-// q*512 + s*16 bytes, and for full FP32 staples the last two reals at
-// NW*512 + s*8 -- 72 bytes per full staple in FP32, 144 in FP64, every
-// access 16- or 8-byte aligned, and the lanes of one staple a constant 512
-// bytes apart, so that a staple costs one address computation (plus one for
-// the FP32 tail) however many lanes it has.  Plane P starts at
-// P * plane_bytes, plane_bytes = the
-// 32-site blocks of the lattice (V rounded up to 32) times the block size.
+// q (3 compact, 4 full) of the staple of site s is at q*512 + s*16 bytes, and
+// of full staples the last two reals at 4*512 + s*8 -- 72 bytes a full staple,
+// every access 16- or 8-byte aligned, and the lanes of one staple a constant
+// 512 bytes apart, so that a staple costs one address computation (plus one
+// for the tail).  Plane P starts at P * plane_bytes, plane_bytes = the 32-site
+// blocks of the lattice (V rounded up to 32) times the block size.  FP64
+// staples have a form of their own (FxPlanes).
 // Pass A writes them with evict-first stores: the 3.6 GB (at 32^3x64) would
 // otherwise push the links that pass A re-reads out of L2.
 constexpr int kStaplePlanes = 24;
 
-template <typename R> struct FullBlock {
-    using V4 = typename Vec<R>::type;
-    static constexpr int W = Vec<R>::W;
-    static constexpr int NW = 18 / W;        // whole 16-byte lanes per staple
-    static constexpr int TAIL = 18 - NW * W; // reals in the FP32 tail (2)
-    static constexpr int LANE = 32 * 16;     // bytes of one lane of a block
-    static constexpr int BYTES = NW * LANE + TAIL * (int)sizeof(R) * 32;
-    static_assert(NW * W + TAIL == 18, "a full staple holds 18 reals");
+struct FullBlock {
+    static constexpr int NW = 4;                 // whole 16-byte lanes per staple
+    static constexpr int LANE = 32 * 16;         // bytes of one lane of a block
+    static constexpr int BYTES = NW * LANE + 32 * 8;
 };
 
 inline size_t full_plane_bytes(int64_t V, int precision)
 {
-    return precision == LQCD_F64 ? fx_plane_bytes(V) : (size_t)((V + 31) / 32) * FullBlock<float>::BYTES;
+    return precision == LQCD_F64 ? fx_plane_bytes(V) : (size_t)((V + 31) / 32) * FullBlock::BYTES;
 }
 
 // Compact planes: the first two rows (12 reals) of every staple, the third
-// rebuilt on load, in the same 32-site blocks (lane q, q < 12/W, of site s at
+// rebuilt on load, in the same 32-site blocks (lane q, q < 3, of site s at
 // q*512 + s*16).
-template <typename R> struct CompactBlock {
-    using V4 = typename Vec<R>::type;
-    static constexpr int W = Vec<R>::W;
-    static constexpr int NW = 12 / W;
+struct CompactBlock {
+    static constexpr int NW = 3;
     static constexpr int LANE = 32 * 16;
     static constexpr int BYTES = NW * LANE;
 };
 
-template <typename R, bool FULL> struct Planes;
+template <bool FULL> struct Planes;
 
-template <typename R> struct Planes<R, false> {
-    using B = CompactBlock<R>;
-    using V4 = typename B::V4;
+template <> struct Planes<false> {
+    using B = CompactBlock;
     char *base;
     int64_t plane_bytes;
     using Ref = char *;
@@ -82,24 +74,19 @@ template <typename R> struct Planes<R, false> {
         return base + (int64_t)(n >> 5) * B::BYTES + (n & 31) * 16;
     }
 
-    __device__ __forceinline__ Mat<R> load(Ref r, int plane) const
+    __device__ __forceinline__ Mat<float> load(Ref r, int plane) const
     {
-        const V4 *p = reinterpret_cast<const V4 *>(r + (int64_t)plane * plane_bytes);
-        R x[12];
+        const float4 *p = reinterpret_cast<const float4 *>(r + (int64_t)plane * plane_bytes);
+        float x[12];
 #pragma unroll
         for (int q = 0; q < B::NW; ++q) {
-            const V4 v = __ldg(p + q * (B::LANE / 16));
-            if constexpr (B::W == 4) {
-                x[4 * q + 0] = v.x;
-                x[4 * q + 1] = v.y;
-                x[4 * q + 2] = v.z;
-                x[4 * q + 3] = v.w;
-            } else {
-                x[2 * q + 0] = v.x;
-                x[2 * q + 1] = v.y;
-            }
+            const float4 v = __ldg(p + q * (B::LANE / 16));
+            x[4 * q + 0] = v.x;
+            x[4 * q + 1] = v.y;
+            x[4 * q + 2] = v.z;
+            x[4 * q + 3] = v.w;
         }
-        Mat<R> u;
+        Mat<float> u;
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -111,10 +98,10 @@ template <typename R> struct Planes<R, false> {
         return u;
     }
 
-    __device__ __forceinline__ void store(Ref r, int plane, const Mat<R> &u) const
+    __device__ __forceinline__ void store(Ref r, int plane, const Mat<float> &u) const
     {
-        V4 *p = reinterpret_cast<V4 *>(r + (int64_t)plane * plane_bytes);
-        R x[12];
+        float4 *p = reinterpret_cast<float4 *>(r + (int64_t)plane * plane_bytes);
+        float x[12];
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -123,18 +110,13 @@ template <typename R> struct Planes<R, false> {
                 x[6 * i + 2 * j + 1] = u.im[i][j];
             }
 #pragma unroll
-        for (int q = 0; q < B::NW; ++q) {
-            V4 v;
-            if constexpr (B::W == 4) v = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-            else v = make_double2(x[2 * q], x[2 * q + 1]);
-            __stcs(p + q * (B::LANE / 16), v);
-        }
+        for (int q = 0; q < B::NW; ++q)
+            __stcs(p + q * (B::LANE / 16), make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]));
     }
 };
 
-template <typename R> struct Planes<R, true> {
-    using B = FullBlock<R>;
-    using V4 = typename B::V4;
+template <> struct Planes<true> {
+    using B = FullBlock;
     char *base;          // plane 0
     int64_t plane_bytes;
 
@@ -151,30 +133,23 @@ template <typename R> struct Planes<R, true> {
         return Ref{b + s * 16, b + B::NW * B::LANE + s * 8};
     }
 
-    __device__ __forceinline__ Mat<R> load(const Ref &r, int plane) const
+    __device__ __forceinline__ Mat<float> load(const Ref &r, int plane) const
     {
         const int64_t off = (int64_t)plane * plane_bytes;
-        const V4 *p = reinterpret_cast<const V4 *>(r.p + off);
-        R x[18];
+        const float4 *p = reinterpret_cast<const float4 *>(r.p + off);
+        float x[18];
 #pragma unroll
         for (int q = 0; q < B::NW; ++q) {
-            const V4 v = __ldg(p + q * (B::LANE / 16));
-            if constexpr (B::W == 4) {
-                x[4 * q + 0] = v.x;
-                x[4 * q + 1] = v.y;
-                x[4 * q + 2] = v.z;
-                x[4 * q + 3] = v.w;
-            } else {
-                x[2 * q + 0] = v.x;
-                x[2 * q + 1] = v.y;
-            }
+            const float4 v = __ldg(p + q * (B::LANE / 16));
+            x[4 * q + 0] = v.x;
+            x[4 * q + 1] = v.y;
+            x[4 * q + 2] = v.z;
+            x[4 * q + 3] = v.w;
         }
-        if constexpr (B::TAIL == 2) {
-            const float2 t = __ldg(reinterpret_cast<const float2 *>(r.t + off));
-            x[16] = t.x;
-            x[17] = t.y;
-        }
-        Mat<R> u;
+        const float2 t = __ldg(reinterpret_cast<const float2 *>(r.t + off));
+        x[16] = t.x;
+        x[17] = t.y;
+        Mat<float> u;
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -185,11 +160,11 @@ template <typename R> struct Planes<R, true> {
         return u;
     }
 
-    __device__ __forceinline__ void store(const Ref &r, int plane, const Mat<R> &u) const
+    __device__ __forceinline__ void store(const Ref &r, int plane, const Mat<float> &u) const
     {
         const int64_t off = (int64_t)plane * plane_bytes;
-        V4 *p = reinterpret_cast<V4 *>(r.p + off);
-        R x[18];
+        float4 *p = reinterpret_cast<float4 *>(r.p + off);
+        float x[18];
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -198,24 +173,20 @@ template <typename R> struct Planes<R, true> {
                 x[2 * (3 * i + j) + 1] = u.im[i][j];
             }
 #pragma unroll
-        for (int q = 0; q < B::NW; ++q) {
-            V4 v;
-            if constexpr (B::W == 4) v = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-            else v = make_double2(x[2 * q], x[2 * q + 1]);
-            __stcs(p + q * (B::LANE / 16), v);
-        }
-        if constexpr (B::TAIL == 2) __stcs(reinterpret_cast<float2 *>(r.t + off), make_float2(x[16], x[17]));
+        for (int q = 0; q < B::NW; ++q)
+            __stcs(p + q * (B::LANE / 16), make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]));
+        __stcs(reinterpret_cast<float2 *>(r.t + off), make_float2(x[16], x[17]));
     }
 };
 
-template <typename R, bool FULL> __device__ __forceinline__ Planes<R, FULL> planes_of(const SfLattice &L)
+template <bool FULL> __device__ __forceinline__ Planes<FULL> planes_of(const SfLattice &L)
 {
     if constexpr (FULL) {
-        return Planes<R, true>{static_cast<char *>(L.staples), L.plane_bytes};
+        return Planes<true>{static_cast<char *>(L.staples), L.plane_bytes};
     } else {
         const int64_t V = (int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3];
-        return Planes<R, false>{static_cast<char *>(L.staples),
-                                ((V + 31) / 32) * CompactBlock<R>::BYTES};
+        return Planes<false>{static_cast<char *>(L.staples),
+                                ((V + 31) / 32) * CompactBlock::BYTES};
     }
 }
 
@@ -418,11 +389,9 @@ __device__ __forceinline__ int batch_entry(const SfBatch &B, int64_t vb)
 
 // Products of two SU(3) factors are accumulated as y += s * (a * op(b)) with
 // the third row of the product rebuilt from its first two (mul_acc_su3: the
-// third row of a is never rebuilt or loaded), or (DIRECT, full FP64 staples)
-// as plain products accumulated in full, the sum scaled once: for FP64 that
-// measured faster (114 vs 122 ms at 32^3x64: at the 255-register limit the
-// extra temporaries spill); for FP32 the rebuilt form is faster (3.65 vs
-// 3.75 ms).
+// third row of a is never rebuilt or loaded; FP32, 3.65 against 3.75 ms at
+// 32^3x64), or (DIRECT, the floating-point path of single FP64 links) as plain
+// products accumulated in full, the sum scaled once.
 template <int FB, bool DIRECT, typename R>
 __device__ __forceinline__ void acc_su3(Mat<R> &y, const Mat<R> &a, const Mat<R> &b, R s)
 {

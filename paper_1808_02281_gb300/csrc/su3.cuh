@@ -37,17 +37,6 @@ template <typename R> __device__ __forceinline__ void set_zero(Mat<R> &m)
         for (int j = 0; j < 3; ++j) m.re[i][j] = m.im[i][j] = R(0);
 }
 
-template <typename R> __device__ __forceinline__ void set_unit(Mat<R> &m)
-{
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            m.re[i][j] = (i == j) ? R(1) : R(0);
-            m.im[i][j] = R(0);
-        }
-}
-
 template <typename R> __device__ __forceinline__ Mat<R> dagger(const Mat<R> &a)
 {
     Mat<R> r;
