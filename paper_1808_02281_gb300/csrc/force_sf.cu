@@ -186,14 +186,15 @@ __device__ __forceinline__ double force_block(const SfLattice &L, const KernelSc
 }
 
 // Split lattices: the links of direction rho of virtual block vb, warp 0 their
-// plaquettes and chains, warps 1 to 3 the terms of one direction d each; warp
-// 0 adds them up.  A quarter of force_block's chain of products (14 against
-// 51 of a thread).  The action's share goes to partial vb*4 + rho.
+// plaquettes and chains, warps 1 to 3 the sums of products that the links +-d
+// of one direction close; warp 0 closes them, in force_link's order, so that
+// force and action have the bits of force_block.  20 products in a row against
+// 51 of a thread.  The action's share goes to partial vb*4 + rho.
 template <typename R, bool ACTION>
 __device__ __forceinline__ void split_force_block(const SfLattice &L, const KernelScalars &sc, const G32 &g,
                                                   const Sweep &sw, int vb, int rho)
 {
-    __shared__ R t_s[3][18][32];
+    __shared__ R y_s[6][18][32]; // of +d, then of -d
     const int part = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
     const int j = vb * 32 + lane;
     const Coord c = swept_site(sw, j < g.V ? j : g.V - 1);
@@ -207,24 +208,36 @@ __device__ __forceinline__ void split_force_block(const SfLattice &L, const Kern
     if (part == 0) {
         chain_terms<R, ACTION, false>(t, tr_pl, links, sf, si, g, c, rho, k, kp, scalar<R>(sc, SC_CPL), c_rt);
     } else {
-        set_zero(t);
-        d_terms<false, false, false>(t, links, sf, si, g, c, rho, k, kp, part - 1, c_rt, c_cb);
-        d_terms<true, false, false>(t, links, sf, si, g, c, rho, k, kp, part - 1, c_rt, c_cb);
+        const auto put = [&](int i, const Mat<R> &y) {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) {
-            t_s[part - 1][2 * e][lane] = t.re[e / 3][e % 3];
-            t_s[part - 1][2 * e + 1][lane] = t.im[e / 3][e % 3];
-        }
+            for (int e = 0; e < 9; ++e) {
+                y_s[i][2 * e][lane] = y.re[e / 3][e % 3];
+                y_s[i][2 * e + 1][lane] = y.im[e / 3][e % 3];
+            }
+        };
+        d_terms<false, false, false, false>(t, links, sf, si, g, c, rho, k, kp, part - 1, c_rt, c_cb);
+        put(part - 1, t);
+        d_terms<true, false, false, false>(t, links, sf, si, g, c, rho, k, kp, part - 1, c_rt, c_cb);
+        put(part + 2, t);
     }
     __syncthreads();
     if (part == 0) {
-#pragma unroll
-        for (int p = 0; p < 3; ++p)
+        const auto get = [&](int i) {
+            Mat<R> y;
 #pragma unroll
             for (int e = 0; e < 9; ++e) {
-                t.re[e / 3][e % 3] += t_s[p][2 * e][lane];
-                t.im[e / 3][e % 3] += t_s[p][2 * e + 1][lane];
+                y.re[e / 3][e % 3] = y_s[i][2 * e][lane];
+                y.im[e / 3][e % 3] = y_s[i][2 * e + 1][lane];
             }
+            return y;
+        };
+#pragma unroll
+        for (int id = 0; id < 3; ++id) mul_acc<N, N>(t, load_link(links, g.V, (rho + 1 + id) & 3, kp), get(id));
+#pragma unroll
+        for (int id = 0; id < 3; ++id) {
+            const int nud = (rho + 1 + id) & 3;
+            mul_acc<D, N>(t, load_link(links, g.V, nud, kp + step32(g, c, nud, -1)), get(3 + id));
+        }
         double share = 0.0;
         if (j < g.V) share = finish_link<R, ACTION>(L, sc, links, g.V, rho, k, t, tr_pl);
         if constexpr (ACTION) {
@@ -232,7 +245,7 @@ __device__ __forceinline__ void split_force_block(const SfLattice &L, const Kern
             if (lane == 0) L.partials[vb * 4 + rho] = share;
         }
     }
-    __syncthreads(); // before t_s is written again
+    __syncthreads(); // before y_s is written again
 }
 
 template <typename R, bool ACTION>
@@ -243,8 +256,10 @@ __global__ void __launch_bounds__(kBlock, 4)
     split_force_block<R, ACTION>(L, sc, g, make_sweep(L, g), (int)(blockIdx.x >> 2), (int)(blockIdx.x & 3));
 }
 
-// The split lattices of a batch, in a launch of their own: with both kinds of
-// block in one kernel the large lattices took 3 to 6 % longer.
+// The same for a batch of split lattices only: a batch with a large lattice
+// among them takes the whole blocks for all (with quarter blocks in one kernel
+// with whole ones the large lattices took 3 to 6 % longer, and a launch of
+// their own is 7 us).
 template <typename R, bool ACTION>
 __global__ void __launch_bounds__(kBlock, 4)
     force_split_batched(const __grid_constant__ SfBatch B, const __grid_constant__ KernelScalars sc)
@@ -296,8 +311,14 @@ __global__ void __launch_bounds__(kBlock, (min_blocks<ACTION, DENSE>()))
         const double acc = force_block<R, ACTION, UNROLLQ, FULL>(
             L, sc, g, make_sweep(L, g), (int)(vb - L.vb_begin));
         if constexpr (ACTION) {
-            const double s = block_sum(acc);
-            if (threadIdx.x == 0) L.partials[vb - L.vb_begin] = s;
+            const int64_t v = vb - L.vb_begin;
+            if (L.split) { // the partial sums of force_split
+                const double s = warp_sum(acc);
+                if ((threadIdx.x & 31) == 0) L.partials[v * 4 + (threadIdx.x >> 5)] = s;
+            } else {
+                const double s = block_sum(acc);
+                if (threadIdx.x == 0) L.partials[v] = s;
+            }
         }
         vb = publish_virtual_block(next);
     }
@@ -497,46 +518,34 @@ cudaError_t launch_passes(const SfLattice &L, const KernelScalars &sc, int varia
     return action ? launch_pass_b<true>(L, sc, variant, st) : launch_pass_b<false>(L, sc, variant, st);
 }
 
-// The lattices of B with (or without) split set, numbered anew in blocks of
-// 32 sites or quarters of one.
-SfBatch part_of(const SfBatch &B, bool split)
-{
-    SfBatch p{};
-    p.counter = B.counter;
-    for (int c = 0; c < B.n; ++c) {
-        if ((B.e[c].split != 0) != split) continue;
-        const int *d = B.e[c].dims;
-        SfLattice &L = p.e[p.n++];
-        L = B.e[c];
-        L.vb_begin = p.total;
-        p.total += virtual_blocks((int64_t)d[0] * d[1] * d[2] * d[3]) * (split ? 4 : 1);
-    }
-    return p;
-}
-
 cudaError_t launch_passes_batched(const SfBatch &B, const KernelScalars &sc, int variant, bool action, cudaStream_t st)
 {
-    const SfBatch split = part_of(B, true);
-    if (split.n == B.n) {
-        staple_fields_split_batched<float, true><<<grid_of(split.total), kBlock, 0, st>>>(split);
-    } else if (full_staples(variant)) {
+    SfBatch quarters = B; // blocks of a quarter each
+    quarters.total = 0;
+    bool all_split = true;
+    for (int c = 0; c < B.n; ++c) {
+        const int *d = B.e[c].dims;
+        quarters.e[c].vb_begin = quarters.total;
+        quarters.total += 4 * virtual_blocks((int64_t)d[0] * d[1] * d[2] * d[3]);
+        all_split = all_split && B.e[c].split;
+    }
+    if (all_split) {
+        staple_fields_split_batched<float, true><<<grid_of(quarters.total), kBlock, 0, st>>>(quarters);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (action) force_split_batched<float, true><<<grid_of(quarters.total), kBlock, 0, st>>>(quarters, sc);
+        else force_split_batched<float, false><<<grid_of(quarters.total), kBlock, 0, st>>>(quarters, sc);
+        return cudaGetLastError();
+    }
+    if (full_staples(variant)) {
         auto ka = staple_fields_batched<float, true>;
         ka<<<persistent_grid(ka, grid_slot(5, false, false), B.total), kBlock, 0, st>>>(B);
     } else {
         auto ka = staple_fields_batched<float, false>;
         ka<<<persistent_grid(ka, grid_slot(4, false, false), B.total), kBlock, 0, st>>>(B);
     }
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (split.n > 0) {
-        if (action) force_split_batched<float, true><<<grid_of(split.total), kBlock, 0, st>>>(split, sc);
-        else force_split_batched<float, false><<<grid_of(split.total), kBlock, 0, st>>>(split, sc);
-        e = cudaGetLastError();
-        if (e != cudaSuccess || split.n == B.n) return e;
-        const SfBatch whole = part_of(B, false);
-        return action ? launch_pass_b_batched<true>(whole, sc, variant, st)
-                      : launch_pass_b_batched<false>(whole, sc, variant, st);
-    }
     return action ? launch_pass_b_batched<true>(B, sc, variant, st) : launch_pass_b_batched<false>(B, sc, variant, st);
 }
 
@@ -560,7 +569,7 @@ bool staple_fields_supported(const int dims[4])
 int staple_force_partials(const int dims[4])
 {
     const int64_t V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
-    return (int)virtual_blocks(V) * (split_lattice(LQCD_F32, V) || split_lattice(LQCD_F64, V) ? 4 : 1);
+    return (int)virtual_blocks(V) * (split_lattice(V) ? 4 : 1);
 }
 
 cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
@@ -571,7 +580,7 @@ cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
     for (int i = 0; i < 4; ++i) L.dims[i] = a.dims[i];
     set_traversal(L, variant);
     L.plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
-    L.split = split_lattice(a.precision, V) && (a.precision == LQCD_F64 || full_staples(variant));
+    L.split = split_lattice(V) && (a.precision == LQCD_F64 || full_staples(variant));
     L.links = a.links;
     L.staples = a.staples;
     L.force = a.force;
@@ -601,7 +610,7 @@ cudaError_t launch_force_staple_fields_batched(const ForceArgs &a, int n, const 
         B.e[c] = items[c];
         set_traversal(B.e[c], variant);
         B.e[c].plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
-        B.e[c].split = split_lattice(a.precision, V) && (a.precision == LQCD_F64 || full_staples(variant));
+        B.e[c].split = split_lattice(V) && (a.precision == LQCD_F64 || full_staples(variant));
         B.e[c].vb_begin = B.total;
         B.total += virtual_blocks(V);
         any_action = any_action || B.e[c].action != nullptr;

@@ -409,11 +409,12 @@ struct LatticeSites {
     __device__ __forceinline__ int nb(int mu, int s) const { return k + step32(*g, *c, mu, s); }
 };
 
-// The staples that start with link(k+rho, d), d = +-nu_d (NEG: minus):
-//   t += B_d [ c_cube sum_{b perp rho, d} S_b(k+d) S^{(d)}_b(k) + c_rect S_d(k+d) A_d^dag ]
+// The staples that start with link(k+rho, d), d = +-nu_d (NEG: minus), t += B_d y:
+//   y = [ c_cube sum_{b perp rho, d} S_b(k+d) S^{(d)}_b(k) + c_rect S_d(k+d) A_d^dag ]
 // (the orientation of the shared links fixed at compile time, so that each
 // sign has one small loop body).
-template <bool NEG, bool UNROLLQ, bool DIRECT, typename R, typename SF, typename SI>
+// CLOSE = false: y into t.
+template <bool NEG, bool UNROLLQ, bool DIRECT, bool CLOSE = true, typename R, typename SF, typename SI>
 __device__ __forceinline__ void d_terms(Mat<R> &t, const R *__restrict__ links,
                                         const SF &sf, const SI &si, const G32 &g,
                                         const Coord &c, int rho, int k, int kp, int id, R c_rt,
@@ -448,11 +449,12 @@ __device__ __forceinline__ void d_terms(Mat<R> &t, const R *__restrict__ links,
     }
     if constexpr (!NEG) {
         acc_su3<D, DIRECT>(y, r3, load_link(links, V, nud, k), c_rt); // A_d = U_nud(k)
-        mul_acc<N, N>(t, load_link(links, V, nud, kp), y);         // B_d = U_nud(k+rho)
+        if constexpr (CLOSE) mul_acc<N, N>(t, load_link(links, V, nud, kp), y); // B_d = U_nud(k+rho)
     } else {
         acc_su3<N, DIRECT>(y, r3, load_link(links, V, nud, kd), c_rt);  // A_d = U_nud(k-nud)^dag
-        mul_acc<D, N>(t, load_link(links, V, nud, kp + (kd - k)), y);  // B_d = U_nud(k+rho-nud)^dag
+        if constexpr (CLOSE) mul_acc<D, N>(t, load_link(links, V, nud, kp + (kd - k)), y); // B_d = U_nud(k+rho-nud)^dag
     }
+    if constexpr (!CLOSE) t = y;
 }
 
 // The plaquettes and the two rectangle chains along rho: t = c_plaq Pl +
@@ -541,14 +543,12 @@ __device__ __forceinline__ double force_link(const SfLattice &L, const KernelSca
 // several warps: four in FP32 (force_sf.cu), eight in FP64 (force_fx.cu).
 // While there are fewer blocks than SMs a launch lasts as long as one thread's
 // chain of products.  Measured, whole | split, force and action: FP32 4^4 24.6
-// | 17.4 us, 64 blocks 26.7 | 17.1, 128 28.7 | 20.5, 256 30.5 | 32.7; FP64 8
-// blocks 73.7 | 30.8, 64 75.6 | 45.2, 128 75.9 | 72.4, 256 97 | 123.  FP32
-// stops at 64 because batches that mix both kinds launch the split ones apart
-// (7 us).
-constexpr int kSplitBlocks[2] = {64, 128}; // FP32, FP64
-inline bool split_lattice(int precision, int64_t V)
+// | 16.7 us, 64 blocks 28.7 | 19.7, 128 26.7 | 22.6, 256 31.8 | 34.0; FP64 8
+// blocks 73.7 | 30.8, 64 75.6 | 45.2, 128 75.9 | 72.4, 256 97 | 123.
+constexpr int kSplitBlocks = 128;
+inline bool split_lattice(int64_t V)
 {
-    return virtual_blocks(V) <= kSplitBlocks[precision == LQCD_F64 ? 1 : 0];
+    return virtual_blocks(V) <= kSplitBlocks;
 }
 
 // Sum over a warp of one double per lane (result in lane 0), the order of

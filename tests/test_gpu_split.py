@@ -11,8 +11,8 @@ from paper_1808_02281_gb300 import hmc, lqcd, synth
 
 pytestmark = pytest.mark.gpu
 
-# 32 sites are a block; lattices of up to 64 (FP32) or 128 (FP64) blocks are split
-SIZES = [(1, 1, 1, 1), (2, 2, 2, 4), (3, 1, 11, 1), (7, 3, 5, 9), (16, 8, 4, 4), (17, 8, 15, 1), (16, 8, 8, 4), (13, 9, 7, 5)]
+# 32 sites are a block; lattices of up to 128 blocks are split
+SIZES = [(1, 1, 1, 1), (2, 2, 2, 4), (3, 1, 11, 1), (7, 3, 5, 9), (16, 8, 4, 4), (17, 8, 15, 1), (16, 8, 8, 4), (13, 9, 7, 5), (13, 9, 9, 4)]
 TOL = {"f64": 1e-12, "f32": 2e-5}
 
 
@@ -56,3 +56,30 @@ def test_batches_equal_single(dims_list, prec):
         lqcd.md_force_step(lat, bs.links[c], force=f, action=S)
         assert torch.equal(f, force[c]), d
         assert float(S) == float(actions[c]), d
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("tile", [(4, 4, 4, 4), (2, 3, 4, 5)])
+def test_split_has_the_bits_of_the_whole(tile, prec):
+    """Links that repeat with period `tile` on a lattice that is not split: every
+    copy has the force of the split lattice of one tile, to the bit, and the
+    action is the tile's times the copies (sums in FP64: 1e-13)."""
+    times = (2, 2, 4, 4) if tile[0] == 4 else (4, 4, 4, 4)
+    big = tuple(a * b for a, b in zip(tile, times))
+    small, large = (lqcd.Lattice.symanzik(d, 6.0, 0.87, prec, force_algo=lqcd.FORCE_STAPLE_FIELDS) for d in (tile, big))
+    grids = np.indices(big[::-1])  # t, z, y, x
+    n = np.zeros(big[::-1], dtype=np.int64)
+    for g, d in zip(grids, tile[::-1]):
+        n = n * d + g % d
+    at = torch.from_numpy(n.reshape(-1)).cuda()
+    links = lqcd.links_from_omega(small, lqcd.algebra_to_device(small, synth.omega(tile, 0.4, 9)))
+    copies = lqcd.pack_links(large, lqcd.unpack_links(small, links)[at].contiguous())
+    out = []
+    for lat, U in ((small, links), (large, copies)):
+        S = torch.empty((), dtype=torch.float64, device="cuda")
+        force = lqcd.empty_algebra(lat)
+        lqcd.md_force_step(lat, U, force=force, action=S)
+        out.append((lqcd.algebra_from_device(force), float(S.item())))
+    (f, s), (f_copies, s_copies) = out
+    assert (f_copies.reshape(large.V, -1) == f.reshape(small.V, -1)[n.reshape(-1)]).all()
+    assert abs(s_copies - s * large.V / small.V) <= 1e-13 * abs(s_copies)
