@@ -3,20 +3,24 @@
 //
 // In floating point a link is about 550 operations on a pipe that issues 2 a
 // clock and SM: 9.5 k clocks a warp where the 256 bytes of a link take 385
-// from memory.  Here the FP64 pipe only scales the momenta and converts the
-// results; inputs are taken apart with integer operations (a conversion on
-// the FP64 pipe costs as much as an FMA).
+// from memory.  Here that pipe scales the momenta, converts the change of the
+// link, adds it and takes the product of the rows; inputs are taken apart with
+// integer operations (a conversion on the FP64 pipe costs as much as an FMA).
 //
 // With c1 = tr Q^2 / 2, c0 = det Q the series of exp(i Q) is
-// f0 + f1 Q + f2 Q^2 (su3.cuh), applied as
-//     U + (f0 - 1) U + f1 (Q U) + f2 (Q (Q U)),
-// so that the rounding of the products is small with Q: they are formed with
-// Q scaled by a power of two to c1 = 1/8 to 1/2.  Where Q itself is larger,
-// exp(i 2^-s Q) is applied 2^s times.
-// The links are unitary to rounding in every molecular-dynamics step, so
-// Gram-Schmidt is a first-order correction by the departures, which are exact
-// whole numbers below 2^-30; links that depart further, scales above s = 2 and
-// what is not finite take the floating-point step (link_step).
+// f0 + f1 Q + f2 Q^2 (su3.cuh), and what is computed in whole numbers is the
+// change of the link,
+//     (f0 - 1) U + f1 (Q U) + f2 (Q (Q U)),
+// in a unit of its own: with Q = 2^-t Q', Q' scaled to c1 = 1/16 to 1/2, it is
+// known to 2^-(57 + t), whatever the size of Q, and is added in FP64 to the link
+// as it was stored.  Small entries of links near 1 (or near a subgroup) so keep
+// their digits.  Where Q itself is larger, exp(i 2^-s Q) is applied 2^s times.
+// rms error of the worst class of entries against extended precision, of its
+// own size (U = exp(i w), w and x normal): 0.9 to 1.7e-16 for w from 0 to 0.5
+// and x from 1e-12 to 1; in floating point 1.1 to 2.9e-16.
+// Components of Q of very different sizes (fx_uneven) and links that are not
+// SU(3) to 2^-30 after the step, scales above s = 2 and what is not finite take
+// the floating-point step (link_step).
 #pragma once
 
 #include "fixed.cuh"
@@ -57,13 +61,14 @@ __constant__ const FxS kInverseFactorial[10] = {
     inverse_factorial(3), inverse_factorial(4), inverse_factorial(5),  inverse_factorial(6),  inverse_factorial(7),
     inverse_factorial(8), inverse_factorial(9), inverse_factorial(10), inverse_factorial(11), inverse_factorial(12)};
 
-// f0 - 1, f1, f2 for c0, c1 in units of 2^-58 (c1 <= 1/2): the forward
-// recurrence of exp_i_hermitian, the terms from n = 13 (below 2^-32) in FP32.
+// (f0 - 1) / c0, f1, f2 for c0, c1 in units of 2^-58 (c1 <= 1/2): the forward
+// recurrence of exp_i_hermitian, where a_n = c0 d_(n-1) for every n > 2, the
+// terms from n = 13 (below 2^-32) in FP32.
 __device__ __forceinline__ void fx_exp_coefficients(long long c0, long long c1, long long f[6])
 {
     const FxS s0 = fxs(c0), s1 = fxs(c1);
     // n = 1, 2: i Q, -Q^2 / 2
-    f[0] = f[1] = f[2] = f[5] = 0; // f0r - 1, f0i, f1r, f2i
+    f[0] = f[1] = f[2] = f[5] = 0; // real and imaginary part of (f0 - 1) / c0, f1r, f2i
     f[3] = 1ll << 58;              // f1i
     f[4] = -(1ll << 57);           // f2r
     // (a, b, d) with the sign of i^n: it turns from odd to even n
@@ -72,20 +77,20 @@ __device__ __forceinline__ void fx_exp_coefficients(long long c0, long long c1, 
     for (int m = 0; m < 5; ++m) {
         const auto odd = kInverseFactorial[2 * m], even = kInverseFactorial[2 * m + 1];
         FxS ds = fxs(d);
+        f[1] += fxs_mul(odd, ds);
         long long an = fxs_mul(s0, ds), bn = a + fxs_mul(s1, ds);
         d = b;
         a = an;
         b = bn;
         ds = fxs(d);
-        f[1] += fxs_mul(odd, fxs(a));
         f[3] += fxs_mul(odd, fxs(b));
         f[5] += fxs_mul(odd, ds);
+        f[0] -= fxs_mul(even, ds);
         an = -fxs_mul(s0, ds);
         bn = -a - fxs_mul(s1, ds);
         d = -b;
         a = an;
         b = bn;
-        f[0] += fxs_mul(even, fxs(a));
         f[2] += fxs_mul(even, fxs(b));
         f[4] += fxs_mul(even, fxs(d));
     }
@@ -96,13 +101,13 @@ __device__ __forceinline__ void fx_exp_coefficients(long long c0, long long c1, 
 #pragma unroll
     for (int n = 13; n <= 19; ++n) {
         const float sign = n & 1 ? 1.f : -1.f;
+        const int o = n & 1;
+        ff *= 1.f / (float)n;
+        t[0 + o] = fmaf(ff, sign * fd, t[0 + o]);
         const float an = sign * g0 * fd, bn = sign * fmaf(g1, fd, fa), dn = sign * fb;
         fa = an;
         fb = bn;
         fd = dn;
-        ff *= 1.f / (float)n;
-        const int o = n & 1;
-        t[0 + o] = fmaf(ff, fa, t[0 + o]);
         t[2 + o] = fmaf(ff, fb, t[2 + o]);
         t[4 + o] = fmaf(ff, fd, t[4 + o]);
     }
@@ -110,17 +115,54 @@ __device__ __forceinline__ void fx_exp_coefficients(long long c0, long long c1, 
     for (int i = 0; i < 6; ++i) f[i] += (long long)__float2int_rn(t[i]); // below 2^-32: fits 27 bits
 }
 
+// Below this exponent field nothing of an exponent shows in a link (2^-900).
+constexpr int kLeastExponent = 123;
+
+// Whether four or more components of x are below 2^-6 of the largest (exponent
+// field em): five links in a million of Gaussian momenta, and all of a field whose
+// momenta lie in a subgroup (diagonal links, an SU(2) or U(2) block, real
+// rotations), beside which the link step has to keep small ones to a precision
+// of their own.
+__device__ __forceinline__ bool fx_uneven(const double x[8], int em)
+{
+    int n = 0;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) n += em - exponent_of(x[a]) > 6;
+    return n >= 4;
+}
+
+// Row i of a b, units 2^-60.
+__device__ __forceinline__ void fx_row_mul(const FLimbs &a, int i, const FLimbs &b, long long re[3], long long im[3])
+{
+    FLimbAcc y; // row 0
+#pragma unroll
+    for (int j = 0; j < 3; ++j) y.h1[0][j] = y.l1[0][j] = y.h2[0][j] = y.l2[0][j] = y.h3[0][j] = y.l3[0][j] = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int sh = a.rh[i][k] + a.ih[i][k], sl = a.rl[i][k] + a.il[i][k];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            fx_mad(y.h1[0][j], y.l1[0][j], a.rh[i][k], a.rl[i][k], b.rh[k][j], b.rl[k][j]);
+            fx_mad(y.h2[0][j], y.l2[0][j], a.ih[i][k], a.il[i][k], b.ih[k][j], b.il[k][j]);
+            fx_mad(y.h3[0][j], y.l3[0][j], sh, sl, b.rh[k][j] + b.ih[k][j], b.rl[k][j] + b.il[k][j]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) fx_total<1>(y, 0, j, re[j], im[j]);
+}
+
 // exp(i sum_a x^a T_a) U with Gram-Schmidt, rows 0 and 1 of both as 12 reals;
 // false where it does not apply (r is then unchanged).
 __device__ __forceinline__ bool fx_link_step(const double x[8], double r[12])
 {
-    // x = 2^(k+1) y with the entries of sum_a y^a lambda_a near 1 or below:
-    // the products then round to 2^-55 of Q and not of 1
-    int em = 1010;
+    // x = 2^(k+1) y, the largest |y^a| 1/4 to 1/2 (1/8 where they are many):
+    // the products then round to 2^-57 of Q and not of 1
+    int em = kLeastExponent;
 #pragma unroll
     for (int a = 0; a < 8; ++a) em = max(em, exponent_of(x[a]));
     int k = em - 1022;
     if (k > 2) return false; // also not finite
+    if (em > kLeastExponent && fx_uneven(x, em)) return false;
     long long y[8];
     float c1f = 0.f;
 #pragma unroll
@@ -136,6 +178,7 @@ __device__ __forceinline__ bool fx_link_step(const double x[8], double r[12])
     }
     const int s = max(k, 0); // 2^s steps
     if (s > 2) return false;
+    const int t = s - k; // of Q 2^-t
     // the link
     FLimbs u;
     {
@@ -143,8 +186,9 @@ __device__ __forceinline__ bool fx_link_step(const double x[8], double r[12])
         fx_row2(u);
     }
     // Q and its invariants
-    FMat q;
-    FScalar g0, g1, g2, m0, m1, m2; // f0 - 1, f1, f2: real and imaginary parts
+    FLimbs q;
+    FxS m1;                     // imaginary part of f1: limbs, the others with FP32 remainders
+    FScalar g0, g1, g2, m0, m2; // f0 - 1, f1, f2: real and imaginary parts
     {
         FxS ys[8];
         long long c1 = 0, l1 = 0;
@@ -166,34 +210,33 @@ __device__ __forceinline__ bool fx_link_step(const double x[8], double r[12])
         long long c0 = fxs_mul(fxs(fxs_mul(d0, d1) - sq(0, 1)), d2) - fxs_mul(d0, fxs(sq(5, 6))) -
                        fxs_mul(d1, fxs(sq(3, 4)));
         c0 += 2 * (fxs_mul(fxs(pr), ys[3]) + fxs_mul(fxs(pi), ys[4]));
-        // back to the scale of one step: Q 2^(k-s)
-        const int t = s - k;
+        // The change of the link in units of 2^-(58 + t): with the invariants
+        // of Q 2^-t, (f0 - 1) 2^t, f1 and f2 2^-t
         long long f[6];
-        fx_exp_coefficients(c0 >> 3 * t, c1 >> 2 * t, f);
-        f[2] >>= t;
-        f[3] >>= t;
-        f[4] >>= 2 * t;
-        f[5] >>= 2 * t;
+        fx_exp_coefficients(c0 >> min(3 * t, 63), c1 >> min(2 * t, 63), f);
+        const FxS c0t = fxs(c0 >> min(2 * t, 63));
+        f[0] = fxs_mul(c0t, fxs(f[0]));
+        f[1] = fxs_mul(c0t, fxs(f[1]));
+        const int down = min(t, 63);
+        f[4] >>= down;
+        f[5] >>= down;
         const auto scalar = [](long long v) {
-            FScalar t;
-            int l;
-            fx_limbs<0>(v, t.h, l);
-            t.l = 0x1p-28f * (float)l;
-            return t;
+            const FxS l = fxs(v);
+            return FScalar{l.h, 0x1p-28f * (float)l.l};
         };
         g0 = scalar(f[0]);
         m0 = scalar(f[1]);
         g1 = scalar(f[2]);
-        m1 = scalar(f[3]);
+        m1 = fxs(f[3]);
         g2 = scalar(f[4]);
         m2 = scalar(f[5]);
         const auto put = [&](int i, int j, const FxS re, const FxS im) {
             q.rh[i][j] = q.rh[j][i] = re.h;
-            q.rl[i][j] = q.rl[j][i] = 0x1p-28f * (float)re.l;
+            q.rl[i][j] = q.rl[j][i] = re.l;
             q.ih[i][j] = -im.h;
-            q.il[i][j] = -0x1p-28f * (float)im.l;
+            q.il[i][j] = -im.l;
             q.ih[j][i] = im.h;
-            q.il[j][i] = 0x1p-28f * (float)im.l;
+            q.il[j][i] = im.l;
         };
         put(0, 1, ys[0], ys[1]);
         put(0, 2, ys[3], ys[4]);
@@ -202,21 +245,31 @@ __device__ __forceinline__ bool fx_link_step(const double x[8], double r[12])
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             q.rh[i][i] = dd[i].h;
-            q.rl[i][i] = 0x1p-28f * (float)dd[i].l;
-            q.ih[i][i] = 0;
-            q.il[i][i] = 0.f;
+            q.rl[i][i] = dd[i].l;
+            q.ih[i][i] = q.il[i][i] = 0;
         }
     }
     long long vr[2][3], vi[2][3]; // rows 0 and 1, units 2^-58
+    long long er[2][3], ei[2][3]; // their change, units 2^-(58 + t)
+    const int tt = min(t, 62);
+    const long long half = (1ll << tt) >> 1;
 #pragma unroll 1
     for (int rep = 0;; ++rep) {
-        const FMat um = fx_remainder(u);
+        // Q U decides the accuracy of the change: whole limbs
+        FLimbs w1;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            long long re[3], im[3];
+            fx_row_mul(q, i, u, re, im);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                fx_limbs<2>(re[j], w1.rh[i][j], w1.rl[i][j]);
+                fx_limbs<2>(im[j], w1.ih[i][j], w1.il[i][j]);
+            }
+        }
         FAcc acc;
         fx_zero(acc);
-        fx_mul_acc<N, N>(acc, q, um);
-        const FMat w1 = fx_round<kUnit>(acc);
-        fx_zero(acc);
-        fx_mul_acc<N, N, 2>(acc, q, w1);
+        fx_mul_acc<N, N, 2>(acc, fx_remainder(q), fx_remainder(w1));
         const FMat w2 = fx_round<kUnit, 1, 2>(acc);
 #pragma unroll
         for (int i = 0; i < 2; ++i)
@@ -227,22 +280,25 @@ __device__ __forceinline__ bool fx_link_step(const double x[8], double r[12])
                     t.v = mad_wide(sign < 0.f ? -c.h : c.h, h, t.v);
                     t.c = fmaf(sign * (float)c.h, l, fmaf(sign * c.l, (float)h, t.c));
                 };
-                add(re, g0, 1.f, um.rh[i][j], um.rl[i][j]);
-                add(re, m0, -1.f, um.ih[i][j], um.il[i][j]);
-                add(re, g1, 1.f, w1.rh[i][j], w1.rl[i][j]);
-                add(re, m1, -1.f, w1.ih[i][j], w1.il[i][j]);
+                const float url = 0x1p-28f * (float)u.rl[i][j], uil = 0x1p-28f * (float)u.il[i][j];
+                const float wrl = 0x1p-28f * (float)w1.rl[i][j], wil = 0x1p-28f * (float)w1.il[i][j];
+                add(re, g0, 1.f, u.rh[i][j], url);
+                add(re, m0, -1.f, u.ih[i][j], uil);
+                add(re, g1, 1.f, w1.rh[i][j], wrl);
                 add(re, g2, 1.f, w2.rh[i][j], w2.rl[i][j]);
                 add(re, m2, -1.f, w2.ih[i][j], w2.il[i][j]);
-                add(im, g0, 1.f, um.ih[i][j], um.il[i][j]);
-                add(im, m0, 1.f, um.rh[i][j], um.rl[i][j]);
-                add(im, g1, 1.f, w1.ih[i][j], w1.il[i][j]);
-                add(im, m1, 1.f, w1.rh[i][j], w1.rl[i][j]);
+                add(im, g0, 1.f, u.ih[i][j], uil);
+                add(im, m0, 1.f, u.rh[i][j], url);
+                add(im, g1, 1.f, w1.ih[i][j], wil);
                 add(im, g2, 1.f, w2.ih[i][j], w2.il[i][j]);
                 add(im, m2, 1.f, w2.rh[i][j], w2.rl[i][j]);
-                vr[i][j] = mad_wide(u.rh[i][j], 1 << 28, (long long)u.rl[i][j]) + ((re.v + 2) >> 2) +
-                           __float2int_rn(0.25f * re.c);
-                vi[i][j] = mad_wide(u.ih[i][j], 1 << 28, (long long)u.il[i][j]) + ((im.v + 2) >> 2) +
-                           __float2int_rn(0.25f * im.c);
+                long long lr = 0, li = 0;
+                fx_mad(re.v, lr, -m1.h, -m1.l, w1.ih[i][j], w1.il[i][j]);
+                fx_mad(im.v, li, m1.h, m1.l, w1.rh[i][j], w1.rl[i][j]);
+                er[i][j] = ((fx_value(re.v, lr) + 2) >> 2) + __float2int_rn(0.25f * re.c);
+                ei[i][j] = ((fx_value(im.v, li) + 2) >> 2) + __float2int_rn(0.25f * im.c);
+                vr[i][j] = mad_wide(u.rh[i][j], 1 << 28, (long long)u.rl[i][j]) + ((er[i][j] + half) >> tt);
+                vi[i][j] = mad_wide(u.ih[i][j], 1 << 28, (long long)u.il[i][j]) + ((ei[i][j] + half) >> tt);
             }
         if (rep + 1 >> s) break; // 2^s steps
 #pragma unroll
@@ -254,61 +310,47 @@ __device__ __forceinline__ bool fx_link_step(const double x[8], double r[12])
             }
         fx_row2(u);
     }
-    // Gram-Schmidt to first order in the departures (units 2^-60)
-    const auto limbs = [&](int i) {
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            fx_limbs<0>(vr[i][j], u.rh[i][j], u.rl[i][j]);
-            fx_limbs<0>(vi[i][j], u.ih[i][j], u.il[i][j]);
-        }
-    };
-    long long worst = 0;
-    const auto normalise = [&](int i) {
+    // Gram-Schmidt to first order in the departures.  Those of the lengths
+    // are whole numbers of 2^-60 ...
+    const auto departure = [&](int i) {
         long long h = 0, l = 0;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            fx_mad(h, l, u.rh[i][j], u.rl[i][j], u.rh[i][j], u.rl[i][j]);
-            fx_mad(h, l, u.ih[i][j], u.il[i][j], u.ih[i][j], u.il[i][j]);
+            const FxS a = fxs(vr[i][j]), b = fxs(vi[i][j]);
+            fx_mad(h, l, a.h, a.l, a.h, a.l);
+            fx_mad(h, l, b.h, b.l, b.h, b.l);
         }
-        const long long d = fx_value(h, l) - (1ll << 60);
-        worst = max(worst, llabs(d));
-        const int dd = (int)d; // u -= u d / 2
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            vr[i][j] -= mad_wide(u.rh[i][j], dd, 1ll << 32) >> 33;
-            vi[i][j] -= mad_wide(u.ih[i][j], dd, 1ll << 32) >> 33;
-        }
+        return fx_value(h, l) - (1ll << 60);
     };
-    limbs(0);
-    limbs(1);
-    normalise(0);
-    limbs(0);
-    {
-        // <row0, row1> = sum conj(u0) u1
-        long long rh = 0, rl = 0, ph = 0, pl = 0, mh = 0, ml = 0;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            fx_mad(rh, rl, u.rh[0][j], u.rl[0][j], u.rh[1][j], u.rl[1][j]);
-            fx_mad(rh, rl, u.ih[0][j], u.il[0][j], u.ih[1][j], u.il[1][j]);
-            fx_mad(ph, pl, u.rh[0][j], u.rl[0][j], u.ih[1][j], u.il[1][j]);
-            fx_mad(mh, ml, u.ih[0][j], u.il[0][j], u.rh[1][j], u.rl[1][j]);
-        }
-        const long long pr = fx_value(rh, rl), pi = fx_value(ph - mh, pl - ml);
-        worst = max(worst, max(llabs(pr), llabs(pi)));
-        const int r32 = (int)pr, i32 = (int)pi, n32 = -i32;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            vr[1][j] -= mad_wide(u.rh[0][j], r32, mad_wide(u.ih[0][j], n32, 1ll << 31)) >> 32;
-            vi[1][j] -= mad_wide(u.ih[0][j], r32, mad_wide(u.rh[0][j], i32, 1ll << 31)) >> 32;
-        }
-    }
-    limbs(1);
-    normalise(1);
-    if (worst >= 1ll << 30) return false;
+    const long long n0 = departure(0), n1 = departure(1);
+    if (llabs(n0) >= 1ll << 30 || llabs(n1) >= 1ll << 30) return false;
+    // ... and the product of the rows is taken in FP64, as the rows
+    // themselves: small entries keep their digits.  One step: the link as it
+    // was stored and its change; several: the link as a whole number.
+    double v[12];
+    const double unit = __hiloint2double((1023 - 58 - (s > 0 ? 0 : t)) << 20, 0);
 #pragma unroll
     for (int e = 0; e < 6; ++e) {
-        r[2 * e] = 0x1p-58 * (double)vr[e / 3][e % 3];
-        r[2 * e + 1] = 0x1p-58 * (double)vi[e / 3][e % 3];
+        const int i = e / 3, j = e % 3;
+        v[2 * e] = fma((double)(s > 0 ? vr[i][j] : er[i][j]), unit, s > 0 ? 0.0 : r[2 * e]);
+        v[2 * e + 1] = fma((double)(s > 0 ? vi[i][j] : ei[i][j]), unit, s > 0 ? 0.0 : r[2 * e + 1]);
+    }
+    double pr = 0.0, pi = 0.0; // <row0, row1> = sum conj(u0) u1
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const double a = v[2 * j], b = v[2 * j + 1], c = v[6 + 2 * j], d = v[7 + 2 * j];
+        pr = fma(a, c, fma(b, d, pr));
+        pi = fma(a, d, fma(-b, c, pi));
+    }
+    if (exponent_of(pr) >= 1023 - 30 || exponent_of(pi) >= 1023 - 30) return false;
+    const double f0 = -0x1p-61 * (double)(int)n0, f1 = -0x1p-61 * (double)(int)n1;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const double a = v[2 * j], b = v[2 * j + 1], c = v[6 + 2 * j], d = v[7 + 2 * j];
+        r[6 + 2 * j] = fma(-pr, a, fma(pi, b, fma(f1, c, c)));
+        r[7 + 2 * j] = fma(-pr, b, fma(-pi, a, fma(f1, d, d)));
+        r[2 * j] = fma(f0, a, a);
+        r[2 * j + 1] = fma(f0, b, b);
     }
     return true;
 }

@@ -129,9 +129,9 @@ __device__ __forceinline__ void update_link(double *__restrict__ links, const do
     }
 }
 
-// Threads of an FP64 link-step block and resident blocks (18x14x22x36: 153 us
-// with 2 blocks of 192, 157 with 3 of 128, 170 with 2 of 128).
-constexpr int kFxStepBlock = 192, kFxStepBlocks = 2;
+// Threads of an FP64 link-step block and resident blocks (18x14x22x36, dt 0.05:
+// 200 us with 3 blocks of 128, 203 with 4 of 128, 210 with 2 of 192).
+constexpr int kFxStepBlock = 128, kFxStepBlocks = 3;
 
 // The link and algebra planes share the site index.
 template <bool FROM_UNIT>

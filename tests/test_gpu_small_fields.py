@@ -1,0 +1,110 @@
+"""FP64 calls on fields with entries of very different sizes: links near 1 or
+near a subgroup of SU(3), steps of any size, spinors whose components differ
+by many orders.  Errors are taken against the size of the entries themselves,
+class by class, not against the largest of the field.
+
+References in long double (80 or 128 bits), from the stored FP64 inputs."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1808_02281_gb300 import build as B
+from paper_1808_02281_gb300 import lqcd, synth
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+DIMS = (3, 4, 2, 5)
+LD, CLD = np.longdouble, np.clongdouble
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _library():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    B.build()
+
+
+def _mm(a, b):
+    return (a[..., :, :, None] * b[..., None, :, :]).sum(-2)
+
+
+def _exp(omega):
+    """exp(i omega.T), T_a = lambda_a / 2, by its series with 6 squarings."""
+    lam = H.gell_mann().astype(CLD)
+    lam[7] = np.diag([1, 1, -2]) / np.sqrt(LD(3))
+    x = np.einsum("...a,aij->...ij", omega.astype(LD), lam) * CLD(1j) / 128
+    one = np.broadcast_to(np.eye(3, dtype=CLD), x.shape)
+    r = one + x / 24
+    for k in range(23, 0, -1):
+        r = _mm(x, r) / LD(k) + one
+    for _ in range(6):
+        r = _mm(r, r)
+    return r
+
+
+def _third(U):
+    U = U.astype(CLD)
+    U[..., 2, :] = np.conj(np.cross(U[..., 0, :], U[..., 1, :]))
+    return U
+
+
+def _gram_schmidt(U):
+    a, b = U[..., 0, :], U[..., 1, :]
+    a = a / np.sqrt((a * a.conj()).real.sum(-1, keepdims=True))
+    b = b - (a.conj() * b).sum(-1, keepdims=True) * a
+    b = b / np.sqrt((b * b.conj()).real.sum(-1, keepdims=True))
+    return np.stack([a, b], -2)
+
+
+def _omega(kind, sigma, seed):
+    """Normal components of size sigma; kind "ab", "su2" or "so3": those of the
+    subgroup of size 0.5 (diagonal links, an SU(2) block, real rotations)."""
+    o = synth.momenta(DIMS, seed) * sigma
+    for a in {"": (), "ab": (2, 7), "su2": (0, 1, 2), "so3": (1, 4, 6)}[kind]:
+        o[..., a] = synth.momenta(DIMS, seed + 50)[..., a] * 0.5
+    return o
+
+
+def _links(lat, U):
+    return lqcd.pack_links(lat, lqcd.full_to_device(lat, U))
+
+
+def _rows(links):
+    """Rows 0, 1 of the stored links [4, 6, V, 2] as [V, 4, 2, 3]."""
+    x = links.cpu().numpy().transpose(2, 0, 1, 3)
+    return (x[..., 0] + 1j * x[..., 1]).reshape(x.shape[0], 4, 2, 3)
+
+
+def _check_classes(got, want, tol):
+    """Every real of the trailing axes against the largest of its kind in the field."""
+    for part in (np.real, np.imag) if np.iscomplexobj(want) else (np.asarray,):
+        g, w = part(got).astype(LD), part(want)
+        size = np.abs(w).max(0)
+        assert (np.abs(g - w).max(0) <= tol * size + 1e-300).all(), (np.abs(g - w).max(0) / (size + 1e-300)).max()
+
+
+# A floating-point step is some 30 roundings of 1.1e-16; the fixed-point one
+# a few.  4e-15 of the largest entry of a class holds for both.
+@pytest.mark.parametrize("kind, sigma, step", [
+    ("", 0.3, 1e-6), ("", 1e-2, 0.05), ("", 1e-2, 1e-2), ("", 1e-4, 1e-4), ("", 1e-8, 1e-8), ("", 1e-8, 1e-3), ("", 1e-3, 1e-12),
+    ("", 0.0, 1e-12), ("", 0.0, 1e-18), ("", 0.0, 1e-200), ("", 1e-8, 0.6), ("ab", 1e-8, 0.05), ("ab", 1e-8, 1e-9),
+    ("su2", 1e-8, 1e-9), ("so3", 1e-8, 1e-6)])
+def test_link_step_of_small_entries(kind, sigma, step):
+    lat = lqcd.Lattice.symanzik(DIMS, 6.0, 0.87, "f64")
+    links = _links(lat, _exp(_omega(kind, sigma, 3)).astype(complex))
+    U = _third(np.concatenate([_rows(links), np.zeros((lat.V, 4, 1, 3))], -2))
+    p = synth.momenta(DIMS, 4)
+    lqcd.md_update_links(lat, links, lqcd.algebra_to_device(lat, p), step)
+    want = _gram_schmidt(_mm(_exp(p * step), U)[..., :2, :])  # p dt in FP64, as the step takes it
+    _check_classes(_rows(links), want, 4e-15)
+
+
+@pytest.mark.parametrize("kind", ["", "ab", "su2", "so3"])
+@pytest.mark.parametrize("sigma", [1.0, 0.05, 1e-3, 1e-8, 1e-16, 1e-30])
+def test_links_from_small_omega(kind, sigma):
+    """Also exponents of a subgroup with small components beside it."""
+    lat = lqcd.Lattice.symanzik(DIMS, 6.0, 0.87, "f64")
+    omega = _omega(kind, sigma, 7)
+    links = lqcd.links_from_omega(lat, lqcd.algebra_to_device(lat, omega))
+    _check_classes(_rows(links), _gram_schmidt(_exp(omega)[..., :2, :]), 4e-15)
