@@ -443,4 +443,29 @@ __device__ __forceinline__ bool fx_limbs_of_rows(const double r[12], FLimbs &u)
 
 template <typename M> __device__ __forceinline__ bool fx_poisoned(const M &m) { return m.rh[0][0] == kPoison; }
 
+// Matrices near 1 or near a subgroup of SU(3) have small entries that count by
+// themselves, and the fixed point keeps only an absolute precision: at least
+// kSmallMost of the 18 reals are below 2^-5, or kSmallSome below 2^-7 (15 of 18
+// are small near 1, 12 near diagonal matrices, 9 or 8 near the real ones and an
+// SU(2) or U(2) block).
+constexpr int kSmallMost = 13, kSmallSome = 8, kSmallMostBits = 5, kSmallSomeBits = 7;
+
+// The number of reals below 2^-BITS.
+template <int BITS> __device__ __forceinline__ int fx_small(const FLimbs &u)
+{
+    constexpr int c = 1 << (kUnit - BITS);
+    int n = 0;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        n += (unsigned)(u.rh[e / 3][e % 3] + c) < 2u * c;
+        n += (unsigned)(u.ih[e / 3][e % 3] + c) < 2u * c;
+    }
+    return n;
+}
+
+__device__ __forceinline__ bool fx_near_subgroup(const FLimbs &u)
+{
+    return fx_small<kSmallMostBits>(u) >= kSmallMost || fx_small<kSmallSomeBits>(u) >= kSmallSome;
+}
+
 } // namespace lqcd

@@ -10,6 +10,17 @@
 // A thread that reads a marked matrix (a link that is not finite or not
 // within 1e-3 of SU(3), or a staple of one) computes its staple or force in
 // floating point from the stored links instead.
+//
+// The force of links near 1, or near a subgroup, is made of small entries, and
+// whole numbers of 2^-58 keep too little of them: rms error against extended
+// precision, of the force's own size (U = exp(i w), w normal, u0 0.87), 1.1 to
+// 1.9e-16 for w of 1 to 0.1, 3.4e-16 at 0.05, below that 1.6e-17 / w; in
+// floating point 3.1 to 4e-16 for all w.  So where a quarter of the links of 32
+// sites, in each direction, are near a subgroup (fx_near_subgroup; or have no
+// fixed-point form) the lattice's flag is set and the other two passes run in
+// floating point, on planes of FP64 staples: the whole lattice, for warps of
+// which some lanes did one and some the other take up to three times as long.
+// 24^3x48: 5.5 ms, in floating point 34.3.
 #include "async_copy.cuh"
 #include "fx_planes.cuh"
 #include "sf_common.cuh"
@@ -75,13 +86,19 @@ FxScalars make_fx_scalars(const KernelScalars &sc)
 
 // ------------------------------------------------------------------ links
 
+// Whether the lattice is computed in floating point.
+__device__ __forceinline__ bool floating(const SfLattice &L) { return *L.flag & L.bit; }
+
 __device__ __forceinline__ void links_block(const SfLattice &L, int V, int vb)
 {
     const int mu = (int)(threadIdx.x >> 5);
     const int x = vb * 32 + (int)(threadIdx.x & 31);
-    if (x >= V) return;
+    const FLimbs u = fx_load_link(static_cast<const double *>(L.links), V, mu, x < V ? x : V - 1);
     const FxPlanes sf = fx_planes(L);
-    sf.store(sf.at(x), kLinkPlane + mu, fx_load_link(static_cast<const double *>(L.links), V, mu, x));
+    if (x < V) sf.store(sf.at(x), kLinkPlane + mu, u);
+    const int n = __popc(__ballot_sync(0xffffffffu, fx_poisoned(u) || fx_near_subgroup(u)));
+    if (__syncthreads_and(n >= 8) && threadIdx.x == 0 && !(*(volatile unsigned long long *)L.flag & L.bit))
+        atomicOr(L.flag, L.bit);
 }
 
 __global__ void __launch_bounds__(kBlock) links_fx(const __grid_constant__ SfLattice L)
@@ -112,12 +129,44 @@ template <int FA, int FB> __device__ __forceinline__ FLimbs fx_mul_top2(const FL
     return fx_round<FA == FB ? 1 : -1, 2>(y);
 }
 
+// Staple plane `plane` of site x in floating point, from the stored links.
+__device__ __forceinline__ Mat<double> direct_staple(const double *links, const G32 &g, const Coord &c, int x, int plane)
+{
+    const int mu = plane / 6, j = plane - 6 * mu, nu = (mu + 1 + (j >> 1)) & 3;
+    const int64_t V = g.V;
+    const int xm = x + step32(g, c, mu, 1);
+    Mat<double> s;
+    if ((j & 1) == 0) {
+        const int vp = step32(g, c, nu, 1);
+        const Mat<double> t = mul<N, D>(load_link(links, V, nu, xm), load_link(links, V, mu, x + vp));
+        s = mul_top2<N, D>(t, load_link(links, V, nu, x));
+    } else {
+        const int vm = step32(g, c, nu, -1);
+        const Mat<double> t = mul<D, D>(load_link(links, V, nu, xm + vm), load_link(links, V, mu, x + vm));
+        s = mul_top2<N, N>(t, load_link(links, V, nu, x + vm));
+    }
+    rebuild_row2(s);
+    return s;
+}
+
+// Staples j0 to j1 - 1 of direction mu at site x in floating point.
+__device__ __noinline__ void staples_floating(const SfLattice &L, int x, int mu, int j0, int j1)
+{
+    const G32 g = make_g32(L.dims);
+    const Coord c = coord32(g, L.div, x);
+    const FxPlanes sf = fx_planes(L);
+#pragma unroll 1
+    for (int j = j0; j < j1; ++j)
+        sf.store(sf.at(x), mu * 6 + j, direct_staple(static_cast<const double *>(L.links), g, c, x, mu * 6 + j));
+}
+
 // Staples j0 to j1 - 1 of each direction.
 __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, int vb, int j0, int j1)
 {
     const int mu = (int)(threadIdx.x >> 5);
     const int x = vb * 32 + (int)(threadIdx.x & 31);
     if (x >= g.V) return;
+    if (floating(L)) return staples_floating(L, x, mu, j0, j1);
     const Coord c = coord32(g, L.div, x);
     const FxPlanes sf = fx_planes(L);
     const int xm = x + step32(g, c, mu, 1); // x + mu
@@ -181,23 +230,16 @@ struct DirectStaples {
 
     __device__ Mat<double> load(int x, int plane) const
     {
-        const int mu = plane / 6, j = plane - 6 * mu, nu = (mu + 1 + (j >> 1)) & 3;
-        const Coord c = coord32(*g, div, x);
-        const int64_t V = g->V;
-        const int xm = x + step32(*g, c, mu, 1);
-        Mat<double> s;
-        if ((j & 1) == 0) {
-            const int vp = step32(*g, c, nu, 1);
-            const Mat<double> t = mul<N, D>(load_link(links, V, nu, xm), load_link(links, V, mu, x + vp));
-            s = mul_top2<N, D>(t, load_link(links, V, nu, x));
-        } else {
-            const int vm = step32(*g, c, nu, -1);
-            const Mat<double> t = mul<D, D>(load_link(links, V, nu, xm + vm), load_link(links, V, mu, x + vm));
-            s = mul_top2<N, N>(t, load_link(links, V, nu, x + vm));
-        }
-        rebuild_row2(s);
-        return s;
+        return direct_staple(links, *g, coord32(*g, div, x), x, plane);
     }
+};
+
+// Staples from FP64 planes.
+struct FloatingStaples {
+    FxPlanes sf;
+
+    __device__ __forceinline__ const char *at(int n) const { return sf.at(n); }
+    __device__ __forceinline__ Mat<double> load(const char *r, int plane) const { return sf.floating(r, plane); }
 };
 
 template <bool ACTION>
@@ -208,6 +250,16 @@ __device__ __noinline__ double force_link_floating(const SfLattice &L, const Ker
     const LatticeSites si{&g, &c, k};
     const DirectStaples sf{static_cast<const double *>(L.links), &g, L.div};
     return force_link<double, ACTION, false, true>(L, sc, g, sf, si, c, k, rho);
+}
+
+// Of a lattice in floating point.
+template <bool ACTION>
+__device__ __noinline__ double force_link_of_planes(const SfLattice &L, const KernelScalars &sc, int k, int rho)
+{
+    const G32 g = make_g32(L.dims);
+    const Coord c = coord32(g, L.div, k);
+    const LatticeSites si{&g, &c, k};
+    return force_link<double, ACTION, false, true>(L, sc, g, FloatingStaples{fx_planes(L)}, si, c, k, rho);
 }
 
 // Where a group of products (fx_group) of a link reads: its left factors at
@@ -465,6 +517,7 @@ __device__ __forceinline__ double fx_force_block(const SfLattice &L, const Kerne
     if (j >= g.V) return 0.0;
     const Coord c = swept_site(sw, j);
     const int k = index32(g, c);
+    if (floating(L)) return force_link_of_planes<ACTION>(L, sc, k, rho);
     const FxPlanes sf = fx_planes(L);
     bool bad = false;
     fx_fetch(slot, sf, fx_group_of(sf, g, c, rho, k, 0), rho, 0);
@@ -531,6 +584,15 @@ __global__ void __launch_bounds__(kSplitBlock, 1)
     const Coord c = swept_site(sw, j < g.V ? j : g.V - 1);
     const int k = index32(g, c);
     const FxPlanes sf = fx_planes(L);
+    if (floating(L)) {
+        if (grp > 0) return;
+        double share = j < g.V ? force_link_of_planes<ACTION>(L, sc, k, rho) : 0.0;
+        if constexpr (ACTION) {
+            share = warp_sum(share);
+            if (lane == 0) L.partials[vb * 4 + rho] = share;
+        }
+        return;
+    }
     longlong2 z[9];
     bool bad = false;
     fx_group<false>(z, bad, sf, fx, g, c, rho, k, grp, nullptr);
@@ -584,8 +646,10 @@ cudaError_t launch_fx_passes(const SfLattice &L, const KernelScalars &sc, bool a
 {
     const unsigned grid = grid_of(virtual_blocks((int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3]));
     const FxScalars fx = make_fx_scalars(sc);
+    cudaError_t e = cudaMemsetAsync(L.flag, 0, sizeof *L.flag, st);
+    if (e != cudaSuccess) return e;
     links_fx<<<grid, kBlock, 0, st>>>(L);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     staples_fx<<<L.split ? 6 * grid : grid, kBlock, 0, st>>>(L);
     e = cudaGetLastError();

@@ -553,12 +553,13 @@ cudaError_t launch_passes_batched(const SfBatch &B, const KernelScalars &sc, int
 
 // FP32: room for the 24 planes in the larger (full, 18-real, in blocks of 32
 // sites) of the two storage forms, so that every schedule fits the same
-// workspace.  FP64: the 24 planes and the 4 planes of the links, in limbs.
+// workspace.  FP64: the 24 planes, the 4 planes of the links in limbs, and the
+// flag.
 size_t staple_field_bytes(const int dims[4], int precision)
 {
     const int64_t V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
     const size_t planes = precision == LQCD_F64 ? fx_planes_count() : kStaplePlanes;
-    return round_up256(planes * full_plane_bytes(V, precision));
+    return round_up256(planes * full_plane_bytes(V, precision)) + (precision == LQCD_F64 ? 256 : 0);
 }
 
 bool staple_fields_supported(const int dims[4])
@@ -589,6 +590,10 @@ cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
     L.action = a.action;
     const KernelScalars sc = make_scalars(a);
     const bool action = a.action != nullptr;
+    if (a.precision == LQCD_F64) {
+        L.flag = reinterpret_cast<unsigned long long *>(static_cast<char *>(a.staples) + fx_planes_count() * L.plane_bytes);
+        L.bit = 1;
+    }
     const cudaError_t e = a.precision == LQCD_F64 ? launch_fx_passes(L, sc, action, st)
                                                   : launch_passes(L, sc, variant, action, st);
     if (e != cudaSuccess || !action) return e;
@@ -611,12 +616,14 @@ cudaError_t launch_force_staple_fields_batched(const ForceArgs &a, int n, const 
         set_traversal(B.e[c], variant);
         B.e[c].plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
         B.e[c].split = split_lattice(V) && (a.precision == LQCD_F64 || full_staples(variant));
+        B.e[c].flag = counter + 3;
+        B.e[c].bit = 1ull << c;
         B.e[c].vb_begin = B.total;
         B.total += virtual_blocks(V);
         any_action = any_action || B.e[c].action != nullptr;
     }
     const KernelScalars sc = make_scalars(a);
-    cudaError_t e = cudaMemsetAsync(counter, 0, 3 * sizeof(unsigned long long), st);
+    cudaError_t e = cudaMemsetAsync(counter, 0, 4 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     e = a.precision == LQCD_F64 ? launch_fx_passes_batched(B, sc, any_action, st)
                                 : launch_passes_batched(B, sc, variant, any_action, st);

@@ -1,7 +1,7 @@
-// Planes of 3x3 matrices in the fixed-point forms of fixed.cuh, in blocks of
-// 32 consecutive sites: 16 bytes for a complex entry (h, l of its real and
-// imaginary part), entry e = 3 i + j of site s at e*512 + s*16 bytes of the
-// block, plane P of a field at P * plane_bytes.
+// Planes of 3x3 matrices in the fixed-point forms of fixed.cuh or in FP64, in
+// blocks of 32 consecutive sites: 16 bytes for a complex entry (h, l of its real
+// and imaginary part, or the two parts), entry e = 3 i + j of site s at
+// e*512 + s*16 bytes of the block, plane P of a field at P * plane_bytes.
 #pragma once
 
 #include "fixed.cuh"
@@ -111,6 +111,27 @@ struct FxPlanes {
 #pragma unroll
         for (int e = 0; e < 9; ++e)
             p[e * S] = make_int4(u.rh[e / 3][e % 3], u.rl[e / 3][e % 3], u.ih[e / 3][e % 3], u.il[e / 3][e % 3]);
+    }
+
+    // A matrix in FP64.
+    __device__ __forceinline__ Mat<double> floating(const char *r, int plane) const
+    {
+        const double2 *p = reinterpret_cast<const double2 *>(ptr(r, plane));
+        Mat<double> u;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const double2 v = __ldg(p + e * S);
+            u.re[e / 3][e % 3] = v.x;
+            u.im[e / 3][e % 3] = v.y;
+        }
+        return u;
+    }
+
+    __device__ __forceinline__ void store(char *r, int plane, const Mat<double> &u) const
+    {
+        double2 *p = reinterpret_cast<double2 *>(const_cast<int4 *>(ptr(r, plane)));
+#pragma unroll
+        for (int e = 0; e < 9; ++e) __stcs(p + e * S, make_double2(u.re[e / 3][e % 3], u.im[e / 3][e % 3]));
     }
 
     template <bool STREAM> __device__ __forceinline__ void store(char *r, int plane, const FMat &u) const

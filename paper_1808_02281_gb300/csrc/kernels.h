@@ -97,6 +97,9 @@ struct SfLattice {
     int64_t plane_bytes; // full staple planes: bytes of one plane
     const void *links;
     void *staples;     // 24 staple planes (FP64: and 4 link planes; workspace)
+    // FP64: `bit` of *flag is set by the first pass where the field wants
+    // floating point
+    unsigned long long *flag, bit;
     void *force;       // written when set
     void *mom;         // p += dt f when set
     double *partials;  // one action partial per virtual block, or four
@@ -108,7 +111,7 @@ constexpr int kMaxBatch = 64;
 struct SfBatch {
     int n;
     int64_t total;                 // virtual blocks of all lattices
-    unsigned long long *counter;   // work counters (3, zeroed before the passes)
+    unsigned long long *counter;   // 3 work counters and the flags of 64 lattices, zeroed before the passes
     SfLattice e[kMaxBatch];
 };
 

@@ -3,14 +3,17 @@ near a subgroup of SU(3), steps of any size, spinors whose components differ
 by many orders.  Errors are taken against the size of the entries themselves,
 class by class, not against the largest of the field.
 
-References in long double (80 or 128 bits), from the stored FP64 inputs."""
+References from the stored FP64 inputs: the link steps in long double (80 or
+128 bits), the others in floating point, which keeps small entries."""
 import numpy as np
 import pytest
 import torch
 
+from oracle import oracle as O
 from paper_1808_02281_gb300 import build as B
 from paper_1808_02281_gb300 import lqcd, synth
 from tests import helpers as H
+from tests.test_gpu_fixed_point import _force as staple_force, _third as _third64
 
 pytestmark = pytest.mark.gpu
 
@@ -108,3 +111,53 @@ def test_links_from_small_omega(kind, sigma):
     omega = _omega(kind, sigma, 7)
     links = lqcd.links_from_omega(lat, lqcd.algebra_to_device(lat, omega))
     _check_classes(_rows(links), _gram_schmidt(_exp(omega)[..., :2, :]), 4e-15)
+
+
+def _field(dims, kind, sigma, seed):
+    V = int(np.prod(dims))
+    o = synth.momenta(dims, seed) * sigma
+    for a in {"ab": (2, 7), "u2": (0, 1, 2, 7), "so3": (1, 4, 6)}.get(kind, ()):
+        o[..., a] = synth.momenta(dims, seed + 50)[..., a] * 0.5
+    if kind in ("scaled", "block", "temporal"):
+        o = synth.momenta(dims, seed + 50) * 0.4
+    if kind == "block":       # 32 sites of small links in a field of large ones
+        o[32:64] = synth.momenta(dims, seed)[32:64] * sigma
+    U = _third64(O.links_from_omega(o).reshape(V, 4, 3, 3))
+    if kind == "scaled":      # no link within 1e-3 of SU(3)
+        U = _third64(U * 1.01)
+    if kind == "temporal":    # one direction of unit links
+        U[:, 3] = np.eye(3)
+    return U
+
+
+# (16, 8, 8, 5) is above the size up to which a link's sums are split over warps.
+# Up to some 1000 roundings of terms of the size of the force: 1e-14 of the
+# largest of a component.  Fields that are not small: 1e-13 of the largest of all.
+@pytest.mark.parametrize("dims", [(3, 4, 2, 5), (16, 8, 8, 5)])
+@pytest.mark.parametrize("kind, sigma", [("", 0.0), ("", 1e-2), ("", 1e-4), ("", 1e-8), ("", 1e-20), ("ab", 1e-8), ("u2", 1e-6),
+                                         ("so3", 1e-8), ("scaled", 0.0), ("block", 1e-8), ("temporal", 0.0)])
+def test_force_of_small_entries(dims, kind, sigma):
+    lat = lqcd.Lattice.symanzik(dims, 6.0, 0.87, "f64", force_algo=lqcd.FORCE_STAPLE_FIELDS)
+    U = _field(dims, kind, sigma, 5)
+    links = _links(lat, U)
+    want = staple_force(U, dims, 6.0, O.coefficients(0.87))
+    p = synth.momenta(dims, 6) * (sigma or 1.0)
+    mom, force, S = lqcd.algebra_to_device(lat, p), lqcd.empty_algebra(lat), torch.empty((), dtype=torch.float64, device="cuda")
+    lqcd.md_force_step(lat, links, force=force, mom=mom, dt=0.5, action=S)
+    got = lqcd.algebra_from_device(force)
+    if kind in ("scaled", "block", "temporal"):
+        assert np.abs(got - want).max() <= 1e-13 * np.abs(want).max()
+    else:
+        _check_classes(got, want, 1e-14)
+    q = p + 0.5 * got
+    assert np.abs(lqcd.algebra_from_device(mom) - q).max() <= 2.3e-16 * np.abs(q).max()
+    if kind != "scaled":   # 34 loops a site, each to 1e-15, under the prefactor 2
+        want = O.gauge_action(dims, U, 6.0, O.coefficients(0.87))
+        assert abs(float(S.item()) - want) <= 68e-15 * lat.V
+    # in a batch with a lattice of large links: the same bits, and those of the other too
+    other = lat.with_(dims=(5, 4, 3, 4))
+    big = lqcd.links_from_omega(other, lqcd.algebra_to_device(other, synth.omega(other.dims, 0.4, 8)))
+    fs, actions = [lqcd.empty_algebra(lat), lqcd.empty_algebra(other)], torch.empty(2, dtype=torch.float64, device="cuda")
+    lqcd.md_force_step_batched(lat, [dims, other.dims], [links, big], force=fs, actions=actions)
+    assert torch.equal(fs[0], force) and float(actions[0]) == float(S)
+    assert torch.equal(fs[1], lqcd.gauge_force(other, big))
