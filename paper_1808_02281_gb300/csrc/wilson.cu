@@ -524,9 +524,23 @@ struct FHalf {
     int rh[2][3], rl[2][3], ih[2][3], il[2][3];
 };
 
+// What the fixed point loses, and how it is seen.  A spinor's reals are known
+// to 2^-58 of the largest, so a result made of much smaller ones only (colours
+// or spin rows that nothing mixes in: links near 1 or diagonal) would have lost
+// its digits.  Such results are themselves small: where a complex one is below
+// 2^-kPairBits of the scale of its spinors, or kFewReals of a site's 24 reals
+// (a spin row, a colour) or kFewComponents of a force's 8 (a colour) below
+// 2^-kRealBits or 2^-kComponentBits, the site or link is computed in floating
+// point.  Of normal spinors on normal links that is one in a million: a single
+// one among the last blocks of a small lattice costs 20 us.
+constexpr int kPairBits = 12, kRealBits = 6, kFewReals = 6, kComponentBits = 7, kFewComponents = 4;
+
+// Exponent field that stands for the scale of a spinor of zeros.
+constexpr int kZeroScale = 64;
+
 // Rows 0 and 1 of (1 + s gamma_mu) x_n, mu at run time, over 2^(e - 1022) with
-// e the largest exponent field of the spinor's 24 reals; false where that is
-// out of range (the scales of two spinors are multiplied) or not finite.
+// e the largest exponent field of the spinor's 24 reals; false where that is out
+// of range (the scales of two spinors are multiplied) or not finite.
 __device__ __forceinline__ bool fx_half(const double *__restrict__ x, int64_t V, int64_t n, int mu, bool minus, FHalf &h,
                                         int &e)
 {
@@ -547,13 +561,13 @@ __device__ __forceinline__ bool fx_half(const double *__restrict__ x, int64_t V,
     e = 0;
 #pragma unroll
     for (int q = 0; q < 12; ++q) e = max(e, max(exponent_of(v[q].x), exponent_of(v[q].y)));
-    if (e < 64 || e > 1900) {
+    if (e <= kZeroScale || e > 1900) {
         if (e != 0) return false;
         bool zero = true; // and no subnormals
 #pragma unroll
         for (int q = 0; q < 12; ++q) zero = zero && v[q].x == 0.0 && v[q].y == 0.0;
         if (!zero) return false;
-        e = 64;
+        e = kZeroScale;
     }
     const int shift = e - 1022;
 #pragma unroll
@@ -639,6 +653,7 @@ __device__ __forceinline__ bool hopping_force_fx(const WilsonArgs &a, int64_t V,
             us[e * kForceBlock] = make_int4(u.rh[e / 3][e % 3], u.rl[e / 3][e % 3], u.ih[e / 3][e % 3], u.il[e / 3][e % 3]);
     }
     double f[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    int scale = 0; // largest sum of the exponent fields of two spinors
 #pragma unroll 1
     for (int t = 0; t < 2; ++t) {
         const double *s0 = static_cast<const double *>(t == 0 ? a.x : a.y), *s1 = static_cast<const double *>(t == 0 ? a.y : a.x);
@@ -657,7 +672,16 @@ __device__ __forceinline__ bool hopping_force_fx(const WilsonArgs &a, int64_t V,
             }
             fx_colour_mul(u, p);
         }
+        // a small colour is a small row of the product: a field of such leaves here
+        bool thin = false;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            constexpr unsigned c = 1u << (27 - kComponentBits);
+            thin = thin || (p.rh[0][i] + c < 2 * c && p.ih[0][i] + c < 2 * c && p.rh[1][i] + c < 2 * c && p.ih[1][i] + c < 2 * c);
+        }
+        if (thin && ep > kZeroScale) return false;
         if (!fx_half(s1, V, k, rho, t == 0, q, eq)) return false;
+        if (ep > kZeroScale && eq > kZeroScale) scale = max(scale, ep + eq);
         long long re[3][3], im[3][3]; // N, units 2^-56 of the two scales
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -688,6 +712,13 @@ __device__ __forceinline__ bool hopping_force_fx(const WilsonArgs &a, int64_t V,
         f[6] = fma(s * (double)(re[1][2] - re[2][1]), w, f[6]);
         f[7] = fma(s * 0.57735026918962576451 * (double)(im[0][0] + im[1][1] - 2 * im[2][2]), w, f[7]);
     }
+    // small results (the diagonal components go together)
+    const int top = exponent_of(a.coef) + scale - 2044;
+    int reals = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) reals += exponent_of(f[q]) < top - kComponentBits;
+    const auto small = [&](int i, int j) { return max(exponent_of(f[i]), exponent_of(f[j])) < top - kPairBits; };
+    if (scale > 0 && (reals >= kFewComponents || small(0, 1) || small(3, 4) || small(5, 6) || small(2, 7))) return false;
     finish_force(a, V, rho, k, f);
     return true;
 }
@@ -790,6 +821,25 @@ __device__ __noinline__ void dslash_site_floating(const WilsonArgs &a, const Sit
     store_dslash(a, x, (int64_t)g.V, (int64_t)n, acc, a.ca, a.cb);
 }
 
+// Whether spinor n has a colour or three spin rows below 2^-kRealBits of the
+// largest: a site of a field of such is left before any work (1.5 % of the
+// time of any other).
+__device__ __forceinline__ bool uneven_spinor(const double *__restrict__ x, int64_t V, int64_t n)
+{
+    const double2 *p = reinterpret_cast<const double2 *>(x) + n;
+    int row[4] = {0, 0, 0, 0}, col[3] = {0, 0, 0};
+#pragma unroll
+    for (int q = 0; q < 12; ++q) {
+        const double2 v = __ldg(p + q * V);
+        const int e = max(exponent_of(v.x), exponent_of(v.y));
+        row[q / 3] = max(row[q / 3], e);
+        col[q % 3] = max(col[q % 3], e);
+    }
+    const int least = max(col[0], max(col[1], col[2])) - kRealBits;
+    return min(col[0], min(col[1], col[2])) < least ||
+           (row[0] < least) + (row[1] < least) + (row[2] < least) + (row[3] < least) >= 3;
+}
+
 // The same in fixed point (hopping_force_fx): the eight hops in one loop, the
 // direction and sign at run time; every neighbour's half spinor in its own
 // scale, the sum in whole numbers of 2^-56 of the largest scale so far.
@@ -798,10 +848,23 @@ __device__ __forceinline__ bool dslash_site_fx(const WilsonArgs &a, const Sites<
 {
     const double *__restrict__ x = static_cast<const double *>(a.x);
     const int64_t V = g.V;
+    if (uneven_spinor(x, V, (int64_t)n)) return false;
     long long sr[12], si[12]; // spin rows 0 to 3, colours 0 to 2
 #pragma unroll
     for (int q = 0; q < 12; ++q) sr[q] = si[q] = 0;
     int scale = 0; // exponent field of the sum's scale
+    // whether a complex result is small, or kFewReals real ones
+    const auto small = [&] {
+        constexpr int cp = 1 << (24 - kPairBits), cr = 1 << (24 - kRealBits);
+        int pairs = 0, reals = 0;
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+            const unsigned r = (unsigned)(int)(sr[q] >> 32), i = (unsigned)(int)(si[q] >> 32);
+            pairs += r + cp < 2u * cp && i + cp < 2u * cp;
+            reals += (r + cr < 2u * cr) + (i + cr < 2u * cr);
+        }
+        return scale > kZeroScale && (pairs > 0 || reals >= kFewReals);
+    };
 #pragma unroll 1
     for (int t = 0; t < 8; ++t) {
         const int mu = t >> 1;
@@ -863,6 +926,7 @@ __device__ __forceinline__ bool dslash_site_fx(const WilsonArgs &a, const Sites<
             }
         }
     }
+    if (small()) return false;
     Spinor<double> acc;
     const double s = 0x1p-56 * __hiloint2double((scale + 1) << 20, 0); // 2^-56 of 2^(scale - 1022)
 #pragma unroll
@@ -874,8 +938,9 @@ __device__ __forceinline__ bool dslash_site_fx(const WilsonArgs &a, const Sites<
     return true;
 }
 
-// 2117 -> 715 us at 32^4, 320 -> 117 at 20x18x14x30; error against extended
-// precision 6.0e-17 where it was 9.0e-17.
+// 32^4: 747 us, 20x18x14x30: 134; in floating point 2153 and 353 (what
+// uneven_spinor finds 2221).  Error against extended precision 6.0e-17, in
+// floating point 9.0e-17.
 template <typename I>
 __global__ void __launch_bounds__(kDslashBlock, 3) wilson_dslash_fx(const __grid_constant__ WilsonArgs a)
 {

@@ -161,3 +161,61 @@ def test_force_of_small_entries(dims, kind, sigma):
     lqcd.md_force_step_batched(lat, [dims, other.dims], [links, big], force=fs, actions=actions)
     assert torch.equal(fs[0], force) and float(actions[0]) == float(S)
     assert torch.equal(fs[1], lqcd.gauge_force(other, big))
+
+
+# Of a spinor: the colour, the spin rows, the complex entries or the parts that
+# are small, by a factor eps
+SMALL = {"colour": lambda x, e: x.__setitem__((slice(None), slice(None), 1), x[:, :, 1] * e),
+         "colours": lambda x, e: x.__setitem__((slice(None), slice(None), 2), x[:, :, 2] * e * e) or
+         x.__setitem__((slice(None), slice(None), 0), x[:, :, 0] * e),
+         "rows": lambda x, e: x.__setitem__((slice(None), slice(1, None)), x[:, 1:] * e),
+         "row": lambda x, e: x.__setitem__((slice(None), 2), x[:, 2] * e),
+         "point": lambda x, e: x.__setitem__(slice(1, None), x[1:] * e) or x.__setitem__((0, slice(1, None)), x[0, 1:] * e),
+         "entry": lambda x, e: x.__setitem__((slice(None), slice(1, None), 0), x[:, 1:, 0] * e),
+         "parts": lambda x, e: x.imag.__imul__(e)}
+
+
+def _gammas():
+    g = np.zeros((4, 4, 4), complex)
+    for mu, (cols, vals) in enumerate([((3, 2, 1, 0), (1j, 1j, -1j, -1j)), ((3, 2, 1, 0), (-1, 1, 1, -1)),
+                                       ((2, 3, 0, 1), (1j, -1j, -1j, 1j)), ((2, 3, 0, 1), (1, 1, 1, 1))]):
+        g[mu, range(4), cols] = vals
+    return g
+
+
+def _sizes(dims, U, X, Y):
+    """Sums of the moduli of the terms of each real or complex result: of
+    calD X, of the hopping-term force of X and Y."""
+    g, grid = np.abs(_gammas()), dims[::-1]
+    sh = lambda a, mu, s: np.roll(a.reshape(*grid, *a.shape[1:]), -s, axis=3 - mu).reshape(a.shape)  # noqa: E731
+    m = lambda a: np.abs(a.real) + np.abs(a.imag)  # noqa: E731
+    out, force = 0, np.zeros((len(X), 4, 8))
+    lam = np.abs(H.gell_mann())
+    for mu in range(4):
+        u, P = m(U[:, mu]), np.eye(4) + g[mu]
+        out = out + np.einsum("st,nab,ntb->nsa", P, u, sh(m(X), mu, 1))
+        out = out + sh(np.einsum("st,nba,ntb->nsa", P, u, m(X)), mu, -1)
+        uX, uY = (np.einsum("st,nab,ntb->nsa", P, u, sh(m(a), mu, 1)) for a in (X, Y))
+        N = np.einsum("nsa,nsb->nab", uX, m(Y)) + np.einsum("nsa,nsb->nab", uY, m(X))
+        force[:, mu] = np.einsum("iab,nba->ni", lam, N + N.transpose(0, 2, 1))
+    return out, force
+
+
+# A result against the sum of the moduli of its terms: 1e-14 of it, some 100
+# roundings, or the 2^-55 of the scale to which the fixed point knows results that
+# are above 2^-7 of it (7e-15).
+@pytest.mark.parametrize("eps", [1e-3, 1e-9, 1e-30])
+@pytest.mark.parametrize("kind", sorted(SMALL))
+@pytest.mark.parametrize("sigma", [0.0, 0.4])
+def test_wilson_of_uneven_spinors(kind, sigma, eps):
+    lat = lqcd.Lattice.symanzik(DIMS, 6.0, 0.87, "f64")
+    U = _third64(O.links_from_omega(synth.momenta(DIMS, 3) * sigma).reshape(lat.V, 4, 3, 3))
+    X, Y = (s[..., 0] + 1j * s[..., 1] for s in (synth.spinor(DIMS, 11), synth.spinor(DIMS, 12)))
+    for s in (X, Y):
+        SMALL[kind](s, eps)
+    links, x, y = _links(lat, U), lqcd.spinor_to_device(lat, X), lqcd.spinor_to_device(lat, Y)
+    size, fsize = _sizes(DIMS, U, X, Y)
+    got = lqcd.spinor_from_device(lqcd.wilson_dslash(lat, links, x, 0.0, 0.7))
+    assert (np.abs(got - 0.7 * O.wilson_hopping(DIMS, U, X)) <= 1e-14 * size).all()
+    f = lqcd.algebra_from_device(lqcd.wilson_hopping_force(lat, links, x, y, coef=0.7))
+    assert (np.abs(f - O.wilson_hopping_force(DIMS, U, X, Y, 0.7)) <= 1e-14 * fsize).all()
