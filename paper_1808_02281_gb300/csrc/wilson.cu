@@ -540,7 +540,7 @@ constexpr int kZeroScale = 64;
 
 // Rows 0 and 1 of (1 + s gamma_mu) x_n, mu at run time, over 2^(e - 1022) with
 // e the largest exponent field of the spinor's 24 reals; false where that is out
-// of range (the scales of two spinors are multiplied) or not finite.
+// of range or not finite.
 __device__ __forceinline__ bool fx_half(const double *__restrict__ x, int64_t V, int64_t n, int mu, bool minus, FHalf &h,
                                         int &e)
 {
@@ -561,7 +561,7 @@ __device__ __forceinline__ bool fx_half(const double *__restrict__ x, int64_t V,
     e = 0;
 #pragma unroll
     for (int q = 0; q < 12; ++q) e = max(e, max(exponent_of(v[q].x), exponent_of(v[q].y)));
-    if (e <= kZeroScale || e > 1900) {
+    if (e <= kZeroScale || e > 2040) { // results up to 2^6 of the scale
         if (e != 0) return false;
         bool zero = true; // and no subnormals
 #pragma unroll
@@ -701,8 +701,11 @@ __device__ __forceinline__ bool hopping_force_fx(const WilsonArgs &a, int64_t V,
 #pragma unroll
             for (int j = 0; j < 3; ++j) fx_total<-1>(y, 0, j, re[i][j], im[i][j]);
         }
-        // Im tr(lambda_a N) times coef and the scales 2^(e - 1022)
-        const double s = a.coef * 0x1p-56 * __hiloint2double((ep + 1) << 20, 0), w = __hiloint2double((eq + 1) << 20, 0);
+        // Im tr(lambda_a N) times coef, and one power of two for all scales
+        const bool zero = ep <= kZeroScale || eq <= kZeroScale;
+        const int power = ep + eq - 2044 - 56;
+        if (!zero && (power < -1022 || power > 900)) return false;
+        const double s = a.coef, w = zero ? 0.0 : __hiloint2double((power + 1023) << 20, 0);
         f[0] = fma(s * (double)(im[0][1] + im[1][0]), w, f[0]);
         f[1] = fma(s * (double)(re[0][1] - re[1][0]), w, f[1]);
         f[2] = fma(s * (double)(im[0][0] - im[1][1]), w, f[2]);
@@ -927,14 +930,19 @@ __device__ __forceinline__ bool dslash_site_fx(const WilsonArgs &a, const Sites<
         }
     }
     if (small()) return false;
+    // 2^-56 of 2^(scale - 1022) by the exponent field, so that cb meets a
+    // number of the result's own size
+    const auto value = [&](long long v) {
+        const double d = (double)v;
+        return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (scale - 1022 - 56) * (1 << 20), __double2loint(d));
+    };
     Spinor<double> acc;
-    const double s = 0x1p-56 * __hiloint2double((scale + 1) << 20, 0); // 2^-56 of 2^(scale - 1022)
 #pragma unroll
     for (int q = 0; q < 12; ++q) {
-        acc.re[q / 3][q % 3] = (double)sr[q];
-        acc.im[q / 3][q % 3] = (double)si[q];
+        acc.re[q / 3][q % 3] = value(sr[q]);
+        acc.im[q / 3][q % 3] = value(si[q]);
     }
-    store_dslash(a, x, V, (int64_t)n, acc, a.ca, a.cb * s);
+    store_dslash(a, x, V, (int64_t)n, acc, a.ca, a.cb);
     return true;
 }
 

@@ -219,3 +219,20 @@ def test_wilson_of_uneven_spinors(kind, sigma, eps):
     assert (np.abs(got - 0.7 * O.wilson_hopping(DIMS, U, X)) <= 1e-14 * size).all()
     f = lqcd.algebra_from_device(lqcd.wilson_hopping_force(lat, links, x, y, coef=0.7))
     assert (np.abs(f - O.wilson_hopping_force(DIMS, U, X, Y, 0.7)) <= 1e-14 * fsize).all()
+
+
+# Scaling a spinor by a power of two scales its results by it, to the bit, as
+# long as they are normal numbers: 2^-955 is next to the smallest scale of the
+# fixed point, and the coefficients are small.
+@pytest.mark.parametrize("px, py", [(-955, 955), (940, -900), (-300, -300), (-955, 100), (870, 40)])
+@pytest.mark.parametrize("coef", [0.7, 0.7 * 2.0 ** -20])
+def test_wilson_scales_with_the_spinors(coef, px, py):
+    lat = lqcd.Lattice.symanzik(DIMS, 6.0, 0.87, "f64")
+    U = O.links_from_omega(synth.momenta(DIMS, 3) * 0.4).reshape(lat.V, 4, 3, 3)
+    links = _links(lat, U)
+    x, y = (lqcd.spinor_to_device(lat, synth.spinor(DIMS, s)) for s in (11, 12))
+    sx, sy = x * 2.0 ** px, y * 2.0 ** py
+    want = lqcd.wilson_dslash(lat, links, x, 0.0, coef)
+    assert torch.equal(lqcd.wilson_dslash(lat, links, sx, 0.0, coef), want * 2.0 ** px)
+    want = lqcd.wilson_hopping_force(lat, links, x, y, coef=coef)
+    assert torch.equal(lqcd.wilson_hopping_force(lat, links, sx, sy, coef=coef), want * 2.0 ** (px + py))
