@@ -118,10 +118,10 @@ LQCD_API int lqcd_links_from_omega(const lqcd_desc *desc, const void *omega, voi
 /* Gauge force of the Symanzik action for every link (Eq. 18_7_25_2 and the
  * force algorithm of Sec. II): f^a = -dS/domega^a.  links: link layout
  * (device, read); force: algebra layout (device, written).  workspace: device
- * scratch, 256-byte aligned, of lqcd_workspace_bytes(desc) bytes for
- * LQCD_FORCE_STAPLE_FIELDS (LQCD_ERR_WORKSPACE if missing or short); the
- * other algorithms ignore it, and LQCD_FORCE_AUTO uses the staple-field
- * algorithm only when the workspace is large enough. */
+ * scratch, 256-byte aligned, of lqcd_workspace_bytes(desc) bytes (or the least
+ * that it names) for LQCD_FORCE_STAPLE_FIELDS (LQCD_ERR_WORKSPACE if missing or
+ * shorter); the other algorithms ignore it, and LQCD_FORCE_AUTO uses the
+ * staple-field algorithm only when the workspace is large enough. */
 LQCD_API int lqcd_gauge_force(const lqcd_desc *desc, const void *links, void *force, void *workspace,
                      size_t workspace_bytes, void *stream);
 
@@ -177,8 +177,8 @@ LQCD_API int lqcd_autotune_force(const lqcd_desc *desc, const void *links, void 
  * lqcd_md_force_step_batched uses the staple-field algorithm (force_algo
  * AUTO or STAPLE_FIELDS, else LQCD_ERR_UNSUPPORTED) with a workspace of
  * lqcd_workspace_bytes_batched bytes (the single-lattice workspaces back to
- * back); every lattice gets exactly the result of its own
- * lqcd_md_force_step, bit for bit.  lqcd_md_update_links_batched is the link
+ * back; or of the least ones); every lattice gets exactly the result of its
+ * own lqcd_md_force_step in such a workspace, bit for bit.  lqcd_md_update_links_batched is the link
  * step U <- exp(i dt p.T) U of every lattice. */
 #define LQCD_MAX_BATCH 64
 typedef struct lqcd_lattice_ref {
@@ -361,12 +361,20 @@ LQCD_API int lqcd_measure_fma_rate(int precision, void *scratch, size_t scratch_
 LQCD_API size_t lqcd_fma_rate_scratch_bytes(void);
 
 /* Bytes of device workspace that this descriptor needs on the current
- * device: the staple planes and action partials of the staple-field force
- * (force_algo STAPLE_FIELDS or AUTO; 24 SU(3) planes per site -- 1728 bytes
- * in FP32, 3456 in FP64, room for either storage form, with V rounded up to
- * a multiple of 32 -- plus one double per 32 sites) and the partial sums of
- * lqcd_gauge_action / lqcd_kinetic_energy (0 on a bad descriptor).  The
- * staple-field algorithm indexes sites with 32-bit integers: for V >= 2^31
+ * device: the planes and action partials of the staple-field force
+ * (force_algo STAPLE_FIELDS or AUTO) and the partial sums of
+ * lqcd_gauge_action / lqcd_kinetic_energy (0 on a bad descriptor).  With V
+ * rounded up to a multiple of 32, FP32 takes 24 SU(3) planes (1728 bytes a
+ * site, room for either storage form), FP64 28 (4032 bytes: the links in fixed
+ * point beside the staples) and a flag, and the partials are one double per 32
+ * sites, four on lattices of up to 4096 sites.
+ * The least that the algorithm runs in is 24 planes (FP64: 3456 bytes a site)
+ * and one double per 32 sites: FP64 then computes in floating point (at
+ * 24^3x48 in 34 ms instead of 5.4) and no lattice is split over more warps; the
+ * results agree to rounding.  This least size is what the function returns for
+ * an FP64 lattice that would take more than 240 GB.  Both hold for
+ * lqcd_workspace_bytes_batched too.
+ * The staple-field algorithm indexes sites with 32-bit integers: for V >= 2^31
  * it returns LQCD_ERR_DIMS (AUTO then takes the factored algorithm). */
 LQCD_API size_t lqcd_workspace_bytes(const lqcd_desc *desc);
 

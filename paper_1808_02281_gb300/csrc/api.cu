@@ -96,11 +96,16 @@ int reduction_setup(const lqcd_desc *desc, void *workspace, size_t workspace_byt
 size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Workspace of the staple-field force: staple planes, then action partials.
-size_t staple_workspace_bytes(const lqcd_desc *d)
+// lean: the least that it runs in (see lqcd_workspace_bytes).
+size_t staple_workspace_bytes(const lqcd_desc *d, bool lean)
 {
-    return lqcd::staple_field_bytes(d->dims, d->precision) +
-           round256((size_t)lqcd::staple_force_partials(d->dims) * sizeof(double));
+    return lqcd::staple_field_bytes(d->dims, d->precision, lean) +
+           round256((size_t)lqcd::staple_force_partials(d->dims, lean) * sizeof(double));
 }
+
+// A workspace above this is recommended lean: with the links and momenta of
+// its lattices the other form would not fit the device's 284 GB.
+constexpr size_t kLeanAbove = (size_t)240 * 1000 * 1000 * 1000;
 
 bool workspace_fits(const void *ws, size_t have, size_t need)
 {
@@ -115,7 +120,8 @@ int run_force(const lqcd_desc *desc, const void *links, void *force, void *mom, 
     int algo = desc->force_algo;
     const bool sf_dims = lqcd::staple_fields_supported(desc->dims);
     if (algo == LQCD_FORCE_STAPLE_FIELDS && !sf_dims) return LQCD_ERR_DIMS;
-    const bool sf_ok = sf_dims && workspace_fits(workspace, workspace_bytes, staple_workspace_bytes(desc));
+    const bool lean = !workspace_fits(workspace, workspace_bytes, staple_workspace_bytes(desc, false));
+    const bool sf_ok = sf_dims && (!lean || workspace_fits(workspace, workspace_bytes, staple_workspace_bytes(desc, true)));
     if (algo == LQCD_FORCE_STAPLE_FIELDS && !sf_ok) return LQCD_ERR_WORKSPACE;
     if (algo == LQCD_FORCE_AUTO) algo = sf_ok ? LQCD_FORCE_STAPLE_FIELDS : LQCD_FORCE_FACTORED;
     int red_blocks = 0;
@@ -139,7 +145,8 @@ int run_force(const lqcd_desc *desc, const void *links, void *force, void *mom, 
     if (algo == LQCD_FORCE_STAPLE_FIELDS) {
         char *ws = static_cast<char *>(workspace);
         a.staples = ws;
-        a.partials = reinterpret_cast<double *>(ws + lqcd::staple_field_bytes(desc->dims, desc->precision));
+        a.lean = lean;
+        a.partials = reinterpret_cast<double *>(ws + lqcd::staple_field_bytes(desc->dims, desc->precision, lean));
         a.action = action;
         return cuda_status(lqcd::launch_force_staple_fields(a, as_stream(stream)));
     }
@@ -252,13 +259,13 @@ int check_batch(const lqcd_desc *desc, int n, const lqcd_lattice_ref *lats)
     return LQCD_OK;
 }
 
-size_t batch_workspace_bytes(const lqcd_desc *desc, int n, const lqcd_lattice_ref *lats)
+size_t batch_workspace_bytes(const lqcd_desc *desc, int n, const lqcd_lattice_ref *lats, bool lean)
 {
     size_t total = 0;
     for (int c = 0; c < n; ++c) {
         lqcd_desc d = *desc;
         for (int i = 0; i < 4; ++i) d.dims[i] = lats[c].dims[i];
-        total += staple_workspace_bytes(&d);
+        total += staple_workspace_bytes(&d, lean);
     }
     return total + lqcd::kBatchCounterBytes;
 }
@@ -269,7 +276,8 @@ size_t lqcd_workspace_bytes_batched(const lqcd_desc *desc, int n, const lqcd_lat
 {
     LQCD_TRACE();
     if (check_batch(desc, n, lats) != LQCD_OK) return 0;
-    return batch_workspace_bytes(desc, n, lats);
+    const size_t need = batch_workspace_bytes(desc, n, lats, false);
+    return need <= kLeanAbove ? need : batch_workspace_bytes(desc, n, lats, true);
 }
 
 int lqcd_md_force_step_batched(const lqcd_desc *desc, int n, const lqcd_lattice_ref *lats,
@@ -286,7 +294,8 @@ int lqcd_md_force_step_batched(const lqcd_desc *desc, int n, const lqcd_lattice_
             return LQCD_ERR_ARG;
         if (!lqcd::staple_fields_supported(lats[c].dims)) return LQCD_ERR_DIMS;
     }
-    if (!workspace_fits(workspace, workspace_bytes, batch_workspace_bytes(desc, n, lats)))
+    const bool lean = !workspace_fits(workspace, workspace_bytes, batch_workspace_bytes(desc, n, lats, false));
+    if (lean && !workspace_fits(workspace, workspace_bytes, batch_workspace_bytes(desc, n, lats, true)))
         return LQCD_ERR_WORKSPACE;
     lqcd::SfLattice items[LQCD_MAX_BATCH];
     char *ws = static_cast<char *>(workspace);
@@ -298,14 +307,15 @@ int lqcd_md_force_step_batched(const lqcd_desc *desc, int n, const lqcd_lattice_
         L.force = lats[c].force;
         L.mom = lats[c].mom;
         L.action = lats[c].action;
-        const size_t sf = lqcd::staple_field_bytes(L.dims, desc->precision);
+        const size_t sf = lqcd::staple_field_bytes(L.dims, desc->precision, lean);
         L.staples = ws;
         L.partials = reinterpret_cast<double *>(ws + sf);
         lqcd_desc d = *desc;
         for (int i = 0; i < 4; ++i) d.dims[i] = lats[c].dims[i];
-        ws += staple_workspace_bytes(&d);
+        ws += staple_workspace_bytes(&d, lean);
     }
     lqcd::ForceArgs a{};
+    a.lean = lean;
     a.precision = desc->precision;
     a.beta = desc->beta;
     a.c_plaq = desc->c_plaq;
@@ -380,7 +390,7 @@ int lqcd_autotune_force(const lqcd_desc *desc, const void *links, void *force, v
         return LQCD_OK;
     }
     if (!lqcd::staple_fields_supported(desc->dims)) return LQCD_ERR_DIMS;
-    if (!workspace_fits(workspace, workspace_bytes, staple_workspace_bytes(desc)))
+    if (!workspace_fits(workspace, workspace_bytes, staple_workspace_bytes(desc, true)))
         return LQCD_ERR_WORKSPACE;
     lqcd_desc d = *desc;
     d.force_algo = LQCD_FORCE_STAPLE_FIELDS;
@@ -701,7 +711,8 @@ size_t lqcd_workspace_bytes(const lqcd_desc *desc)
     if (b <= 0) return 0;
     size_t need = round256((size_t)b * sizeof(double));
     if (desc->force_algo == LQCD_FORCE_AUTO || desc->force_algo == LQCD_FORCE_STAPLE_FIELDS) {
-        const size_t sf = staple_workspace_bytes(desc);
+        size_t sf = staple_workspace_bytes(desc, false);
+        if (sf > kLeanAbove) sf = staple_workspace_bytes(desc, true);
         if (sf > need) need = sf;
     }
     return need;

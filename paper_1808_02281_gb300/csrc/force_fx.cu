@@ -87,7 +87,7 @@ FxScalars make_fx_scalars(const KernelScalars &sc)
 // ------------------------------------------------------------------ links
 
 // Whether the lattice is computed in floating point.
-__device__ __forceinline__ bool floating(const SfLattice &L) { return *L.flag & L.bit; }
+__device__ __forceinline__ bool floating(const SfLattice &L) { return L.flag == nullptr || (*L.flag & L.bit); }
 
 __device__ __forceinline__ void links_block(const SfLattice &L, int V, int vb)
 {
@@ -646,11 +646,14 @@ cudaError_t launch_fx_passes(const SfLattice &L, const KernelScalars &sc, bool a
 {
     const unsigned grid = grid_of(virtual_blocks((int64_t)L.dims[0] * L.dims[1] * L.dims[2] * L.dims[3]));
     const FxScalars fx = make_fx_scalars(sc);
-    cudaError_t e = cudaMemsetAsync(L.flag, 0, sizeof *L.flag, st);
-    if (e != cudaSuccess) return e;
-    links_fx<<<grid, kBlock, 0, st>>>(L);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (L.flag != nullptr) { // not in a lean workspace
+        e = cudaMemsetAsync(L.flag, 0, sizeof *L.flag, st);
+        if (e != cudaSuccess) return e;
+        links_fx<<<grid, kBlock, 0, st>>>(L);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     staples_fx<<<L.split ? 6 * grid : grid, kBlock, 0, st>>>(L);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -669,9 +672,12 @@ cudaError_t launch_fx_passes(const SfLattice &L, const KernelScalars &sc, bool a
 cudaError_t launch_fx_passes_batched(const SfBatch &B, const KernelScalars &sc, bool action, cudaStream_t st)
 {
     const FxScalars fx = make_fx_scalars(sc);
-    links_fx_batched<<<persistent_grid(links_fx_batched, 0, B.total), kBlock, 0, st>>>(B);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (B.e[0].flag != nullptr) { // not in a lean workspace
+        links_fx_batched<<<persistent_grid(links_fx_batched, 0, B.total), kBlock, 0, st>>>(B);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     staples_fx_batched<<<persistent_grid(staples_fx_batched, 1, B.total), kBlock, 0, st>>>(B);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -555,11 +555,11 @@ cudaError_t launch_passes_batched(const SfBatch &B, const KernelScalars &sc, int
 // sites) of the two storage forms, so that every schedule fits the same
 // workspace.  FP64: the 24 planes, the 4 planes of the links in limbs, and the
 // flag.
-size_t staple_field_bytes(const int dims[4], int precision)
+size_t staple_field_bytes(const int dims[4], int precision, bool lean)
 {
     const int64_t V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
-    const size_t planes = precision == LQCD_F64 ? fx_planes_count() : kStaplePlanes;
-    return round_up256(planes * full_plane_bytes(V, precision)) + (precision == LQCD_F64 ? 256 : 0);
+    const bool fixed = precision == LQCD_F64 && !lean;
+    return round_up256((fixed ? fx_planes_count() : kStaplePlanes) * full_plane_bytes(V, precision)) + (fixed ? 256 : 0);
 }
 
 bool staple_fields_supported(const int dims[4])
@@ -567,10 +567,10 @@ bool staple_fields_supported(const int dims[4])
     return (int64_t)dims[0] * dims[1] * dims[2] * dims[3] < ((int64_t)1 << 31);
 }
 
-int staple_force_partials(const int dims[4])
+int staple_force_partials(const int dims[4], bool lean)
 {
     const int64_t V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
-    return (int)virtual_blocks(V) * (split_lattice(V) ? 4 : 1);
+    return (int)virtual_blocks(V) * (split_lattice(V) && !lean ? 4 : 1);
 }
 
 cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
@@ -581,7 +581,7 @@ cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
     for (int i = 0; i < 4; ++i) L.dims[i] = a.dims[i];
     set_traversal(L, variant);
     L.plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
-    L.split = split_lattice(V) && (a.precision == LQCD_F64 || full_staples(variant));
+    L.split = split_lattice(V) && !a.lean && (a.precision == LQCD_F64 || full_staples(variant));
     L.links = a.links;
     L.staples = a.staples;
     L.force = a.force;
@@ -590,7 +590,7 @@ cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
     L.action = a.action;
     const KernelScalars sc = make_scalars(a);
     const bool action = a.action != nullptr;
-    if (a.precision == LQCD_F64) {
+    if (a.precision == LQCD_F64 && !a.lean) {
         L.flag = reinterpret_cast<unsigned long long *>(static_cast<char *>(a.staples) + fx_planes_count() * L.plane_bytes);
         L.bit = 1;
     }
@@ -615,9 +615,11 @@ cudaError_t launch_force_staple_fields_batched(const ForceArgs &a, int n, const 
         B.e[c] = items[c];
         set_traversal(B.e[c], variant);
         B.e[c].plane_bytes = (int64_t)full_plane_bytes(V, a.precision);
-        B.e[c].split = split_lattice(V) && (a.precision == LQCD_F64 || full_staples(variant));
-        B.e[c].flag = counter + 3;
-        B.e[c].bit = 1ull << c;
+        B.e[c].split = split_lattice(V) && !a.lean && (a.precision == LQCD_F64 || full_staples(variant));
+        if (!a.lean) {
+            B.e[c].flag = counter + 3;
+            B.e[c].bit = 1ull << c;
+        }
         B.e[c].vb_begin = B.total;
         B.total += virtual_blocks(V);
         any_action = any_action || B.e[c].action != nullptr;

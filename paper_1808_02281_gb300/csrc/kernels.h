@@ -58,6 +58,7 @@ struct ForceArgs {
     double *partials;  // staple-field algorithm with action: per-block partial sums
     double *action;    // staple-field algorithm: action written here when set
     int variant;       // staple-field force pass schedule; -1 = process-wide choice
+    bool lean;         // staple-field algorithm: the workspace is the lean one
 };
 
 // Unsigned division of n < 2^31 by an invariant d >= 1 (Granlund and
@@ -98,7 +99,7 @@ struct SfLattice {
     const void *links;
     void *staples;     // 24 staple planes (FP64: and 4 link planes; workspace)
     // FP64: `bit` of *flag is set by the first pass where the field wants
-    // floating point
+    // floating point; NULL: there is no such pass, always floating point
     unsigned long long *flag, bit;
     void *force;       // written when set
     void *mom;         // p += dt f when set
@@ -121,12 +122,13 @@ constexpr size_t kBatchCounterBytes = 256;
 
 cudaError_t launch_force(const ForceArgs &a, cudaStream_t st);
 
-// Staple-field algorithm (force_sf.cu): workspace bytes of the 24 staple
-// planes, number of per-block action partials, and the two-pass launch.
-size_t staple_field_bytes(const int dims[4], int precision);
+// Staple-field algorithm (force_sf.cu): workspace bytes of the staple planes,
+// number of per-block action partials, and the launch.  lean: 24 planes and one
+// partial per virtual block (no lattice is split; FP64 in floating point).
+size_t staple_field_bytes(const int dims[4], int precision, bool lean);
 // The staple-field kernels index sites with 32-bit integers: V < 2^31.
 bool staple_fields_supported(const int dims[4]);
-int staple_force_partials(const int dims[4]);
+int staple_force_partials(const int dims[4], bool lean);
 cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st);
 // a: precision, coefficients, dt, variant; items: the lattices (their dims,
 // links, staples, force, mom, partials, action), 1 <= n <= kMaxBatch.
