@@ -1,8 +1,9 @@
 // Box-Muller normals for FP32 fields from 53-bit uniforms without the FP64
 // pipe: log, square root and cosine in pairs of FP32 numbers (a rounded value
-// and its remainder), to about 2^-31 of the result, then rounded to FP32.
-// log and cos in FP64 are some 80 operations on a pipe that issues 2 a clock
-// and SM; these are about 170 instructions on the others.
+// and its remainder).  The remainder tells whether the FP64 evaluation rounds to
+// the same FP32 number; where it may not (one normal in 2900) that is done.  log
+// and cos in FP64 are some 80 operations on a pipe that issues 2 a clock and SM;
+// these are about 190 instructions on the others.
 //
 // log: 53-bit u = 2^-k m, m in [0.70, 1.42), 1/m looked up to 8 bits (exactly 1
 // next to m = 1, so that log u keeps its relative accuracy there), r = m/c - 1
@@ -63,6 +64,16 @@ struct NormalTables {
     }
 };
 
+// a b rounded, where a compiler may not make an FMA of the product and a sum.
+__host__ __device__ inline float product(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+
 // a + b = s + e exactly.
 __host__ __device__ inline void two_sum(float a, float b, float &s, float &e)
 {
@@ -71,8 +82,9 @@ __host__ __device__ inline void two_sum(float a, float b, float &s, float &e)
     e += (a - (s - t)) + (b - t);
 }
 
-// sqrt(-2 log((w1 + 1) 2^-53)) cos(2 pi w2 2^-53) for 53-bit w1, w2.
-__host__ __device__ inline float normal_of(uint64_t w1, uint64_t w2, const NormalTables &tab)
+// sqrt(-2 log((w1 + 1) 2^-53)) cos(2 pi w2 2^-53) for 53-bit w1, w2: the FP32
+// number, its remainder t, and the square root.
+__host__ __device__ inline float normal_of(uint64_t w1, uint64_t w2, const NormalTables &tab, float &t, float &root)
 {
     // -log u
     const uint64_t W = w1 + 1;
@@ -88,31 +100,32 @@ __host__ __device__ inline float normal_of(uint64_t w1, uint64_t w2, const Norma
     const float mh = half * 0x1p-23f * (float)(int)(M >> 40);
     const float ml = half * 0x1p-55f * (float)(uint32_t)(M >> 8);
     const float inv = tab.log[i][0];
-    const float p = mh * inv;
-    const float rh = p - 1.f, rl = fmaf(mh, inv, -p) + ml * inv;
-    const float q = rh * rh, qe = fmaf(rh, rh, -q);
+    const float p = product(mh, inv);
+    float rh = p - 1.f, rl = fmaf(mh, inv, -p) + ml * inv;
+    const int64_t D = (int64_t)((1ull << 53) - W); // u = 1 - D 2^-53
+    if (D < (1ll << 45)) { // next to 1 (k = 0, inv = 1): r = -D 2^-53 exactly
+        const float h = (float)D;
+        rh = -0x1p-53f * h;
+        rl = -0x1p-53f * (float)(D - (int64_t)h);
+    }
+    const float q = product(rh, rh), qe = fmaf(rh, rh, -q);
     float lo = 0.f, s;
     two_sum(k * 0x1.62e4p-1f, tab.log[i][1], s, lo); // log 2 to 16 bits: exact times k
     two_sum(s, -rh, s, lo);
     two_sum(s, 0.5f * q, s, lo);
     const float cub = rh * q * fmaf(rh, fmaf(rh, fmaf(rh, -1.f / 6.f, 0.2f), -0.25f), 1.f / 3.f);
-    lo += fmaf(k, 0x1.7f7d1cp-20f, tab.log[i][2]) - (cub + (fmaf(-rh, rl, rl) - 0.5f * qe));
-    float Lh = s + lo, Ll = (s - Lh) + lo;
-    const int64_t D = (int64_t)((1ull << 53) - W); // u = 1 - D 2^-53
-    if (D < (1ll << 36)) { // -log u = d + d^2 / 2 + d^3 / 3 below 2^-17
-        const float h = (float)D, d = 0x1p-53f * h;
-        Ll = fmaf(d * d, fmaf(d, 1.f / 3.f, 0.5f), 0x1p-53f * (float)(D - (int64_t)h));
-        Lh = d;
-    }
+    lo += fmaf(k, 0x1.7f7d1cp-20f, tab.log[i][2]) - (cub + (fmaf(rl, q - rh, rl) - 0.5f * qe));
+    const float Lh = s + lo, Ll = (s - Lh) + lo;
     // sqrt(2 L)
     const float x = 2.f * Lh;
+    t = root = 0.f;
     if (!(x > 0.f)) return 0.f; // u = 1
 #ifdef __CUDA_ARCH__
     const float is = rsqrtf(x);
 #else
     const float is = 1.f / sqrtf(x);
 #endif
-    const float sh = x * is, sl = 0.5f * is * fmaf(2.f, Ll, fmaf(-sh, sh, x));
+    const float sh = product(x, is), sl = 0.5f * is * fmaf(2.f, Ll, fmaf(-sh, sh, x));
     // cos(2 pi v): quadrant j, |f| <= 2^50
     const int j = (int)((w2 + (1ull << 50)) >> 51);
     const int64_t f = (int64_t)w2 - ((int64_t)j << 51);
@@ -121,27 +134,54 @@ __host__ __device__ inline float normal_of(uint64_t w1, uint64_t w2, const Norma
     const int gh = (int)((g + (1ll << 21)) >> 22);
     const float fh = (float)gh, fl = (float)(int)(g - ((int64_t)gh << 22));
     constexpr float c1 = 0x1.921fb6p-29f, c2 = -0x1.777a5cp-54f; // 2 pi 2^-31 as a pair
-    const float dh = fh * c1;
+    const float dh = product(fh, c1);
     const float dl = fmaf(fh, c1, -dh) + fmaf(fh, c2, fl * 0x1.921fb6p-51f);
-    const float z = dh * dh;
-    const float sl1 = fmaf(dh * z, fmaf(z, 1.f / 120.f, -1.f / 6.f), dl); // sin d = dh + sl1
-    const float vc = z * fmaf(z, -1.f / 24.f, 0.5f) + dh * dl;            // 1 - cos d
+    const float z = product(dh, dh);
+    const float ze = fmaf(dh, dh, -z), d3 = product(dh, z); // d^2 = z + ze, d^3 = d3 + d3e (with dl)
+    const float d3e = fmaf(dh, z, -d3) + fmaf(dh, ze, 3.f * z * dl);
+    constexpr float sixth = 1.f / 6.f, sixth_rest = (float)(1.0 / 6.0 - (double)sixth);
+    const float s3 = product(d3, sixth), s3e = fmaf(d3, sixth, -s3) + fmaf(d3, sixth_rest, d3e * sixth);
+    const float sl1 = (dl - s3) + fmaf(d3 * z, 1.f / 120.f, -s3e); // sin d = dh + sl1
+    const float vh = 0.5f * z; // 1 - cos d as a pair
+    const float vl = fmaf(dh, dl, fmaf(z * z, fmaf(z, 1.f / 720.f, -1.f / 24.f), 0.5f * ze));
     const int b = a < 0 ? -a : a;
     const float ch = tab.trig[b][0], cl = tab.trig[b][1];
     const float nh = a < 0 ? -tab.trig[b][2] : tab.trig[b][2], nl = a < 0 ? -tab.trig[b][3] : tab.trig[b][3];
     // cosine (j even): C - S sin d - C (1 - cos d); sine (odd): S + C sin d - S (1 - cos d)
     const bool odd = j & 1;
     const float bh = odd ? nh : ch, bl = odd ? nl : cl, oh = odd ? ch : -nh, ol = odd ? cl : -nl;
-    const float ph = oh * dh;
+    const float ph = product(oh, dh);
     const float pe = fmaf(oh, dh, -ph) + fmaf(oh, sl1, ol * dh);
     float th, tl = 0.f;
     two_sum(bh, ph, th, tl);
-    tl += (bl + pe) - bh * vc;
+    const float qh = product(bh, vh);
+    two_sum(th, -qh, th, tl);
+    tl += (fmaf(-bl, vh, bl) + pe) - (fmaf(bh, vh, -qh) + bh * vl);
     // quadrants: cos, -sin, -cos, sin
-    const float r = sh * th;
+    const float r = product(sh, th);
     const float e = fmaf(sh, th, -r) + fmaf(sh, tl, sl * th);
     const float y = r + e;
-    return ((j + 1) & 2) ? -y : y;
+    const bool minus = (j + 1) & 2;
+    t = (r - y) + e;
+    if (minus) t = -t;
+    root = sh;
+    return minus ? -y : y;
+}
+__host__ __device__ inline float normal_of(uint64_t w1, uint64_t w2, const NormalTables &tab)
+{
+    float t, root;
+    return normal_of(w1, w2, tab, t, root);
+}
+
+// Whether y is what the FP64 evaluation rounds to: no midpoint of two FP32
+// numbers lies within the errors of the two.  The pairs are within 0.86 of d
+// here (1.4 x 10^9 normals against long double, next to the quadrants and to
+// u = 1 among them), FP64 within 2^-50 of the root (2 pi u2 is rounded before
+// the cosine).
+__host__ __device__ inline bool normal_is_rounded(float y, float t, float root)
+{
+    const float d = fmaf(0x1p-37f, fabsf(y), 0x1p-40f * root);
+    return root > 0.f && y + (t + d) == y && y + (t - d) == y;
 }
 
 } // namespace lqcd
