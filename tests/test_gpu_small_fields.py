@@ -236,3 +236,23 @@ def test_wilson_scales_with_the_spinors(coef, px, py):
     assert torch.equal(lqcd.wilson_dslash(lat, links, sx, 0.0, coef), want * 2.0 ** px)
     want = lqcd.wilson_hopping_force(lat, links, x, y, coef=coef)
     assert torch.equal(lqcd.wilson_hopping_force(lat, links, sx, sy, coef=coef), want * 2.0 ** (px + py))
+
+
+@pytest.mark.parametrize("algo", [lqcd.FORCE_STAPLE_FIELDS, lqcd.FORCE_PATHS])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_what_a_link_that_is_not_finite_reaches(value, algo):
+    """The links that may read it, found from the formulas; every other link
+    has the force that it had, to the bit."""
+    dims = (6, 5, 4, 6)
+    lat = lqcd.Lattice.symanzik(dims, 6.0, 0.87, "f64", force_algo=algo)
+    links = lqcd.links_from_omega(lat, lqcd.algebra_to_device(lat, synth.omega(dims, 0.3, 1)))
+    clean = lqcd.algebra_from_device(lqcd.gauge_force(lat, links))
+    U = lqcd.full_from_device(lqcd.unpack_links(lat, links))
+    links[1, 2, 77, 0] = value
+    U[77, 1] = np.nan
+    with np.errstate(invalid="ignore"):
+        reach = ~np.isfinite(staple_force(U, dims, 6.0, O.coefficients(0.87))).all(-1)
+    assert 40 < reach.sum() < reach.size // 2
+    f = lqcd.algebra_from_device(lqcd.gauge_force(lat, links))
+    assert np.isfinite(f[~reach]).all() and np.array_equal(f[~reach], clean[~reach])
+    assert not np.isfinite(f[reach]).all(-1).any()
