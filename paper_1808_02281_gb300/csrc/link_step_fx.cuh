@@ -118,17 +118,18 @@ __device__ __forceinline__ void fx_exp_coefficients(long long c0, long long c1, 
 // Below this exponent field nothing of an exponent shows in a link (2^-900).
 constexpr int kLeastExponent = 123;
 
-// Whether four or more components of x are below 2^-6 of the largest (exponent
-// field em): five links in a million of Gaussian momenta, and all of a field whose
-// momenta lie in a subgroup (diagonal links, an SU(2) or U(2) block, real
-// rotations), beside which the link step has to keep small ones to a precision
-// of their own.
+// Whether the components of x beside a subgroup are below 2^-6 of the largest
+// (exponent field em): the four that leave a U(2) block, or any five (of an
+// SU(2) block, of real rotations, of diagonal links).  The link step then has to
+// keep small ones to a precision of their own.  Of Gaussian momenta it is one
+// link in four million: a single one among the last blocks of a small lattice
+// costs 18 us.
 __device__ __forceinline__ bool fx_uneven(const double x[8], int em)
 {
-    int n = 0;
+    unsigned m = 0;
 #pragma unroll
-    for (int a = 0; a < 8; ++a) n += em - exponent_of(x[a]) > 6;
-    return n >= 4;
+    for (int a = 0; a < 8; ++a) m |= (em - exponent_of(x[a]) > 6 ? 1u : 0u) << a;
+    return __popc(m) >= 5 || (m & 0x78) == 0x78 || (m & 0x1b) == 0x1b || (m & 0x63) == 0x63;
 }
 
 // Row i of a b, units 2^-60.

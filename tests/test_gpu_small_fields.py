@@ -61,10 +61,11 @@ def _gram_schmidt(U):
 
 
 def _omega(kind, sigma, seed):
-    """Normal components of size sigma; kind "ab", "su2" or "so3": those of the
-    subgroup of size 0.5 (diagonal links, an SU(2) block, real rotations)."""
+    """Normal components of size sigma; with a kind, those of the subgroup of
+    size 0.5 (diagonal links, an SU(2) block, the three U(2) blocks, real rotations)."""
     o = synth.momenta(DIMS, seed) * sigma
-    for a in {"": (), "ab": (2, 7), "su2": (0, 1, 2), "so3": (1, 4, 6)}[kind]:
+    for a in {"": (), "ab": (2, 7), "su2": (0, 1, 2), "u2": (0, 1, 2, 7), "u2b": (2, 3, 4, 7), "u2c": (2, 5, 6, 7),
+              "so3": (1, 4, 6)}[kind]:
         o[..., a] = synth.momenta(DIMS, seed + 50)[..., a] * 0.5
     return o
 
@@ -103,7 +104,7 @@ def test_link_step_of_small_entries(kind, sigma, step):
     _check_classes(_rows(links), want, 4e-15)
 
 
-@pytest.mark.parametrize("kind", ["", "ab", "su2", "so3"])
+@pytest.mark.parametrize("kind", ["", "ab", "su2", "u2", "u2b", "u2c", "so3"])
 @pytest.mark.parametrize("sigma", [1.0, 0.05, 1e-3, 1e-8, 1e-16, 1e-30])
 def test_links_from_small_omega(kind, sigma):
     """Also exponents of a subgroup with small components beside it."""
