@@ -86,8 +86,16 @@ FxScalars make_fx_scalars(const KernelScalars &sc)
 
 // ------------------------------------------------------------------ links
 
-// Whether the lattice is computed in floating point.
-__device__ __forceinline__ bool floating(const SfLattice &L) { return L.flag == nullptr || (*L.flag & L.bit); }
+// Whether the lattice is computed in floating point; for whole warps.
+__device__ __forceinline__ bool floating(const SfLattice &L)
+{
+    if (L.flag == nullptr) return true;
+    if (L.near == nullptr) return *L.flag & L.bit;
+    const int n = (int)virtual_blocks(make_g32(L.dims).V);
+    int any = 0;
+    for (int i = (int)(threadIdx.x & 31); i < n; i += 32) any |= L.near[i];
+    return __any_sync(0xffffffffu, any);
+}
 
 __device__ __forceinline__ void links_block(const SfLattice &L, int V, int vb)
 {
@@ -97,8 +105,10 @@ __device__ __forceinline__ void links_block(const SfLattice &L, int V, int vb)
     const FxPlanes sf = fx_planes(L);
     if (x < V) sf.store(sf.at(x), kLinkPlane + mu, u);
     const int n = __popc(__ballot_sync(0xffffffffu, fx_poisoned(u) || fx_near_subgroup(u)));
-    if (__syncthreads_and(n >= 8) && threadIdx.x == 0 && !(*(volatile unsigned long long *)L.flag & L.bit))
-        atomicOr(L.flag, L.bit);
+    const int near = __syncthreads_and(n >= 8);
+    if (threadIdx.x > 0) return;
+    if (L.near != nullptr) L.near[vb] = near;
+    else if (near && !(*(volatile unsigned long long *)L.flag & L.bit)) atomicOr(L.flag, L.bit);
 }
 
 __global__ void __launch_bounds__(kBlock) links_fx(const __grid_constant__ SfLattice L)
@@ -165,8 +175,9 @@ __device__ __forceinline__ void staples_block(const SfLattice &L, const G32 &g, 
 {
     const int mu = (int)(threadIdx.x >> 5);
     const int x = vb * 32 + (int)(threadIdx.x & 31);
+    const bool fl = floating(L);
     if (x >= g.V) return;
-    if (floating(L)) return staples_floating(L, x, mu, j0, j1);
+    if (fl) return staples_floating(L, x, mu, j0, j1);
     const Coord c = coord32(g, L.div, x);
     const FxPlanes sf = fx_planes(L);
     const int xm = x + step32(g, c, mu, 1); // x + mu
@@ -514,10 +525,11 @@ __device__ __forceinline__ double fx_force_block(const SfLattice &L, const Kerne
     longlong2 *zs = reinterpret_cast<longlong2 *>(ahead_s + kAheadWords * kBlock) + threadIdx.x;
     const int rho = (int)(threadIdx.x >> 5);
     const int j = vb * 32 + (int)(threadIdx.x & 31);
+    const bool fl = floating(L);
     if (j >= g.V) return 0.0;
     const Coord c = swept_site(sw, j);
     const int k = index32(g, c);
-    if (floating(L)) return force_link_of_planes<ACTION>(L, sc, k, rho);
+    if (fl) return force_link_of_planes<ACTION>(L, sc, k, rho);
     const FxPlanes sf = fx_planes(L);
     bool bad = false;
     fx_fetch(slot, sf, fx_group_of(sf, g, c, rho, k, 0), rho, 0);
@@ -648,7 +660,7 @@ cudaError_t launch_fx_passes(const SfLattice &L, const KernelScalars &sc, bool a
     const FxScalars fx = make_fx_scalars(sc);
     cudaError_t e = cudaSuccess;
     if (L.flag != nullptr) { // not in a lean workspace
-        e = cudaMemsetAsync(L.flag, 0, sizeof *L.flag, st);
+        if (L.near == nullptr) e = cudaMemsetAsync(L.flag, 0, sizeof *L.flag, st);
         if (e != cudaSuccess) return e;
         links_fx<<<grid, kBlock, 0, st>>>(L);
         e = cudaGetLastError();

@@ -553,13 +553,14 @@ cudaError_t launch_passes_batched(const SfBatch &B, const KernelScalars &sc, int
 
 // FP32: room for the 24 planes in the larger (full, 18-real, in blocks of 32
 // sites) of the two storage forms, so that every schedule fits the same
-// workspace.  FP64: the 24 planes, the 4 planes of the links in limbs, and the
-// flag.
+// workspace.  FP64: the 24 planes, the 4 planes of the links in limbs, 256 bytes
+// for the flag, and the words of small lattices.
 size_t staple_field_bytes(const int dims[4], int precision, bool lean)
 {
     const int64_t V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
     const bool fixed = precision == LQCD_F64 && !lean;
-    return round_up256((fixed ? fx_planes_count() : kStaplePlanes) * full_plane_bytes(V, precision)) + (fixed ? 256 : 0);
+    return round_up256((fixed ? fx_planes_count() : kStaplePlanes) * full_plane_bytes(V, precision)) +
+           (fixed ? 256 + (near_words(V) ? round_up256(virtual_blocks(V) * sizeof(int)) : 0) : 0);
 }
 
 bool staple_fields_supported(const int dims[4])
@@ -593,6 +594,7 @@ cudaError_t launch_force_staple_fields(const ForceArgs &a, cudaStream_t st)
     if (a.precision == LQCD_F64 && !a.lean) {
         L.flag = reinterpret_cast<unsigned long long *>(static_cast<char *>(a.staples) + fx_planes_count() * L.plane_bytes);
         L.bit = 1;
+        if (near_words(V)) L.near = reinterpret_cast<int *>(L.flag + 32);
     }
     const cudaError_t e = a.precision == LQCD_F64 ? launch_fx_passes(L, sc, action, st)
                                                   : launch_passes(L, sc, variant, action, st);

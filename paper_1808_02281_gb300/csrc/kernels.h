@@ -98,9 +98,11 @@ struct SfLattice {
     int64_t plane_bytes; // full staple planes: bytes of one plane
     const void *links;
     void *staples;     // 24 staple planes (FP64: and 4 link planes; workspace)
-    // FP64: `bit` of *flag is set by the first pass where the field wants
-    // floating point; NULL: there is no such pass, always floating point
+    // FP64: where the field wants floating point the first pass sets its virtual
+    // block's word of `near`, or (NULL) `bit` of *flag; flag NULL: there is no
+    // such pass, always floating point
     unsigned long long *flag, bit;
+    int *near;
     void *force;       // written when set
     void *mom;         // p += dt f when set
     double *partials;  // one action partial per virtual block, or four
