@@ -200,11 +200,14 @@ LQCD_API int lqcd_md_update_links_batched(const lqcd_desc *desc, int n,
 
 /* Gauge action S_G = (beta/3) sum_n sum_{34 loops P} c_P [3 - Re tr P_n]
  * (Eq. 18_6_4_1).  links: link layout (device, read).  action: ONE double in
- * device memory (written, FP64 in both precisions: per-loop terms and all
- * sums are accumulated in double, in a fixed order, so the result is
- * bitwise reproducible).  workspace: device scratch of at least
- * lqcd_workspace_bytes(desc) bytes, 256-byte aligned, used for per-block
- * partial sums. */
+ * device memory (written, FP64 in both precisions).  All sums are taken in a
+ * fixed order, so the result is bitwise reproducible: FP32 adds the traces of a
+ * site's loops of one kind as a pair of FP32 numbers (to 2^-45; a trace is good
+ * to 2^-23), FP64 as whole numbers of 2^-56, and everything above a site in
+ * double.  workspace: device scratch of at least lqcd_workspace_bytes(desc)
+ * bytes, 256-byte aligned, for per-block partial sums; FP64 links that are
+ * converted once (576 bytes a site) take the rest of it where it has room, so
+ * no part of it survives the call. */
 LQCD_API int lqcd_gauge_action(const lqcd_desc *desc, const void *links, double *action, void *workspace,
                       size_t workspace_bytes, void *stream);
 
@@ -249,7 +252,10 @@ LQCD_API int lqcd_md_update_momenta(const lqcd_desc *desc, void *mom, const void
 /* Link step U <- exp(i dt sum_a p^a T_a) U for every link (the flow of the
  * left parametrisation of Eq. 18_1_29_3), then Gram-Schmidt of rows 0, 1
  * (row 2 is always rebuilt as conj(row0 x row1)).  links: link layout (read
- * and written); mom: algebra layout (read). */
+ * and written); mom: algebra layout (read).  FP64: the change of a link is
+ * known to 2^-57 of the largest component of dt p and added to the link as
+ * stored, so small entries keep their digits (components of dt p beside a
+ * subgroup that are below 2^-6 of the largest: in floating point). */
 LQCD_API int lqcd_md_update_links(const lqcd_desc *desc, void *links, const void *mom, double dt,
                          void *stream);
 
@@ -325,7 +331,12 @@ LQCD_API int lqcd_gaussian_momenta(const lqcd_desc *desc, uint64_t seed, void *m
  *   (calD x)_n = sum_mu (1 - gamma_mu) U_{n,mu} x_{n+mu}
  *              + (1 + gamma_mu) U_{n-mu,mu}^dagger x_{n-mu}  (periodic).
  * a = 1, b = -kappa gives Y = D X of Eq. 18_7_17_2 without the clover term.
- * x (read) and y (written) must not overlap; a, b finite. */
+ * x (read) and y (written) must not overlap; a, b finite.  FP64: a site is
+ * computed in fixed point, to about 2^-56 of the largest real of its eight
+ * neighbours, unless a complex result is below 2^-12 of that, or six real ones
+ * are below 2^-6 (a colour or spin row that the links do not mix with the
+ * others): then in floating point, where each result has a rounding of its own.
+ * lqcd_wilson_hopping_force likewise, for components of the force. */
 LQCD_API int lqcd_wilson_dslash(const lqcd_desc *desc, const void *links, const void *x, double a,
                                 double b, void *y, void *stream);
 

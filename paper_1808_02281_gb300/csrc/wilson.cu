@@ -262,8 +262,8 @@ constexpr int kDslashBlock = 128;
 // 32^3x64: 159 -> 133 us (5.1 -> 6.1 TB/s of 384 B a site), 32^4: 84 -> 69 us,
 // 24^3x48: 55 -> 51 us; below that the launch is what counts.
 // A ring of two hops and 4 blocks an SM (147 KB of shared memory, up to 128
-// registers): 133 us at 32^3x64; 3 blocks of three hops 131, but more shared
-// memory than a static allocation may have; 5 blocks of two hops at 96
+// registers): 133 us at 32^3x64; 3 blocks of three hops 131, if it were
+// dynamic shared memory (55 KB a block); 5 blocks of two hops at 96
 // registers 145, 4 of three hops 144; 64 or 256 threads a block the same; one
 // site a thread instead of as many blocks as are resident 139.
 constexpr int kRing = 2;
@@ -785,10 +785,9 @@ __global__ void __launch_bounds__(kForceBlock) wilson_hopping_force(const __grid
     }
 }
 
-// 4 blocks per SM (128 registers, 172 bytes spilled): 146 us at 20x18x14x30
-// against 149 with 3 and 158 with 5; in floating point 431.  What bounds it
-// now are three pipes alike: instruction issue, the integer half of the FMA
-// pipe and the ALUs would each take about 67 us.
+// 4 blocks per SM (128 registers, 236 bytes spilled): 149 us at 20x18x14x30; in
+// floating point 431.  What bounds it are three pipes alike: instruction issue,
+// the integer half of the FMA pipe and the ALUs would each take about 67 us.
 template <typename I>
 __global__ void __launch_bounds__(kForceBlock, 4) wilson_hopping_force_fx(const __grid_constant__ WilsonArgs a)
 {
@@ -946,7 +945,7 @@ __device__ __forceinline__ bool dslash_site_fx(const WilsonArgs &a, const Sites<
     return true;
 }
 
-// 32^4: 747 us, 20x18x14x30: 134; in floating point 2153 and 353 (what
+// 32^4: 752 us, 20x18x14x30: 136; in floating point 2153 and 353 (what
 // uneven_spinor finds 2221).  Error against extended precision 6.0e-17, in
 // floating point 9.0e-17.
 template <typename I>
