@@ -704,7 +704,7 @@ __device__ __forceinline__ bool hopping_force_fx(const WilsonArgs &a, int64_t V,
         // Im tr(lambda_a N) times coef, and one power of two for all scales
         const bool zero = ep <= kZeroScale || eq <= kZeroScale;
         const int power = ep + eq - 2044 - 56;
-        if (!zero && (power < -1022 || power > 900)) return false;
+        if (!zero && (power < -1022 || power > 900 || exponent_of(a.coef) > 1023 + 900)) return false;
         const double s = a.coef, w = zero ? 0.0 : __hiloint2double((power + 1023) << 20, 0);
         f[0] = fma(s * (double)(im[0][1] + im[1][0]), w, f[0]);
         f[1] = fma(s * (double)(re[0][1] - re[1][0]), w, f[1]);

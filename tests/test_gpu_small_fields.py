@@ -257,3 +257,13 @@ def test_what_a_link_that_is_not_finite_reaches(value, algo):
     f = lqcd.algebra_from_device(lqcd.gauge_force(lat, links))
     assert np.isfinite(f[~reach]).all() and np.array_equal(f[~reach], clean[~reach])
     assert not np.isfinite(f[reach]).all(-1).any()
+
+
+def test_hopping_force_of_a_large_coefficient():
+    """A coefficient of 2^990 and spinors that make up for it."""
+    lat = lqcd.Lattice.symanzik(DIMS, 6.0, 0.87, "f64")
+    links = _links(lat, O.links_from_omega(synth.momenta(DIMS, 3) * 0.4).reshape(lat.V, 4, 3, 3))
+    x, y = (lqcd.spinor_to_device(lat, synth.spinor(DIMS, s)) for s in (11, 12))
+    want = lqcd.wilson_hopping_force(lat, links, x, y, coef=0.7)
+    got = lqcd.wilson_hopping_force(lat, links, x * 2.0 ** -500, y * 2.0 ** -490, coef=0.7 * 2.0 ** 990)
+    assert (got - want).abs().max() <= 1e-14 * want.abs().max()
