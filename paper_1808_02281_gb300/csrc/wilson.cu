@@ -785,7 +785,7 @@ __global__ void __launch_bounds__(kForceBlock) wilson_hopping_force(const __grid
     }
 }
 
-// 4 blocks per SM (128 registers, 236 bytes spilled): 149 us at 20x18x14x30; in
+// 4 blocks per SM (128 registers, 236 bytes spilled): 151 us at 20x18x14x30; in
 // floating point 431.  What bounds it are three pipes alike: instruction issue,
 // the integer half of the FMA pipe and the ALUs would each take about 67 us.
 template <typename I>
